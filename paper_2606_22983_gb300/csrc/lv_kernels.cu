@@ -894,19 +894,42 @@ k_exchange_plan(DevPool p, const lv_victim* __restrict__ v, long long n_out, int
   }
 }
 
-// Unit u = (task t, sub-page j): the out half copies hbm_kv[j][page] to host[slot][j],
-// the in half host[slot'][j] to hbm_kv[j][page']; each thread loads both before it
-// stores either, so a paired task reads the old page before overwriting it.  CTAs take
-// units in order from a shared cursor (zeroed by the plan), the next one fetched while
-// the current one is copied: a CTA that starts late, or runs on an SM crowded by other
-// work, simply takes fewer units.
+// Unit u = (task t, chunk c): kUnitVecs 16-byte vectors of the task's page, taken as one
+// run of J * P bytes (which it is in the host slot; in HBM vector q of the page lies in
+// sub-page q / nvec).  The out half copies the HBM page to its host slot, the in half a
+// host slot to its HBM page; each thread loads both before it stores either, so a paired
+// task reads the old page before overwriting it.  CTAs take units in order from a shared
+// cursor (zeroed by the plan), the next one fetched while the current one is copied: a CTA
+// that starts late, or runs on an SM crowded by other work, simply takes fewer units.
+//
+// What bounds it: the host link, as long as enough bytes are on their way.  A CTA has one
+// unit in flight and 45 CTAs have to cover the link's latency, so a unit is 16 KiB each way
+// whatever the sub-page size.  With one sub-page per unit, pages of 4 KiB sub-pages kept a
+// quarter of that in flight: a turn that moves 45 pages of 192 KiB each way (1000 sessions)
+// took 140 us and takes 106 us; pages of 16 KiB sub-pages are as before (1.90 ms for 203
+// pages of 1.5 MiB each way, 336 GB/s).
+constexpr int kUnitVecs = kCopyThreads * kCopyUnroll;
+constexpr int kCopyKv = 512;      // sub-page arrays whose addresses a CTA keeps in shared memory
+
+__host__ __device__ __forceinline__ long long copy_chunks(const DevPool& p) {
+  return ((p.P >> 4) * p.J + kUnitVecs - 1) / kUnitVecs;
+}
+
 __global__ void __launch_bounds__(kCopyThreads)
 k_exchange_copy(DevPool p, const int4* __restrict__ tasks, const long long* __restrict__ n_tasks,
                 long long* __restrict__ cursor) {
-  pdl_entry();
-  const long long units = *n_tasks * p.J;
-  const int nvec = (int)(p.P >> 4);
+  __shared__ uint8_t* kv_s[kCopyKv];
   __shared__ long long next;
+  // the arrays' addresses never change: read before the plan is waited for
+  for (int j = threadIdx.x; j < p.J && j < kCopyKv; j += kCopyThreads) kv_s[j] = p.kv[j];
+  pdl_entry();
+  const uint32_t nvec = (uint32_t)(p.P >> 4);
+  const long long page_vecs = (long long)nvec * p.J;
+  const long long chunks = copy_chunks(p);
+  const long long units = *n_tasks * chunks;
+  // x / nvec for x < nvec + kUnitVecs: at most 1 for sub-pages of a unit or more, else the
+  // high half of x times ceil(2^32 / nvec) (exact: x < 2^11, nvec < 2^10)
+  const uint32_t inverse = 0xffffffffu / nvec + 1u;
   if (threadIdx.x == 0) next = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(cursor), 1ull);
   __syncthreads();
   for (long long u = next; u < units; u = next) {
@@ -914,30 +937,37 @@ k_exchange_copy(DevPool p, const int4* __restrict__ tasks, const long long* __re
     // warp does not wait for the atomic's result meanwhile
     unsigned long long fetched = 0;
     if (threadIdx.x == 0) fetched = atomicAdd(reinterpret_cast<unsigned long long*>(cursor), 1ull);
-    const int4 t = tasks[u / p.J];
-    const int j = (int)(u % p.J);
+    const long long ti = u / chunks;
+    const int4 t = tasks[ti];
+    const long long q0 = (u - ti * chunks) * kUnitVecs;       // the unit's first vector
+    const long long j0 = q0 / nvec;
+    const uint32_t r0 = (uint32_t)(q0 - j0 * nvec);
+    const int left = (int)(page_vecs - q0 < kUnitVecs ? page_vecs - q0 : kUnitVecs);
     const bool has_out = t.x >= 0, has_in = t.z >= 0;
-    const int4* so = has_out ? reinterpret_cast<const int4*>(p.kv[j] + (size_t)t.x * p.P) : nullptr;
-    int4* dout = has_out ? reinterpret_cast<int4*>(p.host + ((size_t)t.y * p.J + j) * p.P) : nullptr;
-    const int4* si = has_in ? reinterpret_cast<const int4*>(p.host + ((size_t)t.z * p.J + j) * p.P) : nullptr;
-    int4* din = has_in ? reinterpret_cast<int4*>(p.kv[j] + (size_t)t.w * p.P) : nullptr;
-    for (int base = threadIdx.x; base < nvec; base += kCopyThreads * kCopyUnroll) {
-      int4 ro[kCopyUnroll], ri[kCopyUnroll];
+    int4* dout = has_out ? reinterpret_cast<int4*>(p.host) + (size_t)t.y * page_vecs + q0 : nullptr;
+    const int4* si = has_in ? reinterpret_cast<const int4*>(p.host) + (size_t)t.z * page_vecs + q0 : nullptr;
+    int4 ro[kCopyUnroll], ri[kCopyUnroll];
+    int4* din[kCopyUnroll];
 #pragma unroll
-      for (int k = 0; k < kCopyUnroll; ++k) {
-        const int q = base + k * kCopyThreads;
-        if (q < nvec) {
-          if (has_in) ri[k] = si[q];
-          if (has_out) ro[k] = so[q];
-        }
+    for (int k = 0; k < kCopyUnroll; ++k) {
+      const int q = threadIdx.x + k * kCopyThreads;
+      if (q < left) {
+        if (has_in) ri[k] = si[q];
+        const uint32_t x = r0 + q;
+        const uint32_t dj = nvec >= kUnitVecs ? (uint32_t)(x >= nvec) : nvec == 1 ? x : __umulhi(x, inverse);
+        const long long j = j0 + dj;
+        uint8_t* base = j < kCopyKv ? kv_s[j] : p.kv[j];
+        const size_t at = (size_t)(x - dj * nvec);
+        din[k] = reinterpret_cast<int4*>(base + (size_t)t.w * p.P) + at;
+        if (has_out) ro[k] = *(reinterpret_cast<const int4*>(base + (size_t)t.x * p.P) + at);
       }
+    }
 #pragma unroll
-      for (int k = 0; k < kCopyUnroll; ++k) {
-        const int q = base + k * kCopyThreads;
-        if (q < nvec) {
-          if (has_out) dout[q] = ro[k];
-          if (has_in) din[q] = ri[k];
-        }
+    for (int k = 0; k < kCopyUnroll; ++k) {
+      const int q = threadIdx.x + k * kCopyThreads;
+      if (q < left) {
+        if (has_out) dout[q] = ro[k];
+        if (has_in) *din[k] = ri[k];
       }
     }
     __syncthreads();   // every thread holds u before `next` is replaced
@@ -2154,7 +2184,8 @@ cudaError_t launch_exchange(const DevPool& p, const lv_victim* v, int64_t n_out,
   }
   if (ev) cudaEventRecord(ev->start, cs);
   else if (off && off->started) cudaEventRecord(off->started, cs);
-  const unsigned grid = blocks_for(units, 1, copy_ctas);
+  // the 16-byte copy takes whole pages in chunks, the TMA copy sub-pages
+  const unsigned grid = blocks_for(p.xstages > 0 ? units : units / p.J * copy_chunks(p), 1, copy_ctas);
   if (p.xstages > 0) {
     const size_t smem = (size_t)p.xstages * 2 * p.P;
     if (off || ev) {
