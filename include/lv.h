@@ -227,10 +227,7 @@ typedef struct lv_stats {
    LV_REMAP_ENTRIES_PER_THREAD = 1, 2 or 4 (lv_remap's entries per thread,
    default 1 while the GPU holds one thread per entry at once, else 2 or 4);
    LV_EXCHANGE_KERNEL=tma (the exchange copy by TMA bulk copies, one issuing
-   thread per CTA, with LV_EXCHANGE_STAGES stages of 2P bytes, default 4);
-   LV_STEP_GRAPHS=0 (a device-driven step whose kernels all run on the caller's
-   stream is issued kernel by kernel instead of as one CUDA graph launch; the
-   results are the same). */
+   thread per CTA, with LV_EXCHANGE_STAGES stages of 2P bytes, default 4). */
 lv_status lv_pool_create(const lv_pool_desc* desc, lv_stream stream, lv_pool** out);
 
 /* Waits for the pool's outstanding work on `stream`, then frees everything the
@@ -448,8 +445,7 @@ lv_status lv_evict(lv_pool* pool, int64_t now_us, int64_t k, uint32_t flags, lv_
    or host memory, indexed by block id) sets the order in which the session's
    host-tier blocks are loaded -- ascending (key, block id) instead of
    ascending block id -- and so which of the lowest free HBM pages each block
-   takes; blocks_out then lists them in that order.  Ordering costs one warp
-   per host block, each comparing it with every other.  Host-detected:
+   takes; blocks_out then lists them in that order.  Host-detected:
    LV_ERR_INVALID.  Device-detected: as lv_make_resident, LV_ERR_BOUNDS for a
    candidate out of range. */
 typedef struct lv_turn_desc {

@@ -93,20 +93,6 @@ struct lv_pool {
   void* host_base = nullptr;       // host-visible address of the host pool
   std::vector<void*> dev_allocs;
   cudaMemPool_t mp = nullptr;      // stream-ordered staging memory
-  // device-driven steps whose kernels all run on the caller's stream go out as one
-  // CUDA graph launch: one instantiated graph per shape of the launch sequence, its
-  // kernel nodes' arguments replaced for every step
-  struct StepGraph {
-    std::vector<const void*> funcs;
-    std::vector<dim3> grids, blocks;
-    std::vector<size_t> smems;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    std::vector<cudaGraphNode_t> nodes;   // kernel nodes in launch order
-  };
-  std::vector<StepGraph> step_graphs;
-  bool step_graphs_on = true;
-  cudaStream_t s_capture = nullptr;
 };
 
 namespace {
@@ -503,12 +489,6 @@ cudaError_t next_scratch(lv_pool* pool, cudaStream_t s, bool async, const lv::Re
 }
 
 void free_pool(lv_pool* pool) {
-  for (auto& g : pool->step_graphs) {
-    if (g.exec) cudaGraphExecDestroy(g.exec);
-    if (g.graph) cudaGraphDestroy(g.graph);
-  }
-  pool->step_graphs.clear();
-  if (pool->s_capture) cudaStreamDestroy(pool->s_capture);
   if (pool->s_unpack) cudaStreamSynchronize(pool->s_unpack);
   if (pool->s_unpack) cudaStreamDestroy(pool->s_unpack);
   for (cudaEvent_t e : {pool->ev_st_d2h, pool->ev_st_h2d, pool->ev_st_unpack, pool->ev_st_packed,
@@ -637,6 +617,7 @@ lv_status create_impl(const lv_pool_desc* desc, cudaStream_t s, lv_pool** out) {
       (st = dev_alloc(pool, &d.table, tb)) != LV_OK ||
       (st = dev_alloc(pool, &d.mark, tb)) != LV_OK ||
       (st = dev_alloc(pool, &d.shadow, tb)) != LV_OK ||
+      (st = dev_alloc(pool, &d.cnt, d.S)) != LV_OK ||
       (st = dev_alloc(pool, &d.own_hbm, (size_t)d.hbm_pages)) != LV_OK ||
       (st = dev_alloc(pool, &d.own_host, (size_t)d.host_pages)) != LV_OK ||
       (st = dev_alloc(pool, &d.bits_hbm, wh)) != LV_OK ||
@@ -656,7 +637,6 @@ lv_status create_impl(const lv_pool_desc* desc, cudaStream_t s, lv_pool** out) {
       (st = dev_alloc(pool, &rs.append, (size_t)d.maxB + 2)) != LV_OK ||
       (st = dev_alloc(pool, &rs.tasks, (size_t)d.budget + d.maxB)) != LV_OK ||
       (st = dev_alloc(pool, &rs.words, 16)) != LV_OK ||
-      (st = dev_alloc(pool, &rs.hits, (size_t)d.S)) != LV_OK ||
       (st = dev_alloc(pool, &pool->sched_scratch, (size_t)32 * LV_SCHED_MAX_REQUESTS)) != LV_OK)
     return fail(st);
   pool->rs_alt = rs;
@@ -679,6 +659,7 @@ lv_status create_impl(const lv_pool_desc* desc, cudaStream_t s, lv_pool** out) {
       cudaMemsetAsync(d.table, 0xff, tb * sizeof(int32_t), s) != cudaSuccess ||
       cudaMemsetAsync(d.mark, 0, tb * sizeof(int32_t), s) != cudaSuccess ||
       cudaMemsetAsync(d.shadow, 0xff, tb * sizeof(int32_t), s) != cudaSuccess ||
+      cudaMemsetAsync(d.cnt, 0, d.S * sizeof(int2), s) != cudaSuccess ||
       cudaMemsetAsync(d.own_hbm, 0xff, (size_t)d.hbm_pages * 4, s) != cudaSuccess ||
       cudaMemsetAsync(d.own_host, 0xff, (size_t)(d.host_pages ? d.host_pages : 1) * 4, s) != cudaSuccess ||
       cudaMemsetAsync(d.bits_hbm, 0, wh * 4, s) != cudaSuccess ||
@@ -717,6 +698,7 @@ lv_status create_impl(const lv_pool_desc* desc, cudaStream_t s, lv_pool** out) {
     }
   }
   if (lv::configure_exchange_tma(d) != cudaSuccess) return fail(LV_ERR_CUDA);
+  if (lv::configure_step_kernels() != cudaSuccess) return fail(LV_ERR_CUDA);
   if (const char* env = std::getenv("LV_STAGE_STAGES")) {   // TMA pack/unpack stages per CTA
     const int st = std::atoi(env);
     if (st >= 2 && st <= 16) d.stages = st;
@@ -751,9 +733,6 @@ lv_status create_impl(const lv_pool_desc* desc, cudaStream_t s, lv_pool** out) {
     if (per >= 1 && per <= 4) pool->stage_ctas = pool->num_sms * per;
   }
   if (const char* env = std::getenv("LV_STAGE_KERNEL")) pool->stage_tma = std::strcmp(env, "lsu") != 0;
-  // device-driven steps on the caller's stream as graph launches (LV_STEP_GRAPHS=0: one
-  // kernel launch at a time)
-  if (const char* env = std::getenv("LV_STEP_GRAPHS")) pool->step_graphs_on = std::strcmp(env, "0") != 0;
   if (const char* env = std::getenv("LV_REMAP_ENTRIES_PER_THREAD")) {   // 1, 2 or 4
     const int e = std::atoi(env);
     if (e == 1 || e == 2 || e == 4) pool->remap_per_thread = e;
@@ -776,114 +755,6 @@ lv_status create_impl(const lv_pool_desc* desc, cudaStream_t s, lv_pool** out) {
   if (cudaStreamSynchronize(s) != cudaSuccess) return fail(LV_ERR_CUDA);
   *out = pool;
   return LV_OK;
-}
-
-// The kernel nodes of a captured launch chain, in launch order (each node depends on
-// the one before it); false unless the graph is exactly such a chain of n nodes.
-bool chain_nodes(cudaGraph_t graph, size_t n, std::vector<cudaGraphNode_t>* order) {
-  size_t count = 0;
-  if (cudaGraphGetNodes(graph, nullptr, &count) != cudaSuccess || count != n) return false;
-  std::vector<cudaGraphNode_t> nodes(count);
-  if (cudaGraphGetNodes(graph, nodes.data(), &count) != cudaSuccess) return false;
-  std::vector<cudaGraphNode_t> prev(count, nullptr);
-  cudaGraphNode_t root = nullptr;
-  for (size_t i = 0; i < count; ++i) {
-    // with room for two, so that a node with more than one dependency is seen; the edge
-    // data is asked for too (programmatic edges are not default edges)
-    cudaGraphNode_t deps[2] = {nullptr, nullptr};
-    cudaGraphEdgeData edge[2] = {};
-    size_t nd = 2;
-    if (cudaGraphNodeGetDependencies(nodes[i], deps, edge, &nd) != cudaSuccess || nd > 1) return false;
-    if (nd == 1) {
-      prev[i] = deps[0];
-    } else if (root) {
-      return false;
-    } else {
-      root = nodes[i];
-    }
-  }
-  order->clear();
-  for (cudaGraphNode_t cur = root; cur && order->size() < count;) {
-    order->push_back(cur);
-    cudaGraphNode_t next = nullptr;
-    for (size_t i = 0; i < count; ++i)
-      if (prev[i] == cur) next = nodes[i];
-    cur = next;
-  }
-  for (cudaGraphNode_t nd : *order) {
-    cudaGraphNodeType t;
-    if (cudaGraphNodeGetType(nd, &t) != cudaSuccess || t != cudaGraphNodeTypeKernel) return false;
-  }
-  return order->size() == count;
-}
-
-// Issues a device-driven step whose kernels all run on `s` (`launch(stream)` makes its
-// launches): the launches are recorded, and the instantiated graph of the same shape
-// (built by stream capture on first use) is launched with every kernel node's arguments
-// replaced by this step's.  A shape that cannot be captured as a chain turns the graphs
-// off for the pool, and the recorded launches are issued one by one.
-template <typename F>
-cudaError_t run_step(lv_pool* pool, cudaStream_t s, F&& launch) {
-  if (!pool->step_graphs_on) return launch(s);
-  std::vector<lv::LaunchRecord> recs;
-  lv::set_launch_recorder(&recs);
-  cudaError_t e = launch(s);
-  lv::set_launch_recorder(nullptr);
-  if (e != cudaSuccess || recs.empty()) return e;
-  lv_pool::StepGraph* g = nullptr;
-  for (auto& c : pool->step_graphs) {
-    if (c.funcs.size() != recs.size()) continue;
-    bool same = true;
-    for (size_t i = 0; i < recs.size() && same; ++i)
-      same = c.funcs[i] == recs[i].func && c.grids[i].x == recs[i].grid.x && c.grids[i].y == recs[i].grid.y &&
-             c.blocks[i].x == recs[i].block.x && c.smems[i] == recs[i].smem;
-    if (same) {
-      g = &c;
-      break;
-    }
-  }
-  if (g) {
-    for (size_t i = 0; i < recs.size(); ++i) {
-      cudaKernelNodeParams kp{};
-      kp.func = const_cast<void*>(recs[i].func);
-      kp.gridDim = recs[i].grid;
-      kp.blockDim = recs[i].block;
-      kp.sharedMemBytes = (unsigned)recs[i].smem;
-      kp.kernelParams = const_cast<void**>(recs[i].args.data());
-      e = cudaGraphExecKernelNodeSetParams(g->exec, g->nodes[i], &kp);
-      if (e != cudaSuccess) return e;
-    }
-    return cudaGraphLaunch(g->exec, s);
-  }
-  // a new shape: capture the launches on the pool's capture stream (past 32 shapes,
-  // further shapes are issued launch by launch)
-  if (pool->step_graphs.size() >= 32) return lv::replay_launches(recs, s);
-  lv_pool::StepGraph c;
-  bool ok = true;
-  if (!pool->s_capture) ok = cudaStreamCreateWithFlags(&pool->s_capture, cudaStreamNonBlocking) == cudaSuccess;
-  if (ok) ok = cudaStreamBeginCapture(pool->s_capture, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-  if (ok) {
-    const cudaError_t le = lv::replay_launches(recs, pool->s_capture);
-    const cudaError_t ce = cudaStreamEndCapture(pool->s_capture, &c.graph);
-    ok = le == cudaSuccess && ce == cudaSuccess && c.graph;
-  }
-  if (ok) ok = chain_nodes(c.graph, recs.size(), &c.nodes);
-  if (ok) ok = cudaGraphInstantiate(&c.exec, c.graph, 0) == cudaSuccess;
-  if (!ok) {
-    cudaGetLastError();
-    if (c.exec) cudaGraphExecDestroy(c.exec);
-    if (c.graph) cudaGraphDestroy(c.graph);
-    pool->step_graphs_on = false;
-    return lv::replay_launches(recs, s);
-  }
-  for (const auto& r : recs) {
-    c.funcs.push_back(r.func);
-    c.grids.push_back(r.grid);
-    c.blocks.push_back(r.block);
-    c.smems.push_back(r.smem);
-  }
-  pool->step_graphs.push_back(std::move(c));
-  return cudaGraphLaunch(pool->step_graphs.back().exec, s);
 }
 
 }  // namespace
@@ -944,6 +815,7 @@ lv_status lv_pool_import(lv_pool* pool, const int32_t* placement, const int32_t*
     if (d.host_pages) LV_TRY(cudaMemsetAsync(d.bits_host, 0, (size_t)((d.host_pages + 31) / 32) * 4, s));
     LV_TRY(cudaMemsetAsync(d.ctl, 0, 2 * sizeof(long long), s));   // allocation counts
     LV_TRY(cudaMemsetAsync(d.ctl + lv::C_CLEAN, 0, sizeof(long long), s));   // no clean copies
+    LV_TRY(cudaMemsetAsync(d.cnt, 0, (size_t)d.S * sizeof(int2), s));
     LV_TRY(lv::launch_import(d, static_cast<const int32_t*>(pl), static_cast<const int32_t*>(cx), s));
     LV_TRY(lv::launch_check_budget(d, s));
     return st.finish();
@@ -1015,8 +887,7 @@ lv_status lv_select_victims(lv_pool* pool, int64_t now_us, int64_t k, uint32_t f
     if ((r = st.out(out, (size_t)keff * sizeof(lv_victim), &vdev, false)) != LV_OK) return r;
     if ((r = st.out(count_out, sizeof(int64_t), &cdev, false)) != LV_OK) return r;
     LV_TRY(lv::launch_select(pool->d, now_us, keff, (flags & LV_SELECT_FALLBACK) != 0,
-                             static_cast<lv_victim*>(vdev), static_cast<long long*>(cdev), s,
-                             pool->num_sms));
+                             static_cast<lv_victim*>(vdev), static_cast<long long*>(cdev), s));
     return st.finish();
   } catch (const std::bad_alloc&) {
     return LV_ERR_OOM;
@@ -1151,8 +1022,8 @@ lv_status lv_swap_exchange(lv_pool* pool, const lv_victim* victims, int64_t n_ou
                                static_cast<const int32_t*>(bin), n_in, static_cast<int32_t*>(sdev),
                                static_cast<int32_t*>(pdev), static_cast<int4*>(tdev),
                                static_cast<long long*>(ndev), pool->epoch, pool->d.page_tag, s,
-                               pool->exchange_ctas, nullptr, 0, timing_pair(pool, LV_TIMING_EXCHANGE),
-                               nullptr, nullptr, 0, static_cast<long long*>(ndev) + 1));
+                               pool->exchange_ctas, timing_pair(pool, LV_TIMING_EXCHANGE),
+                               static_cast<long long*>(ndev) + 1));
     return st.finish();
   } catch (const std::bad_alloc&) {
     return LV_ERR_OOM;
@@ -1205,13 +1076,9 @@ lv_status lv_make_resident(lv_pool* pool, int32_t sid, int64_t now_us, int32_t a
     lv::CopyOffload off{};
     LV_TRY(next_scratch(pool, s, async, &rs, &off));
     const lv::EventPair* ev = timing_pair(pool, LV_TIMING_EXCHANGE);
-    auto launch = [&](cudaStream_t cs) {
-      return lv::launch_make_resident(d, *rs, sid, now_us, append_tokens, preload, max_load_pages,
-                                      pool->epoch, cs, pool->exchange_ctas,
-                                      static_cast<lv_resident_result*>(rdev), ev, nullptr,
-                                      async ? &off : nullptr);
-    };
-    LV_TRY(async || ev ? launch(s) : run_step(pool, s, launch));
+    const lv::StepCall c{sid, nullptr, 0, now_us, append_tokens, false, preload, max_load_pages, -1, 0, 0,
+                         nullptr, static_cast<lv_resident_result*>(rdev)};
+    LV_TRY(lv::launch_step(d, *rs, c, pool->epoch, s, pool->exchange_ctas, ev, async ? &off : nullptr));
     LV_TRY(copy_resident_outputs(pool, append_tokens, victims_out, slots_out, blocks_out, pages_out,
                                  append_out, s));
     return st.finish();
@@ -1239,11 +1106,9 @@ lv_status lv_evict(lv_pool* pool, int64_t now_us, int64_t k, uint32_t flags, lv_
     LV_TRY(next_scratch(pool, s, async, &rs, &off));
     const int64_t kk = k < (int64_t)pool->d.budget ? k : (int64_t)pool->d.budget;
     const lv::EventPair* ev = timing_pair(pool, LV_TIMING_EXCHANGE);
-    auto launch = [&](cudaStream_t cs) {
-      return lv::launch_evict(pool->d, *rs, now_us, kk, pool->epoch, cs, pool->exchange_ctas,
-                              static_cast<lv_resident_result*>(rdev), ev, async ? &off : nullptr);
-    };
-    LV_TRY(async || ev ? launch(s) : run_step(pool, s, launch));
+    const lv::StepCall c{-1, nullptr, 0, now_us, 0, false, false, -1, kk, 0, 0, nullptr,
+                         static_cast<lv_resident_result*>(rdev)};
+    LV_TRY(lv::launch_step(pool->d, *rs, c, pool->epoch, s, pool->exchange_ctas, ev, async ? &off : nullptr));
     LV_TRY(copy_resident_outputs(pool, 0, victims_out, slots_out, nullptr, nullptr, nullptr, s));
     return st.finish();
   } catch (const std::bad_alloc&) {
@@ -1290,14 +1155,10 @@ lv_status lv_turn(lv_pool* pool, const lv_turn_desc* d, lv_victim* victims_out, 
     lv::CopyOffload off{};
     LV_TRY(next_scratch(pool, s, async, &rs, &off));
     const lv::EventPair* ev = timing_pair(pool, LV_TIMING_EXCHANGE);
-    auto launch = [&](cudaStream_t cs) {
-      return lv::launch_turn(pool->d, *rs, d->sid, static_cast<const int32_t*>(cdev),
-                             d->sid == -1 ? d->num_candidates : 0, d->now_us, d->append_tokens,
-                             d->reply_audio_us, d->reply_units, pool->epoch, cs, pool->exchange_ctas,
-                             static_cast<lv_resident_result*>(rdev), ev, async ? &off : nullptr,
-                             static_cast<const unsigned long long*>(kdev));
-    };
-    LV_TRY(async || ev ? launch(s) : run_step(pool, s, launch));
+    const lv::StepCall c{d->sid, static_cast<const int32_t*>(cdev), d->sid == -1 ? d->num_candidates : 0,
+                         d->now_us, d->append_tokens, true, false, -1, -1, d->reply_audio_us, d->reply_units,
+                         static_cast<const unsigned long long*>(kdev), static_cast<lv_resident_result*>(rdev)};
+    LV_TRY(lv::launch_step(pool->d, *rs, c, pool->epoch, s, pool->exchange_ctas, ev, async ? &off : nullptr));
     LV_TRY(copy_resident_outputs(pool, d->append_tokens, victims_out, slots_out, blocks_out, pages_out,
                                  append_out, s, d->load_keys != nullptr));
     return st.finish();

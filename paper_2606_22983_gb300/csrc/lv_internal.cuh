@@ -2,8 +2,6 @@
 #pragma once
 
 #include <cstdint>
-#include <memory>
-#include <vector>
 #include <cuda_runtime.h>
 
 #include "lv.h"
@@ -66,6 +64,7 @@ struct DevPool {
   int32_t* table;         // [S][maxB]
   int32_t* mark;          // [S][maxB] epoch of the last remap that touched the block
   int32_t* shadow;        // [S][maxB] host slot holding the block's clean copy, or -1
+  int2* cnt;              // [S] blocks in HBM (x) and in the host tier (y), kept with the table
   uint32_t* own_hbm;      // [hbm_pages] owner word (kOwnerNone / kOwnerReserved / sid << 16 | blk)
   uint32_t* own_host;     // [host_pages]
   uint32_t* bits_hbm;     // allocation bitmap, 1 = reserved or owned
@@ -110,8 +109,7 @@ cudaError_t launch_session_set(const DevPool& p, const lv_session_state* in, int
                                int32_t n, cudaStream_t s);
 cudaError_t launch_events(const DevPool& p, const lv_event* ev, int64_t n, cudaStream_t s);
 cudaError_t launch_select(const DevPool& p, int64_t now_us, int64_t k, bool fallback,
-                          lv_victim* out, long long* count_dev, cudaStream_t s, int num_sms,
-                          const long long* k_dev = nullptr);
+                          lv_victim* out, long long* count_dev, cudaStream_t s);
 cudaError_t launch_alloc(const DevPool& p, bool hbm, int64_t n, int32_t* out, cudaStream_t s,
                          bool injected_fail = false);
 // host slots for n victims: a clean copy where the block has one (inclusive
@@ -128,38 +126,14 @@ cudaError_t launch_exchange(const DevPool& p, const lv_victim* v, int64_t n_out,
                             const int32_t* blks, int64_t n_in, int32_t* slots, int32_t* pages,
                             int4* tasks, long long* n_tasks, int32_t epoch,
                             unsigned long long* page_tag, cudaStream_t s, int copy_ctas,
-                            const long long* counts_dev = nullptr, long long max_units = 0,
-                            const EventPair* ev = nullptr, const long long* sid_dev = nullptr,
-                            const CopyOffload* off = nullptr, int gate = 0,
-                            long long* cursor = nullptr, const struct StepFinish* fin = nullptr);
+                            const EventPair* ev, long long* cursor);
 cudaError_t launch_remap(const DevPool& p, const lv_remap_entry* e, int64_t n, int32_t epoch,
                          cudaStream_t s, int num_sms, int per_thread);
 cudaError_t launch_cancel(const DevPool& p, const int32_t* locs, int64_t n, cudaStream_t s);
 // Zeroes bytes (a multiple of 4) at q: device memory or mapped page-locked host memory.
 cudaError_t launch_zero(void* q, int64_t bytes, cudaStream_t s);
-// fin (with R, the step's control words): a device-driven step's end, done by the
-// append kernel after the growth
 cudaError_t launch_append(const DevPool& p, int32_t sid, int32_t n_tokens, int32_t* pages,
-                          int32_t* count, cudaStream_t s, const long long* gate = nullptr,
-                          const long long* sid_dev = nullptr, const struct StepFinish* fin = nullptr,
-                          const long long* R = nullptr);
-
-// One kernel launch of a device-driven step, recorded instead of issued (for replay
-// through a CUDA graph): the kernel, its launch shape, whether it is a programmatic
-// dependent launch, and its argument values (`args` points into `holder`).
-struct LaunchRecord {
-  const void* func;
-  dim3 grid, block;
-  size_t smem;
-  bool pdl;
-  std::shared_ptr<void> holder;
-  std::vector<void*> args;
-};
-// While a recorder is set on the calling host thread, the step launchers append their
-// programmatic dependent launches to it instead of issuing them.
-void set_launch_recorder(std::vector<LaunchRecord>* rec);
-// Issues recorded launches on s (the same launches the launchers would have made).
-cudaError_t replay_launches(const std::vector<LaunchRecord>& recs, cudaStream_t s);
+                          int32_t* count, cudaStream_t s);
 
 // Device buffers of lv_make_resident, owned by the pool.
 struct ResidentScratch {
@@ -171,47 +145,24 @@ struct ResidentScratch {
   int32_t* append;      // [maxB + 2]
   int4* tasks;          // [budget + maxB]
   long long* words;     // [16]
-  int32_t* hits;        // [S] lv_turn's pick
 };
-// The end of a device-driven step (lv_make_resident, lv_turn, lv_evict): the turn's
-// LV_EV_TURN_END, a completed preload's protection, and the result record.
-struct StepFinish {
-  bool on;
-  int32_t sid;                    // the session, or read from sid_dev when that is set
-  const long long* sid_dev;
-  long long now_us;
-  bool preload;
-  bool turn_end;
-  long long audio_us, units;      // LV_EV_TURN_END's a and b
-  lv_resident_result* out;        // may be null
-};
-// lv_turn's start, done by the first kernel of the make-resident chain: pick the
-// session when sid < 0 (the first of cand[0..n_cand) with hit set), then TURN_BEGIN.
-struct TurnStart {
-  bool on;
+// A device-driven step: lv_turn, lv_make_resident or lv_evict.
+struct StepCall {
+  int32_t sid;                          // -1: lv_turn picks from cand
   const int32_t* cand;
   int32_t n_cand;
-  const int32_t* hit;
-  long long now_us;
+  int64_t now_us;
+  int32_t append_tokens;
+  bool turn, preload;
+  int64_t max_load;                     // preload admission (< 0: no limit)
+  int64_t evict;                        // lv_evict's k, -1 for the others
+  int64_t audio_us, units;              // LV_EV_TURN_END's a and b
+  const unsigned long long* load_keys;  // or null
+  lv_resident_result* out;              // or null
 };
-cudaError_t launch_make_resident(const DevPool& p, const ResidentScratch& rs, int32_t sid,
-                                 int64_t now_us, int32_t append_tokens, bool preload,
-                                 int64_t max_load, int32_t epoch, cudaStream_t s, int copy_ctas,
-                                 lv_resident_result* result, const EventPair* ev = nullptr,
-                                 const long long* sid_dev = nullptr, const CopyOffload* off = nullptr,
-                                 const unsigned long long* load_keys = nullptr, bool turn_end = false,
-                                 int64_t audio_us = 0, int64_t units = 0,
-                                 const TurnStart* ts = nullptr);
-// lv_turn: pick (sid < 0), LV_EV_TURN_BEGIN, make resident, LV_EV_TURN_END
-// lv_evict: rank, evict up to k victims (no loads), finish
-cudaError_t launch_evict(const DevPool& p, const ResidentScratch& rs, int64_t now_us, int64_t k,
-                         int32_t epoch, cudaStream_t s, int copy_ctas, lv_resident_result* result,
-                         const EventPair* ev, const CopyOffload* off);
-cudaError_t launch_turn(const DevPool& p, const ResidentScratch& rs, int32_t sid, const int32_t* cand,
-                        int32_t n_cand, int64_t now_us, int32_t append_tokens, int64_t audio_us,
-                        int64_t units, int32_t epoch, cudaStream_t s, int copy_ctas,
-                        lv_resident_result* result, const EventPair* ev = nullptr,
-                        const CopyOffload* off = nullptr, const unsigned long long* load_keys = nullptr);
+cudaError_t configure_step_kernels();
+cudaError_t launch_step(const DevPool& p, const ResidentScratch& rs, const StepCall& c, int32_t epoch,
+                        cudaStream_t s, int copy_ctas, const EventPair* ev, const CopyOffload* off);
 cudaError_t launch_counts(const DevPool& p, int32_t* hbm, int32_t* host, cudaStream_t s);
 // sums[i] = position-weighted 64-bit sum of page pages[i] (sums zeroed by the caller)
 cudaError_t launch_checksums(const DevPool& p, const int32_t* pages, int64_t n,
@@ -228,7 +179,7 @@ cudaError_t launch_tasks_in(const DevPool& p, int32_t sid, const int32_t* blks, 
 cudaError_t launch_exchange_plan(const DevPool& p, const lv_victim* v, int64_t n_out, int32_t sid,
                                  const int32_t* blks, int64_t n_in, int32_t* slots, int32_t* pages,
                                  int4* tasks, long long* n_tasks, int32_t epoch,
-                                 unsigned long long* page_tag, cudaStream_t s);
+                                 unsigned long long* page_tag, cudaStream_t s, long long* cursor = nullptr);
 // pack (staging[t] <- out pages) or unpack (in pages <- staging[t]) for tasks [t_begin, t_end)
 cudaError_t launch_stage(const DevPool& p, bool pack, const int4* tasks, int64_t t_begin,
                          int64_t t_end, uint8_t* staging, cudaStream_t s, int ctas,

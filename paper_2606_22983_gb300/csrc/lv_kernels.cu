@@ -17,8 +17,6 @@
 // index read from memory is range-checked and a bad item is skipped with the
 // sticky error set.
 #include <cstdint>
-#include <memory>
-#include <tuple>
 #include <utility>
 
 #include "lv_internal.cuh"
@@ -167,54 +165,100 @@ __device__ void block_alloc_out(const DevPool& p, const lv_victim* __restrict__ 
   }
 }
 
+// ---------------------------------------------------------------- counts
+// p.cnt[s] holds session s's blocks in HBM (x) and in the host tier (y): what a scan of its
+// table row for entries >= 0 and <= -2 would count.  Every kernel that writes a table entry
+// keeps it (import, remap, the exchange's plan, append), so that a decision reads S counts
+// instead of S table rows.
+__device__ __forceinline__ int2 tier_of(int32_t e) { return make_int2(e >= 0 ? 1 : 0, e <= -2 ? 1 : 0); }
+
+// Adds (dh, dd) to the counts of session s, for the whole warp at once: lanes that share the
+// first adding lane's session add through one pair of reductions, the others by themselves.
+// All 32 lanes must call it; a lane with nothing to add passes zeros.
+__device__ __forceinline__ void warp_count(const DevPool& p, int32_t s, int dh, int dd) {
+  const unsigned act = __ballot_sync(0xffffffffu, dh != 0 || dd != 0);
+  if (!act) return;
+  const int lead = __ffs(act) - 1;
+  const int32_t s0 = __shfl_sync(0xffffffffu, s, lead);
+  const bool adds = act >> (threadIdx.x & 31) & 1u, mine = adds && s == s0;
+  const int h = __reduce_add_sync(0xffffffffu, mine ? dh : 0);
+  const int d = __reduce_add_sync(0xffffffffu, mine ? dd : 0);
+  if ((int)(threadIdx.x & 31) == lead) {
+    if (h) atomicAdd(&p.cnt[s0].x, h);
+    if (d) atomicAdd(&p.cnt[s0].y, d);
+  } else if (adds && !mine) {
+    if (dh) atomicAdd(&p.cnt[s].x, dh);
+    if (dd) atomicAdd(&p.cnt[s].y, dd);
+  }
+}
+
 // ---------------------------------------------------------------- import
+__device__ __forceinline__ int32_t import_block(const DevPool& p, const int32_t* __restrict__ placement,
+                                                const int32_t* __restrict__ ctx, long long idx, int32_t s,
+                                                int32_t b);
+
+// One thread per table entry; whole warps stay in the loop so that they can add up counts.
 __global__ void k_import(DevPool p, const int32_t* __restrict__ placement,
                          const int32_t* __restrict__ ctx) {
   const long long total = (long long)p.S * p.maxB;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int32_t s = (int32_t)(idx / p.maxB), b = (int32_t)(idx % p.maxB);
-    const long long c = ctx[s];
-    long long nb = (c + p.T - 1) / p.T;
-    if (b == 0) {
-      if (c < 0 || nb > p.maxB) {
-        set_error(p.ctl, LV_ERR_BOUNDS, s);
-      }
-      p.sess[s].ctx_tokens = (c < 0 || nb > p.maxB) ? 0 : (int32_t)c;
+  for (long long base = blockIdx.x * (long long)blockDim.x; base < total;
+       base += (long long)gridDim.x * blockDim.x) {
+    const long long idx = base + threadIdx.x;
+    int32_t s = 0, e = -1;
+    if (idx < total) {
+      s = (int32_t)(idx / p.maxB);
+      e = import_block(p, placement, ctx, idx, s, (int32_t)(idx % p.maxB));
     }
-    if (c < 0 || nb > p.maxB) nb = 0;
-    const int32_t e = placement[idx];
-    p.table[idx] = -1;
-    p.mark[idx] = 0;
-    p.shadow[idx] = -1;
-    if (b >= nb) {
-      if (e != -1) set_error(p.ctl, LV_ERR_BOUNDS, idx);
-      continue;
-    }
-    const uint32_t key = owner_key(s, b);
-    if (e >= 0) {
-      if (e >= p.hbm_pages) { set_error(p.ctl, LV_ERR_BOUNDS, idx); continue; }
-      if (atomicCAS(&p.own_hbm[e], kOwnerNone, key) != kOwnerNone) {
-        set_error(p.ctl, LV_ERR_DOUBLE_MAP, idx);
-        continue;
-      }
-      atomicOr(&p.bits_hbm[e >> 5], 1u << (e & 31));
-      atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]), 1ull);
-    } else if (e <= -2) {
-      const long long h = -(long long)e - 2;
-      if (h >= p.host_pages) { set_error(p.ctl, LV_ERR_BOUNDS, idx); continue; }
-      if (atomicCAS(&p.own_host[h], kOwnerNone, key) != kOwnerNone) {
-        set_error(p.ctl, LV_ERR_DOUBLE_MAP, idx);
-        continue;
-      }
-      atomicOr(&p.bits_host[h >> 5], 1u << (h & 31));
-      atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HOST_ALLOC]), 1ull);
-    } else {
-      set_error(p.ctl, LV_ERR_BOUNDS, idx);   // a block inside the context with no location
-      continue;
-    }
-    p.table[idx] = e;
+    const int2 t = tier_of(e);
+    warp_count(p, s, t.x, t.y);
   }
+}
+
+// The table entry that block b of session s gets (-1: none, or refused).
+__device__ __forceinline__ int32_t import_block(const DevPool& p, const int32_t* __restrict__ placement,
+                                                const int32_t* __restrict__ ctx, long long idx, int32_t s,
+                                                int32_t b) {
+  const long long c = ctx[s];
+  long long nb = (c + p.T - 1) / p.T;
+  if (b == 0) {
+    if (c < 0 || nb > p.maxB) {
+      set_error(p.ctl, LV_ERR_BOUNDS, s);
+    }
+    p.sess[s].ctx_tokens = (c < 0 || nb > p.maxB) ? 0 : (int32_t)c;
+  }
+  if (c < 0 || nb > p.maxB) nb = 0;
+  const int32_t e = placement[idx];
+  p.table[idx] = -1;
+  p.mark[idx] = 0;
+  p.shadow[idx] = -1;
+  if (b >= nb) {
+    if (e != -1) set_error(p.ctl, LV_ERR_BOUNDS, idx);
+    return -1;
+  }
+  const uint32_t key = owner_key(s, b);
+  if (e >= 0) {
+    if (e >= p.hbm_pages) { set_error(p.ctl, LV_ERR_BOUNDS, idx); return -1; }
+    if (atomicCAS(&p.own_hbm[e], kOwnerNone, key) != kOwnerNone) {
+      set_error(p.ctl, LV_ERR_DOUBLE_MAP, idx);
+      return -1;
+    }
+    atomicOr(&p.bits_hbm[e >> 5], 1u << (e & 31));
+    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]), 1ull);
+  } else if (e <= -2) {
+    const long long h = -(long long)e - 2;
+    if (h >= p.host_pages) { set_error(p.ctl, LV_ERR_BOUNDS, idx); return -1; }
+    if (atomicCAS(&p.own_host[h], kOwnerNone, key) != kOwnerNone) {
+      set_error(p.ctl, LV_ERR_DOUBLE_MAP, idx);
+      return -1;
+    }
+    atomicOr(&p.bits_host[h >> 5], 1u << (h & 31));
+    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HOST_ALLOC]), 1ull);
+  } else {
+    set_error(p.ctl, LV_ERR_BOUNDS, idx);   // a block inside the context with no location
+    return -1;
+  }
+  p.table[idx] = e;
+  return e;
 }
 
 __global__ void k_check_budget(DevPool p) {
@@ -379,9 +423,8 @@ constexpr int kEmitScanMax = LV_EMIT_SCAN_MAX;
 
 // One CTA per session: its key and its count of HBM-resident blocks.
 __global__ void __launch_bounds__(kCensusThreads)
-k_rank_census(DevPool p, long long now_us, bool fallback, const long long* __restrict__ k_dev) {
+k_rank_census(DevPool p, long long now_us, bool fallback) {
   pdl_wait();
-  if (k_dev && *k_dev == 0) return;   // a device-driven step with no deficit ranks nothing
   const int32_t s = blockIdx.x;
   __shared__ unsigned long long key;
   if (threadIdx.x == 0) {
@@ -419,9 +462,8 @@ constexpr int kPrefixChunk = 256;   // keys staged by one CTA in shared memory
 // once: a broadcast), and adds its partial sums; the CTAs of tile 0 also add up
 // all candidates' blocks into C_RANK_TOTAL.  The census zeroed both.
 __global__ void __launch_bounds__(kPrefixTile)
-k_rank_prefix(DevPool p, const long long* __restrict__ k_dev) {
+k_rank_prefix(DevPool p) {
   pdl_wait();   // the census is complete and visible
-  if (k_dev && *k_dev == 0) return;
   __shared__ unsigned long long kc[kPrefixChunk];
   __shared__ int32_t cc[kPrefixChunk];
   __shared__ long long part[kPrefixTile / 32];
@@ -466,22 +508,10 @@ constexpr int kEmitThreads = 256;
 // the selection count min(k, all resident candidates).  CTA 0 publishes the
 // count and the counters.
 __global__ void __launch_bounds__(kEmitThreads)
-k_rank_emit(DevPool p, long long k, const long long* k_dev, bool fallback, long long* count_dev,
+k_rank_emit(DevPool p, long long k, bool fallback, long long* count_dev,
             lv_victim* __restrict__ out) {
   pdl_wait();   // the census (and the places) are complete and visible
   const int32_t sid = blockIdx.x;
-  if (k_dev) {            // k decided on the device (lv_make_resident, lv_evict)
-    k = *k_dev;
-    if (k == 0) {         // no deficit: the census did not run, nothing is selected
-      if (sid == 0 && threadIdx.x == 0) {
-        p.ctl[C_SEL_COUNT] = 0;
-        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_SELECTS]), 1ull);
-        if (fallback) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_FALLBACK]), 1ull);
-        if (count_dev) *count_dev = 0;
-      }
-      return;
-    }
-  }
   const unsigned long long key = p.skey[sid];
   if (key == 0ull && sid != 0) return;
   long long off, total;
@@ -675,212 +705,327 @@ k_swap_in(DevPool p, int32_t sid, const int32_t* __restrict__ blks,
   }
 }
 
+// ------------------------------------------------------- one-CTA decisions
+// The decision kernels (k_step, k_exchange_plan, k_append) run as one CTA: what they do is a
+// chain of dependent reads of a few hundred table words, so their time is the number of
+// links, each a trip to L2 or a barrier, and not the work in them.  Lists of up to
+// kStepItems entries and the allocation bitmaps are therefore kept in shared memory, reads
+// that depend on nothing are issued at the start, and a scan costs one barrier.
+constexpr int kStepThreads = 512;
+constexpr int kStepWarps = kStepThreads / 32;
+constexpr int kStepItems = 1024;   // victims, and loads, whose lists stay in shared memory
+
+// Prefix sums over the CTA with one barrier each: consecutive calls alternate between two
+// sets of warp totals, so a set is written again only after the barrier of the call between.
+struct BlockScan {
+  int* ws;   // [2][kStepWarps] in shared memory
+  int ph;
+  __device__ int sum(int v, int* total) {          // exclusive prefix of v
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    return warps(x, lane, wid, total) + x - v;
+  }
+  __device__ int rank(bool flag, int* total) {      // flagged threads before this one
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned m = __ballot_sync(0xffffffffu, flag);
+    return warps(__popc(m & (0xffffffffu >> (31 - lane))), lane, wid, total) +
+           __popc(m & ((1u << lane) - 1u));
+  }
+
+ private:
+  // x: the warp's inclusive sums (lane 31 holds its total); returns the total of the warps before
+  __device__ int warps(int x, int lane, int wid, int* total) {
+    int* w = ws + ph * kStepWarps;
+    ph ^= 1;
+    if (lane == 31) w[wid] = x;
+    __syncthreads();
+    int y = lane < kStepWarps ? w[lane] : 0;
+#pragma unroll
+    for (int o = 1; o < kStepWarps; o <<= 1) {
+      const int z = __shfl_up_sync(0xffffffffu, y, o);
+      if (lane >= o) y += z;
+    }
+    *total = __shfl_sync(0xffffffffu, y, kStepWarps - 1);
+    const int before = __shfl_sync(0xffffffffu, y, wid > 0 ? wid - 1 : 0);
+    return wid > 0 ? before : 0;
+  }
+};
+
+// One tier's allocation bitmap: the pool's words, and the copy that this kernel reads
+// (in shared memory where it fits, else the words themselves).
+struct TierBits {
+  uint32_t* gl;
+  uint32_t* cur;
+  long long nbits;
+  __device__ void set(long long w, uint32_t m) const {     // a word only this thread changes
+    atomicOr(&gl[w], m);
+    if (cur != gl) cur[w] |= m;
+  }
+  __device__ void clear(long long i) const {
+    const uint32_t m = ~(1u << (i & 31));
+    atomicAnd(&gl[i >> 5], m);
+    if (cur != gl) atomicAnd(&cur[i >> 5], m);
+  }
+};
+
+// The n lowest free bits, ascending, into out[0..n); sets them.  Each thread owns a
+// contiguous run of words.  The caller has checked that n are free; a barrier is needed
+// before other threads read out or the bitmap.
+__device__ void take_lowest(const TierBits& t, long long n, int32_t* out, BlockScan& scan) {
+  const long long W = (t.nbits + 31) >> 5;
+  const long long per = (W + kStepThreads - 1) / kStepThreads;
+  const long long w0 = min(W, (long long)threadIdx.x * per);
+  const long long w1 = min(W, w0 + per);
+  int cnt = 0;
+#pragma unroll 4
+  for (long long w = w0; w < w1; ++w) cnt += __popc(free_bits(t.cur, w, W, t.nbits));
+  int total;
+  long long r = scan.sum(cnt, &total);
+  const long long r_end = min(n, r + cnt);
+  for (long long w = w0; w < w1 && r < r_end; ++w) {
+    uint32_t f = free_bits(t.cur, w, W, t.nbits);
+    uint32_t take = 0;
+    while (f && r < r_end) {
+      const int b = __ffs(f) - 1;
+      f &= f - 1;
+      out[r++] = (int32_t)(w * 32 + b);
+      take |= 1u << b;
+    }
+    if (take) t.set(w, take);
+  }
+}
+
 // -------------------------------------------------------------- exchange
 // Evict n_out victims and load n_in host blocks of one session in a single
 // stream-ordered step whose result equals swap-out, commit, swap-in, commit
-// done one after the other.  k_exchange_plan (one CTA) takes every metadata
-// decision in that order -- validation, host slots (lowest free, victim
-// order), out-commit, HBM pages (lowest free after the frees, list order),
-// in-commit -- and emits copy tasks {out page, out slot, in slot, in page}.
+// done one after the other.  plan_moves takes every metadata decision in that
+// order -- validation, host slots (lowest free, victim order), out-commit, HBM
+// pages (lowest free after the frees, list order), in-commit -- and emits copy
+// tasks {out page, out slot, in slot, in page}.
 // An incoming block that lands on a victim's old page shares that victim's
 // task, so one thread reads the old bytes before it writes the new ones and
 // both directions of the host link carry data at the same time.
-constexpr int kPlanThreads = 1024;
 constexpr unsigned long long kPairedBit = 1ull << 31;
 
-// Words shared by the steps of one lv_make_resident call.
+// Words that a device-driven step leaves for the kernels after it.
 enum ResWord : int {
-  R_K_SELECT = 0,   // k handed to the ranker (0 when nothing is to be evicted)
-  R_N_OUT = 1,      // victims the exchange evicts
-  R_N_IN = 2,       // host blocks the exchange loads
-  R_STATUS = 3,     // LV_RESIDENT_*
-  R_K = 4,          // pages the budget was short
-  R_GATE = 5,       // 0: the append may run
+  R_N_IN = 2,       // host blocks listed (for k_order_loads)
   R_N_TASKS = 6,
-  R_APPENDED = 7,   // int32 count of appended pages, in the low half
-  R_FOUND = 8,      // victims the ranking found
   R_SID = 9,        // lv_turn: the turn's session (-1 when the pick failed)
   R_CURSOR = 10     // the exchange copy's next unit (zeroed by the plan)
 };
 
-// The gate after a device-driven step's ranking, run by the exchange plan's first
-// thread before it reads the counts.  GATE_RESIDENT / GATE_PRELOAD (lv_make_resident):
-// a shortfall stops the step (a preload is skipped, a foreground turn fails),
-// otherwise the exchange evicts exactly k victims.  GATE_EVICT (lv_evict): every
-// victim found is evicted; none found is LV_RESIDENT_NOTHING.
-enum { GATE_NONE = 0, GATE_RESIDENT = 1, GATE_PRELOAD = 2, GATE_EVICT = 3 };
+// What plan_moves works on.  v, slots, blks, gslot and pages may lie in shared memory
+// (lists of up to kStepItems entries) or in global memory.
+struct MovePlan {
+  const lv_victim* v;
+  int64_t n_out;
+  int32_t sid;
+  const int32_t* blks;
+  const int32_t* gslot;     // the loads' host slots, or null: read from the table
+  int64_t n_in;
+  int32_t* slots;
+  int32_t* pages;
+  int32_t* slots_out;       // global results
+  int32_t* pages_out;
+  int4* tasks;
+  long long* n_tasks;
+  int32_t epoch;
+  unsigned long long* page_tag;
+};
 
-__device__ __forceinline__ void step_gate(const DevPool& p, long long* __restrict__ R, int gate) {
-  const long long found = p.ctl[C_SEL_COUNT];   // min(k, candidates)
-  if (gate == GATE_EVICT) {
-    R[R_FOUND] = found;
-    R[R_N_OUT] = found;
-    if (found == 0) R[R_STATUS] = LV_RESIDENT_NOTHING;
-    return;
-  }
-  if (R[R_STATUS] != LV_RESIDENT_DONE) return;
-  const long long k = R[R_K];
-  R[R_FOUND] = found;
-  if (found < k) {
-    if (gate == GATE_PRELOAD) {
-      R[R_STATUS] = LV_RESIDENT_SKIPPED;
-      atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_PRELOADS_SKIPPED]), 1ull);
-    } else {
-      set_error(p.ctl, LV_ERR_NO_HBM, k);
-      R[R_STATUS] = LV_RESIDENT_FAILED;
-    }
-    R[R_N_OUT] = 0;
-    R[R_N_IN] = 0;
-    R[R_GATE] = 1;
-  } else {
-    R[R_N_OUT] = k;
-  }
-}
+// Shared memory of the one-CTA kernels.
+struct StepShared {
+  int ws[2 * kStepWarps];
+  unsigned long long best[2][kStepWarps];
+  int sums[kStepWarps];
+  int2 pick[kStepWarps + 1];
+  int bad;
+  int sel_sid[8], sel_off[8];
+  uint32_t paired[kStepItems / 32];
+  lv_victim v[kStepItems];
+  int32_t slots[kStepItems], blks[kStepItems], gslot[kStepItems], pages[kStepItems];
+};
 
-__device__ void finish_step(const DevPool& p, const StepFinish& f, const long long* __restrict__ R);
-
-__global__ void __launch_bounds__(kPlanThreads)
-k_exchange_plan(DevPool p, const lv_victim* __restrict__ v, long long n_out, int32_t sid,
-                const int32_t* __restrict__ blks, long long n_in, int32_t* __restrict__ slots,
-                int32_t* __restrict__ pages, int4* __restrict__ tasks, long long* n_tasks,
-                int32_t epoch, unsigned long long* __restrict__ page_tag,
-                const long long* counts_dev, const long long* __restrict__ sid_dev,
-                long long* R, int gate, long long* __restrict__ cursor, StepFinish fin) {
-  pdl_entry();
-  __shared__ int bad;
-  if (threadIdx.x == 0) {
-    bad = 0;
-    if (cursor) *cursor = 0;
-    if (gate != GATE_NONE) step_gate(p, R, gate);   // a device-driven step: may set the counts
-  }
-  __syncthreads();
-  if (counts_dev) {          // counts decided on the device (lv_make_resident, lv_evict)
-    n_out = counts_dev[0];
-    n_in = counts_dev[1];
-  }
-  if (sid_dev) sid = (int32_t)*sid_dev;
-  const bool sid_ok = sid >= 0 && sid < p.S;
-  const int32_t nb_in = sid_ok ? nblocks_of(p, sid) : 0;
-  // validation: every victim is resident where it says, every incoming block is in
-  // the host tier, and no block appears twice (victims and incoming blocks side by
-  // side: item i < n_out is victim i, item n_out + i incoming block i)
-  for (long long it = threadIdx.x; it < n_out + n_in; it += kPlanThreads) {
+// Plans and commits m's moves; every thread of the CTA calls it.  kListed: the lists come
+// from the caller and may be wrong or hold a block twice (checked, with the epoch marks);
+// else they were just read from the tables.  Returns false, with nothing changed, the
+// outputs -1 and no tasks, when an item is refused or a tier is too full.
+// hbm_alloc and host_alloc: the tiers' allocation counts as the kernel found them.
+template <bool kListed>
+__device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& hbm, const TierBits& host,
+                           long long hbm_alloc, long long host_alloc, StepShared& sh, BlockScan& scan) {
+  const long long n_out = m.n_out, n_in = m.n_in;
+  const bool sid_ok = m.sid >= 0 && m.sid < p.S;
+  const size_t row = sid_ok ? (size_t)m.sid * p.maxB : 0;
+  const int32_t nb_in = kListed && sid_ok ? nblocks_of(p, m.sid) : 0;
+  const bool few = n_out <= kStepItems;      // victims are tracked in shared memory
+  if (few && threadIdx.x < kStepItems / 32) sh.paired[threadIdx.x] = 0u;
+  // validation: every victim is resident where it says, every incoming block is in the
+  // host tier, and no block appears twice (victims and incoming blocks side by side: item
+  // i < n_out is victim i, item n_out + i incoming block i)
+  bool bad = false;
+  int dirty = 0;             // victims without a clean copy: all of them unless the tiers are inclusive
+  for (long long it = threadIdx.x; it < n_out + n_in; it += kStepThreads) {
+    bool ok;
     if (it < n_out) {
-      const lv_victim x = v[it];
-      bool ok = x.sid >= 0 && x.sid < p.S && x.blk >= 0 && x.page >= 0 && x.page < p.hbm_pages;
-      ok = ok && x.blk < nblocks_of(p, x.sid);
-      ok = ok && p.table[(size_t)x.sid * p.maxB + x.blk] == x.page &&
-           p.own_hbm[x.page] == owner_key(x.sid, x.blk);
-      ok = ok && atomicExch(&p.mark[(size_t)x.sid * p.maxB + x.blk], epoch) != epoch;
-      if (!ok) { set_error(p.ctl, LV_ERR_STATE, it); bad = 1; }
-    } else {
-      const int32_t b = blks[it - n_out];
-      bool ok = sid_ok && b >= 0 && b < nb_in;
-      if (ok) {
-        const int32_t e = p.table[(size_t)sid * p.maxB + b];
-        const long long h = -(long long)e - 2;
-        ok = e <= -2 && h < p.host_pages && p.own_host[h] == owner_key(sid, b);
-        ok = ok && atomicExch(&p.mark[(size_t)sid * p.maxB + b], epoch) != epoch;
+      const lv_victim x = m.v[it];
+      if (kListed) {
+        ok = x.sid >= 0 && x.sid < p.S && x.blk >= 0 && x.page >= 0 && x.page < p.hbm_pages;
+        ok = ok && x.blk < nblocks_of(p, x.sid);
+        ok = ok && p.table[(size_t)x.sid * p.maxB + x.blk] == x.page &&
+             p.own_hbm[x.page] == owner_key(x.sid, x.blk);
+        ok = ok && atomicExch(&p.mark[(size_t)x.sid * p.maxB + x.blk], m.epoch) != m.epoch;
+      } else {
+        ok = x.page < p.hbm_pages && p.own_hbm[x.page] == owner_key(x.sid, x.blk);
       }
-      if (!ok) { set_error(p.ctl, sid_ok ? LV_ERR_STATE : LV_ERR_BOUNDS, it); bad = 1; }
+      dirty += clean_copy_of(p, x) < 0 ? 1 : 0;
+    } else {
+      const int32_t b = m.blks[it - n_out];
+      if (kListed) {
+        ok = sid_ok && b >= 0 && b < nb_in;
+        if (ok) {
+          const int32_t e = p.table[row + b];
+          const long long h = -(long long)e - 2;
+          ok = e <= -2 && h < p.host_pages && p.own_host[h] == owner_key(m.sid, b);
+          ok = ok && atomicExch(&p.mark[row + b], m.epoch) != m.epoch;
+        }
+      } else {
+        const long long h = m.gslot ? (long long)m.gslot[it - n_out] : -(long long)p.table[row + b] - 2;
+        ok = h < p.host_pages && p.own_host[h] == owner_key(m.sid, b);
+      }
     }
+    if (!ok) { set_error(p.ctl, sid_ok || it < n_out ? LV_ERR_STATE : LV_ERR_BOUNDS, it); bad = true; }
   }
-  __syncthreads();   // every validation verdict is in `bad` before the capacity check
-  // victims without a clean copy: all of them unless the tiers are inclusive
-  long long n_dirty = n_out;
-  if (p.incl) {
-    long long cnt = 0;
-    for (long long i = threadIdx.x; i < n_out; i += kPlanThreads) cnt += clean_copy_of(p, v[i]) < 0;
-    block_excl_scan<kPlanThreads>(cnt, &n_dirty);
-  }
-  if (threadIdx.x == 0 && !bad) {
+  bad = __syncthreads_or(bad);
+  int n_dirty = (int)n_out;
+  if (p.incl) scan.sum(dirty, &n_dirty);
+  if (!bad) {
     // capacity, as the sequential calls see it: host slots before any is freed,
     // HBM pages after the victims' pages are freed
-    if (p.ctl[C_HOST_ALLOC] + n_dirty > p.host_pages) {
-      set_error(p.ctl, LV_ERR_NO_HOST, n_dirty);
-      bad = 1;
-    } else if (p.ctl[C_HBM_ALLOC] - n_out + n_in > p.budget) {
-      set_error(p.ctl, LV_ERR_NO_HBM, n_in);
-      bad = 1;
+    if (host_alloc + n_dirty > p.host_pages) {
+      if (threadIdx.x == 0) set_error(p.ctl, LV_ERR_NO_HOST, n_dirty);
+      bad = true;
+    } else if (hbm_alloc - n_out + n_in > p.budget) {
+      if (threadIdx.x == 0) set_error(p.ctl, LV_ERR_NO_HBM, n_in);
+      bad = true;
     }
   }
-  __syncthreads();
   if (bad) {
-    for (long long i = threadIdx.x; i < n_out; i += kPlanThreads) slots[i] = -1;
-    for (long long i = threadIdx.x; i < n_in; i += kPlanThreads) pages[i] = -1;
-    if (threadIdx.x == 0) {
-      *n_tasks = 0;
-      if (fin.on) finish_step(p, fin, R);
-    }
-    return;
+    for (long long i = threadIdx.x; i < n_out; i += kStepThreads) m.slots_out[i] = -1;
+    for (long long i = threadIdx.x; i < n_in; i += kStepThreads) m.pages_out[i] = -1;
+    if (threadIdx.x == 0) *m.n_tasks = 0;
+    return false;
   }
-  // host slots for the victims: a clean copy, or the lowest free slots in victim order
-  if (n_out > 0) block_alloc_out<kPlanThreads>(p, v, n_out, n_dirty, slots);
+  // host slots for the victims: a clean copy, or the lowest free slots in victim order.
+  // The compact list of new slots is spread in place from the last chunk to the first: a
+  // victim's rank among those without a copy is at most its index, so each read position
+  // still holds its compact value when it is read.
+  if (n_dirty > 0) take_lowest(host, n_dirty, m.slots, scan);
   __syncthreads();
+  if (n_dirty < n_out) {
+    long long after = 0;   // victims without a copy in the chunks already spread
+    for (long long c = (n_out + kStepThreads - 1) / kStepThreads - 1; c >= 0; --c) {
+      const long long i = c * kStepThreads + threadIdx.x;
+      const int32_t cp = i < n_out ? clean_copy_of(p, m.v[i]) : 0;
+      int chunk;
+      const int excl = scan.rank(cp < 0, &chunk);
+      const int32_t val = cp < 0 ? m.slots[n_dirty - after - chunk + excl] : cp;
+      __syncthreads();
+      if (i < n_out) m.slots[i] = val;
+      __syncthreads();
+      after += chunk;
+    }
+  }
   // out-commit: victims now live in their slots, their pages are free; only a
   // victim that moves bytes tags its page (a clean one has nothing to read)
-  const unsigned long long tag = (unsigned long long)(uint32_t)epoch << 32;
-  for (long long i = threadIdx.x; i < n_out; i += kPlanThreads) {
-    const lv_victim x = v[i];
-    const uint32_t key = owner_key(x.sid, x.blk);
-    const size_t ti = (size_t)x.sid * p.maxB + x.blk;
-    const bool clean = p.incl && p.shadow[ti] == slots[i];
-    p.table[ti] = -(slots[i] + 2);
-    if (clean) p.shadow[ti] = -1;
-    p.own_host[slots[i]] = key;
-    p.own_hbm[x.page] = kOwnerNone;
-    atomicAnd(&p.bits_hbm[x.page >> 5], ~(1u << (x.page & 31)));
-    if (!clean) page_tag[x.page] = tag | (unsigned long long)i;
+  const unsigned long long tag = (unsigned long long)(uint32_t)m.epoch << 32;
+  for (long long i0 = 0; i0 < n_out; i0 += kStepThreads) {
+    const long long i = i0 + threadIdx.x;
+    if (i < n_out) {
+      const lv_victim x = m.v[i];
+      const int32_t slot = m.slots[i];
+      const size_t ti = (size_t)x.sid * p.maxB + x.blk;
+      const bool clean = p.incl && p.shadow[ti] == slot;
+      p.table[ti] = -(slot + 2);
+      if (clean) p.shadow[ti] = -1;
+      p.own_host[slot] = owner_key(x.sid, x.blk);
+      p.own_hbm[x.page] = kOwnerNone;
+      hbm.clear(x.page);
+      if (!clean) m.page_tag[x.page] = tag | (unsigned long long)i;
+      else if (few) atomicOr(&sh.paired[i >> 5], 1u << (i & 31));   // no out task of its own
+      if (m.slots_out != m.slots) m.slots_out[i] = slot;
+    }
+    if (kListed) {
+      const bool mine = i < n_out;
+      warp_count(p, mine ? m.v[i].sid : 0, mine ? -1 : 0, mine ? 1 : 0);
+    }
   }
   __syncthreads();
   // HBM pages for the incoming blocks
-  if (n_in > 0) block_alloc_lowest<kPlanThreads>(p.bits_hbm, p.hbm_pages, n_in, pages);
+  if (n_in > 0) take_lowest(hbm, n_in, m.pages, scan);
   __syncthreads();
   // in-commit, and one task per incoming block (paired with the victim whose page it takes)
-  for (long long i = threadIdx.x; i < n_in; i += kPlanThreads) {
-    const int32_t b = blks[i];
-    const size_t ti = (size_t)sid * p.maxB + b;
-    const long long g = -(long long)p.table[ti] - 2;
-    const int32_t pg = pages[i];
-    const unsigned long long pt = page_tag[pg];   // read before this thread's stores
+  for (long long i = threadIdx.x; i < n_in; i += kStepThreads) {
+    const int32_t b = m.blks[i];
+    const size_t ti = row + b;
+    const long long g = m.gslot ? (long long)m.gslot[i] : -(long long)p.table[ti] - 2;
+    const int32_t pg = m.pages[i];
+    const unsigned long long pt = n_out > 0 ? m.page_tag[pg] : 0ull;   // read before this thread's stores
     p.table[ti] = pg;
-    p.own_hbm[pg] = owner_key(sid, b);
+    p.own_hbm[pg] = owner_key(m.sid, b);
     if (p.incl) {
       p.shadow[ti] = (int32_t)g;             // the host slot stays as its clean copy
     } else {
       p.own_host[g] = kOwnerNone;
-      atomicAnd(&p.bits_host[g >> 5], ~(1u << (g & 31)));
+      host.clear(g);
     }
     int4 t = make_int4(-1, -1, (int32_t)g, pg);
-    if ((pt >> 32) == (unsigned long long)(uint32_t)epoch && !(pt & kPairedBit)) {
+    if ((pt >> 32) == (unsigned long long)(uint32_t)m.epoch && !(pt & kPairedBit)) {
       const long long vi = (long long)(pt & 0x7fffffffull);
       t.x = pg;
-      t.y = slots[vi];
-      page_tag[pg] = pt | kPairedBit;
+      t.y = m.slots[vi];
+      if (few) atomicOr(&sh.paired[vi >> 5], 1u << (vi & 31));
+      else m.page_tag[pg] = pt | kPairedBit;
     }
-    tasks[i] = t;
+    m.tasks[i] = t;
+    if (m.pages_out != m.pages) m.pages_out[i] = pg;
   }
   __syncthreads();
   // victims whose page no incoming block takes: out-only tasks, in victim order
   long long run = 0;
-  for (long long i0 = 0; i0 < n_out; i0 += kPlanThreads) {
+  for (long long i0 = 0; i0 < n_out; i0 += kStepThreads) {
     const long long i = i0 + threadIdx.x;
-    long long flag = 0;
+    bool flag = false;
     int32_t pg = -1;
     if (i < n_out) {
-      pg = v[i].page;
-      const unsigned long long pt = page_tag[pg];
-      flag = ((pt >> 32) == (unsigned long long)(uint32_t)epoch && !(pt & kPairedBit)) ? 1 : 0;
+      pg = m.v[i].page;
+      if (few) {
+        flag = !(sh.paired[i >> 5] >> (i & 31) & 1u);
+      } else {
+        const unsigned long long pt = m.page_tag[pg];
+        flag = (pt >> 32) == (unsigned long long)(uint32_t)m.epoch && !(pt & kPairedBit) &&
+               (long long)(pt & 0x7fffffffull) == i;
+      }
     }
-    long long chunk;
-    const long long pos = run + block_excl_scan<kPlanThreads>(flag, &chunk);
-    if (flag) tasks[n_in + pos] = make_int4(pg, slots[i], -1, -1);
+    int chunk;
+    const long long pos = run + scan.rank(flag, &chunk);
+    if (flag) m.tasks[n_in + pos] = make_int4(pg, m.slots[i], -1, -1);
     run += chunk;
   }
   if (threadIdx.x == 0) {
-    *n_tasks = n_in + run;
+    *m.n_tasks = n_in + run;
     const long long n_clean = n_out - n_dirty;
     const long long host_delta = p.incl ? n_dirty : n_dirty - n_in;
+    if (n_in) {
+      atomicAdd(&p.cnt[m.sid].x, (int)n_in);
+      atomicAdd(&p.cnt[m.sid].y, -(int)n_in);
+    }
     atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HOST_ALLOC]), (unsigned long long)host_delta);
     if (p.incl) {
       atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_CLEAN]), (unsigned long long)(n_in - n_clean));
@@ -890,8 +1035,109 @@ k_exchange_plan(DevPool p, const lv_victim* __restrict__ v, long long n_out, int
     atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_PAGES_OUT]), (unsigned long long)n_out);
     atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_PAGES_IN]), (unsigned long long)n_in);
     atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_REMAP]), (unsigned long long)(n_out + n_in));
-    if (fin.on) finish_step(p, fin, R);   // the step's end when nothing follows the plan
   }
+  return true;
+}
+
+// The bitmaps of both tiers, copied to shared memory at `copy` (null: used in place).
+__device__ void tier_bits(const DevPool& p, uint32_t* copy, TierBits* hbm, TierBits* host) {
+  const long long wh = (p.hbm_pages + 31) >> 5, wo = (p.host_pages + 31) >> 5;
+  *hbm = TierBits{p.bits_hbm, copy ? copy : p.bits_hbm, p.hbm_pages};
+  *host = TierBits{p.bits_host, copy ? copy + wh : p.bits_host, p.host_pages};
+  if (copy) {
+#pragma unroll 4
+    for (long long w = threadIdx.x; w < wh; w += kStepThreads) copy[w] = p.bits_hbm[w];
+#pragma unroll 4
+    for (long long w = threadIdx.x; w < wo; w += kStepThreads) copy[wh + w] = p.bits_host[w];
+  }
+}
+
+// The exchange of a caller's lists (lv_swap_exchange).
+__global__ void __launch_bounds__(kStepThreads)
+k_exchange_plan(DevPool p, const lv_victim* __restrict__ v, long long n_out, int32_t sid,
+                const int32_t* __restrict__ blks, long long n_in, int32_t* slots, int32_t* pages,
+                int4* tasks, long long* n_tasks, int32_t epoch, unsigned long long* page_tag,
+                long long* cursor, int copy_bits) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ StepShared sh;
+  pdl_entry();
+  BlockScan scan{sh.ws, 0};
+  TierBits hbm, host;
+  tier_bits(p, copy_bits ? reinterpret_cast<uint32_t*>(dyn) : nullptr, &hbm, &host);
+  const long long hbm_alloc = p.ctl[C_HBM_ALLOC], host_alloc = p.ctl[C_HOST_ALLOC];
+  if (threadIdx.x == 0 && cursor) *cursor = 0;
+  MovePlan m{v, n_out, sid, blks, nullptr, n_in, n_out <= kStepItems ? sh.slots : slots,
+             n_in <= kStepItems ? sh.pages : pages, slots, pages, tasks, n_tasks, epoch, page_tag};
+  plan_moves<true>(p, m, hbm, host, hbm_alloc, host_alloc, sh, scan);
+}
+
+// Grows session sid by n_tokens (every thread of the CTA calls it): the new blocks take the
+// lowest free HBM pages, in block order.  Returns the pages appended, -1 on an error.
+__device__ long long append_tokens_to(const DevPool& p, int32_t sid, int32_t n_tokens, int32_t* pages,
+                                      const TierBits& hbm, BlockScan& scan, int* s_ok) {
+  const long long ctx = p.sess[sid].ctx_tokens;
+  const long long nb = (ctx + p.T - 1) / p.T;
+  const long long nctx = ctx + n_tokens;
+  const long long nnb = (nctx + p.T - 1) / p.T;
+  const long long m = nnb - nb;
+  if (threadIdx.x == 0) {
+    int ok = 1;
+    if (nnb > p.maxB || nctx > 0x7fffffffll) {
+      set_error(p.ctl, LV_ERR_BOUNDS, sid);
+      ok = 0;
+    } else if (m > 0) {
+      const long long before = (long long)atomicAdd(
+          reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]), (unsigned long long)m);
+      if (before + m > p.budget) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]), (unsigned long long)(-m));
+        set_error(p.ctl, LV_ERR_NO_HBM, sid);
+        ok = 0;
+      }
+    }
+    *s_ok = ok;
+  }
+  __syncthreads();   // the verdict; and every thread has read the context length
+  if (!*s_ok) return -1;
+  if (m > 0) {
+    take_lowest(hbm, m, pages, scan);
+    __syncthreads();
+    for (long long i = threadIdx.x; i < m; i += kStepThreads) {
+      const int32_t pg = pages[i];
+      const int32_t b = (int32_t)(nb + i);
+      p.table[(size_t)sid * p.maxB + b] = pg;
+      p.own_hbm[pg] = owner_key(sid, b);
+    }
+  }
+  if (threadIdx.x == 0) {
+    if (m > 0) atomicAdd(&p.cnt[sid].x, (int)m);
+    // inclusive tiers: the partially filled last block gains rows, its clean copy is stale
+    if (p.incl && n_tokens > 0 && nb > 0 && ctx % p.T != 0) {
+      const size_t ti = (size_t)sid * p.maxB + (nb - 1);
+      const int32_t g = p.shadow[ti];
+      if (g >= 0 && g < p.host_pages) {
+        p.shadow[ti] = -1;
+        p.own_host[g] = kOwnerNone;
+        atomicAnd(&p.bits_host[g >> 5], ~(1u << (g & 31)));
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HOST_ALLOC]), (unsigned long long)-1ll);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_CLEAN]), (unsigned long long)-1ll);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_CLEAN_DROPPED]), 1ull);
+      }
+    }
+    p.sess[sid].ctx_tokens = (int32_t)nctx;
+    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_APPENDED]), (unsigned long long)m);
+  }
+  return m;
+}
+
+__global__ void __launch_bounds__(kStepThreads)
+k_append(DevPool p, int32_t sid, int32_t n_tokens, int32_t* pages, int32_t* count) {
+  __shared__ int ws[2 * kStepWarps];
+  __shared__ int ok;
+  pdl_entry();
+  BlockScan scan{ws, 0};
+  const TierBits hbm{p.bits_hbm, p.bits_hbm, p.hbm_pages};
+  const long long m = append_tokens_to(p, sid, n_tokens, pages, hbm, scan, &ok);
+  if (threadIdx.x == 0 && count) *count = m > 0 ? (int32_t)m : 0;
 }
 
 // Unit u = (task t, chunk c): kUnitVecs 16-byte vectors of the task's page, taken as one
@@ -1352,6 +1598,7 @@ struct RemapRead {
 
 struct RemapCounts {
   int ok, hbm, host, clean;
+  int dh, dd;           // the last settled entry's change of its session's counts
 };
 
 __device__ __forceinline__ void remap_read_entry(const DevPool& p, const lv_remap_entry* e, long long i,
@@ -1446,10 +1693,14 @@ __device__ __forceinline__ void remap_settle(const DevPool& p, const RemapRead& 
       else if (old_host && !(p.incl && x.loc >= 0)) p.own_host[old_slot] = was;
     }
   }
+  c.dh = c.dd = 0;
   if (err) {
     set_error(p.ctl, err, i);
     return;
   }
+  const int2 from = tier_of(old), to = tier_of(x.loc);
+  c.dh = to.x - from.x;
+  c.dd = to.y - from.y;
   if (x.loc <= -2 && g >= 0) {          // the copy becomes the location, or goes
     p.shadow[r.ti] = -1;
     c.clean -= 1;
@@ -1515,10 +1766,13 @@ k_remap(DevPool p, const lv_remap_entry* __restrict__ e, long long n, int32_t ep
     err[j] = i0 + j * stride < n ? remap_judge(r[j], epoch, seen[j]) : -1;
     if (err[j] >= 0) err[j] = remap_claim(p, r[j], err[j], got[j], was[j]);
   }
-  RemapCounts c{0, 0, 0, 0};
+  RemapCounts c{0, 0, 0, 0, 0, 0};
 #pragma unroll
-  for (int j = 0; j < E; ++j)
+  for (int j = 0; j < E; ++j) {
+    c.dh = c.dd = 0;
     if (err[j] >= 0) remap_settle(p, r[j], err[j], got[j], was[j], i0 + j * stride, c);
+    warp_count(p, r[j].x.sid, c.dh, c.dd);
+  }
   // block totals: warp sums, one shared atomic per warp, one global atomic per block
   __shared__ int tot[4];
   if (threadIdx.x < 4) tot[threadIdx.x] = 0;
@@ -1637,195 +1891,493 @@ __global__ void k_cancel(DevPool p, const int32_t* __restrict__ locs, long long 
   atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_CANCELS]), 1ull);
 }
 
-__global__ void __launch_bounds__(kAllocThreads)
-k_append(DevPool p, int32_t sid, int32_t n_tokens, int32_t* __restrict__ pages,
-         int32_t* __restrict__ count, const long long* __restrict__ gate,
-         const long long* __restrict__ sid_dev, StepFinish fin, const long long* __restrict__ R) {
-  pdl_entry();
-  __shared__ long long m_s, nb_s, ctx_s;
-  if (gate && *gate != 0) {   // an earlier step of lv_make_resident did not complete
-    if (threadIdx.x == 0) {
-      if (count) *count = 0;
-      if (fin.on) finish_step(p, fin, R);
-    }
-    return;
-  }
-  if (sid_dev) sid = (int32_t)*sid_dev;
-  if (threadIdx.x == 0) {
-    long long m = -1;
-    if (sid >= 0 && sid < p.S && n_tokens >= 0) {
-      const long long ctx = p.sess[sid].ctx_tokens;
-      const long long nb = (ctx + p.T - 1) / p.T;
-      const long long nctx = ctx + n_tokens;
-      const long long nnb = (nctx + p.T - 1) / p.T;
-      if (nnb > p.maxB || nctx > 0x7fffffffll) {
-        set_error(p.ctl, LV_ERR_BOUNDS, sid);
-      } else {
-        m = nnb - nb;
-        if (m > 0) {
-          const long long before = (long long)atomicAdd(
-              reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]), (unsigned long long)m);
-          if (before + m > p.budget) {
-            atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]),
-                      (unsigned long long)(-m));
-            set_error(p.ctl, LV_ERR_NO_HBM, sid);
-            m = -1;
+// ---------------------------------------------------------------- step
+// A device-driven step -- lv_turn, lv_make_resident, lv_evict -- as one kernel of one CTA,
+// followed by the exchange copy: pick the turn's session, begin the turn, list its host-tier
+// blocks, the deficit, the ranking, the victims, the plan and its commits, the growth, and
+// the step's end.  It reads per-session counts, the rows of the sessions concerned and the
+// bitmaps, so what bounds it is the chain of dependent reads.  As six to eight kernels in a
+// row (pick, prepare, order, census of every table row, emission, plan, append) these
+// decisions took 25-27 us of a turn of 16 or 1000 sessions, and 24 us of an eviction; as
+// one they take 17-19 and 12 us, and a turn of eight sessions that moves 24 pages of
+// 16 KiB each way went from 47.2 to 34.6 us (45 pages of 192 KiB with 1000 sessions: from
+// 106 to 97).
+constexpr int kSelectRounds = 8;    // sessions taken by repeated maximum before the keys are sorted
+
+// The step's arguments beyond the pool.
+struct StepArgs {
+  ResidentScratch rs;
+  int32_t sid;                      // -1: lv_turn picks from cand
+  const int32_t* cand;
+  int32_t n_cand;
+  const unsigned long long* keys;   // the loads' order, or null: ascending block id
+  long long now_us;
+  long long audio_us, units;        // lv_turn: LV_EV_TURN_END's a and b
+  long long max_load;               // preload admission (< 0: no limit)
+  long long evict;                  // lv_evict: pages to free; -1 for the other steps
+  int32_t append_tokens;
+  int32_t epoch;
+  int turn, preload;
+  // kStepAll, or in two parts around k_order_loads: kStepList up to the list of loads,
+  // kStepMove the rest
+  int part;
+  int copy_bits;                    // the bitmaps fit in shared memory
+  lv_resident_result* out;          // may be null
+};
+enum { kStepAll = 0, kStepList = 1, kStepMove = 2 };
+
+// Dynamic shared memory of k_step: [n2] keys and [n2] places and [n2] counts of the ranking,
+// [kStepItems] keys and [kStepItems] indexes of the loads' order, both bitmaps.
+struct StepLayout {
+  int n2;
+  size_t off, cnt, load, bits, total;
+};
+
+__host__ __device__ inline StepLayout step_layout(const DevPool& p, bool ordered, bool copy_bits) {
+  StepLayout l{};
+  l.n2 = 32;
+  while (l.n2 < p.S) l.n2 *= 2;
+  l.off = (size_t)l.n2 * 8;
+  l.cnt = l.off + (size_t)l.n2 * 4;
+  l.load = l.cnt + (size_t)l.n2 * 4;
+  l.bits = l.load + (ordered ? (size_t)kStepItems * 12 : 0);
+  l.total = l.bits + (copy_bits ? (size_t)(((p.hbm_pages + 31) >> 5) + ((p.host_pages + 31) >> 5)) * 4 : 0);
+  return l;
+}
+
+// Bitonic sort of n (a power of two) entries in shared memory: keys descending, or, with an
+// index per key, (key, index) ascending.  Up to 64 entries take one warp.
+template <bool kIndexed>
+__device__ void sort_entries(unsigned long long* key, int* idx, int n) {
+  const bool one_warp = n <= 64;
+  const int step = one_warp ? 32 : kStepThreads;
+  if (!one_warp || threadIdx.x < 32) {
+    for (int k = 2; k <= n; k <<= 1) {
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        for (int i = threadIdx.x; i < n / 2; i += step) {
+          const int lo = ((i & ~(j - 1)) << 1) | (i & (j - 1)), hi = lo | j;
+          const unsigned long long x = key[lo], y = key[hi];
+          const bool first = (lo & k) == 0;
+          bool less = x < y;                     // lo's entry belongs after hi's in descending order
+          bool more = x > y;
+          if (kIndexed && x == y) {
+            less = idx[lo] < idx[hi];
+            more = idx[lo] > idx[hi];
+          }
+          const bool swap = kIndexed ? (first ? more : less) : (first ? less : more);
+          if (swap) {
+            key[lo] = y;
+            key[hi] = x;
+            if (kIndexed) {
+              const int t = idx[lo];
+              idx[lo] = idx[hi];
+              idx[hi] = t;
+            }
           }
         }
+        if (one_warp) __syncwarp();
+        else __syncthreads();
       }
-      nb_s = nb;
-      ctx_s = nctx;
-    } else {
-      set_error(p.ctl, LV_ERR_BOUNDS, sid);
     }
-    m_s = m;
   }
   __syncthreads();
-  const long long m = m_s;
-  if (m < 0) {
+}
+
+// The largest of every thread's v, to all of them (one barrier; two buffers as BlockScan).
+__device__ __forceinline__ unsigned long long block_max(unsigned long long v, StepShared& sh, int ph) {
+  const int lane = threadIdx.x & 31;
+  auto warp_max = [](unsigned long long x) {
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(x >> 32));
+    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(x >> 32) == hi ? (unsigned)x : 0u);
+    return (unsigned long long)hi << 32 | lo;
+  };
+  v = warp_max(v);
+  if (lane == 0) sh.best[ph][threadIdx.x >> 5] = v;
+  __syncthreads();
+  return warp_max(lane < kStepWarps ? sh.best[ph][lane] : 0ull);
+}
+
+__device__ __forceinline__ int32_t session_of_key(unsigned long long key) {
+  return 0x7fffffff - (int32_t)(key & 0x7fffffffull);
+}
+
+// Writes the victims of one session, positions off.. of the order while below n_out.  By the
+// whole CTA (kWhole) or by one warp.
+template <bool kWhole>
+__device__ void emit_session(const DevPool& p, int32_t s, long long off, long long n_out, lv_victim* near,
+                             lv_victim* far, BlockScan& scan) {
+  const int32_t nb = nblocks_of(p, s);
+  const int32_t* row = p.table + (size_t)s * p.maxB;
+  const bool suffix = p.within == LV_SUFFIX_FIRST;
+  long long pos0 = off;
+  auto put = [&](long long pos, int32_t b, int32_t e) {
+    if (near) near[pos] = lv_victim{s, b, e};
+    far[pos] = lv_victim{s, b, e};
+  };
+  if (kWhole) {
+    for (int32_t q0 = 0; q0 < nb && pos0 < n_out; q0 += kStepThreads) {
+      const int32_t q = q0 + threadIdx.x;
+      const int32_t b = suffix ? nb - 1 - q : q;
+      const int32_t e = q < nb ? row[b] : -1;
+      int chunk;
+      const long long pos = pos0 + scan.rank(e >= 0, &chunk);
+      if (e >= 0 && pos < n_out) put(pos, b, e);
+      pos0 += chunk;
+    }
+  } else {
+    const int lane = threadIdx.x & 31;
+    for (int32_t q0 = 0; q0 < nb && pos0 < n_out; q0 += 128) {
+      int32_t e[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int32_t q = q0 + u * 32 + lane;
+        e[u] = q < nb ? row[suffix ? nb - 1 - q : q] : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int32_t q = q0 + u * 32 + lane;
+        const unsigned has = __ballot_sync(0xffffffffu, e[u] >= 0);
+        const long long pos = pos0 + __popc(has & ((1u << lane) - 1u));
+        if (e[u] >= 0 && pos < n_out) put(pos, suffix ? nb - 1 - q : q, e[u]);
+        pos0 += __popc(has);
+      }
+    }
+  }
+}
+
+// The sessions that the first n_out positions of the victim order touch.
+struct Selected {
+  int m;                // sessions
+  bool sorted;          // in keys / off (the sorted keys), else in sh.sel_sid / sh.sel_off
+  long long n_out;      // min(k, total)
+  long long total;      // resident blocks of all candidates
+};
+
+// Ranks by the keys and counts in shared memory (keys[s] != 0 for candidates with at least
+// one resident block) and finds the sessions of the first k victims.  Mostly a few sessions
+// hold k blocks: they are found by repeated maximum, about 0.15 us each; after kSelectRounds
+// the keys are sorted.  Keys are distinct (each holds its session).
+__device__ Selected select_sessions(const DevPool& p, unsigned long long* keys, int* off, const int* cnt,
+                                    int n2, long long k, StepShared& sh, BlockScan& scan) {
+  int mine = 0;
+  for (int s = threadIdx.x; s < p.S; s += kStepThreads)
+    if (keys[s]) mine += cnt[s];
+  Selected r{};
+  int total;
+  scan.sum(mine, &total);
+  r.total = total;
+  r.n_out = k < total ? k : total;
+  unsigned long long last = ~0ull;
+  long long at = 0;
+  while (at < r.n_out && r.m < kSelectRounds) {
+    unsigned long long v = 0;
+    for (int s = threadIdx.x; s < p.S; s += kStepThreads) {
+      const unsigned long long x = keys[s];
+      if ((r.m == 0 || x < last) && x > v) v = x;
+    }
+    last = block_max(v, sh, r.m & 1);
+    const int32_t s = session_of_key(last);
     if (threadIdx.x == 0) {
-      if (count) *count = 0;
-      if (fin.on) finish_step(p, fin, R);
+      sh.sel_sid[r.m] = s;
+      sh.sel_off[r.m] = (int)at;
     }
-    return;
+    at += cnt[s];
+    ++r.m;
   }
-  if (m > 0) block_alloc_lowest<kAllocThreads>(p.bits_hbm, p.hbm_pages, m, pages);
+  if (at < r.n_out) {
+    r.sorted = true;
+    __syncthreads();
+    for (int s = p.S + threadIdx.x; s < n2; s += kStepThreads) keys[s] = 0ull;
+    __syncthreads();
+    sort_entries<false>(keys, nullptr, n2);
+    long long run = 0;
+    int m = 0;
+    for (int i0 = 0; i0 < n2 && run < r.n_out; i0 += kStepThreads) {
+      const int i = i0 + threadIdx.x;
+      const unsigned long long x = i < n2 ? keys[i] : 0ull;
+      int chunk;
+      const long long pos = run + scan.sum(x ? cnt[session_of_key(x)] : 0, &chunk);
+      const bool in = x && pos < r.n_out;
+      if (in) off[i] = (int)pos;
+      m += __syncthreads_count(in);
+      run += chunk;
+    }
+    r.m = m;
+  }
   __syncthreads();
-  for (long long i = threadIdx.x; i < m; i += kAllocThreads) {
-    const int32_t pg = pages[i];
-    const int32_t b = (int32_t)(nb_s + i);
-    p.table[(size_t)sid * p.maxB + b] = pg;
-    p.own_hbm[pg] = owner_key(sid, b);
-  }
-  if (threadIdx.x == 0) {
-    // inclusive tiers: the partially filled last block gains rows, its clean copy is stale
-    const long long old_ctx = ctx_s - n_tokens;
-    if (p.incl && n_tokens > 0 && nb_s > 0 && old_ctx % p.T != 0) {
-      const size_t ti = (size_t)sid * p.maxB + (nb_s - 1);
-      const int32_t g = p.shadow[ti];
-      if (g >= 0 && g < p.host_pages) {
-        p.shadow[ti] = -1;
-        p.own_host[g] = kOwnerNone;
-        atomicAnd(&p.bits_host[g >> 5], ~(1u << (g & 31)));
-        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HOST_ALLOC]), (unsigned long long)-1ll);
-        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_CLEAN]), (unsigned long long)-1ll);
-        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_CLEAN_DROPPED]), 1ull);
-      }
-    }
-    p.sess[sid].ctx_tokens = (int32_t)ctx_s;
-    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_APPENDED]), (unsigned long long)m);
-    if (count) *count = (int32_t)m;
-    if (fin.on) finish_step(p, fin, R);   // a device-driven step's end, after its growth
-  }
+  return r;
 }
 
-// -------------------------------------------------------- make_resident
-
-// lv_turn's start, run first by k_resident_prepare: the turn's session (sid, or the
-// first candidate with a hit, else the first candidate) into R[R_SID], then
-// LV_EV_TURN_BEGIN for it.  Returns the session, -1 when the pick failed.
-__device__ int32_t turn_begin(const DevPool& p, int32_t sid, const TurnStart& ts, long long* R) {
-  __shared__ int first;
-  __shared__ int32_t picked;
-  if (threadIdx.x == 0) first = ts.n_cand;
-  __syncthreads();
-  if (sid < 0) {
-    int mine = ts.n_cand;
-    for (int c = threadIdx.x; c < ts.n_cand; c += blockDim.x)
-      if (ts.hit[c]) { mine = c; break; }
-    if (mine < ts.n_cand) atomicMin(&first, mine);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int32_t s = sid;
-    if (s < 0) {
-      const int c = first < ts.n_cand ? first : 0;
-      s = ts.cand[c];
-      if (s < 0 || s >= p.S) {
-        set_error(p.ctl, LV_ERR_BOUNDS, c);
-        s = -1;
-      }
-    }
-    R[R_SID] = s;
-    if (s >= 0) {
-      lv_session_state st = p.sess[s];
-      lv_event x{};
-      x.kind = LV_EV_TURN_BEGIN;
-      x.sid = s;
-      x.t_us = ts.now_us;
-      apply_event(p, st, x);
-      p.sess[s] = st;
-      atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_EVENTS]), 1ull);
-    }
-    picked = s;
-  }
-  __syncthreads();
-  return picked;
-}
-
-// One CTA: sid's host-tier blocks (ascending), the deficit k and the admission; for
-// lv_turn (ts.on) the turn's start first.
-__global__ void __launch_bounds__(kCensusThreads)
-k_resident_prepare(DevPool p, int32_t sid, int32_t append_tokens, bool preload,
-                   long long max_load, int32_t* __restrict__ blocks, long long* __restrict__ R,
-                   const long long* __restrict__ sid_dev, TurnStart ts) {
+__global__ void __launch_bounds__(kStepThreads)
+k_step(DevPool p, StepArgs a) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ StepShared sh;
   pdl_entry();
-  if (ts.on) sid = turn_begin(p, sid, ts, R);
-  else if (sid_dev) sid = (int32_t)*sid_dev;
-  if (sid < 0 || sid >= p.S) {        // lv_turn's pick failed (already reported)
-    if (threadIdx.x == 0) {
-      R[R_K_SELECT] = 0; R[R_N_OUT] = 0; R[R_N_IN] = 0; R[R_STATUS] = LV_RESIDENT_FAILED;
-      R[R_K] = 0; R[R_GATE] = 1; R[R_APPENDED] = 0; R[R_FOUND] = 0;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const StepLayout lay = step_layout(p, a.keys != nullptr && a.part == kStepAll, a.copy_bits != 0);
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(dyn);
+  int* off = reinterpret_cast<int*>(dyn + lay.off);
+  int* cnt = reinterpret_cast<int*>(dyn + lay.cnt);
+  BlockScan scan{sh.ws, 0};
+  long long* R = a.rs.words;
+  const bool evict = a.evict >= 0;
+
+  // reads that depend on nothing: allocation counts, bitmaps, every session's key and count
+  const long long hbm_alloc = p.ctl[C_HBM_ALLOC], host_alloc = p.ctl[C_HOST_ALLOC];
+  TierBits hbm{}, host{};
+  if (a.part != kStepList) {
+    tier_bits(p, a.copy_bits ? reinterpret_cast<uint32_t*>(dyn + lay.bits) : nullptr, &hbm, &host);
+    const bool fallback = !evict && !a.preload;
+    for (int s = tid; s < p.S; s += kStepThreads) {
+      const int c = p.cnt[s].x;
+      cnt[s] = c;
+      keys[s] = c > 0 ? session_key(p, s, a.now_us, fallback) : 0ull;
     }
-    return;
+    if (tid == 0) R[R_CURSOR] = 0;
   }
-  const int32_t nb = nblocks_of(p, sid);
-  const int32_t* row = p.table + (size_t)sid * p.maxB;
-  long long run = 0;
-  for (int32_t q0 = 0; q0 < nb; q0 += kCensusThreads) {
-    const int32_t b = q0 + threadIdx.x;
-    const long long flag = (b < nb && row[b] <= -2) ? 1 : 0;
-    long long chunk;
-    const long long pos = run + block_excl_scan<kCensusThreads>(flag, &chunk);
-    if (flag) blocks[pos] = b;
-    run += chunk;
+
+  // the session: given, picked (the first candidate with a host-tier block, else the first), or none
+  int32_t sid = a.sid;
+  if (a.part == kStepMove) {
+    sid = (int32_t)R[R_SID];
+  } else if (a.turn && sid < 0) {
+    unsigned c = 0x7fffffffu;
+    int32_t s = -1;
+    for (int i = tid; i < a.n_cand; i += kStepThreads) {
+      const int32_t x = a.cand[i];
+      if (tid == 0 && i == 0) sh.pick[kStepWarps] = make_int2(0, x);
+      if (x >= 0 && x < p.S && p.cnt[x].y > 0) {
+        c = (unsigned)i;
+        s = x;
+        break;
+      }
+    }
+    __syncwarp();
+    const unsigned low = __reduce_min_sync(0xffffffffu, c);
+    if (c == low && (low != 0x7fffffffu || lane == 0)) sh.pick[tid >> 5] = make_int2((int)low, s);
+    __syncthreads();
+    const int2 w = lane < kStepWarps ? sh.pick[lane] : make_int2(0x7fffffff, -1);
+    const unsigned first = __reduce_min_sync(0xffffffffu, (unsigned)w.x);
+    if (first != 0x7fffffffu) {
+      const unsigned who = __ballot_sync(0xffffffffu, (unsigned)w.x == first);
+      sid = __shfl_sync(0xffffffffu, w.y, __ffs(who) - 1);
+    } else {
+      sid = sh.pick[kStepWarps].y;
+      if (sid < 0 || sid >= p.S) {
+        if (tid == 0) set_error(p.ctl, LV_ERR_BOUNDS, 0);
+        sid = -1;
+      }
+    }
   }
-  if (threadIdx.x == 0) {
-    const long long nh = run;
+  const bool have = sid >= 0 && sid < p.S;      // lv_evict has no session; a failed pick neither
+  if (a.turn && a.part != kStepMove && have && tid == 0) {
+    // LV_EV_TURN_BEGIN; only the fields it changes are written (others read this state now)
+    lv_session_state st = p.sess[sid];
+    lv_event x{};
+    x.kind = LV_EV_TURN_BEGIN;
+    x.sid = sid;
+    x.t_us = a.now_us;
+    apply_event(p, st, x);
+    p.sess[sid].flags = st.flags;
+    p.sess[sid].protect_until_us = st.protect_until_us;
+    p.sess[sid].last_use_us = st.last_use_us;
+    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_EVENTS]), 1ull);
+  }
+
+  // the session's host-tier blocks, in load order
+  int status = evict || have ? LV_RESIDENT_DONE : LV_RESIDENT_FAILED;
+  long long nh = 0, new_blocks = 0, k = 0;
+  const int32_t* blks = a.keys ? a.rs.loads : a.rs.blocks;
+  const int32_t* gslot = nullptr;
+  if (!evict && have) {
     const long long ctx = p.sess[sid].ctx_tokens;
-    const long long nctx = ctx + append_tokens;
+    const int32_t nb = nblocks_of(p, sid);
+    const long long nctx = ctx + a.append_tokens;
     const long long nnb = (nctx + p.T - 1) / p.T;
-    int status = LV_RESIDENT_DONE;
-    long long k = 0;
-    if (nnb > p.maxB || nctx > 0x7fffffffll) {
-      set_error(p.ctl, LV_ERR_BOUNDS, sid);
+    const bool over = nnb > p.maxB || nctx > 0x7fffffffll;
+    new_blocks = nnb - nb;
+    if (a.part == kStepMove) {
+      nh = R[R_N_IN];
+    } else if (p.cnt[sid].y > 0) {
+      const int32_t* row = p.table + (size_t)sid * p.maxB;
+      for (int32_t q0 = 0; q0 < nb; q0 += kStepThreads) {
+        const int32_t b = q0 + tid;
+        const int32_t e = b < nb ? row[b] : -1;
+        int chunk;
+        const long long pos = nh + scan.rank(e <= -2, &chunk);
+        if (e <= -2) {
+          if (pos < kStepItems) {
+            sh.blks[pos] = b;
+            sh.gslot[pos] = (int32_t)(-(long long)e - 2);
+          }
+          a.rs.blocks[pos] = b;
+        }
+        nh += chunk;
+      }
+      __syncthreads();
+      if (nh <= kStepItems) {
+        if (a.keys && a.part == kStepAll) {
+          // the caller's order: ascending (key, block id); the list is in block order already
+          unsigned long long* lk = reinterpret_cast<unsigned long long*>(dyn + lay.load);
+          int* li = reinterpret_cast<int*>(lk + kStepItems);
+          int n = 32;
+          while (n < nh) n *= 2;
+          for (int i = tid; i < n; i += kStepThreads) {
+            lk[i] = i < nh ? a.keys[sh.blks[i]] : ~0ull;
+            li[i] = i;
+          }
+          __syncthreads();
+          sort_entries<true>(lk, li, n);
+          static_assert(kStepItems <= 2 * kStepThreads, "two loads per thread");
+          int32_t b[2], g[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int i = tid + u * kStepThreads;
+            if (i < nh) {
+              b[u] = sh.blks[li[i]];
+              g[u] = sh.gslot[li[i]];
+            }
+          }
+          __syncthreads();
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int i = tid + u * kStepThreads;
+            if (i < nh) {
+              sh.blks[i] = b[u];
+              sh.gslot[i] = g[u];
+              a.rs.loads[i] = b[u];
+            }
+          }
+          __syncthreads();
+        }
+        blks = sh.blks;
+        gslot = sh.gslot;
+      }
+    }
+    if (over) {
+      if (tid == 0 && a.part != kStepMove) set_error(p.ctl, LV_ERR_BOUNDS, sid);
       status = LV_RESIDENT_FAILED;
     } else {
-      const long long need = nh + (nnb - nb);
-      const long long free_pages = p.budget - p.ctl[C_HBM_ALLOC];
+      const long long need = nh + new_blocks, free_pages = p.budget - hbm_alloc;
       k = need - free_pages > 0 ? need - free_pages : 0;
-      if (preload && nh == 0) status = LV_RESIDENT_NOTHING;
-      else if (preload && max_load >= 0 && nh > max_load) status = LV_RESIDENT_SKIPPED;
+      if (a.preload && nh == 0) status = LV_RESIDENT_NOTHING;
+      else if (a.preload && a.max_load >= 0 && nh > a.max_load) status = LV_RESIDENT_SKIPPED;
+      if (tid == 0 && status == LV_RESIDENT_SKIPPED)
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_PRELOADS_SKIPPED]), 1ull);
     }
-    const bool go = status == LV_RESIDENT_DONE;
-    R[R_K_SELECT] = go ? k : 0;
-    R[R_N_OUT] = 0;
-    R[R_N_IN] = go ? nh : 0;
-    R[R_STATUS] = status;
-    R[R_K] = k;
-    R[R_GATE] = go ? 0 : 1;
-    R[R_APPENDED] = 0;
-    R[R_FOUND] = 0;
-    if (preload && status == LV_RESIDENT_SKIPPED)
-      atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_PRELOADS_SKIPPED]), 1ull);
+  }
+  if (a.part == kStepList) {
+    if (tid == 0) {
+      R[R_SID] = sid;
+      R[R_N_IN] = nh;
+    }
+    return;
+  }
+  if (evict) k = a.evict;
+  const bool go = status == LV_RESIDENT_DONE;
+  const long long want = go ? k : 0;            // victims asked for
+  __syncthreads();                              // keys and counts are complete
+  if (a.turn && have && tid == 0) keys[sid] = 0ull;   // RUNNING: never a victim (its key may predate that)
+  __syncthreads();
+
+  Selected sel{};
+  if (want > 0) sel = select_sessions(p, keys, off, cnt, lay.n2, want, sh, scan);
+  if (tid == 0) {
+    p.ctl[C_SEL_COUNT] = sel.n_out;
+    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_SELECTS]), 1ull);
+    if (!evict && !a.preload) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_FALLBACK]), 1ull);
+    if (want > 0) {
+      p.ctl[C_SEL_TOTAL] = sel.total;
+      atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_VICTIMS]), (unsigned long long)sel.n_out);
+      if (sel.total < want) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_SHORTFALLS]), 1ull);
+    }
+  }
+  // the victims of the order's first n_out positions
+  lv_victim* near = sel.n_out <= kStepItems ? sh.v : nullptr;
+  if (sel.m <= 2 && !sel.sorted) {
+    for (int r = 0; r < sel.m; ++r)
+      emit_session<true>(p, sh.sel_sid[r], sh.sel_off[r], sel.n_out, near, a.rs.victims, scan);
+  } else {
+    for (int r = tid >> 5; r < sel.m; r += kStepWarps)
+      emit_session<false>(p, sel.sorted ? session_of_key(keys[r]) : sh.sel_sid[r],
+                          sel.sorted ? off[r] : sh.sel_off[r], sel.n_out, near, a.rs.victims, scan);
+  }
+  // the gate: a shortfall stops the step (a preload is skipped, a foreground turn fails);
+  // lv_evict takes what there is
+  long long n_out = sel.n_out, n_in = go ? nh : 0;
+  bool grow = go;
+  if (evict) {
+    if (n_out == 0) status = LV_RESIDENT_NOTHING;
+    grow = false;
+  } else if (go && sel.n_out < k) {
+    if (a.preload) {
+      status = LV_RESIDENT_SKIPPED;
+      if (tid == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_PRELOADS_SKIPPED]), 1ull);
+    } else {
+      status = LV_RESIDENT_FAILED;
+      if (tid == 0) set_error(p.ctl, LV_ERR_NO_HBM, k);
+    }
+    n_out = n_in = 0;
+    grow = false;
+  }
+  __syncthreads();                              // the victims are listed
+  MovePlan m{near ? near : a.rs.victims, n_out, sid, blks, gslot, n_in, near ? sh.slots : a.rs.slots,
+             n_in <= kStepItems ? sh.pages : a.rs.pages, a.rs.slots, a.rs.pages, a.rs.tasks,
+             R + R_N_TASKS, a.epoch, p.page_tag};
+  if (plan_moves<false>(p, m, hbm, host, hbm_alloc, host_alloc, sh, scan) && n_out > 0) {
+    // the victims' sessions: fewer blocks in HBM, more in the host tier
+    for (int r = tid; r < sel.m; r += kStepThreads) {
+      const int32_t s = sel.sorted ? session_of_key(keys[r]) : sh.sel_sid[r];
+      const long long at = sel.sorted ? off[r] : sh.sel_off[r];
+      const int take = (int)(n_out - at < cnt[s] ? n_out - at : cnt[s]);
+      atomicAdd(&p.cnt[s].x, -take);
+      atomicAdd(&p.cnt[s].y, take);
+    }
+  }
+  long long appended = 0;
+  if (grow && a.append_tokens > 0) {
+    __syncthreads();                            // the commits of the plan
+    appended = append_tokens_to(p, sid, a.append_tokens, a.rs.append, hbm, scan, &sh.bad);
+    if (appended < 0) appended = 0;
+  }
+  if (tid != 0) return;
+  // the step's end: LV_EV_TURN_END unless the turn failed, a completed preload's protection,
+  // and the result
+  if (a.turn && have && status != LV_RESIDENT_FAILED) {
+    lv_session_state st = p.sess[sid];
+    lv_event x{};
+    x.kind = LV_EV_TURN_END;
+    x.sid = sid;
+    x.t_us = a.now_us;
+    x.a = a.audio_us;
+    x.b = a.units;
+    apply_event(p, st, x);
+    p.sess[sid] = st;
+    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_EVENTS]), 1ull);
+  }
+  if (a.preload && status == LV_RESIDENT_DONE) {
+    p.sess[sid].protect_until_us = a.now_us + p.protect_us;   // warmed KV (Section 5.2)
+    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_PRELOADS]), 1ull);
+  }
+  if (a.out) {
+    lv_resident_result r;
+    r.k = k;
+    r.n_found = go ? sel.n_out : 0;
+    r.n_victims = n_out;
+    r.n_loaded = n_in;
+    r.n_appended = appended;
+    r.status = status;
+    r.sid = sid;
+    *a.out = r;
   }
 }
 
 constexpr int kOrderThreads = 256;
 
-// The caller's load order: host-tier block i of the session (ascending in
-// `blocks`, R[R_N_IN] of them) goes to position #{j : (key[b_j], b_j) <
-// (key[b_i], b_i)} of `loads` -- ascending (key, block id).  One warp per block.
+// The caller's load order where a session may have more host-tier blocks than k_step sorts
+// in shared memory: host-tier block i of the session (ascending in `blocks`, R[R_N_IN] of
+// them) goes to position #{j : (key[b_j], b_j) < (key[b_i], b_i)} of `loads` -- ascending
+// (key, block id).  One warp per block.
 __global__ void __launch_bounds__(kOrderThreads)
 k_order_loads(const long long* __restrict__ R, const int32_t* __restrict__ blocks,
               const unsigned long long* __restrict__ key, int32_t* __restrict__ loads) {
@@ -1845,75 +2397,6 @@ k_order_loads(const long long* __restrict__ R, const int32_t* __restrict__ block
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
   if (lane == 0) loads[rank] = bi;
-}
-
-
-// The step's result and, for lv_turn (turn_end), LV_EV_TURN_END for the turn's session
-// unless its KV could not be made resident.
-__device__ void finish_step(const DevPool& p, const StepFinish& f, const long long* __restrict__ R) {
-  int32_t sid = f.sid_dev ? (int32_t)*f.sid_dev : f.sid;
-  const int status = (int)R[R_STATUS];
-  if (f.turn_end && sid >= 0 && sid < p.S && status != LV_RESIDENT_FAILED) {
-    lv_session_state st = p.sess[sid];
-    lv_event x{};
-    x.kind = LV_EV_TURN_END;
-    x.sid = sid;
-    x.t_us = f.now_us;
-    x.a = f.audio_us;
-    x.b = f.units;
-    apply_event(p, st, x);
-    p.sess[sid] = st;
-    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_EVENTS]), 1ull);
-  }
-  if (f.preload && status == LV_RESIDENT_DONE) {
-    p.sess[sid].protect_until_us = f.now_us + p.protect_us;   // warmed KV (Section 5.2)
-    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_PRELOADS]), 1ull);
-  }
-  if (f.out) {
-    lv_resident_result r;
-    r.k = R[R_K];
-    r.n_found = R[R_FOUND];
-    r.n_victims = R[R_N_OUT];
-    r.n_loaded = R[R_N_IN];
-    r.n_appended = (int32_t)R[R_APPENDED];
-    r.status = status;
-    r.sid = sid;
-    *f.out = r;
-  }
-}
-
-// ----------------------------------------------------------------- evict
-// lv_evict: up to k victims by the normal order (no fallback tier), fewer when
-// there are fewer candidates (GATE_EVICT); nothing is loaded.
-__global__ void k_evict_prepare(long long k, long long* __restrict__ R) {
-  pdl_entry();
-  if (threadIdx.x != 0) return;
-  R[R_K_SELECT] = k;
-  R[R_N_OUT] = 0;
-  R[R_N_IN] = 0;
-  R[R_STATUS] = LV_RESIDENT_DONE;
-  R[R_K] = k;
-  R[R_GATE] = 1;
-  R[R_APPENDED] = 0;
-  R[R_FOUND] = 0;
-  R[R_SID] = -1;
-}
-
-
-// ------------------------------------------------------------------ turn
-// lv_turn's pick: CTA c reports whether candidate c has a block in the host tier.
-__global__ void __launch_bounds__(kCensusThreads)
-k_pick_scan(DevPool p, const int32_t* __restrict__ cand, int32_t* __restrict__ hit) {
-  pdl_entry();
-  const int32_t s = cand[blockIdx.x];
-  int any = 0;
-  if (s >= 0 && s < p.S) {
-    const int32_t nb = nblocks_of(p, s);
-    const int32_t* row = p.table + (size_t)s * p.maxB;
-    for (int32_t b = threadIdx.x; b < nb && !any; b += kCensusThreads) any = row[b] <= -2;
-  }
-  any = __syncthreads_or(any);
-  if (threadIdx.x == 0) hit[blockIdx.x] = any;
 }
 
 // ------------------------------------------------------------- checksums
@@ -2052,43 +2535,11 @@ cudaError_t launch_session_set(const DevPool& p, const lv_session_state* in, int
   return cudaGetLastError();
 }
 
-thread_local std::vector<LaunchRecord>* t_recorder = nullptr;
-
-void set_launch_recorder(std::vector<LaunchRecord>* rec) { t_recorder = rec; }
-
-cudaError_t replay_launches(const std::vector<LaunchRecord>& recs, cudaStream_t s) {
-  for (const LaunchRecord& r : recs) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = r.grid;
-    cfg.blockDim = r.block;
-    cfg.dynamicSmemBytes = r.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = r.pdl ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelExC(&cfg, r.func, const_cast<void**>(r.args.data()));
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
 // A launch that lets the kernel be scheduled while the previous kernel on `s`
-// still runs; the kernel must begin with pdl_entry().  With a recorder set on this
-// thread the launch is recorded (its arguments converted to the kernel's parameter
-// types and kept) instead of issued.
+// still runs; the kernel must begin with pdl_entry() or pdl_wait().
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem,
                        cudaStream_t s, Args&&... args) {
-  if (t_recorder) {
-    using Values = std::tuple<std::decay_t<KArgs>...>;
-    auto values = std::make_shared<Values>(std::forward<Args>(args)...);
-    LaunchRecord r{reinterpret_cast<const void*>(kernel), grid, dim3(block), smem, true, values, {}};
-    std::apply([&r](auto&... x) { (r.args.push_back(static_cast<void*>(&x)), ...); }, *values);
-    t_recorder->push_back(std::move(r));
-    return cudaSuccess;
-  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
@@ -2108,18 +2559,17 @@ cudaError_t launch_events(const DevPool& p, const lv_event* ev, int64_t n, cudaS
 }
 
 cudaError_t launch_select(const DevPool& p, int64_t now_us, int64_t k, bool fallback,
-                          lv_victim* out, long long* count_dev, cudaStream_t s, int /*num_sms*/,
-                          const long long* k_dev) {
+                          lv_victim* out, long long* count_dev, cudaStream_t s) {
   cudaError_t e = launch_pdl(k_rank_census, (unsigned)p.S, kCensusThreads, 0, s, p, (long long)now_us,
-                             fallback, k_dev);
+                             fallback);
   if (e != cudaSuccess) return e;
   if (p.S > kEmitScanMax) {
     const dim3 grid((unsigned)((p.S + kPrefixTile - 1) / kPrefixTile),
                     (unsigned)((p.S + kPrefixChunk - 1) / kPrefixChunk));
-    e = launch_pdl(k_rank_prefix, grid, kPrefixTile, 0, s, p, k_dev);
+    e = launch_pdl(k_rank_prefix, grid, kPrefixTile, 0, s, p);
     if (e != cudaSuccess) return e;
   }
-  e = launch_pdl(k_rank_emit, (unsigned)p.S, kEmitThreads, 0, s, p, (long long)k, k_dev, fallback,
+  e = launch_pdl(k_rank_emit, (unsigned)p.S, kEmitThreads, 0, s, p, (long long)k, fallback,
                  count_dev, out);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
@@ -2160,21 +2610,35 @@ cudaError_t launch_swap_in(const DevPool& p, int32_t sid, const int32_t* blks, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_exchange(const DevPool& p, const lv_victim* v, int64_t n_out, int32_t sid,
-                            const int32_t* blks, int64_t n_in, int32_t* slots, int32_t* pages,
-                            int4* tasks, long long* n_tasks, int32_t epoch,
-                            unsigned long long* page_tag, cudaStream_t s, int copy_ctas,
-                            const long long* counts_dev, long long max_units, const EventPair* ev,
-                            const long long* sid_dev, const CopyOffload* off, int gate,
-                            long long* cursor, const StepFinish* fin) {
-  long long* R = gate != GATE_NONE ? const_cast<long long*>(counts_dev) - R_N_OUT : nullptr;
-  if (R) cursor = R + R_CURSOR;
-  const StepFinish no_fin{};
-  cudaError_t le = launch_pdl(k_exchange_plan, 1, kPlanThreads, 0, s, p, v, (long long)n_out, sid,
-                              blks, (long long)n_in, slots, pages, tasks, n_tasks, epoch, page_tag,
-                              counts_dev, sid_dev, R, gate, cursor, fin && R ? *fin : no_fin);
-  if (le != cudaSuccess) return le;
-  const long long units = counts_dev ? max_units : (n_out + n_in) * (long long)p.J;
+// The largest dynamic shared memory of the one-CTA kernels beside their static lists.
+constexpr size_t kStepDynamic = 190 * 1024;
+
+bool bits_fit(const DevPool& p, size_t others) {
+  const size_t words = (size_t)(((p.hbm_pages + 31) >> 5) + ((p.host_pages + 31) >> 5));
+  return others + words * 4 <= kStepDynamic;
+}
+
+cudaError_t configure_step_kernels() {
+  cudaError_t e = cudaFuncSetAttribute(k_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStepDynamic);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_exchange_plan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStepDynamic);
+}
+
+cudaError_t launch_exchange_plan(const DevPool& p, const lv_victim* v, int64_t n_out, int32_t sid,
+                                 const int32_t* blks, int64_t n_in, int32_t* slots, int32_t* pages,
+                                 int4* tasks, long long* n_tasks, int32_t epoch,
+                                 unsigned long long* page_tag, cudaStream_t s, long long* cursor) {
+  const bool fit = bits_fit(p, 0);
+  const size_t smem = fit ? (size_t)(((p.hbm_pages + 31) >> 5) + ((p.host_pages + 31) >> 5)) * 4 : 0;
+  return launch_pdl(k_exchange_plan, 1, kStepThreads, smem, s, p, v, (long long)n_out, sid, blks,
+                    (long long)n_in, slots, pages, tasks, n_tasks, epoch, page_tag, cursor, fit ? 1 : 0);
+}
+
+// The copy of a plan's tasks (at most max_pages of them), on s or, with `off`, on the copy
+// stream after everything queued on s.
+static cudaError_t launch_copy(const DevPool& p, const int4* tasks, const long long* n_tasks,
+                               long long* cursor, long long max_pages, cudaStream_t s, int copy_ctas,
+                               const EventPair* ev, const CopyOffload* off) {
   cudaStream_t cs = s;
   if (off) {
     cudaError_t e = cudaEventRecord(off->planned, s);
@@ -2185,23 +2649,18 @@ cudaError_t launch_exchange(const DevPool& p, const lv_victim* v, int64_t n_out,
   if (ev) cudaEventRecord(ev->start, cs);
   else if (off && off->started) cudaEventRecord(off->started, cs);
   // the 16-byte copy takes whole pages in chunks, the TMA copy sub-pages
-  const unsigned grid = blocks_for(p.xstages > 0 ? units : units / p.J * copy_chunks(p), 1, copy_ctas);
+  const unsigned grid = blocks_for(max_pages * (p.xstages > 0 ? p.J : copy_chunks(p)), 1, copy_ctas);
+  cudaError_t le = cudaSuccess;
   if (p.xstages > 0) {
     const size_t smem = (size_t)p.xstages * 2 * p.P;
-    if (off || ev) {
-      k_exchange_copy_tma<<<grid, kStageThreads, smem, cs>>>(p, tasks, n_tasks, cursor);
-    } else {
-      le = launch_pdl(k_exchange_copy_tma, grid, kStageThreads, smem, cs, p, (const int4*)tasks,
-                      (const long long*)n_tasks, cursor);
-      if (le != cudaSuccess) return le;
-    }
+    if (off || ev) k_exchange_copy_tma<<<grid, kStageThreads, smem, cs>>>(p, tasks, n_tasks, cursor);
+    else le = launch_pdl(k_exchange_copy_tma, grid, kStageThreads, smem, cs, p, tasks, n_tasks, cursor);
   } else if (off || ev) {   // after an event wait or record: an ordinary launch
     k_exchange_copy<<<grid, kCopyThreads, 0, cs>>>(p, tasks, n_tasks, cursor);
   } else {
-    le = launch_pdl(k_exchange_copy, grid, kCopyThreads, 0, cs, p, (const int4*)tasks,
-                    (const long long*)n_tasks, cursor);
-    if (le != cudaSuccess) return le;
+    le = launch_pdl(k_exchange_copy, grid, kCopyThreads, 0, cs, p, tasks, n_tasks, cursor);
   }
+  if (le != cudaSuccess) return le;
   if (ev) cudaEventRecord(ev->end, cs);
   else if (off && off->finished) cudaEventRecord(off->finished, cs);
   if (off) {
@@ -2211,79 +2670,54 @@ cudaError_t launch_exchange(const DevPool& p, const lv_victim* v, int64_t n_out,
   return cudaGetLastError();
 }
 
-cudaError_t launch_make_resident(const DevPool& p, const ResidentScratch& rs, int32_t sid,
-                                 int64_t now_us, int32_t append_tokens, bool preload,
-                                 int64_t max_load, int32_t epoch, cudaStream_t s, int copy_ctas,
-                                 lv_resident_result* result, const EventPair* ev,
-                                 const long long* sid_dev, const CopyOffload* off,
-                                 const unsigned long long* load_keys, bool turn_end,
-                                 int64_t audio_us, int64_t units, const TurnStart* ts) {
-  long long* R = rs.words;
-  const TurnStart none{};
-  cudaError_t e = launch_pdl(k_resident_prepare, 1, kCensusThreads, 0, s, p, sid, append_tokens,
-                             preload, (long long)max_load, rs.blocks, R, sid_dev, ts ? *ts : none);
+cudaError_t launch_exchange(const DevPool& p, const lv_victim* v, int64_t n_out, int32_t sid,
+                            const int32_t* blks, int64_t n_in, int32_t* slots, int32_t* pages,
+                            int4* tasks, long long* n_tasks, int32_t epoch,
+                            unsigned long long* page_tag, cudaStream_t s, int copy_ctas,
+                            const EventPair* ev, long long* cursor) {
+  const cudaError_t e = launch_exchange_plan(p, v, n_out, sid, blks, n_in, slots, pages, tasks, n_tasks,
+                                             epoch, page_tag, s, cursor);
   if (e != cudaSuccess) return e;
-  if (load_keys) {
-    e = launch_pdl(k_order_loads, blocks_for(p.maxB, kOrderThreads / 32, 1ll << 30), kOrderThreads, 0,
-                   s, (const long long*)R, (const int32_t*)rs.blocks, load_keys, rs.loads);
-    if (e != cudaSuccess) return e;
-  }
-  e = launch_select(p, now_us, 0, !preload, rs.victims, nullptr, s, 0, R + R_K_SELECT);
-  if (e != cudaSuccess) return e;
-  const long long max_units = ((long long)p.budget + p.maxB) * p.J;
-  // the step's end (turn end, preload protection, result): in the plan kernel when no
-  // append follows it, else in a kernel of its own after the append
-  const StepFinish fin{true, sid, sid_dev, (long long)now_us, preload, turn_end, (long long)audio_us,
-                       (long long)units, result};
-  e = launch_exchange(p, rs.victims, 0, sid, load_keys ? rs.loads : rs.blocks, 0, rs.slots, rs.pages,
-                      rs.tasks, R + R_N_TASKS, epoch, p.page_tag, s, copy_ctas, R + R_N_OUT, max_units,
-                      ev, sid_dev, off, preload ? GATE_PRELOAD : GATE_RESIDENT, nullptr,
-                      append_tokens > 0 ? nullptr : &fin);
-  if (e != cudaSuccess) return e;
-  if (append_tokens > 0) {   // the growth, then the step's end in the same kernel
-    e = launch_append(p, sid, append_tokens, rs.append, reinterpret_cast<int32_t*>(R + R_APPENDED), s,
-                      R + R_GATE, sid_dev, &fin, R);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaGetLastError();
+  return launch_copy(p, tasks, n_tasks, cursor, n_out + n_in, s, copy_ctas, ev, nullptr);
 }
 
-cudaError_t launch_evict(const DevPool& p, const ResidentScratch& rs, int64_t now_us, int64_t k,
-                         int32_t epoch, cudaStream_t s, int copy_ctas, lv_resident_result* result,
-                         const EventPair* ev, const CopyOffload* off) {
-  long long* R = rs.words;
-  cudaError_t e = launch_pdl(k_evict_prepare, 1, 32, 0, s, (long long)k, R);
+cudaError_t launch_step(const DevPool& p, const ResidentScratch& rs, const StepCall& c, int32_t epoch,
+                        cudaStream_t s, int copy_ctas, const EventPair* ev, const CopyOffload* off) {
+  StepArgs a{};
+  a.rs = rs;
+  a.sid = c.sid;
+  a.cand = c.cand;
+  a.n_cand = c.n_cand;
+  a.keys = c.load_keys;
+  a.now_us = c.now_us;
+  a.audio_us = c.audio_us;
+  a.units = c.units;
+  a.max_load = c.max_load;
+  a.evict = c.evict;
+  a.append_tokens = c.append_tokens;
+  a.epoch = epoch;
+  a.turn = c.turn;
+  a.preload = c.preload;
+  a.out = c.out;
+  // up to kStepItems loads are ordered inside the step; a session that may have more takes
+  // the grid-wide ordering kernel between two parts of it (one warp per block: n^2
+  // comparisons over the whole GPU instead of over one CTA)
+  const bool split = c.load_keys && p.maxB > kStepItems;
+  a.copy_bits = bits_fit(p, step_layout(p, c.load_keys && !split, false).total) ? 1 : 0;
+  a.part = split ? kStepList : kStepAll;
+  const size_t smem = step_layout(p, c.load_keys && !split, a.copy_bits != 0).total;
+  cudaError_t e = launch_pdl(k_step, 1, kStepThreads, split ? 0 : smem, s, p, a);
   if (e != cudaSuccess) return e;
-  e = launch_select(p, now_us, 0, false, rs.victims, nullptr, s, 0, R + R_K_SELECT);
-  if (e != cudaSuccess) return e;
-  const long long max_units = (long long)p.budget * p.J;
-  const StepFinish fin{true, -1, nullptr, (long long)now_us, false, false, 0, 0, result};
-  e = launch_exchange(p, rs.victims, 0, -1, rs.blocks, 0, rs.slots, rs.pages, rs.tasks,
-                      R + R_N_TASKS, epoch, p.page_tag, s, copy_ctas, R + R_N_OUT, max_units, ev,
-                      nullptr, off, GATE_EVICT, nullptr, &fin);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
-}
-
-cudaError_t launch_turn(const DevPool& p, const ResidentScratch& rs, int32_t sid, const int32_t* cand,
-                        int32_t n_cand, int64_t now_us, int32_t append_tokens, int64_t audio_us,
-                        int64_t units, int32_t epoch, cudaStream_t s, int copy_ctas,
-                        lv_resident_result* result, const EventPair* ev, const CopyOffload* off,
-                        const unsigned long long* load_keys) {
-  long long* R = rs.words;
-  cudaError_t e0 = cudaSuccess;
-  if (sid < 0) {
-    e0 = launch_pdl(k_pick_scan, (unsigned)n_cand, kCensusThreads, 0, s, p, cand, rs.hits);
-    if (e0 != cudaSuccess) return e0;
+  if (split) {
+    e = launch_pdl(k_order_loads, blocks_for(p.maxB, kOrderThreads / 32, 1ll << 30), kOrderThreads, 0, s,
+                   (const long long*)rs.words, (const int32_t*)rs.blocks, c.load_keys, rs.loads);
+    if (e != cudaSuccess) return e;
+    a.part = kStepMove;
+    e = launch_pdl(k_step, 1, kStepThreads, smem, s, p, a);
+    if (e != cudaSuccess) return e;
   }
-  // turn start (in the prepare kernel), make resident, then (in its finish kernel)
-  // LV_EV_TURN_END
-  const TurnStart ts{true, cand, n_cand, rs.hits, (long long)now_us};
-  cudaError_t e = launch_make_resident(p, rs, sid, now_us, append_tokens, false, -1, epoch, s,
-                                       copy_ctas, result, ev, R + R_SID, off, load_keys, true,
-                                       audio_us, units, &ts);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  const long long most = c.evict >= 0 ? (long long)p.budget : (long long)p.budget + p.maxB;
+  return launch_copy(p, rs.tasks, rs.words + R_N_TASKS, rs.words + R_CURSOR, most, s, copy_ctas, ev, off);
 }
 
 // Zeroes `words` 32-bit words at p, which may be device memory or the device alias of
@@ -2387,16 +2821,6 @@ cudaError_t launch_tasks_pages(const DevPool& p, const int32_t* pages, int64_t n
   return cudaGetLastError();
 }
 
-cudaError_t launch_exchange_plan(const DevPool& p, const lv_victim* v, int64_t n_out, int32_t sid,
-                                 const int32_t* blks, int64_t n_in, int32_t* slots, int32_t* pages,
-                                 int4* tasks, long long* n_tasks, int32_t epoch,
-                                 unsigned long long* page_tag, cudaStream_t s) {
-  k_exchange_plan<<<1, kPlanThreads, 0, s>>>(p, v, n_out, sid, blks, n_in, slots, pages, tasks,
-                                             n_tasks, epoch, page_tag, nullptr, nullptr, nullptr,
-                                             (int)GATE_NONE, nullptr, StepFinish{});
-  return cudaGetLastError();
-}
-
 cudaError_t launch_remap(const DevPool& p, const lv_remap_entry* e, int64_t n, int32_t epoch,
                          cudaStream_t s, int num_sms, int per_thread) {
   if (n <= 0) return cudaSuccess;
@@ -2429,13 +2853,8 @@ cudaError_t launch_cancel(const DevPool& p, const int32_t* locs, int64_t n, cuda
 }
 
 cudaError_t launch_append(const DevPool& p, int32_t sid, int32_t n_tokens, int32_t* pages,
-                          int32_t* count, cudaStream_t s, const long long* gate,
-                          const long long* sid_dev, const StepFinish* fin, const long long* R) {
-  const StepFinish none{};
-  const cudaError_t e = launch_pdl(k_append, 1, kAllocThreads, 0, s, p, sid, n_tokens, pages, count,
-                                   gate, sid_dev, fin ? *fin : none, R);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+                          int32_t* count, cudaStream_t s) {
+  return launch_pdl(k_append, 1, kStepThreads, 0, s, p, sid, n_tokens, pages, count);
 }
 
 cudaError_t launch_counts(const DevPool& p, int32_t* hbm, int32_t* host, cudaStream_t s) {

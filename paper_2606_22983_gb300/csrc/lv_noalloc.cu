@@ -117,7 +117,7 @@ extern "C" lv_status lv_select_victims_noalloc(const lv_rank_params* prm,
   // keys and counts are rewritten for every session each call
   if (cudaMemsetAsync(p.ctl, 0, kCtlBytes, s) != cudaSuccess) return LV_ERR_CUDA;
   if (lv::launch_select(p, now_us, keff, (prm->flags & LV_SELECT_FALLBACK) != 0,
-                        static_cast<lv_victim*>(vout), static_cast<long long*>(cout), s, 0) !=
+                        static_cast<lv_victim*>(vout), static_cast<long long*>(cout), s) !=
       cudaSuccess)
     return LV_ERR_CUDA;
   return LV_OK;

@@ -32,6 +32,7 @@ LV_POLICY_NEXT_USE, LV_POLICY_LRU = 0, 1
 LV_TIERS_EXCLUSIVE, LV_TIERS_INCLUSIVE = 0, 1
 LV_RESIDENT_ASYNC_COPY = 2
 LV_VERSION = 3                     # include/lv.h
+STEP_ITEMS = 1024                  # loads of one turn that a device-driven step orders by itself
 EMIT_SCAN_MAX = 1024               # above this many sessions a ranking runs one more kernel
 LV_MODE_ASYNC = 16
 LV_RUNNING, LV_IMMEDIATE, LV_RESP_OPEN, LV_DONE_VALID = 1, 2, 4, 8

@@ -139,8 +139,7 @@ class KVManager:
             self.timer.start("resident")
         lv.lv_make_resident(pool.handle, sid, now_us, append_tokens, flags, -1, *outs,
                             self.res_h, pool.stream)
-        # prepare, census, emit, plan (with the step's end), copy; or the append with the end
-        pool.launches += 5 + pool.rank_extra + (1 if append_tokens else 0)
+        pool.launches += 2          # the step's decisions, the copy
         if self.timer:
             self.timer.stop("resident", None)
         if not rec_bufs:
@@ -193,8 +192,9 @@ class KVManager:
         lv.lv_turn(pool.handle, sid, now_us, append_tokens, reply_us, reply_units, outs, self.res_h,
                    cand, n_cand, pool.stream, lv.LV_RESIDENT_ASYNC_COPY if self.async_copy else 0,
                    load_keys)
-        pool.launches += 1 if load_keys is not None else 0
-        pool.launches += 5 + pool.rank_extra + (1 if sid < 0 else 0) + (1 if append_tokens else 0)
+        # the decisions and the copy; the decisions in two parts around the ordering kernel
+        # where a session may have more loads than one CTA sorts
+        pool.launches += 4 if load_keys is not None and pool.max_blocks > lv.STEP_ITEMS else 2
         if not rec_bufs:
             return sid
         pool.sync(raise_on_error=False)
@@ -405,7 +405,7 @@ class KVManager:
         outs = (pool.victims, pool.slots) if self.record else (None, None)
         lv.lv_evict(pool.handle, now_us, int(k), lv.LV_RESIDENT_ASYNC_COPY if self.async_copy else 0,
                     *outs, self.res_h, pool.stream)
-        pool.launches += 5 + pool.rank_extra
+        pool.launches += 2
         rec["k"] = int(k)
         if not self.record:
             return
