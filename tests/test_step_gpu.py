@@ -101,3 +101,54 @@ def test_turn_decisions(S, blocks, away, scatter, cap, grow):
         assert pool.victims[:len(want)].cpu().numpy().tolist() == [list(v) for v in want]
     finally:
         pool.close()
+
+
+@pytest.mark.parametrize("where", ["device", "pinned", "pageable", "overlapping", "misaligned"])
+@pytest.mark.parametrize("n_blocks", [20, 1500])
+def test_step_outputs_wherever_they_lie(where, n_blocks):
+    """The lists of a step are the same in device memory, where the kernel writes them itself, as
+    in host memory and in device arrays that it may not write: overlapping ones (each list is
+    copied in turn, so the last one stands) and one that is not aligned for 32-bit words."""
+    import torch
+    from paper_2606_22983_gb300 import lv
+    from paper_2606_22983_gb300.pool import KVPool
+    rng = np.random.default_rng(n_blocks)
+    S, away = 4, n_blocks - 3
+    budget, host = S * n_blocks - away, 2 * away + 8
+    pool = KVPool(layers=1, kv_heads=1, head_dim=8, max_sessions=S, max_blocks=n_blocks, hbm_pages=budget,
+                  hbm_budget_pages=budget, host_pages=host)
+    try:
+        table = np.full((S, n_blocks), -1, np.int32)
+        pages = rng.permutation(budget)
+        slots = rng.permutation(host)[:away]
+        table[0, 3:] = -(slots + 2)
+        table[0, :3] = pages[:3]
+        table[1:] = pages[3:].reshape(S - 1, n_blocks)
+        st = np.zeros(S, dtype=lv.SESSION_DTYPE)
+        st["gen_us"] = [0, 9_000_000, 8_000_000, 7_000_000]
+        pool.import_placement(table, np.full(S, n_blocks * T, np.int32))
+        pool.set_sessions(st)
+        sizes = [budget * 12, budget * 4, n_blocks * 4, n_blocks * 4]        # victims, slots, blocks, pages
+        at = np.concatenate([[0], np.cumsum([s + 16 for s in sizes])])
+        kw = dict(dtype=torch.uint8, device=pool.device) if where in ("device", "overlapping", "misaligned") else dict(dtype=torch.uint8)
+        buf = torch.zeros(int(at[-1]) + 16, **kw)
+        buf = buf.pin_memory() if where == "pinned" else buf
+        off = [int(x) for x in at[:4]]
+        if where == "misaligned":
+            off[1] += 2
+        if where == "overlapping":
+            off[2] = off[3] = off[0]           # pages lie over blocks and over the first victims
+        outs = tuple(buf.data_ptr() + o for o in off) + (None,)
+        lv.lv_turn(pool.handle, 0, 0, 0, 1_000_000, 10, outs, None, None, 0, pool.stream)
+        pool.sync()
+        got = [buf[o:o + s].cpu().numpy() for o, s in zip(off, sizes)]
+        want_victims = [(1, b, table[1, b]) for b in range(n_blocks - 1, 2, -1)]
+        want_slots = sorted(set(range(host)) - set(slots.tolist()))[:away]
+        want_pages = sorted(v[2] for v in want_victims)
+        assert got[1][:4 * away].copy().view(np.int32).tolist() == want_slots
+        assert got[3][:4 * away].copy().view(np.int32).tolist() == want_pages
+        if where != "overlapping":
+            assert got[0][:12 * away].copy().view(np.int32).reshape(-1, 3).tolist() == [list(v) for v in want_victims]
+            assert got[2][:4 * away].copy().view(np.int32).tolist() == list(range(3, n_blocks))
+    finally:
+        pool.close()
