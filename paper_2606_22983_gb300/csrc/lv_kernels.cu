@@ -53,12 +53,16 @@ __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Blocks of a context of `ctx` tokens, at most maxB (a 32-bit division: a 64-bit one costs
+// some 100 instructions in the chain of dependent reads).
+__device__ __forceinline__ int32_t blocks_of_context(const DevPool& p, int32_t ctx) {
+  if (ctx <= 0) return 0;
+  const uint32_t nb = ((uint32_t)ctx + (uint32_t)p.T - 1u) / (uint32_t)p.T;
+  return nb > (uint32_t)p.maxB ? p.maxB : (int32_t)nb;
+}
+
 __device__ __forceinline__ int32_t nblocks_of(const DevPool& p, int32_t sid) {
-  long long c = p.sess[sid].ctx_tokens;
-  long long nb = (c + p.T - 1) / p.T;
-  if (nb < 0) nb = 0;
-  if (nb > p.maxB) nb = p.maxB;
-  return (int32_t)nb;
+  return blocks_of_context(p, p.sess[sid].ctx_tokens);
 }
 
 // Exclusive scan over the block of NT threads; *total receives the sum.
@@ -344,6 +348,7 @@ constexpr int kEventChunk = 512;   // events staged in shared memory at a time (
 // every event's kind and session and counts them.
 __global__ void __launch_bounds__(kEventThreads)
 k_events(DevPool p, const lv_event* __restrict__ ev, long long n) {
+  pdl_entry();
   __shared__ lv_event chunk[kEventChunk];
   const int s = blockIdx.x * kEventThreads + threadIdx.x;
   lv_session_state st;
@@ -377,9 +382,8 @@ k_events(DevPool p, const lv_event* __restrict__ ev, long long n) {
 // Order key of a session, 0 when it is not a candidate.  Larger keys are
 // evicted first: bit 63 = normal tier, bits 31..62 = T_next (Eq. 4), bits
 // 0..30 = 2^31-1-sid so that equal T_next rank by ascending session id.
-__device__ __forceinline__ unsigned long long session_key(const DevPool& p, int32_t s,
-                                                          long long now_us, bool fallback) {
-  const lv_session_state st = p.sess[s];
+__device__ __forceinline__ unsigned long long session_key(const DevPool& p, const lv_session_state& st,
+                                                          int32_t s, long long now_us, bool fallback) {
   if (p.policy == LV_POLICY_LRU) {
     // least recently used first: every non-running session is a candidate
     if (st.flags & LV_RUNNING) return 0ull;
@@ -428,7 +432,7 @@ k_rank_census(DevPool p, long long now_us, bool fallback) {
   const int32_t s = blockIdx.x;
   __shared__ unsigned long long key;
   if (threadIdx.x == 0) {
-    key = session_key(p, s, now_us, fallback);
+    key = session_key(p, p.sess[s], s, now_us, fallback);
     if (p.S > kEmitScanMax) {       // k_rank_prefix accumulates into these
       p.sbefore[s] = 0;
       if (s == 0) p.ctl[C_RANK_TOTAL] = 0;
@@ -710,7 +714,18 @@ k_swap_in(DevPool p, int32_t sid, const int32_t* __restrict__ blks,
 // chain of dependent reads of a few hundred table words, so their time is the number of
 // links, each a trip to L2 or a barrier, and not the work in them.  Lists of up to
 // kStepItems entries and the allocation bitmaps are therefore kept in shared memory, reads
-// that depend on nothing are issued at the start, and a scan costs one barrier.
+// that depend on nothing are issued at the start, and a scan costs one barrier.  The other
+// cost is scattered access: a warp's 32 stores or reductions to 32 places keep the SM's
+// memory pipe busy for 32 cycles (measured: 31 a warp), and whatever comes next, a barrier's
+// shared-memory word too, queues behind them.  So the bitmaps change in shared memory alone
+// and only the words that differ at the end are written, a page that is freed and taken
+// again in one step gets one owner word, and the session table is read in whole lines.
+// The third cost is instructions: a jump to a line outside the small instruction buffer costs
+// about 110 cycles, warm or not (measured with 160 taken branches over short blocks), while
+// straight code is fetched ahead.  So these kernels do not unroll loops that mostly run once,
+// and what is rare is marked and laid out of line.
+#define LV_RARE(x) __builtin_expect(!!(x), 0)
+#define LV_MOSTLY(x) __builtin_expect(!!(x), 1)
 constexpr int kStepThreads = 512;
 constexpr int kStepWarps = kStepThreads / 32;
 constexpr int kStepItems = 1024;   // victims, and loads, whose lists stay in shared memory
@@ -756,47 +771,101 @@ struct BlockScan {
   }
 };
 
-// One tier's allocation bitmap: the pool's words, and the copy that this kernel reads
-// (in shared memory where it fits, else the words themselves).
+// One tier's allocation bitmap: the pool's words, and what this kernel works on: a copy in
+// shared memory (with the words as they were beside it, for bits_back), or where that does
+// not fit the pool's words themselves.
 struct TierBits {
   uint32_t* gl;
   uint32_t* cur;
+  uint32_t* old;
   long long nbits;
-  __device__ void set(long long w, uint32_t m) const {     // a word only this thread changes
-    atomicOr(&gl[w], m);
+  __device__ uint32_t word(int w) const { return cur != gl ? cur[w] : __ldcg(&gl[w]); }
+  __device__ bool has(int32_t i) const { return word(i >> 5) >> (i & 31) & 1u; }
+  __device__ void set(int w, uint32_t m) const {           // a word only this thread changes now
     if (cur != gl) cur[w] |= m;
+    else atomicOr(&gl[w], m);
   }
-  __device__ void clear(long long i) const {
-    const uint32_t m = ~(1u << (i & 31));
-    atomicAnd(&gl[i >> 5], m);
-    if (cur != gl) atomicAnd(&cur[i >> 5], m);
-  }
+  __device__ void clear(int32_t i) const { atomicAnd(&cur[i >> 5], ~(1u << (i & 31))); }
 };
 
-// The n lowest free bits, ascending, into out[0..n); sets them.  Each thread owns a
-// contiguous run of words.  The caller has checked that n are free; a barrier is needed
-// before other threads read out or the bitmap.
-__device__ void take_lowest(const TierBits& t, long long n, int32_t* out, BlockScan& scan) {
-  const long long W = (t.nbits + 31) >> 5;
-  const long long per = (W + kStepThreads - 1) / kStepThreads;
-  const long long w0 = min(W, (long long)threadIdx.x * per);
-  const long long w1 = min(W, w0 + per);
-  int cnt = 0;
-#pragma unroll 4
-  for (long long w = w0; w < w1; ++w) cnt += __popc(free_bits(t.cur, w, W, t.nbits));
-  int total;
-  long long r = scan.sum(cnt, &total);
-  const long long r_end = min(n, r + cnt);
-  for (long long w = w0; w < w1 && r < r_end; ++w) {
-    uint32_t f = free_bits(t.cur, w, W, t.nbits);
-    uint32_t take = 0;
-    while (f && r < r_end) {
-      const int b = __ffs(f) - 1;
-      f &= f - 1;
-      out[r++] = (int32_t)(w * 32 + b);
-      take |= 1u << b;
+// Reads a bitmap of W words into shared memory at `copy` (2 W words; null: used in place).
+__device__ __forceinline__ TierBits bits_copy(uint32_t* gl, long long nbits, uint32_t* copy) {
+  const int W = (int)((nbits + 31) >> 5);
+  if (!copy) return TierBits{gl, gl, gl, nbits};
+#pragma unroll 1
+  for (int w = threadIdx.x; w < W; w += kStepThreads) copy[w] = copy[W + w] = gl[w];
+  return TierBits{gl, copy, copy + W, nbits};
+}
+
+// Writes the words that changed, as reductions of the bits that changed: a free of other
+// pages on another stream may run meanwhile.  After a barrier.
+__device__ __forceinline__ void bits_back(const TierBits& t) {
+  if (t.cur == t.gl) return;
+  const int W = (int)((t.nbits + 31) >> 5);
+#pragma unroll 1
+  for (int w = threadIdx.x; w < W; w += kStepThreads) {
+    const uint32_t now = t.cur[w], was = t.old[w];
+    if (now & ~was) atomicOr(&t.gl[w], now & ~was);
+    if (was & ~now) atomicAnd(&t.gl[w], ~(was & ~now));
+  }
+}
+
+// Position of the k-th set bit of f (k counted from 0, below popc(f)).
+__device__ __forceinline__ int nth_bit(uint32_t f, int k) {
+  int at = 0;
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1) {
+    const int c = __popc(f & ((1u << w) - 1u));
+    if (k >= c) {
+      k -= c;
+      at += w;
+      f >>= w;
     }
-    if (take) t.set(w, take);
+  }
+  return at;
+}
+
+// The n lowest free bits, ascending, into out[0..n); sets them.  Each thread owns a
+// contiguous run of words and counts its free bits; then thread i finds the i-th one by
+// binary search among the threads' counts (in `base`), so that a tier with whole free words
+// takes as long as one with a free bit here and there.  The caller has checked that n are
+// free; other threads may read out when it returns.
+__device__ void take_lowest(const TierBits& t, int n, int32_t* out, BlockScan& scan, int* base) {
+  const int W = (int)((t.nbits + 31) >> 5);
+  const int per = (W + kStepThreads - 1) / kStepThreads;
+  const int w0 = threadIdx.x * per;
+  const uint32_t last = (t.nbits & 31) ? (1u << (t.nbits & 31)) - 1u : 0xffffffffu;
+  auto free_of = [&](int w) { return w < W ? ~t.word(w) & (w == W - 1 ? last : 0xffffffffu) : 0u; };
+  int cnt = 0;
+#pragma unroll 1
+  for (int i = 0; i < per; ++i) cnt += __popc(free_of(w0 + i));
+  int total;
+  int r = scan.sum(cnt, &total);
+  base[threadIdx.x] = r;
+  __syncthreads();
+#pragma unroll 1
+  for (int i = threadIdx.x; i < n; i += kStepThreads) {
+    int o = 0;                 // the last thread whose run starts at or before the i-th bit
+#pragma unroll
+    for (int step = kStepThreads / 2; step > 0; step >>= 1)
+      if (base[o + step] <= i) o += step;
+    int left = i - base[o], w = o * per;
+    uint32_t f = free_of(w);
+#pragma unroll 1
+    for (int c = __popc(f); left >= c; c = __popc(f)) {
+      left -= c;
+      f = free_of(++w);
+    }
+    out[i] = w * 32 + nth_bit(f, left);
+  }
+  __syncthreads();             // every thread has read the words
+#pragma unroll 1
+  for (int i = 0; i < per && r < n; ++i) {
+    const uint32_t f = free_of(w0 + i);
+    const int c = __popc(f);
+    const uint32_t take = c <= n - r ? f : f & ((1u << nth_bit(f, n - r)) - 1u);
+    if (take) t.set(w0 + i, take);
+    r += c;
   }
 }
 
@@ -840,54 +909,60 @@ struct MovePlan {
 };
 
 // Shared memory of the one-CTA kernels.
+struct StepLists {
+  lv_victim v[kStepItems];
+  int32_t slots[kStepItems], blks[kStepItems], gslot[kStepItems], pages[kStepItems], pair[kStepItems];
+};
 struct StepShared {
   int ws[2 * kStepWarps];
   unsigned long long best[2][kStepWarps];
-  int sums[kStepWarps];
+  int sums[2][kStepWarps];
   int2 pick[kStepWarps + 1];
-  int bad;
   int sel_sid[8], sel_off[8];
-  uint32_t paired[kStepItems / 32];
-  lv_victim v[kStepItems];
-  int32_t slots[kStepItems], blks[kStepItems], gslot[kStepItems], pages[kStepItems];
+  uint32_t done[kStepItems / 32];   // victims that need no out task of their own
+  int base[kStepThreads];
+  union {
+    StepLists l;
+    // at the start, 32 sessions' states of each warp
+    __align__(16) long long states[kStepWarps][32 * sizeof(lv_session_state) / 8];
+  };
 };
 
 // Plans and commits m's moves; every thread of the CTA calls it.  kListed: the lists come
 // from the caller and may be wrong or hold a block twice (checked, with the epoch marks);
-// else they were just read from the tables.  Returns false, with nothing changed, the
+// else they were just read from the tables, and checked there: bad_out and bad_in are a
+// thread's first wrong victim and load, or -1.  Returns false, with nothing changed, the
 // outputs -1 and no tasks, when an item is refused or a tier is too full.
 // hbm_alloc and host_alloc: the tiers' allocation counts as the kernel found them.
 template <bool kListed>
 __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& hbm, const TierBits& host,
-                           long long hbm_alloc, long long host_alloc, StepShared& sh, BlockScan& scan) {
+                           long long hbm_alloc, long long host_alloc, long long bad_out, long long bad_in,
+                           StepShared& sh, BlockScan& scan) {
   const long long n_out = m.n_out, n_in = m.n_in;
   const bool sid_ok = m.sid >= 0 && m.sid < p.S;
   const size_t row = sid_ok ? (size_t)m.sid * p.maxB : 0;
   const int32_t nb_in = kListed && sid_ok ? nblocks_of(p, m.sid) : 0;
   const bool few = n_out <= kStepItems;      // victims are tracked in shared memory
-  if (few && threadIdx.x < kStepItems / 32) sh.paired[threadIdx.x] = 0u;
+  static_assert(kStepItems / 32 <= kStepThreads, "one word of `done` per thread");
+  if (few && threadIdx.x < kStepItems / 32) sh.done[threadIdx.x] = 0u;
   // validation: every victim is resident where it says, every incoming block is in the
   // host tier, and no block appears twice (victims and incoming blocks side by side: item
   // i < n_out is victim i, item n_out + i incoming block i)
   bool bad = false;
   int dirty = 0;             // victims without a clean copy: all of them unless the tiers are inclusive
-  for (long long it = threadIdx.x; it < n_out + n_in; it += kStepThreads) {
-    bool ok;
-    if (it < n_out) {
-      const lv_victim x = m.v[it];
-      if (kListed) {
+  if (kListed) {
+#pragma unroll 1
+    for (long long it = threadIdx.x; it < n_out + n_in; it += kStepThreads) {
+      bool ok;
+      if (it < n_out) {
+        const lv_victim x = m.v[it];
         ok = x.sid >= 0 && x.sid < p.S && x.blk >= 0 && x.page >= 0 && x.page < p.hbm_pages;
         ok = ok && x.blk < nblocks_of(p, x.sid);
         ok = ok && p.table[(size_t)x.sid * p.maxB + x.blk] == x.page &&
              p.own_hbm[x.page] == owner_key(x.sid, x.blk);
         ok = ok && atomicExch(&p.mark[(size_t)x.sid * p.maxB + x.blk], m.epoch) != m.epoch;
       } else {
-        ok = x.page < p.hbm_pages && p.own_hbm[x.page] == owner_key(x.sid, x.blk);
-      }
-      dirty += clean_copy_of(p, x) < 0 ? 1 : 0;
-    } else {
-      const int32_t b = m.blks[it - n_out];
-      if (kListed) {
+        const int32_t b = m.blks[it - n_out];
         ok = sid_ok && b >= 0 && b < nb_in;
         if (ok) {
           const int32_t e = p.table[row + b];
@@ -895,29 +970,29 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
           ok = e <= -2 && h < p.host_pages && p.own_host[h] == owner_key(m.sid, b);
           ok = ok && atomicExch(&p.mark[row + b], m.epoch) != m.epoch;
         }
-      } else {
-        const long long h = m.gslot ? (long long)m.gslot[it - n_out] : -(long long)p.table[row + b] - 2;
-        ok = h < p.host_pages && p.own_host[h] == owner_key(m.sid, b);
       }
+      if (!ok) { set_error(p.ctl, sid_ok || it < n_out ? LV_ERR_STATE : LV_ERR_BOUNDS, it); bad = true; }
     }
-    if (!ok) { set_error(p.ctl, sid_ok || it < n_out ? LV_ERR_STATE : LV_ERR_BOUNDS, it); bad = true; }
+  } else {
+    if (LV_RARE(n_out > 0 && bad_out >= 0)) { set_error(p.ctl, LV_ERR_STATE, bad_out); bad = true; }
+    if (LV_RARE(n_in > 0 && bad_in >= 0)) { set_error(p.ctl, LV_ERR_STATE, n_out + bad_in); bad = true; }
   }
+  if (LV_RARE(p.incl))
+#pragma unroll 1
+    for (long long i = threadIdx.x; i < n_out; i += kStepThreads) dirty += clean_copy_of(p, m.v[i]) < 0 ? 1 : 0;
   bad = __syncthreads_or(bad);
   int n_dirty = (int)n_out;
-  if (p.incl) scan.sum(dirty, &n_dirty);
-  if (!bad) {
-    // capacity, as the sequential calls see it: host slots before any is freed,
-    // HBM pages after the victims' pages are freed
-    if (host_alloc + n_dirty > p.host_pages) {
-      if (threadIdx.x == 0) set_error(p.ctl, LV_ERR_NO_HOST, n_dirty);
-      bad = true;
-    } else if (hbm_alloc - n_out + n_in > p.budget) {
-      if (threadIdx.x == 0) set_error(p.ctl, LV_ERR_NO_HBM, n_in);
-      bad = true;
-    }
-  }
-  if (bad) {
+  if (LV_RARE(p.incl)) scan.sum(dirty, &n_dirty);
+  // capacity, as the sequential calls see it: host slots before any is freed,
+  // HBM pages after the victims' pages are freed
+  const bool no_host = host_alloc + n_dirty > p.host_pages;
+  const bool no_hbm = hbm_alloc - n_out + n_in > p.budget;
+  if (LV_RARE(bad || no_host || no_hbm)) {
+    if (!bad && threadIdx.x == 0)
+      set_error(p.ctl, no_host ? LV_ERR_NO_HOST : LV_ERR_NO_HBM, no_host ? (long long)n_dirty : n_in);
+#pragma unroll 1
     for (long long i = threadIdx.x; i < n_out; i += kStepThreads) m.slots_out[i] = -1;
+#pragma unroll 1
     for (long long i = threadIdx.x; i < n_in; i += kStepThreads) m.pages_out[i] = -1;
     if (threadIdx.x == 0) *m.n_tasks = 0;
     return false;
@@ -926,10 +1001,10 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
   // The compact list of new slots is spread in place from the last chunk to the first: a
   // victim's rank among those without a copy is at most its index, so each read position
   // still holds its compact value when it is read.
-  if (n_dirty > 0) take_lowest(host, n_dirty, m.slots, scan);
-  __syncthreads();
-  if (n_dirty < n_out) {
+  if (n_dirty > 0) take_lowest(host, n_dirty, m.slots, scan, sh.base);
+  if (LV_RARE(n_dirty < n_out)) {
     long long after = 0;   // victims without a copy in the chunks already spread
+#pragma unroll 1
     for (long long c = (n_out + kStepThreads - 1) / kStepThreads - 1; c >= 0; --c) {
       const long long i = c * kStepThreads + threadIdx.x;
       const int32_t cp = i < n_out ? clean_copy_of(p, m.v[i]) : 0;
@@ -942,71 +1017,110 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
       after += chunk;
     }
   }
-  // out-commit: victims now live in their slots, their pages are free; only a
-  // victim that moves bytes tags its page (a clean one has nothing to read)
+  // out-commit: victims now live in their slots, their pages are free.  A page that an
+  // incoming block takes pairs that block's task with its victim's: found by looking the
+  // victim's page up among the pages taken (ascending), or for longer lists through a tag
+  // that the victim leaves in page_tag.  A clean victim has nothing to read and no pair.
+  const bool look_up = few && n_in <= kStepItems;
   const unsigned long long tag = (unsigned long long)(uint32_t)m.epoch << 32;
+#pragma unroll 1
   for (long long i0 = 0; i0 < n_out; i0 += kStepThreads) {
     const long long i = i0 + threadIdx.x;
     if (i < n_out) {
       const lv_victim x = m.v[i];
       const int32_t slot = m.slots[i];
       const size_t ti = (size_t)x.sid * p.maxB + x.blk;
-      const bool clean = p.incl && p.shadow[ti] == slot;
+      bool clean = false;
+      if (LV_RARE(p.incl)) clean = p.shadow[ti] == slot;
       p.table[ti] = -(slot + 2);
-      if (clean) p.shadow[ti] = -1;
+      if (LV_RARE(clean)) p.shadow[ti] = -1;
       p.own_host[slot] = owner_key(x.sid, x.blk);
-      p.own_hbm[x.page] = kOwnerNone;
       hbm.clear(x.page);
-      if (!clean) m.page_tag[x.page] = tag | (unsigned long long)i;
-      else if (few) atomicOr(&sh.paired[i >> 5], 1u << (i & 31));   // no out task of its own
-      if (m.slots_out != m.slots) m.slots_out[i] = slot;
+      if (LV_RARE(clean && few)) atomicOr(&sh.done[i >> 5], 1u << (i & 31));
+      if (LV_RARE(!clean && !look_up)) m.page_tag[x.page] = tag | (unsigned long long)i;
+      if (LV_MOSTLY(m.slots_out != m.slots)) m.slots_out[i] = slot;
     }
     if (kListed) {
       const bool mine = i < n_out;
       warp_count(p, mine ? m.v[i].sid : 0, mine ? -1 : 0, mine ? 1 : 0);
     }
   }
+  if (LV_MOSTLY(look_up))
+#pragma unroll 1
+    for (int i = threadIdx.x; i < n_in; i += kStepThreads) sh.l.pair[i] = -1;
   __syncthreads();
   // HBM pages for the incoming blocks
-  if (n_in > 0) take_lowest(hbm, n_in, m.pages, scan);
-  __syncthreads();
-  // in-commit, and one task per incoming block (paired with the victim whose page it takes)
+  if (n_in > 0) {
+    take_lowest(hbm, (int)n_in, m.pages, scan, sh.base);
+    __syncthreads();
+  }
+  // a victim's page is now taken again, or free
+  int paired = 0;
+#pragma unroll 1
+  for (long long i = threadIdx.x; i < n_out; i += kStepThreads) {
+    const int32_t pg = m.v[i].page;
+    if (LV_RARE(!hbm.has(pg))) {
+      p.own_hbm[pg] = kOwnerNone;
+    } else if (LV_MOSTLY(look_up && !(sh.done[i >> 5] >> (i & 31) & 1u))) {
+      int lo = 0;
+#pragma unroll
+      for (int step = kStepItems / 2; step > 0; step >>= 1)
+        if (lo + step < n_in && m.pages[lo + step] <= pg) lo += step;
+      sh.l.pair[lo] = m.slots[i];
+      atomicOr(&sh.done[i >> 5], 1u << (i & 31));
+      ++paired;
+    }
+  }
+  int all_paired = 0;
+  if (LV_MOSTLY(look_up)) scan.sum(paired, &all_paired);
+  else __syncthreads();
+  // in-commit, and one task per incoming block
+#pragma unroll 1
   for (long long i = threadIdx.x; i < n_in; i += kStepThreads) {
     const int32_t b = m.blks[i];
     const size_t ti = row + b;
     const long long g = m.gslot ? (long long)m.gslot[i] : -(long long)p.table[ti] - 2;
     const int32_t pg = m.pages[i];
-    const unsigned long long pt = n_out > 0 ? m.page_tag[pg] : 0ull;   // read before this thread's stores
+    int4 t = make_int4(-1, -1, (int32_t)g, pg);
+    if (LV_MOSTLY(look_up)) {
+      t.y = sh.l.pair[i];
+      if (t.y >= 0) t.x = pg;
+    } else if (n_out > 0) {
+      const unsigned long long pt = m.page_tag[pg];
+      if ((pt >> 32) == (unsigned long long)(uint32_t)m.epoch && !(pt & kPairedBit)) {
+        const long long vi = (long long)(pt & 0x7fffffffull);
+        t.x = pg;
+        t.y = m.slots[vi];
+        ++paired;
+        if (few) atomicOr(&sh.done[vi >> 5], 1u << (vi & 31));
+        else m.page_tag[pg] = pt | kPairedBit;
+      }
+    }
     p.table[ti] = pg;
     p.own_hbm[pg] = owner_key(m.sid, b);
-    if (p.incl) {
+    if (LV_RARE(p.incl)) {
       p.shadow[ti] = (int32_t)g;             // the host slot stays as its clean copy
     } else {
       p.own_host[g] = kOwnerNone;
-      host.clear(g);
-    }
-    int4 t = make_int4(-1, -1, (int32_t)g, pg);
-    if ((pt >> 32) == (unsigned long long)(uint32_t)m.epoch && !(pt & kPairedBit)) {
-      const long long vi = (long long)(pt & 0x7fffffffull);
-      t.x = pg;
-      t.y = m.slots[vi];
-      if (few) atomicOr(&sh.paired[vi >> 5], 1u << (vi & 31));
-      else m.page_tag[pg] = pt | kPairedBit;
+      host.clear((int32_t)g);
     }
     m.tasks[i] = t;
-    if (m.pages_out != m.pages) m.pages_out[i] = pg;
+    if (LV_MOSTLY(m.pages_out != m.pages)) m.pages_out[i] = pg;
   }
-  __syncthreads();
-  // victims whose page no incoming block takes: out-only tasks, in victim order
+  if (LV_RARE(!look_up)) scan.sum(paired, &all_paired);
+  // victims whose page no incoming block takes: out-only tasks, in victim order.  (Mostly
+  // there are none: a full tier's lowest free pages are the victims' own.)
+  const bool more = all_paired < n_dirty;
   long long run = 0;
-  for (long long i0 = 0; i0 < n_out; i0 += kStepThreads) {
+#pragma unroll 1
+  for (long long i0 = 0; LV_RARE(more && i0 < n_out); i0 += kStepThreads) {
     const long long i = i0 + threadIdx.x;
     bool flag = false;
     int32_t pg = -1;
     if (i < n_out) {
       pg = m.v[i].page;
       if (few) {
-        flag = !(sh.paired[i >> 5] >> (i & 31) & 1u);
+        flag = !(sh.done[i >> 5] >> (i & 31) & 1u);
       } else {
         const unsigned long long pt = m.page_tag[pg];
         flag = (pt >> 32) == (unsigned long long)(uint32_t)m.epoch && !(pt & kPairedBit) &&
@@ -1027,7 +1141,7 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
       atomicAdd(&p.cnt[m.sid].y, -(int)n_in);
     }
     atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HOST_ALLOC]), (unsigned long long)host_delta);
-    if (p.incl) {
+    if (LV_RARE(p.incl)) {
       atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_CLEAN]), (unsigned long long)(n_in - n_clean));
       atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_CLEAN_OUT]), (unsigned long long)n_clean);
     }
@@ -1039,21 +1153,13 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
   return true;
 }
 
-// The bitmaps of both tiers, copied to shared memory at `copy` (null: used in place).
-__device__ void tier_bits(const DevPool& p, uint32_t* copy, TierBits* hbm, TierBits* host) {
-  const long long wh = (p.hbm_pages + 31) >> 5, wo = (p.host_pages + 31) >> 5;
-  *hbm = TierBits{p.bits_hbm, copy ? copy : p.bits_hbm, p.hbm_pages};
-  *host = TierBits{p.bits_host, copy ? copy + wh : p.bits_host, p.host_pages};
-  if (copy) {
-#pragma unroll 4
-    for (long long w = threadIdx.x; w < wh; w += kStepThreads) copy[w] = p.bits_hbm[w];
-#pragma unroll 4
-    for (long long w = threadIdx.x; w < wo; w += kStepThreads) copy[wh + w] = p.bits_host[w];
-  }
+// The words of both bitmaps, twice each (bits_copy).
+__host__ __device__ inline size_t bits_words(const DevPool& p) {
+  return 2 * (size_t)(((p.hbm_pages + 31) >> 5) + ((p.host_pages + 31) >> 5));
 }
 
 // The exchange of a caller's lists (lv_swap_exchange).
-__global__ void __launch_bounds__(kStepThreads)
+__global__ void __launch_bounds__(kStepThreads, 1)
 k_exchange_plan(DevPool p, const lv_victim* __restrict__ v, long long n_out, int32_t sid,
                 const int32_t* __restrict__ blks, long long n_in, int32_t* slots, int32_t* pages,
                 int4* tasks, long long* n_tasks, int32_t epoch, unsigned long long* page_tag,
@@ -1062,62 +1168,65 @@ k_exchange_plan(DevPool p, const lv_victim* __restrict__ v, long long n_out, int
   __shared__ StepShared sh;
   pdl_entry();
   BlockScan scan{sh.ws, 0};
-  TierBits hbm, host;
-  tier_bits(p, copy_bits ? reinterpret_cast<uint32_t*>(dyn) : nullptr, &hbm, &host);
+  uint32_t* copy = copy_bits ? reinterpret_cast<uint32_t*>(dyn) : nullptr;
+  const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, copy);
+  const TierBits host = bits_copy(p.bits_host, p.host_pages, copy ? copy + 2 * ((p.hbm_pages + 31) >> 5) : nullptr);
   const long long hbm_alloc = p.ctl[C_HBM_ALLOC], host_alloc = p.ctl[C_HOST_ALLOC];
   if (threadIdx.x == 0 && cursor) *cursor = 0;
-  MovePlan m{v, n_out, sid, blks, nullptr, n_in, n_out <= kStepItems ? sh.slots : slots,
-             n_in <= kStepItems ? sh.pages : pages, slots, pages, tasks, n_tasks, epoch, page_tag};
-  plan_moves<true>(p, m, hbm, host, hbm_alloc, host_alloc, sh, scan);
+  MovePlan m{v, n_out, sid, blks, nullptr, n_in, n_out <= kStepItems ? sh.l.slots : slots,
+             n_in <= kStepItems ? sh.l.pages : pages, slots, pages, tasks, n_tasks, epoch, page_tag};
+  plan_moves<true>(p, m, hbm, host, hbm_alloc, host_alloc, -1, -1, sh, scan);
+  __syncthreads();
+  bits_back(hbm);
+  bits_back(host);
 }
 
-// Grows session sid by n_tokens (every thread of the CTA calls it): the new blocks take the
-// lowest free HBM pages, in block order.  Returns the pages appended, -1 on an error.
-__device__ long long append_tokens_to(const DevPool& p, int32_t sid, int32_t n_tokens, int32_t* pages,
-                                      const TierBits& hbm, BlockScan& scan, int* s_ok) {
-  const long long ctx = p.sess[sid].ctx_tokens;
-  const long long nb = (ctx + p.T - 1) / p.T;
-  const long long nctx = ctx + n_tokens;
-  const long long nnb = (nctx + p.T - 1) / p.T;
+// Grows session sid, of ctx tokens, by n_tokens (every thread of the CTA calls it): the new
+// blocks take the lowest free HBM pages, in block order.  hbm_alloc: pages allocated now.
+// near: room for kStepItems page ids in shared memory.  Returns the pages appended, -1 on an
+// error.
+__device__ long long append_tokens_to(const DevPool& p, int32_t sid, int32_t ctx, int32_t n_tokens,
+                                      int32_t* pages, long long hbm_alloc, const TierBits& hbm,
+                                      const TierBits& host,
+                                      int32_t* near, BlockScan& scan, int* base) {
+  const int32_t nb = (int32_t)(((uint32_t)ctx + (uint32_t)p.T - 1u) / (uint32_t)p.T);
+  const uint32_t nctx = (uint32_t)ctx + (uint32_t)n_tokens;
+  // (nctx past 2^31 is refused: its block count only has to be defined)
+  const long long nnb = nctx > 0x7fffffffu ? 0 : (nctx + (uint32_t)p.T - 1u) / (uint32_t)p.T;
   const long long m = nnb - nb;
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    if (nnb > p.maxB || nctx > 0x7fffffffll) {
-      set_error(p.ctl, LV_ERR_BOUNDS, sid);
-      ok = 0;
-    } else if (m > 0) {
-      const long long before = (long long)atomicAdd(
-          reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]), (unsigned long long)m);
-      if (before + m > p.budget) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]), (unsigned long long)(-m));
-        set_error(p.ctl, LV_ERR_NO_HBM, sid);
-        ok = 0;
-      }
-    }
-    *s_ok = ok;
+  if (LV_RARE(nnb > p.maxB || nctx > 0x7fffffffu)) {
+    if (threadIdx.x == 0) set_error(p.ctl, LV_ERR_BOUNDS, sid);
+    return -1;
   }
-  __syncthreads();   // the verdict; and every thread has read the context length
-  if (!*s_ok) return -1;
+  if (LV_RARE(m > 0 && hbm_alloc + m > p.budget)) {
+    if (threadIdx.x == 0) set_error(p.ctl, LV_ERR_NO_HBM, sid);
+    return -1;
+  }
   if (m > 0) {
-    take_lowest(hbm, m, pages, scan);
-    __syncthreads();
+    int32_t* list = m <= kStepItems ? near : pages;
+    take_lowest(hbm, (int)m, list, scan, base);
+#pragma unroll 1
     for (long long i = threadIdx.x; i < m; i += kStepThreads) {
-      const int32_t pg = pages[i];
+      const int32_t pg = list[i];
       const int32_t b = (int32_t)(nb + i);
       p.table[(size_t)sid * p.maxB + b] = pg;
       p.own_hbm[pg] = owner_key(sid, b);
+      if (list != pages) pages[i] = pg;
     }
   }
   if (threadIdx.x == 0) {
-    if (m > 0) atomicAdd(&p.cnt[sid].x, (int)m);
+    if (m > 0) {
+      atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]), (unsigned long long)m);
+      atomicAdd(&p.cnt[sid].x, (int)m);
+    }
     // inclusive tiers: the partially filled last block gains rows, its clean copy is stale
-    if (p.incl && n_tokens > 0 && nb > 0 && ctx % p.T != 0) {
+    if (LV_RARE(p.incl) && n_tokens > 0 && nb > 0 && ctx % p.T != 0) {
       const size_t ti = (size_t)sid * p.maxB + (nb - 1);
       const int32_t g = p.shadow[ti];
       if (g >= 0 && g < p.host_pages) {
         p.shadow[ti] = -1;
         p.own_host[g] = kOwnerNone;
-        atomicAnd(&p.bits_host[g >> 5], ~(1u << (g & 31)));
+        host.clear(g);
         atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HOST_ALLOC]), (unsigned long long)-1ll);
         atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_CLEAN]), (unsigned long long)-1ll);
         atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_CLEAN_DROPPED]), 1ull);
@@ -1132,11 +1241,16 @@ __device__ long long append_tokens_to(const DevPool& p, int32_t sid, int32_t n_t
 __global__ void __launch_bounds__(kStepThreads)
 k_append(DevPool p, int32_t sid, int32_t n_tokens, int32_t* pages, int32_t* count) {
   __shared__ int ws[2 * kStepWarps];
-  __shared__ int ok;
+  __shared__ int32_t near[kStepItems];
+  __shared__ int base[kStepThreads];
   pdl_entry();
   BlockScan scan{ws, 0};
-  const TierBits hbm{p.bits_hbm, p.bits_hbm, p.hbm_pages};
-  const long long m = append_tokens_to(p, sid, n_tokens, pages, hbm, scan, &ok);
+  const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, nullptr);
+  const TierBits host = bits_copy(p.bits_host, p.host_pages, nullptr);
+  const int32_t ctx = p.sess[sid].ctx_tokens;
+  const long long hbm_alloc = p.ctl[C_HBM_ALLOC];
+  __syncthreads();      // every thread has read both
+  const long long m = append_tokens_to(p, sid, ctx, n_tokens, pages, hbm_alloc, hbm, host, near, scan, base);
   if (threadIdx.x == 0 && count) *count = m > 0 ? (int32_t)m : 0;
 }
 
@@ -1896,13 +2010,16 @@ __global__ void k_cancel(DevPool p, const int32_t* __restrict__ locs, long long 
 // followed by the exchange copy: pick the turn's session, begin the turn, list its host-tier
 // blocks, the deficit, the ranking, the victims, the plan and its commits, the growth, and
 // the step's end.  It reads per-session counts, the rows of the sessions concerned and the
-// bitmaps, so what bounds it is the chain of dependent reads.  As six to eight kernels in a
-// row (pick, prepare, order, census of every table row, emission, plan, append) these
-// decisions took 25-27 us of a turn of 16 or 1000 sessions, and 24 us of an eviction; as
-// one they take 17-19 and 12 us, and a turn of eight sessions that moves 24 pages of
-// 16 KiB each way went from 47.2 to 34.6 us (45 pages of 192 KiB with 1000 sessions: from
-// 106 to 97).
+// bitmaps, so what bounds it is the chain of dependent reads and the instructions between
+// them.  As six to eight kernels in a row (pick, prepare, order, census of every table row,
+// emission, plan, append) these decisions took 25-27 us of a turn of 16 or 1000 sessions, and
+// 24 us of an eviction; as one kernel 17-19 and 12 us; with the session table read in whole
+// lines, the bitmaps changed in shared memory and rare branches out of line 11 us for 16
+// sessions.  Whole turns, when the copy took 16 KiB units already: eight sessions that move 24
+// pages of 16 KiB each way 47 us with the kernels in a row, 22.8 as one, 19.2 now; 1000
+// sessions and 45 pages of 192 KiB in scattered order 106, 81.8 and 75.8.
 constexpr int kSelectRounds = 8;    // sessions taken by repeated maximum before the keys are sorted
+constexpr int kCountedLoads = 128;  // loads ordered by counting; more are sorted
 
 // The step's arguments beyond the pool.
 struct StepArgs {
@@ -1926,22 +2043,25 @@ struct StepArgs {
 };
 enum { kStepAll = 0, kStepList = 1, kStepMove = 2 };
 
-// Dynamic shared memory of k_step: [n2] keys and [n2] places and [n2] counts of the ranking,
-// [kStepItems] keys and [kStepItems] indexes of the loads' order, both bitmaps.
+// Dynamic shared memory of k_step: [n2] keys, places, blocks in HBM, blocks in the host tier
+// and blocks of the sessions, [kStepItems] keys and indexes of the loads' order, both bitmaps.
 struct StepLayout {
   int n2;
-  size_t off, cnt, load, bits, total;
+  size_t off, cnt, away, nb, load, bits, total;
 };
 
 __host__ __device__ inline StepLayout step_layout(const DevPool& p, bool ordered, bool copy_bits) {
   StepLayout l{};
   l.n2 = 32;
+#pragma unroll 1
   while (l.n2 < p.S) l.n2 *= 2;
   l.off = (size_t)l.n2 * 8;
   l.cnt = l.off + (size_t)l.n2 * 4;
-  l.load = l.cnt + (size_t)l.n2 * 4;
+  l.away = l.cnt + (size_t)l.n2 * 4;
+  l.nb = l.away + (size_t)l.n2 * 4;
+  l.load = l.nb + (size_t)l.n2 * 4;
   l.bits = l.load + (ordered ? (size_t)kStepItems * 12 : 0);
-  l.total = l.bits + (copy_bits ? (size_t)(((p.hbm_pages + 31) >> 5) + ((p.host_pages + 31) >> 5)) * 4 : 0);
+  l.total = l.bits + (copy_bits ? bits_words(p) * 4 : 0);
   return l;
 }
 
@@ -1952,8 +2072,11 @@ __device__ void sort_entries(unsigned long long* key, int* idx, int n) {
   const bool one_warp = n <= 64;
   const int step = one_warp ? 32 : kStepThreads;
   if (!one_warp || threadIdx.x < 32) {
+#pragma unroll 1
     for (int k = 2; k <= n; k <<= 1) {
+#pragma unroll 1
       for (int j = k >> 1; j > 0; j >>= 1) {
+#pragma unroll 1
         for (int i = threadIdx.x; i < n / 2; i += step) {
           const int lo = ((i & ~(j - 1)) << 1) | (i & (j - 1)), hi = lo | j;
           const unsigned long long x = key[lo], y = key[hi];
@@ -1983,17 +2106,25 @@ __device__ void sort_entries(unsigned long long* key, int* idx, int n) {
   __syncthreads();
 }
 
-// The largest of every thread's v, to all of them (one barrier; two buffers as BlockScan).
-__device__ __forceinline__ unsigned long long block_max(unsigned long long v, StepShared& sh, int ph) {
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long x) {
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(x >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(x >> 32) == hi ? (unsigned)x : 0u);
+  return (unsigned long long)hi << 32 | lo;
+}
+
+// The largest of every thread's v and the sum of every thread's n, to all of them (one
+// barrier; two buffers as BlockScan).
+__device__ __forceinline__ unsigned long long block_max(unsigned long long v, int n, int* sum, StepShared& sh,
+                                                        int ph) {
   const int lane = threadIdx.x & 31;
-  auto warp_max = [](unsigned long long x) {
-    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(x >> 32));
-    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(x >> 32) == hi ? (unsigned)x : 0u);
-    return (unsigned long long)hi << 32 | lo;
-  };
   v = warp_max(v);
-  if (lane == 0) sh.best[ph][threadIdx.x >> 5] = v;
+  n = __reduce_add_sync(0xffffffffu, n);
+  if (lane == 0) {
+    sh.best[ph][threadIdx.x >> 5] = v;
+    sh.sums[ph][threadIdx.x >> 5] = n;
+  }
   __syncthreads();
+  *sum = __reduce_add_sync(0xffffffffu, lane < kStepWarps ? sh.sums[ph][lane] : 0);
   return warp_max(lane < kStepWarps ? sh.best[ph][lane] : 0ull);
 }
 
@@ -2001,24 +2132,46 @@ __device__ __forceinline__ int32_t session_of_key(unsigned long long key) {
   return 0x7fffffff - (int32_t)(key & 0x7fffffffull);
 }
 
-// Writes the victims of one session, positions off.. of the order while below n_out.  By the
-// whole CTA (kWhole) or by one warp.
+// A check of owner words that does not wait for them: a word is compared when the next one
+// is read, or at the end, so that the read is not a link of the chain.
+struct OwnerCheck {
+  uint32_t owner, key;
+  long long pos, bad;       // -1: none
+  __device__ void settle() {
+    if (pos >= 0 && owner != key && bad < 0) bad = pos;
+    pos = -1;
+  }
+  __device__ void read(const uint32_t* own, long long i, long long n) {
+    settle();
+    owner = kOwnerNone;
+    if (i >= 0 && i < n) owner = own[i];
+  }
+  __device__ void expect(uint32_t k, long long at) {
+    key = k;
+    pos = at;
+  }
+};
+
+// Writes the victims of one session of nb blocks, positions off.. of the order while below
+// n_out, by the whole CTA (kWhole) or by one warp.  A block's page has to be its own.
 template <bool kWhole>
-__device__ void emit_session(const DevPool& p, int32_t s, long long off, long long n_out, lv_victim* near,
-                             lv_victim* far, BlockScan& scan) {
-  const int32_t nb = nblocks_of(p, s);
+__device__ void emit_session(const DevPool& p, int32_t s, int32_t nb, long long off, long long n_out,
+                             lv_victim* near, lv_victim* far, OwnerCheck& check, BlockScan& scan) {
   const int32_t* row = p.table + (size_t)s * p.maxB;
   const bool suffix = p.within == LV_SUFFIX_FIRST;
   long long pos0 = off;
   auto put = [&](long long pos, int32_t b, int32_t e) {
     if (near) near[pos] = lv_victim{s, b, e};
     far[pos] = lv_victim{s, b, e};
+    check.expect(owner_key(s, b), pos);
   };
   if (kWhole) {
+#pragma unroll 1
     for (int32_t q0 = 0; q0 < nb && pos0 < n_out; q0 += kStepThreads) {
       const int32_t q = q0 + threadIdx.x;
       const int32_t b = suffix ? nb - 1 - q : q;
       const int32_t e = q < nb ? row[b] : -1;
+      check.read(p.own_hbm, e, p.hbm_pages);
       int chunk;
       const long long pos = pos0 + scan.rank(e >= 0, &chunk);
       if (e >= 0 && pos < n_out) put(pos, b, e);
@@ -2026,6 +2179,7 @@ __device__ void emit_session(const DevPool& p, int32_t s, long long off, long lo
     }
   } else {
     const int lane = threadIdx.x & 31;
+#pragma unroll 1
     for (int32_t q0 = 0; q0 < nb && pos0 < n_out; q0 += 128) {
       int32_t e[4];
 #pragma unroll
@@ -2036,6 +2190,7 @@ __device__ void emit_session(const DevPool& p, int32_t s, long long off, long lo
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int32_t q = q0 + u * 32 + lane;
+        check.read(p.own_hbm, e[u], p.hbm_pages);
         const unsigned has = __ballot_sync(0xffffffffu, e[u] >= 0);
         const long long pos = pos0 + __popc(has & ((1u << lane) - 1u));
         if (e[u] >= 0 && pos < n_out) put(pos, suffix ? nb - 1 - q : q, e[u]);
@@ -2054,28 +2209,30 @@ struct Selected {
 };
 
 // Ranks by the keys and counts in shared memory (keys[s] != 0 for candidates with at least
-// one resident block) and finds the sessions of the first k victims.  Mostly a few sessions
-// hold k blocks: they are found by repeated maximum, about 0.15 us each; after kSelectRounds
-// the keys are sorted.  Keys are distinct (each holds its session).
+// one resident block; session `running` is none, whatever its key) and finds the sessions of
+// the first k victims.  Mostly a few sessions hold k blocks: they are found by repeated
+// maximum, one barrier each; after kSelectRounds the keys are sorted.  Keys are distinct
+// (each holds its session).  A thread may call it with only its own sessions' keys and
+// counts (s = thread, thread + kStepThreads, ...) written.
 __device__ Selected select_sessions(const DevPool& p, unsigned long long* keys, int* off, const int* cnt,
-                                    int n2, long long k, StepShared& sh, BlockScan& scan) {
-  int mine = 0;
-  for (int s = threadIdx.x; s < p.S; s += kStepThreads)
-    if (keys[s]) mine += cnt[s];
+                                    int n2, long long k, int32_t running, StepShared& sh, BlockScan& scan) {
   Selected r{};
+  int mine = 0;
+  unsigned long long v = 0;
+#pragma unroll 1
+  for (int s = threadIdx.x; s < p.S; s += kStepThreads) {
+    if (s == running) keys[s] = 0ull;
+    const unsigned long long x = keys[s];
+    if (x) mine += cnt[s];
+    if (x > v) v = x;
+  }
   int total;
-  scan.sum(mine, &total);
+  unsigned long long last = block_max(v, mine, &total, sh, 0);
   r.total = total;
   r.n_out = k < total ? k : total;
-  unsigned long long last = ~0ull;
   long long at = 0;
-  while (at < r.n_out && r.m < kSelectRounds) {
-    unsigned long long v = 0;
-    for (int s = threadIdx.x; s < p.S; s += kStepThreads) {
-      const unsigned long long x = keys[s];
-      if ((r.m == 0 || x < last) && x > v) v = x;
-    }
-    last = block_max(v, sh, r.m & 1);
+#pragma unroll 1
+  while (at < r.n_out) {
     const int32_t s = session_of_key(last);
     if (threadIdx.x == 0) {
       sh.sel_sid[r.m] = s;
@@ -2083,15 +2240,26 @@ __device__ Selected select_sessions(const DevPool& p, unsigned long long* keys, 
     }
     at += cnt[s];
     ++r.m;
+    if (at >= r.n_out || r.m == kSelectRounds) break;
+    v = 0;
+#pragma unroll 1
+    for (int s2 = threadIdx.x; s2 < p.S; s2 += kStepThreads) {
+      const unsigned long long x = keys[s2];
+      if (x < last && x > v) v = x;
+    }
+    int unused;
+    last = block_max(v, 0, &unused, sh, r.m & 1);
   }
-  if (at < r.n_out) {
+  if (LV_RARE(at < r.n_out)) {
     r.sorted = true;
     __syncthreads();
+#pragma unroll 1
     for (int s = p.S + threadIdx.x; s < n2; s += kStepThreads) keys[s] = 0ull;
     __syncthreads();
     sort_entries<false>(keys, nullptr, n2);
     long long run = 0;
     int m = 0;
+#pragma unroll 1
     for (int i0 = 0; i0 < n2 && run < r.n_out; i0 += kStepThreads) {
       const int i = i0 + threadIdx.x;
       const unsigned long long x = i < n2 ? keys[i] : 0ull;
@@ -2108,7 +2276,33 @@ __device__ Selected select_sessions(const DevPool& p, unsigned long long* keys, 
   return r;
 }
 
-__global__ void __launch_bounds__(kStepThreads)
+// The states of 32 consecutive sessions (of `left` that there are), one per lane: read by the
+// warp as whole lines through its buffer in shared memory.  (Read by each lane for itself,
+// 72 bytes apart, every load touches 32 sectors: 3.4 us for 1000 sessions.)
+__device__ __forceinline__ lv_session_state load_states(const lv_session_state* q, int left, long long* buf) {
+  static_assert(sizeof(lv_session_state) == 72, "nine words");
+  const int lane = threadIdx.x & 31;
+  const int words = 9 * (left < 32 ? left : 32);
+  long long w[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    w[i] = 0;
+    if (i * 32 + lane < words) w[i] = reinterpret_cast<const long long*>(q)[i * 32 + lane];
+  }
+  __syncwarp();                  // the buffer's last reads are over
+#pragma unroll
+  for (int i = 0; i < 9; ++i) buf[i * 32 + lane] = w[i];
+  __syncwarp();
+  union {
+    lv_session_state st;
+    long long w[9];
+  } u;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) u.w[i] = buf[lane * 9 + i];
+  return u.st;
+}
+
+__global__ void __launch_bounds__(kStepThreads, 1)
 k_step(DevPool p, StepArgs a) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ StepShared sh;
@@ -2118,35 +2312,49 @@ k_step(DevPool p, StepArgs a) {
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(dyn);
   int* off = reinterpret_cast<int*>(dyn + lay.off);
   int* cnt = reinterpret_cast<int*>(dyn + lay.cnt);
+  int* away = reinterpret_cast<int*>(dyn + lay.away);
+  int* nblk = reinterpret_cast<int*>(dyn + lay.nb);
   BlockScan scan{sh.ws, 0};
   long long* R = a.rs.words;
   const bool evict = a.evict >= 0;
 
-  // reads that depend on nothing: allocation counts, bitmaps, every session's key and count
+  // reads that depend on nothing: the candidates, allocation counts, bitmaps, every session's
+  // state (whole, before anything is decided from it) and counts
+  const bool picks = a.turn && a.sid < 0 && a.part != kStepMove;
+  int32_t first_cand = -1;
+  if (picks && tid < a.n_cand) first_cand = a.cand[tid];
   const long long hbm_alloc = p.ctl[C_HBM_ALLOC], host_alloc = p.ctl[C_HOST_ALLOC];
-  TierBits hbm{}, host{};
-  if (a.part != kStepList) {
-    tier_bits(p, a.copy_bits ? reinterpret_cast<uint32_t*>(dyn + lay.bits) : nullptr, &hbm, &host);
-    const bool fallback = !evict && !a.preload;
-    for (int s = tid; s < p.S; s += kStepThreads) {
-      const int c = p.cnt[s].x;
-      cnt[s] = c;
-      keys[s] = c > 0 ? session_key(p, s, a.now_us, fallback) : 0ull;
+  uint32_t* copy = a.copy_bits && a.part != kStepList ? reinterpret_cast<uint32_t*>(dyn + lay.bits) : nullptr;
+  const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, copy);
+  const TierBits host = bits_copy(p.bits_host, p.host_pages, copy ? copy + 2 * ((p.hbm_pages + 31) >> 5) : nullptr);
+  const bool fallback = !evict && !a.preload;
+#pragma unroll 1
+  for (int s0 = tid & ~31; s0 < p.S; s0 += kStepThreads) {      // 32 sessions of a warp
+    const int x = s0 + lane;
+    const int2 c = x < p.S ? p.cnt[x] : make_int2(0, 0);
+    const lv_session_state st = load_states(p.sess + s0, p.S - s0, sh.states[tid >> 5]);
+    if (x < p.S) {
+      cnt[x] = c.x;
+      away[x] = c.y;
+      nblk[x] = blocks_of_context(p, st.ctx_tokens);
+      keys[x] = c.x > 0 ? session_key(p, st, x, a.now_us, fallback) : 0ull;
     }
-    if (tid == 0) R[R_CURSOR] = 0;
   }
+  if (tid == 0) R[R_CURSOR] = 0;
+  __syncthreads();
 
   // the session: given, picked (the first candidate with a host-tier block, else the first), or none
   int32_t sid = a.sid;
-  if (a.part == kStepMove) {
+  if (LV_RARE(a.part == kStepMove)) {
     sid = (int32_t)R[R_SID];
-  } else if (a.turn && sid < 0) {
+  } else if (picks) {
+    if (tid == 0) sh.pick[kStepWarps] = make_int2(0, first_cand);
     unsigned c = 0x7fffffffu;
     int32_t s = -1;
+#pragma unroll 1
     for (int i = tid; i < a.n_cand; i += kStepThreads) {
-      const int32_t x = a.cand[i];
-      if (tid == 0 && i == 0) sh.pick[kStepWarps] = make_int2(0, x);
-      if (x >= 0 && x < p.S && p.cnt[x].y > 0) {
+      const int32_t x = i == tid ? first_cand : a.cand[i];
+      if (x >= 0 && x < p.S && away[x] > 0) {
         c = (unsigned)i;
         s = x;
         break;
@@ -2158,7 +2366,7 @@ k_step(DevPool p, StepArgs a) {
     __syncthreads();
     const int2 w = lane < kStepWarps ? sh.pick[lane] : make_int2(0x7fffffff, -1);
     const unsigned first = __reduce_min_sync(0xffffffffu, (unsigned)w.x);
-    if (first != 0x7fffffffu) {
+    if (LV_MOSTLY(first != 0x7fffffffu)) {
       const unsigned who = __ballot_sync(0xffffffffu, (unsigned)w.x == first);
       sid = __shfl_sync(0xffffffffu, w.y, __ffs(who) - 1);
     } else {
@@ -2170,18 +2378,25 @@ k_step(DevPool p, StepArgs a) {
     }
   }
   const bool have = sid >= 0 && sid < p.S;      // lv_evict has no session; a failed pick neither
-  if (a.turn && a.part != kStepMove && have && tid == 0) {
-    // LV_EV_TURN_BEGIN; only the fields it changes are written (others read this state now)
-    lv_session_state st = p.sess[sid];
-    lv_event x{};
-    x.kind = LV_EV_TURN_BEGIN;
-    x.sid = sid;
-    x.t_us = a.now_us;
-    apply_event(p, st, x);
-    p.sess[sid].flags = st.flags;
-    p.sess[sid].protect_until_us = st.protect_until_us;
-    p.sess[sid].last_use_us = st.last_use_us;
-    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_EVENTS]), 1ull);
+  const int32_t ctx = have ? p.sess[sid].ctx_tokens : 0;
+  int32_t flags = 0;                            // the turn's session's, in thread 0
+  if (a.turn && have && tid == 0) {
+    flags = p.sess[sid].flags;
+    if (a.part != kStepMove) {
+      // LV_EV_TURN_BEGIN; only the fields it changes are written (others read this state now)
+      lv_session_state st{};
+      st.flags = flags;
+      lv_event x{};
+      x.kind = LV_EV_TURN_BEGIN;
+      x.sid = sid;
+      x.t_us = a.now_us;
+      apply_event(p, st, x);
+      flags = st.flags;
+      p.sess[sid].flags = flags;
+      p.sess[sid].protect_until_us = st.protect_until_us;
+      p.sess[sid].last_use_us = st.last_use_us;
+      atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_EVENTS]), 1ull);
+    }
   }
 
   // the session's host-tier blocks, in load order
@@ -2189,72 +2404,103 @@ k_step(DevPool p, StepArgs a) {
   long long nh = 0, new_blocks = 0, k = 0;
   const int32_t* blks = a.keys ? a.rs.loads : a.rs.blocks;
   const int32_t* gslot = nullptr;
+  OwnerCheck out_check{0, 0, -1, -1}, in_check{0, 0, -1, -1};
   if (!evict && have) {
-    const long long ctx = p.sess[sid].ctx_tokens;
-    const int32_t nb = nblocks_of(p, sid);
-    const long long nctx = ctx + a.append_tokens;
-    const long long nnb = (nctx + p.T - 1) / p.T;
-    const bool over = nnb > p.maxB || nctx > 0x7fffffffll;
+    const int32_t nb = nblk[sid];
+    const uint32_t nctx = (uint32_t)ctx + (uint32_t)a.append_tokens;
+    // (nctx past 2^31 is refused anyway: its block count only has to be defined)
+    const long long nnb = nctx > 0x7fffffffu ? 0 : (nctx + (uint32_t)p.T - 1u) / (uint32_t)p.T;
+    const bool over = nnb > p.maxB || nctx > 0x7fffffffu;
     new_blocks = nnb - nb;
-    if (a.part == kStepMove) {
+    if (LV_RARE(a.part == kStepMove)) {
       nh = R[R_N_IN];
-    } else if (p.cnt[sid].y > 0) {
+#pragma unroll 1
+      for (long long i = tid; i < nh; i += kStepThreads) {
+        const int32_t b = a.rs.loads[i];
+        const long long h = -(long long)p.table[(size_t)sid * p.maxB + b] - 2;
+        in_check.read(p.own_host, h, p.host_pages);
+        in_check.expect(owner_key(sid, b), i);
+      }
+    } else if (away[sid] > 0) {
       const int32_t* row = p.table + (size_t)sid * p.maxB;
+#pragma unroll 1
       for (int32_t q0 = 0; q0 < nb; q0 += kStepThreads) {
         const int32_t b = q0 + tid;
         const int32_t e = b < nb ? row[b] : -1;
+        const long long h = -(long long)e - 2;
+        in_check.read(p.own_host, h, p.host_pages);     // (h < 0 where there is no slot)
         int chunk;
         const long long pos = nh + scan.rank(e <= -2, &chunk);
         if (e <= -2) {
-          if (pos < kStepItems) {
-            sh.blks[pos] = b;
-            sh.gslot[pos] = (int32_t)(-(long long)e - 2);
+          if (LV_MOSTLY(pos < kStepItems)) {
+            sh.l.blks[pos] = b;
+            sh.l.gslot[pos] = (int32_t)h;
           }
           a.rs.blocks[pos] = b;
+          in_check.expect(owner_key(sid, b), pos);
         }
         nh += chunk;
       }
       __syncthreads();
-      if (nh <= kStepItems) {
-        if (a.keys && a.part == kStepAll) {
+      if (LV_MOSTLY(nh <= kStepItems)) {
+        if (LV_RARE(a.keys && a.part == kStepAll)) {
           // the caller's order: ascending (key, block id); the list is in block order already
           unsigned long long* lk = reinterpret_cast<unsigned long long*>(dyn + lay.load);
           int* li = reinterpret_cast<int*>(lk + kStepItems);
-          int n = 32;
-          while (n < nh) n *= 2;
-          for (int i = tid; i < n; i += kStepThreads) {
-            lk[i] = i < nh ? a.keys[sh.blks[i]] : ~0ull;
-            li[i] = i;
+          if (nh <= kCountedLoads) {
+            // few: a warp per load counts the loads before it
+#pragma unroll 1
+            for (int i = tid; i < nh; i += kStepThreads) lk[i] = a.keys[sh.l.blks[i]];
+            __syncthreads();
+#pragma unroll 1
+            for (int i = tid >> 5; i < nh; i += kStepWarps) {
+              const unsigned long long ki = lk[i];
+              int before = 0;
+#pragma unroll 1
+              for (int j = lane; j < nh; j += 32) before += lk[j] < ki || (lk[j] == ki && j < i) ? 1 : 0;
+              before = __reduce_add_sync(0xffffffffu, before);
+              if (lane == 0) li[before] = i;
+            }
+            __syncthreads();
+          } else {
+            int n = 2 * kCountedLoads;
+#pragma unroll 1
+            while (n < nh) n *= 2;
+#pragma unroll 1
+            for (int i = tid; i < n; i += kStepThreads) {
+              lk[i] = i < nh ? a.keys[sh.l.blks[i]] : ~0ull;
+              li[i] = i;
+            }
+            __syncthreads();
+            sort_entries<true>(lk, li, n);
           }
-          __syncthreads();
-          sort_entries<true>(lk, li, n);
-          static_assert(kStepItems <= 2 * kStepThreads, "two loads per thread");
-          int32_t b[2], g[2];
+          constexpr int kEach = kStepItems / kStepThreads;
+          int32_t b[kEach], g[kEach];
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
+          for (int u = 0; u < kEach; ++u) {
             const int i = tid + u * kStepThreads;
             if (i < nh) {
-              b[u] = sh.blks[li[i]];
-              g[u] = sh.gslot[li[i]];
+              b[u] = sh.l.blks[li[i]];
+              g[u] = sh.l.gslot[li[i]];
             }
           }
           __syncthreads();
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
+          for (int u = 0; u < kEach; ++u) {
             const int i = tid + u * kStepThreads;
             if (i < nh) {
-              sh.blks[i] = b[u];
-              sh.gslot[i] = g[u];
+              sh.l.blks[i] = b[u];
+              sh.l.gslot[i] = g[u];
               a.rs.loads[i] = b[u];
             }
           }
           __syncthreads();
         }
-        blks = sh.blks;
-        gslot = sh.gslot;
+        blks = sh.l.blks;
+        gslot = sh.l.gslot;
       }
     }
-    if (over) {
+    if (LV_RARE(over)) {
       if (tid == 0 && a.part != kStepMove) set_error(p.ctl, LV_ERR_BOUNDS, sid);
       status = LV_RESIDENT_FAILED;
     } else {
@@ -2262,11 +2508,11 @@ k_step(DevPool p, StepArgs a) {
       k = need - free_pages > 0 ? need - free_pages : 0;
       if (a.preload && nh == 0) status = LV_RESIDENT_NOTHING;
       else if (a.preload && a.max_load >= 0 && nh > a.max_load) status = LV_RESIDENT_SKIPPED;
-      if (tid == 0 && status == LV_RESIDENT_SKIPPED)
+      if (LV_RARE(status == LV_RESIDENT_SKIPPED) && tid == 0)
         atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_PRELOADS_SKIPPED]), 1ull);
     }
   }
-  if (a.part == kStepList) {
+  if (LV_RARE(a.part == kStepList)) {
     if (tid == 0) {
       R[R_SID] = sid;
       R[R_N_IN] = nh;
@@ -2276,12 +2522,10 @@ k_step(DevPool p, StepArgs a) {
   if (evict) k = a.evict;
   const bool go = status == LV_RESIDENT_DONE;
   const long long want = go ? k : 0;            // victims asked for
-  __syncthreads();                              // keys and counts are complete
-  if (a.turn && have && tid == 0) keys[sid] = 0ull;   // RUNNING: never a victim (its key may predate that)
-  __syncthreads();
 
   Selected sel{};
-  if (want > 0) sel = select_sessions(p, keys, off, cnt, lay.n2, want, sh, scan);
+  // the turn's session is RUNNING by now: never a victim
+  if (want > 0) sel = select_sessions(p, keys, off, cnt, lay.n2, want, a.turn ? sid : -1, sh, scan);
   if (tid == 0) {
     p.ctl[C_SEL_COUNT] = sel.n_out;
     atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_SELECTS]), 1ull);
@@ -2293,14 +2537,19 @@ k_step(DevPool p, StepArgs a) {
     }
   }
   // the victims of the order's first n_out positions
-  lv_victim* near = sel.n_out <= kStepItems ? sh.v : nullptr;
-  if (sel.m <= 2 && !sel.sorted) {
+  lv_victim* near = sel.n_out <= kStepItems ? sh.l.v : nullptr;
+  if (LV_MOSTLY(sel.m <= 2 && !sel.sorted)) {
+#pragma unroll 1
     for (int r = 0; r < sel.m; ++r)
-      emit_session<true>(p, sh.sel_sid[r], sh.sel_off[r], sel.n_out, near, a.rs.victims, scan);
+      emit_session<true>(p, sh.sel_sid[r], nblk[sh.sel_sid[r]], sh.sel_off[r], sel.n_out, near, a.rs.victims,
+                         out_check, scan);
   } else {
-    for (int r = tid >> 5; r < sel.m; r += kStepWarps)
-      emit_session<false>(p, sel.sorted ? session_of_key(keys[r]) : sh.sel_sid[r],
-                          sel.sorted ? off[r] : sh.sel_off[r], sel.n_out, near, a.rs.victims, scan);
+#pragma unroll 1
+    for (int r = tid >> 5; r < sel.m; r += kStepWarps) {
+      const int32_t x = sel.sorted ? session_of_key(keys[r]) : sh.sel_sid[r];
+      emit_session<false>(p, x, nblk[x], sel.sorted ? off[r] : sh.sel_off[r], sel.n_out, near, a.rs.victims,
+                          out_check, scan);
+    }
   }
   // the gate: a shortfall stops the step (a preload is skipped, a foreground turn fails);
   // lv_evict takes what there is
@@ -2309,7 +2558,7 @@ k_step(DevPool p, StepArgs a) {
   if (evict) {
     if (n_out == 0) status = LV_RESIDENT_NOTHING;
     grow = false;
-  } else if (go && sel.n_out < k) {
+  } else if (LV_RARE(go && sel.n_out < k)) {
     if (a.preload) {
       status = LV_RESIDENT_SKIPPED;
       if (tid == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_PRELOADS_SKIPPED]), 1ull);
@@ -2321,11 +2570,16 @@ k_step(DevPool p, StepArgs a) {
     grow = false;
   }
   __syncthreads();                              // the victims are listed
-  MovePlan m{near ? near : a.rs.victims, n_out, sid, blks, gslot, n_in, near ? sh.slots : a.rs.slots,
-             n_in <= kStepItems ? sh.pages : a.rs.pages, a.rs.slots, a.rs.pages, a.rs.tasks,
+  MovePlan m{near ? near : a.rs.victims, n_out, sid, blks, gslot, n_in, near ? sh.l.slots : a.rs.slots,
+             n_in <= kStepItems ? sh.l.pages : a.rs.pages, a.rs.slots, a.rs.pages, a.rs.tasks,
              R + R_N_TASKS, a.epoch, p.page_tag};
-  if (plan_moves<false>(p, m, hbm, host, hbm_alloc, host_alloc, sh, scan) && n_out > 0) {
+  out_check.settle();
+  in_check.settle();
+  const bool planned =
+      plan_moves<false>(p, m, hbm, host, hbm_alloc, host_alloc, out_check.bad, in_check.bad, sh, scan);
+  if (LV_MOSTLY(planned && n_out > 0)) {
     // the victims' sessions: fewer blocks in HBM, more in the host tier
+#pragma unroll 1
     for (int r = tid; r < sel.m; r += kStepThreads) {
       const int32_t s = sel.sorted ? session_of_key(keys[r]) : sh.sel_sid[r];
       const long long at = sel.sorted ? off[r] : sh.sel_off[r];
@@ -2335,16 +2589,22 @@ k_step(DevPool p, StepArgs a) {
     }
   }
   long long appended = 0;
-  if (grow && a.append_tokens > 0) {
+  if (LV_RARE(grow && a.append_tokens > 0)) {
     __syncthreads();                            // the commits of the plan
-    appended = append_tokens_to(p, sid, a.append_tokens, a.rs.append, hbm, scan, &sh.bad);
+    appended = append_tokens_to(p, sid, ctx, a.append_tokens, a.rs.append,
+                                planned ? hbm_alloc - n_out + n_in : hbm_alloc, hbm, host, sh.l.pages, scan,
+                                sh.base);
     if (appended < 0) appended = 0;
   }
+  __syncthreads();
+  bits_back(hbm);
+  bits_back(host);
   if (tid != 0) return;
   // the step's end: LV_EV_TURN_END unless the turn failed, a completed preload's protection,
   // and the result
   if (a.turn && have && status != LV_RESIDENT_FAILED) {
-    lv_session_state st = p.sess[sid];
+    lv_session_state st{};
+    st.flags = flags;
     lv_event x{};
     x.kind = LV_EV_TURN_END;
     x.sid = sid;
@@ -2352,7 +2612,13 @@ k_step(DevPool p, StepArgs a) {
     x.a = a.audio_us;
     x.b = a.units;
     apply_event(p, st, x);
-    p.sess[sid] = st;
+    lv_session_state& to = p.sess[sid];
+    to.flags = st.flags;
+    to.gen_us = st.gen_us;
+    to.play_us = st.play_us;
+    to.reply_tokens = st.reply_tokens;
+    to.last_use_us = st.last_use_us;
+    if (st.flags & LV_DONE_VALID) to.t_done_us = st.t_done_us;
     atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_EVENTS]), 1ull);
   }
   if (a.preload && status == LV_RESIDENT_DONE) {
@@ -2554,8 +2820,7 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, unsigned block, size
 }
 
 cudaError_t launch_events(const DevPool& p, const lv_event* ev, int64_t n, cudaStream_t s) {
-  k_events<<<blocks_for(p.S, kEventThreads, 1 << 20), kEventThreads, 0, s>>>(p, ev, n);
-  return cudaGetLastError();
+  return launch_pdl(k_events, blocks_for(p.S, kEventThreads, 1 << 20), kEventThreads, 0, s, p, ev, (long long)n);
 }
 
 cudaError_t launch_select(const DevPool& p, int64_t now_us, int64_t k, bool fallback,
@@ -2611,11 +2876,10 @@ cudaError_t launch_swap_in(const DevPool& p, int32_t sid, const int32_t* blks, c
 }
 
 // The largest dynamic shared memory of the one-CTA kernels beside their static lists.
-constexpr size_t kStepDynamic = 190 * 1024;
+constexpr size_t kStepDynamic = 180 * 1024;
 
 bool bits_fit(const DevPool& p, size_t others) {
-  const size_t words = (size_t)(((p.hbm_pages + 31) >> 5) + ((p.host_pages + 31) >> 5));
-  return others + words * 4 <= kStepDynamic;
+  return others + bits_words(p) * 4 <= kStepDynamic;
 }
 
 cudaError_t configure_step_kernels() {
@@ -2629,7 +2893,7 @@ cudaError_t launch_exchange_plan(const DevPool& p, const lv_victim* v, int64_t n
                                  int4* tasks, long long* n_tasks, int32_t epoch,
                                  unsigned long long* page_tag, cudaStream_t s, long long* cursor) {
   const bool fit = bits_fit(p, 0);
-  const size_t smem = fit ? (size_t)(((p.hbm_pages + 31) >> 5) + ((p.host_pages + 31) >> 5)) * 4 : 0;
+  const size_t smem = fit ? bits_words(p) * 4 : 0;
   return launch_pdl(k_exchange_plan, 1, kStepThreads, smem, s, p, v, (long long)n_out, sid, blks,
                     (long long)n_in, slots, pages, tasks, n_tasks, epoch, page_tag, cursor, fit ? 1 : 0);
 }
@@ -2706,7 +2970,7 @@ cudaError_t launch_step(const DevPool& p, const ResidentScratch& rs, const StepC
   a.copy_bits = bits_fit(p, step_layout(p, c.load_keys && !split, false).total) ? 1 : 0;
   a.part = split ? kStepList : kStepAll;
   const size_t smem = step_layout(p, c.load_keys && !split, a.copy_bits != 0).total;
-  cudaError_t e = launch_pdl(k_step, 1, kStepThreads, split ? 0 : smem, s, p, a);
+  cudaError_t e = launch_pdl(k_step, 1, kStepThreads, smem, s, p, a);
   if (e != cudaSuccess) return e;
   if (split) {
     e = launch_pdl(k_order_loads, blocks_for(p.maxB, kOrderThreads / 32, 1ll << 30), kOrderThreads, 0, s,
