@@ -193,9 +193,9 @@ int exchange_stage_limit(long long P);
 cudaError_t configure_exchange_tma(const DevPool& p);
 cudaError_t launch_selftest_wait(const DevPool& p, long long limit_ns, cudaStream_t s);
 // lv_sched.cu
-// scratch: device memory of 32 * LV_SCHED_MAX_REQUESTS bytes (keys and costs)
+cudaError_t configure_schedule();
 cudaError_t launch_schedule(const lv_sched_params& q, const lv_request* reqs, int n, int32_t* order,
-                            int32_t* batch, long long* ctl, void* scratch, cudaStream_t s);
+                            int32_t* batch, long long* ctl, cudaStream_t s);
 // lv_api.cu: the shape of a pool (for the controller)
 void pool_shape(const lv_pool* pool, int32_t* sessions, int32_t* max_blocks, int64_t* page_bytes,
                 int64_t* budget, int64_t* host_pages);
