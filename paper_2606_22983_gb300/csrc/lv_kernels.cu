@@ -1,25 +1,29 @@
 // CUDA kernels of the KV swap path (sm_103a).
 //
-//   ranking   k_rank_census -> k_rank_emit                (Section 5.1, Eq. 4)
+//   ranking   k_select; k_rank_census -> k_rank_emit          (Section 5.1, Eq. 4)
 //   allocate  k_alloc, k_alloc_out                           (lowest free, Section 5.1)
 //   move      k_swap_out / k_swap_in                         (Section 5, Fig. 6; Section 5.2)
 //             k_exchange_plan -> k_exchange_copy             (both directions in one step)
 //             k_stage_tasks (TMA) / k_stage_tasks_lsu         (staged copy-engine path)
 //   commit    k_remap, k_cancel, k_append                    (Section 6 side tables)
 //   monitor   k_events                                       (Section 3, Sections 5.1-5.2)
-//   turn      k_resident_*, k_pick_scan,                      (a whole turn on the device;
-//             k_order_loads, k_evict_prepare                 the gate runs in the plan)
+//   step      k_step -> k_exchange_copy                      (a whole turn, preload or eviction
+//                                                             decided on the device)
 //   verify    k_checksum                                     (page checksums)
 //
 // The only waits are the TMA stage kernel's mbarrier waits for its own copies,
 // each limited by %globaltimer to one second, after which the kernel reports
-// LV_ERR_TIMEOUT and returns; no kernel waits on another kernel or agent.  Every
+// LV_ERR_TIMEOUT and returns, and the barriers of a cluster's CTAs, which run together; no
+// kernel waits on another kernel or agent.  Every
 // index read from memory is range-checked and a bad item is skipped with the
 // sticky error set.
+#include <cooperative_groups.h>
 #include <cstdint>
 #include <utility>
 
 #include "lv_internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace lv {
 
@@ -205,6 +209,7 @@ __device__ __forceinline__ int32_t import_block(const DevPool& p, const int32_t*
 __global__ void k_import(DevPool p, const int32_t* __restrict__ placement,
                          const int32_t* __restrict__ ctx) {
   const long long total = (long long)p.S * p.maxB;
+  int in_hbm = 0, in_host = 0;
   for (long long base = blockIdx.x * (long long)blockDim.x; base < total;
        base += (long long)gridDim.x * blockDim.x) {
     const long long idx = base + threadIdx.x;
@@ -215,6 +220,15 @@ __global__ void k_import(DevPool p, const int32_t* __restrict__ placement,
     }
     const int2 t = tier_of(e);
     warp_count(p, s, t.x, t.y);
+    in_hbm += t.x;
+    in_host += t.y;
+  }
+  // the allocation counts, once per warp (a million blocks counted one by one queue on two words)
+  in_hbm = __reduce_add_sync(0xffffffffu, in_hbm);
+  in_host = __reduce_add_sync(0xffffffffu, in_host);
+  if ((threadIdx.x & 31) == 0) {
+    if (in_hbm) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]), (unsigned long long)in_hbm);
+    if (in_host) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HOST_ALLOC]), (unsigned long long)in_host);
   }
 }
 
@@ -247,7 +261,6 @@ __device__ __forceinline__ int32_t import_block(const DevPool& p, const int32_t*
       return -1;
     }
     atomicOr(&p.bits_hbm[e >> 5], 1u << (e & 31));
-    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]), 1ull);
   } else if (e <= -2) {
     const long long h = -(long long)e - 2;
     if (h >= p.host_pages) { set_error(p.ctl, LV_ERR_BOUNDS, idx); return -1; }
@@ -256,7 +269,6 @@ __device__ __forceinline__ int32_t import_block(const DevPool& p, const int32_t*
       return -1;
     }
     atomicOr(&p.bits_host[h >> 5], 1u << (h & 31));
-    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HOST_ALLOC]), 1ull);
   } else {
     set_error(p.ctl, LV_ERR_BOUNDS, idx);   // a block inside the context with no location
     return -1;
@@ -425,33 +437,42 @@ constexpr int kCensusThreads = 256;
 #endif
 constexpr int kEmitScanMax = LV_EMIT_SCAN_MAX;
 
-// One CTA per session: its key and its count of HBM-resident blocks.
+// Every session's key and its count of HBM-resident blocks.  kRow: threads of a row's
+// session -- a CTA, or a warp (eight sessions a CTA) where rows are short: 4096 rows of 256
+// words took 8.8 us with a CTA each.
+template <int kRow>
 __global__ void __launch_bounds__(kCensusThreads)
 k_rank_census(DevPool p, long long now_us, bool fallback) {
   pdl_wait();
-  const int32_t s = blockIdx.x;
-  __shared__ unsigned long long key;
-  if (threadIdx.x == 0) {
+  const int32_t s = (blockIdx.x * kCensusThreads + threadIdx.x) / kRow;
+  const int t = threadIdx.x % kRow;
+  unsigned long long key = 0ull;
+  int c = 0;
+  if (s < p.S) {
     key = session_key(p, p.sess[s], s, now_us, fallback);
+    if (key != 0ull) {
+      const int32_t nb = nblocks_of(p, s);
+      const int32_t* row = p.table + (size_t)s * p.maxB;
+#pragma unroll 4
+      for (int32_t b = t; b < nb; b += kRow) c += row[b] >= 0 ? 1 : 0;
+    }
+  }
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (kRow > 32) {
+    __shared__ int part[kCensusThreads / 32];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
+    __syncthreads();
+    c = 0;
+    if (t == 0)
+      for (int w = 0; w < kCensusThreads / 32; ++w) c += part[w];
+  }
+  if (t == 0 && s < p.S) {
+    p.skey[s] = key;
+    p.scount[s] = c;
     if (p.S > kEmitScanMax) {       // k_rank_prefix accumulates into these
       p.sbefore[s] = 0;
       if (s == 0) p.ctl[C_RANK_TOTAL] = 0;
     }
-  }
-  __syncthreads();
-  if (key == 0ull) {
-    if (threadIdx.x == 0) { p.skey[s] = 0ull; p.scount[s] = 0; }
-    return;
-  }
-  const int32_t nb = nblocks_of(p, s);
-  const int32_t* row = p.table + (size_t)s * p.maxB;
-  long long c = 0;
-  for (int32_t b = threadIdx.x; b < nb; b += kCensusThreads) c += row[b] >= 0 ? 1 : 0;
-  long long total;
-  block_excl_scan<kCensusThreads>(c, &total);
-  if (threadIdx.x == 0) {
-    p.skey[s] = key;
-    p.scount[s] = (int32_t)total;
   }
   pdl_trigger();
 }
@@ -918,7 +939,7 @@ struct StepShared {
   unsigned long long best[2][kStepWarps];
   int sums[2][kStepWarps];
   int2 pick[kStepWarps + 1];
-  int sel_sid[8], sel_off[8];
+  int sel_sid[12], sel_off[12];     // [kSelectRounds]
   uint32_t done[kStepItems / 32];   // victims that need no out task of their own
   int base[kStepThreads];
   union {
@@ -2018,7 +2039,7 @@ __global__ void k_cancel(DevPool p, const int32_t* __restrict__ locs, long long 
 // sessions.  Whole turns, when the copy took 16 KiB units already: eight sessions that move 24
 // pages of 16 KiB each way 47 us with the kernels in a row, 22.8 as one, 19.2 now; 1000
 // sessions and 45 pages of 192 KiB in scattered order 106, 81.8 and 75.8.
-constexpr int kSelectRounds = 8;    // sessions taken by repeated maximum before the keys are sorted
+constexpr int kSelectRounds = 12;   // sessions found by repeated maximum at most
 constexpr int kCountedLoads = 128;  // loads ordered by counting; more are sorted
 
 // The step's arguments beyond the pool.
@@ -2152,49 +2173,85 @@ struct OwnerCheck {
   }
 };
 
-// Writes the victims of one session of nb blocks, positions off.. of the order while below
-// n_out, by the whole CTA (kWhole) or by one warp.  A block's page has to be its own.
-template <bool kWhole>
-__device__ void emit_session(const DevPool& p, int32_t s, int32_t nb, long long off, long long n_out,
-                             lv_victim* near, lv_victim* far, OwnerCheck& check, BlockScan& scan) {
-  const int32_t* row = p.table + (size_t)s * p.maxB;
-  const bool suffix = p.within == LV_SUFFIX_FIRST;
-  long long pos0 = off;
-  auto put = [&](long long pos, int32_t b, int32_t e) {
+// Where victims go, and what their pages' owner words are checked against.
+struct VictimList {
+  lv_victim* near;          // shared memory, or null
+  lv_victim* far;
+  const uint32_t* own;      // null: not checked
+  long long n_own;
+  long long n_out;          // positions below this are written
+  __device__ void put(long long pos, int32_t s, int32_t b, int32_t e) const {
     if (near) near[pos] = lv_victim{s, b, e};
     far[pos] = lv_victim{s, b, e};
-    check.expect(owner_key(s, b), pos);
-  };
-  if (kWhole) {
+  }
+};
+
+// The blocks of session s (nb of them) in victim order: positions pos0.. of the list, by the
+// whole CTA.  A block's page has to be its own.
+__device__ void emit_whole(const DevPool& p, int32_t s, int32_t nb, long long pos0, const VictimList& l,
+                           OwnerCheck& check, BlockScan& scan) {
+  const int32_t* row = p.table + (size_t)s * p.maxB;
+  const bool suffix = p.within == LV_SUFFIX_FIRST;
 #pragma unroll 1
-    for (int32_t q0 = 0; q0 < nb && pos0 < n_out; q0 += kStepThreads) {
-      const int32_t q = q0 + threadIdx.x;
-      const int32_t b = suffix ? nb - 1 - q : q;
-      const int32_t e = q < nb ? row[b] : -1;
-      check.read(p.own_hbm, e, p.hbm_pages);
-      int chunk;
-      const long long pos = pos0 + scan.rank(e >= 0, &chunk);
-      if (e >= 0 && pos < n_out) put(pos, b, e);
-      pos0 += chunk;
+  for (int32_t q0 = 0; q0 < nb && pos0 < l.n_out; q0 += kStepThreads) {
+    const int32_t q = q0 + threadIdx.x;
+    const int32_t b = suffix ? nb - 1 - q : q;
+    const int32_t e = q < nb ? row[b] : -1;
+    check.read(l.own, e, l.n_own);
+    int chunk;
+    const long long pos = pos0 + scan.rank(e >= 0, &chunk);
+    if (e >= 0 && pos < l.n_out) {
+      l.put(pos, s, b, e);
+      if (l.own) check.expect(owner_key(s, b), pos);
     }
-  } else {
-    const int lane = threadIdx.x & 31;
+    pos0 += chunk;
+  }
+}
+
+// The same for sessions `of(r)`, r = first, first + kStepWarps, ... below m, by one warp, four
+// sessions at a time: the first 32 blocks of each are read together (a session of a few
+// blocks costs a read's latency, whoever reads it).
+template <typename Of>
+__device__ void emit_warp(const DevPool& p, const int* nblk, int m, const VictimList& l, OwnerCheck& check,
+                          Of of) {
+  const int lane = threadIdx.x & 31;
+  const bool suffix = p.within == LV_SUFFIX_FIRST;
 #pragma unroll 1
-    for (int32_t q0 = 0; q0 < nb && pos0 < n_out; q0 += 128) {
-      int32_t e[4];
+  for (int r0 = threadIdx.x >> 5; r0 < m; r0 += 4 * kStepWarps) {
+    int32_t e[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int32_t q = q0 + u * 32 + lane;
-        e[u] = q < nb ? row[suffix ? nb - 1 - q : q] : -1;
+    for (int u = 0; u < 4; ++u) {
+      const int r = r0 + u * kStepWarps;
+      e[u] = -1;
+      if (r < m) {
+        const int32_t s = of(r).x, nb = nblk[s];
+        if (lane < nb) e[u] = p.table[(size_t)s * p.maxB + (suffix ? nb - 1 - lane : lane)];
       }
+    }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int32_t q = q0 + u * 32 + lane;
-        check.read(p.own_hbm, e[u], p.hbm_pages);
-        const unsigned has = __ballot_sync(0xffffffffu, e[u] >= 0);
+    for (int u = 0; u < 4; ++u) {
+      const int r = r0 + u * kStepWarps;
+      if (r >= m) break;
+      const int2 so = of(r);
+      const int32_t s = so.x, nb = nblk[s];
+      const int32_t* row = p.table + (size_t)s * p.maxB;
+      long long pos0 = so.y;
+      int32_t x = e[u];
+#pragma unroll 1
+      for (int32_t q0 = 0;; ) {
+        const int32_t q = q0 + lane;
+        check.read(l.own, x, l.n_own);
+        const unsigned has = __ballot_sync(0xffffffffu, x >= 0);
         const long long pos = pos0 + __popc(has & ((1u << lane) - 1u));
-        if (e[u] >= 0 && pos < n_out) put(pos, suffix ? nb - 1 - q : q, e[u]);
+        if (x >= 0 && pos < l.n_out) {
+          const int32_t b = suffix ? nb - 1 - q : q;
+          l.put(pos, s, b, x);
+          if (l.own) check.expect(owner_key(s, b), pos);
+        }
         pos0 += __popc(has);
+        q0 += 32;
+        if (q0 >= nb || pos0 >= l.n_out) break;
+        x = q0 + lane < nb ? row[suffix ? nb - 1 - q0 - lane : q0 + lane] : -1;
       }
     }
   }
@@ -2208,22 +2265,78 @@ struct Selected {
   long long total;      // resident blocks of all candidates
 };
 
+// The lowest key among those of the first n positions (n of the order's blocks are found for
+// certain): the range of the keys that hold position n is narrowed by histograms of
+// kStepThreads bins, weighted by the sessions' blocks, over the tight range of the keys left;
+// two or three rounds for spread keys, three or four where T_next ties.
+__device__ unsigned long long threshold_key(const DevPool& p, const unsigned long long* keys, const int* cnt,
+                                            long long n, StepShared& sh, BlockScan& scan) {
+  unsigned long long lo = 1, hi = ~0ull;
+  long long above = 0;
+#pragma unroll 1
+  for (;;) {
+    unsigned long long high = 0, low = 0;        // low: the largest complement
+#pragma unroll 1
+    for (int s = threadIdx.x; s < p.S; s += kStepThreads) {
+      const unsigned long long x = keys[s];
+      const bool in = x >= lo && x <= hi;
+      if (in && x > high) high = x;
+      if (in && ~x > low) low = ~x;
+    }
+    int unused;
+    high = block_max(high, 0, &unused, sh, 0);
+    low = ~block_max(low, 0, &unused, sh, 1);
+    if (low == high) return low;
+    const int bits = 64 - __clzll((long long)(high - low));
+    const int shift = bits > 9 ? bits - 9 : 0;
+    static_assert(kStepThreads == 512, "nine bits of bins");
+    sh.base[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll 1
+    for (int s = threadIdx.x; s < p.S; s += kStepThreads) {
+      const unsigned long long x = keys[s];
+      if (x >= low && x <= high) atomicAdd(&sh.base[(x - low) >> shift], cnt[s]);
+    }
+    __syncthreads();
+    const int bin = kStepThreads - 1 - (int)threadIdx.x;    // largest first
+    const int w = sh.base[bin];
+    int total;
+    const long long before = above + scan.sum(w, &total);
+    if (before < n && n <= before + w) {
+      sh.sel_sid[0] = bin;
+      sh.sel_off[0] = (int)before;
+    }
+    __syncthreads();
+    above = sh.sel_off[0];
+    lo = low + ((unsigned long long)sh.sel_sid[0] << shift);
+    hi = lo + ((1ull << shift) - 1);
+    if (hi < lo || hi > high) hi = high;
+  }
+}
+
 // Ranks by the keys and counts in shared memory (keys[s] != 0 for candidates with at least
 // one resident block; session `running` is none, whatever its key) and finds the sessions of
-// the first k victims.  Mostly a few sessions hold k blocks: they are found by repeated
-// maximum, one barrier each; after kSelectRounds the keys are sorted.  Keys are distinct
-// (each holds its session).  A thread may call it with only its own sessions' keys and
-// counts (s = thread, thread + kStepThreads, ...) written.
+// the first k victims.  Where few sessions should hold k blocks they are found by repeated
+// maximum, one barrier each; else, or when kSelectRounds were not enough, by the threshold
+// key, and the sessions' places by comparing them with one another, or by a sort of more
+// than kCompared.  (4096 sessions, 1500 victims of 7 or 8 sessions: 9.1 us by maximum, 12.6
+// by the threshold; 256 victims of 128 sessions: 48 us by maximum and a sort of all keys,
+// 13.1 by the threshold.)  Keys are distinct (each holds its session).  A thread may call it with
+// only its own sessions' keys and counts (s = thread, thread + kStepThreads, ...) written.
+constexpr int kCompared = 256;
 __device__ Selected select_sessions(const DevPool& p, unsigned long long* keys, int* off, const int* cnt,
-                                    int n2, long long k, int32_t running, StepShared& sh, BlockScan& scan) {
+                                    long long k, int32_t running, StepShared& sh, BlockScan& scan) {
   Selected r{};
-  int mine = 0;
+  int mine = 0, cand = 0;
   unsigned long long v = 0;
 #pragma unroll 1
   for (int s = threadIdx.x; s < p.S; s += kStepThreads) {
     if (s == running) keys[s] = 0ull;
     const unsigned long long x = keys[s];
-    if (x) mine += cnt[s];
+    if (x) {
+      mine += cnt[s];
+      ++cand;
+    }
     if (x > v) v = x;
   }
   int total;
@@ -2231,49 +2344,97 @@ __device__ Selected select_sessions(const DevPool& p, unsigned long long* keys, 
   r.total = total;
   r.n_out = k < total ? k : total;
   long long at = 0;
+  int cands;
+  scan.sum(cand, &cands);
+  const bool few = r.n_out * cands <= 8ll * total;      // eight sessions of average size
+  if (LV_MOSTLY(few)) {
 #pragma unroll 1
-  while (at < r.n_out) {
-    const int32_t s = session_of_key(last);
-    if (threadIdx.x == 0) {
-      sh.sel_sid[r.m] = s;
-      sh.sel_off[r.m] = (int)at;
-    }
-    at += cnt[s];
-    ++r.m;
-    if (at >= r.n_out || r.m == kSelectRounds) break;
-    v = 0;
+    while (at < r.n_out) {
+      const int32_t s = session_of_key(last);
+      if (threadIdx.x == 0) {
+        sh.sel_sid[r.m] = s;
+        sh.sel_off[r.m] = (int)at;
+      }
+      at += cnt[s];
+      ++r.m;
+      if (at >= r.n_out || r.m == kSelectRounds) break;
+      v = 0;
 #pragma unroll 1
-    for (int s2 = threadIdx.x; s2 < p.S; s2 += kStepThreads) {
-      const unsigned long long x = keys[s2];
-      if (x < last && x > v) v = x;
+      for (int s2 = threadIdx.x; s2 < p.S; s2 += kStepThreads) {
+        const unsigned long long x = keys[s2];
+        if (x < last && x > v) v = x;
+      }
+      int unused;
+      last = block_max(v, 0, &unused, sh, r.m & 1);
     }
-    int unused;
-    last = block_max(v, 0, &unused, sh, r.m & 1);
   }
   if (LV_RARE(at < r.n_out)) {
     r.sorted = true;
     __syncthreads();
-#pragma unroll 1
-    for (int s = p.S + threadIdx.x; s < n2; s += kStepThreads) keys[s] = 0ull;
-    __syncthreads();
-    sort_entries<false>(keys, nullptr, n2);
-    long long run = 0;
-    int m = 0;
-#pragma unroll 1
-    for (int i0 = 0; i0 < n2 && run < r.n_out; i0 += kStepThreads) {
-      const int i = i0 + threadIdx.x;
-      const unsigned long long x = i < n2 ? keys[i] : 0ull;
-      int chunk;
-      const long long pos = run + scan.sum(x ? cnt[session_of_key(x)] : 0, &chunk);
-      const bool in = x && pos < r.n_out;
-      if (in) off[i] = (int)pos;
-      m += __syncthreads_count(in);
-      run += chunk;
+    const unsigned long long least = threshold_key(p, keys, cnt, r.n_out, sh, scan);
+    // the chosen keys to the front of the array
+    constexpr int kEach = 4096 / kStepThreads;      // a pool's sessions per thread at most
+    unsigned long long x[kEach];
+    int chosen = 0;
+#pragma unroll
+    for (int u = 0; u < kEach; ++u) {
+      const int s = threadIdx.x + u * kStepThreads;
+      x[u] = s < p.S ? keys[s] : 0ull;
+      if (x[u] < least) x[u] = 0ull;
+      chosen += x[u] ? 1 : 0;
     }
-    r.m = m;
+    int at2 = scan.sum(chosen, &r.m);               // (every thread has read its keys)
+#pragma unroll
+    for (int u = 0; u < kEach; ++u)
+      if (x[u]) keys[at2++] = x[u];
+    __syncthreads();
+    if (r.m <= kCompared) {
+      const int i = threadIdx.x;
+      const unsigned long long key = i < r.m ? keys[i] : 0ull;
+      if (i < r.m) off[i] = cnt[session_of_key(key)];
+      __syncthreads();
+      int before = 0;
+      if (i < r.m) {
+#pragma unroll 4
+        for (int j = 0; j < r.m; ++j) before += keys[j] > key ? off[j] : 0;
+      }
+      __syncthreads();
+      if (i < r.m) off[i] = before;
+    } else {
+      int n2 = 2 * kCompared;
+      while (n2 < r.m) n2 *= 2;
+#pragma unroll 1
+      for (int i = r.m + threadIdx.x; i < n2; i += kStepThreads) keys[i] = 0ull;
+      __syncthreads();
+      sort_entries<false>(keys, nullptr, n2);
+      int run = 0;
+#pragma unroll 1
+      for (int i0 = 0; i0 < r.m; i0 += kStepThreads) {
+        const int i = i0 + threadIdx.x;
+        int chunk;
+        const int pos = run + scan.sum(i < r.m ? cnt[session_of_key(keys[i])] : 0, &chunk);
+        if (i < r.m) off[i] = pos;
+        run += chunk;
+      }
+    }
   }
   __syncthreads();
   return r;
+}
+
+// Writes the victims of the selected sessions.
+__device__ void emit_selected(const DevPool& p, const Selected& sel, const unsigned long long* keys,
+                              const int* off, const int* nblk, const VictimList& l, OwnerCheck& check,
+                              StepShared& sh, BlockScan& scan) {
+  if (LV_MOSTLY(sel.m <= 2 && !sel.sorted)) {
+#pragma unroll 1
+    for (int r = 0; r < sel.m; ++r)
+      emit_whole(p, sh.sel_sid[r], nblk[sh.sel_sid[r]], sh.sel_off[r], l, check, scan);
+  } else if (sel.sorted) {
+    emit_warp(p, nblk, sel.m, l, check, [&](int r) { return make_int2(session_of_key(keys[r]), off[r]); });
+  } else {
+    emit_warp(p, nblk, sel.m, l, check, [&](int r) { return make_int2(sh.sel_sid[r], sh.sel_off[r]); });
+  }
 }
 
 // The states of 32 consecutive sessions (of `left` that there are), one per lane: read by the
@@ -2525,7 +2686,7 @@ k_step(DevPool p, StepArgs a) {
 
   Selected sel{};
   // the turn's session is RUNNING by now: never a victim
-  if (want > 0) sel = select_sessions(p, keys, off, cnt, lay.n2, want, a.turn ? sid : -1, sh, scan);
+  if (want > 0) sel = select_sessions(p, keys, off, cnt, want, a.turn ? sid : -1, sh, scan);
   if (tid == 0) {
     p.ctl[C_SEL_COUNT] = sel.n_out;
     atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_SELECTS]), 1ull);
@@ -2538,19 +2699,8 @@ k_step(DevPool p, StepArgs a) {
   }
   // the victims of the order's first n_out positions
   lv_victim* near = sel.n_out <= kStepItems ? sh.l.v : nullptr;
-  if (LV_MOSTLY(sel.m <= 2 && !sel.sorted)) {
-#pragma unroll 1
-    for (int r = 0; r < sel.m; ++r)
-      emit_session<true>(p, sh.sel_sid[r], nblk[sh.sel_sid[r]], sh.sel_off[r], sel.n_out, near, a.rs.victims,
-                         out_check, scan);
-  } else {
-#pragma unroll 1
-    for (int r = tid >> 5; r < sel.m; r += kStepWarps) {
-      const int32_t x = sel.sorted ? session_of_key(keys[r]) : sh.sel_sid[r];
-      emit_session<false>(p, x, nblk[x], sel.sorted ? off[r] : sh.sel_off[r], sel.n_out, near, a.rs.victims,
-                          out_check, scan);
-    }
-  }
+  const VictimList list{near, a.rs.victims, p.own_hbm, p.hbm_pages, sel.n_out};
+  emit_selected(p, sel, keys, off, nblk, list, out_check, sh, scan);
   // the gate: a shortfall stops the step (a preload is skipped, a foreground turn fails);
   // lv_evict takes what there is
   long long n_out = sel.n_out, n_in = go ? nh : 0;
@@ -2635,6 +2785,88 @@ k_step(DevPool p, StepArgs a) {
     r.status = status;
     r.sid = sid;
     *a.out = r;
+  }
+}
+
+// ------------------------------------------------------ ranking by itself
+// lv_select_victims for up to kSelectMost victims: one kernel.  The keys of kStepThreads
+// sessions are made by each CTA of a cluster and written into the first CTA's shared memory,
+// which then selects and lists the victims; it reads one count per session and the rows of
+// the sessions chosen, where the census reads every row.  kCensus: no counts are kept for
+// these tables (lv_select_victims_noalloc); one CTA takes keys and counts from the census.
+// 256 victims of 1024 sessions with 1024 blocks each: 7.1 us as census and emission, 3.9 as
+// one kernel; 1500 of 4096 sessions with 256 blocks: 20.7 and 9.1 us.
+// More victims, or victims of some hundred sessions, are written by many CTAs: 4096 victims
+// of 1024 sessions take 11.8 us here and 9.2 there, 2048 of at least 1024 sessions with two
+// blocks each 32 and 9.2, 256 of 128 such sessions 10.1 and 9.2 (13.1 and 14.9 with 4096
+// sessions).
+constexpr int kSelectMost = 2048;
+constexpr int kSelectSessions = 128;   // k victims are blocks of k / maxB sessions at least
+
+struct SelectLayout {
+  int n2;
+  size_t off, cnt, nb, total;
+};
+__host__ __device__ inline SelectLayout select_layout(int S) {
+  SelectLayout l{};
+  l.n2 = 32;
+  while (l.n2 < S) l.n2 *= 2;
+  l.off = (size_t)l.n2 * 8;
+  l.cnt = l.off + (size_t)l.n2 * 4;
+  l.nb = l.cnt + (size_t)l.n2 * 4;
+  l.total = l.nb + (size_t)l.n2 * 4;
+  return l;
+}
+
+template <bool kCensus>
+__global__ void __launch_bounds__(kStepThreads, 1)
+k_select(DevPool p, long long now_us, long long k, bool fallback, long long* count_dev, lv_victim* out) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ StepShared sh;
+  pdl_entry();
+  const int tid = threadIdx.x;
+  const SelectLayout lay = select_layout(p.S);
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(dyn);
+  int* off = reinterpret_cast<int*>(dyn + lay.off);
+  int* cnt = reinterpret_cast<int*>(dyn + lay.cnt);
+  int* nblk = reinterpret_cast<int*>(dyn + lay.nb);
+  BlockScan scan{sh.ws, 0};
+  if (kCensus) {
+    for (int s = tid; s < p.S; s += kStepThreads) {
+      const int c = p.scount[s];
+      cnt[s] = c;
+      keys[s] = c > 0 ? p.skey[s] : 0ull;
+      nblk[s] = nblocks_of(p, s);
+    }
+    __syncthreads();
+  } else {
+    cg::cluster_group cluster = cg::this_cluster();
+    const int x = blockIdx.x * kStepThreads + tid, s0 = x & ~31;
+    if (s0 < p.S) {
+      const int c = x < p.S ? p.cnt[x].x : 0;
+      const lv_session_state st = load_states(p.sess + s0, p.S - s0, sh.states[tid >> 5]);
+      if (x < p.S) {
+        const unsigned long long key = c > 0 ? session_key(p, st, x, now_us, fallback) : 0ull;
+        cluster.map_shared_rank(keys, 0)[x] = key;
+        cluster.map_shared_rank(cnt, 0)[x] = c;
+        cluster.map_shared_rank(nblk, 0)[x] = blocks_of_context(p, st.ctx_tokens);
+      }
+    }
+    cluster.sync();
+    if (blockIdx.x > 0) return;
+  }
+  const Selected sel = select_sessions(p, keys, off, cnt, k, -1, sh, scan);
+  OwnerCheck check{0, 0, -1, -1};
+  const VictimList list{nullptr, out, nullptr, 0, sel.n_out};
+  emit_selected(p, sel, keys, off, nblk, list, check, sh, scan);
+  if (tid == 0) {
+    p.ctl[C_SEL_COUNT] = sel.n_out;
+    p.ctl[C_SEL_TOTAL] = sel.total;
+    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_SELECTS]), 1ull);
+    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_VICTIMS]), (unsigned long long)sel.n_out);
+    if (sel.total < k) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_SHORTFALLS]), 1ull);
+    if (fallback) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_FALLBACK]), 1ull);
+    if (count_dev) *count_dev = sel.n_out;
   }
 }
 
@@ -2823,23 +3055,51 @@ cudaError_t launch_events(const DevPool& p, const lv_event* ev, int64_t n, cudaS
   return launch_pdl(k_events, blocks_for(p.S, kEventThreads, 1 << 20), kEventThreads, 0, s, p, ev, (long long)n);
 }
 
+// One kernel up to kSelectMost victims (after a census where no counts are kept); more are
+// written by a CTA per session.
 cudaError_t launch_select(const DevPool& p, int64_t now_us, int64_t k, bool fallback,
                           lv_victim* out, long long* count_dev, cudaStream_t s) {
-  cudaError_t e = launch_pdl(k_rank_census, (unsigned)p.S, kCensusThreads, 0, s, p, (long long)now_us,
-                             fallback);
+  const size_t smem = select_layout(p.S).total;
+  const bool one = k <= kSelectMost && k <= (long long)kSelectSessions * p.maxB;
+  if (one && p.cnt) {
+    unsigned ctas = 1;
+    while ((int)ctas * kStepThreads < p.S) ctas *= 2;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(kStepThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = ctas;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = ctas > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, k_select<false>, p, (long long)now_us, (long long)k, fallback, count_dev, out);
+  }
+  const bool by_warp = p.maxB <= 1024;
+  cudaError_t e = by_warp ? launch_pdl(k_rank_census<32>, blocks_for(p.S, kCensusThreads / 32, 1 << 20), kCensusThreads,
+                                       0, s, p, (long long)now_us, fallback)
+                          : launch_pdl(k_rank_census<kCensusThreads>, (unsigned)p.S, kCensusThreads, 0, s, p,
+                                       (long long)now_us, fallback);
   if (e != cudaSuccess) return e;
+  if (one) {
+    e = cudaFuncSetAttribute(k_select<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)select_layout(4096).total);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(k_select<true>, 1, kStepThreads, smem, s, p, (long long)now_us, (long long)k, fallback, count_dev,
+                      out);
+  }
   if (p.S > kEmitScanMax) {
     const dim3 grid((unsigned)((p.S + kPrefixTile - 1) / kPrefixTile),
                     (unsigned)((p.S + kPrefixChunk - 1) / kPrefixChunk));
     e = launch_pdl(k_rank_prefix, grid, kPrefixTile, 0, s, p);
     if (e != cudaSuccess) return e;
   }
-  e = launch_pdl(k_rank_emit, (unsigned)p.S, kEmitThreads, 0, s, p, (long long)k, fallback,
-                 count_dev, out);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return launch_pdl(k_rank_emit, (unsigned)p.S, kEmitThreads, 0, s, p, (long long)k, fallback, count_dev, out);
 }
-
 
 cudaError_t launch_alloc(const DevPool& p, bool hbm, int64_t n, int32_t* out, cudaStream_t s,
                          bool injected_fail) {
@@ -2884,6 +3144,8 @@ bool bits_fit(const DevPool& p, size_t others) {
 
 cudaError_t configure_step_kernels() {
   cudaError_t e = cudaFuncSetAttribute(k_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStepDynamic);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_select<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)select_layout(4096).total);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_exchange_plan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStepDynamic);
 }

@@ -39,7 +39,7 @@ class KVPool:
         self.S, self.max_blocks = max_sessions, max_blocks
         self.hbm_pages, self.budget, self.host_pages = hbm_pages, hbm_budget_pages, host_pages
         self.launches = 0      # liblv kernels launched through this object
-        # a ranking is two kernels, three above 1024 sessions (liblv's k_rank_prefix)
+        # a ranking of many victims is two kernels, three above 1024 sessions
         self.rank_extra = 1 if max_sessions > lv.EMIT_SCAN_MAX else 0
         self.policy = policy
         self.tiers = tiers
@@ -137,7 +137,8 @@ class KVPool:
                                                                 device=self.device)
         lv.lv_select_victims(self.handle, now_us, min(k, lv.LV_ALL), flags, out, cap,
                              self.count_h[0:1], self.stream)
-        self.launches += 2 + self.rank_extra
+        self.launches += 1 if min(k, cap) <= min(lv.SELECT_MOST, lv.SELECT_SESSIONS * self.max_blocks) \
+            else 2 + self.rank_extra
         self.sync()
         n = int(self.count_h[0])
         return out[:n], n
