@@ -982,10 +982,7 @@ lv_status lv_swap_out(lv_pool* pool, const lv_victim* victims, int64_t n, int32_
     if ((r = st.out(commit_out, (size_t)n * sizeof(lv_remap_entry), &cdev, false)) != LV_OK) return r;
     int32_t* slots = static_cast<int32_t*>(sdev);
     const bool fail_alloc = fault_fires(pool, LV_FAULT_HOST_ALLOC);
-    if (pool->d.incl)
-      LV_TRY(lv::launch_alloc_out(pool->d, static_cast<const lv_victim*>(vin), n, slots, s, fail_alloc));
-    else
-      LV_TRY(lv::launch_alloc(pool->d, false, n, slots, s, fail_alloc));
+    LV_TRY(lv::launch_alloc(pool->d, false, static_cast<const lv_victim*>(vin), n, slots, s, fail_alloc));
     if (mode == LV_MODE_STAGED) {
       void* tdev = nullptr;
       if ((r = st.out(nullptr, (size_t)n * sizeof(int4), &tdev, true)) != LV_OK) return r;
@@ -1023,7 +1020,7 @@ lv_status lv_swap_in(lv_pool* pool, int32_t sid, const int32_t* blks, int64_t n,
     if ((r = st.out(pages_out, (size_t)n * 4, &pdev, true)) != LV_OK) return r;
     if ((r = st.out(commit_out, (size_t)n * sizeof(lv_remap_entry), &cdev, false)) != LV_OK) return r;
     int32_t* pages = static_cast<int32_t*>(pdev);
-    LV_TRY(lv::launch_alloc(pool->d, true, n, pages, s, fault_fires(pool, LV_FAULT_HBM_ALLOC)));
+    LV_TRY(lv::launch_alloc(pool->d, true, nullptr, n, pages, s, fault_fires(pool, LV_FAULT_HBM_ALLOC)));
     if (mode == LV_MODE_STAGED) {
       void* tdev = nullptr;
       if ((r = st.out(nullptr, (size_t)n * sizeof(int4), &tdev, true)) != LV_OK) return r;

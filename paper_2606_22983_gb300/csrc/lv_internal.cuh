@@ -110,12 +110,10 @@ cudaError_t launch_session_set(const DevPool& p, const lv_session_state* in, int
 cudaError_t launch_events(const DevPool& p, const lv_event* ev, int64_t n, cudaStream_t s);
 cudaError_t launch_select(const DevPool& p, int64_t now_us, int64_t k, bool fallback,
                           lv_victim* out, long long* count_dev, cudaStream_t s);
-cudaError_t launch_alloc(const DevPool& p, bool hbm, int64_t n, int32_t* out, cudaStream_t s,
-                         bool injected_fail = false);
-// host slots for n victims: a clean copy where the block has one (inclusive
-// tiers), else the lowest free slots in victim order (reserved)
-cudaError_t launch_alloc_out(const DevPool& p, const lv_victim* v, int64_t n, int32_t* out,
-                             cudaStream_t s, bool injected_fail = false);
+// Reserves the n lowest free pages (in_hbm) or slots.  Inclusive tiers, slots: one of v's
+// victims that has a clean copy gets that one and reserves nothing.
+cudaError_t launch_alloc(const DevPool& p, bool in_hbm, const lv_victim* v, int64_t n, int32_t* out,
+                         cudaStream_t s, bool injected_fail);
 cudaError_t launch_swap_out(const DevPool& p, const lv_victim* v, const int32_t* slots,
                             int64_t n, lv_remap_entry* commit, cudaStream_t s, int num_sms,
                             const EventPair* ev = nullptr);

@@ -99,78 +99,10 @@ __device__ long long block_excl_scan(long long v, long long* total) {
   return before + x - v;
 }
 
-__device__ __forceinline__ uint32_t free_bits(const uint32_t* bits, long long w, long long W,
-                                              long long nbits) {
-  uint32_t valid = 0xffffffffu;
-  if (w == W - 1 && (nbits & 31)) valid = (1u << (nbits & 31)) - 1u;
-  return ~bits[w] & valid;
-}
-
-// The n lowest free bits of a bitmap, ascending, into out[0..n); sets them.
-// Each thread owns a contiguous run of words and writes only the ranks it
-// counted, so a concurrent free elsewhere cannot make two threads write one rank.
-template <int NT>
-__device__ void block_alloc_lowest(uint32_t* bits, long long nbits, long long n, int32_t* out) {
-  const long long W = (nbits + 31) >> 5;
-  const long long per = (W + NT - 1) / NT;
-  const long long w0 = min(W, (long long)threadIdx.x * per);
-  const long long w1 = min(W, w0 + per);
-  long long cnt = 0;
-  for (long long w = w0; w < w1; ++w) cnt += __popc(free_bits(bits, w, W, nbits));
-  long long total;
-  const long long base = block_excl_scan<NT>(cnt, &total);
-  long long r = base;
-  const long long r_end = min(n, base + cnt);
-  for (long long w = w0; w < w1 && r < r_end; ++w) {
-    uint32_t f = free_bits(bits, w, W, nbits);
-    uint32_t take = 0;
-    while (f && r < r_end) {
-      int b = __ffs(f) - 1;
-      f &= f - 1;
-      out[r++] = (int32_t)(w * 32 + b);
-      take |= 1u << b;
-    }
-    if (take) atomicOr(&bits[w], take);
-  }
-}
-
 // Inclusive tiers: the host slot holding victim x's clean copy, or -1.
 __device__ __forceinline__ int32_t clean_copy_of(const DevPool& p, const lv_victim& x) {
   if (!p.incl || x.sid < 0 || x.sid >= p.S || x.blk < 0 || x.blk >= p.maxB) return -1;
   return p.shadow[(size_t)x.sid * p.maxB + x.blk];
-}
-
-// Host slots for n victims when nd of them have no clean copy: the nd lowest
-// free slots are taken (ascending) into out[0..nd), then spread in place so
-// that the r-th victim without a copy gets the r-th slot and every other
-// victim its copy.  The spreading runs from the last chunk to the first: a
-// victim's rank r is at most its index, so each read position still holds its
-// compact value when it is read.
-template <int NT>
-__device__ void block_alloc_out(const DevPool& p, const lv_victim* __restrict__ v, long long n,
-                                long long nd, int32_t* out) {
-  if (nd > 0) block_alloc_lowest<NT>(p.bits_host, p.host_pages, nd, out);
-  __syncthreads();
-  for (long long r = threadIdx.x; r < nd; r += NT) p.own_host[out[r]] = kOwnerReserved;
-  __syncthreads();
-  if (nd == n) return;
-  long long after = 0;   // victims without a copy in the chunks already spread
-  for (long long c = (n + NT - 1) / NT - 1; c >= 0; --c) {
-    const long long i = c * NT + threadIdx.x;
-    int32_t cp = -1;
-    long long d = 0;
-    if (i < n) {
-      cp = clean_copy_of(p, v[i]);
-      d = cp < 0;
-    }
-    long long chunk;
-    const long long excl = block_excl_scan<NT>(d, &chunk);
-    const int32_t val = (i < n && d) ? out[nd - after - chunk + excl] : cp;
-    __syncthreads();
-    if (i < n) out[i] = val;
-    __syncthreads();
-    after += chunk;
-  }
 }
 
 // ---------------------------------------------------------------- counts
@@ -180,8 +112,15 @@ __device__ void block_alloc_out(const DevPool& p, const lv_victim* __restrict__ 
 // instead of S table rows.
 __device__ __forceinline__ int2 tier_of(int32_t e) { return make_int2(e >= 0 ? 1 : 0, e <= -2 ? 1 : 0); }
 
+// Both counts change by one 64-bit addition of dd * 2^32 + dh (a negative dh borrows from the
+// upper half what the sum gives back).
+__device__ __forceinline__ void add_counts(const DevPool& p, int32_t s, int dh, int dd) {
+  atomicAdd(reinterpret_cast<unsigned long long*>(&p.cnt[s]),
+            ((unsigned long long)(unsigned)dd << 32) + (unsigned long long)(long long)dh);
+}
+
 // Adds (dh, dd) to the counts of session s, for the whole warp at once: lanes that share the
-// first adding lane's session add through one pair of reductions, the others by themselves.
+// first adding lane's session add through one reduction, the others by themselves.
 // All 32 lanes must call it; a lane with nothing to add passes zeros.
 __device__ __forceinline__ void warp_count(const DevPool& p, int32_t s, int dh, int dd) {
   const unsigned act = __ballot_sync(0xffffffffu, dh != 0 || dd != 0);
@@ -192,11 +131,9 @@ __device__ __forceinline__ void warp_count(const DevPool& p, int32_t s, int dh, 
   const int h = __reduce_add_sync(0xffffffffu, mine ? dh : 0);
   const int d = __reduce_add_sync(0xffffffffu, mine ? dd : 0);
   if ((int)(threadIdx.x & 31) == lead) {
-    if (h) atomicAdd(&p.cnt[s0].x, h);
-    if (d) atomicAdd(&p.cnt[s0].y, d);
+    add_counts(p, s0, h, d);
   } else if (adds && !mine) {
-    if (dh) atomicAdd(&p.cnt[s].x, dh);
-    if (dd) atomicAdd(&p.cnt[s].y, dd);
+    add_counts(p, s, dh, dd);
   }
 }
 
@@ -584,66 +521,6 @@ k_rank_emit(DevPool p, long long k, bool fallback, long long* count_dev,
   pdl_trigger();
 }
 
-// ------------------------------------------------------------ allocation
-constexpr int kAllocThreads = 1024;
-
-__global__ void __launch_bounds__(kAllocThreads)
-k_alloc(DevPool p, bool hbm, long long n, int32_t* __restrict__ out, bool injected_fail) {
-  __shared__ int ok;
-  uint32_t* bits = hbm ? p.bits_hbm : p.bits_host;
-  const long long nbits = hbm ? p.hbm_pages : p.host_pages;
-  const long long cap = hbm ? p.budget : p.host_pages;
-  long long* counter = &p.ctl[hbm ? C_HBM_ALLOC : C_HOST_ALLOC];
-  if (threadIdx.x == 0) {
-    const long long before = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(counter),
-                                                  (unsigned long long)n);
-    ok = before + n <= cap && !injected_fail;
-    if (!ok) {
-      atomicAdd(reinterpret_cast<unsigned long long*>(counter), (unsigned long long)(-n));
-      set_error(p.ctl, hbm ? LV_ERR_NO_HBM : LV_ERR_NO_HOST, n);
-    }
-  }
-  __syncthreads();
-  if (!ok) {
-    for (long long i = threadIdx.x; i < n; i += kAllocThreads) out[i] = -1;
-    return;
-  }
-  block_alloc_lowest<kAllocThreads>(bits, nbits, n, out);
-  __syncthreads();
-  uint32_t* own = hbm ? p.own_hbm : p.own_host;
-  for (long long i = threadIdx.x; i < n; i += kAllocThreads) own[out[i]] = kOwnerReserved;
-}
-
-// Host slots of a swap-out under inclusive tiers (one CTA): victims with a clean
-// copy take it; only the others count against the host tier and reserve slots.
-__global__ void __launch_bounds__(kAllocThreads)
-k_alloc_out(DevPool p, const lv_victim* __restrict__ v, long long n, int32_t* __restrict__ out,
-            bool injected_fail) {
-  __shared__ int ok;
-  __shared__ long long nd_s;
-  long long cnt = 0;
-  for (long long i = threadIdx.x; i < n; i += kAllocThreads) cnt += clean_copy_of(p, v[i]) < 0;
-  long long nd;
-  block_excl_scan<kAllocThreads>(cnt, &nd);
-  if (threadIdx.x == 0) {
-    long long* counter = &p.ctl[C_HOST_ALLOC];
-    const long long before = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(counter),
-                                                  (unsigned long long)nd);
-    ok = before + nd <= p.host_pages && !injected_fail;
-    if (!ok) {
-      atomicAdd(reinterpret_cast<unsigned long long*>(counter), (unsigned long long)(-nd));
-      set_error(p.ctl, LV_ERR_NO_HOST, nd);
-    }
-    nd_s = nd;
-  }
-  __syncthreads();
-  if (!ok) {
-    for (long long i = threadIdx.x; i < n; i += kAllocThreads) out[i] = -1;
-    return;
-  }
-  block_alloc_out<kAllocThreads>(p, v, n, nd_s, out);
-}
-
 // ------------------------------------------------------------------ copy
 constexpr int kCopyThreads = 256;
 constexpr int kCopyUnroll = 4;
@@ -670,6 +547,7 @@ __device__ __forceinline__ void copy_subpage(const int4* __restrict__ src, int4*
 __global__ void __launch_bounds__(kCopyThreads)
 k_swap_out(DevPool p, const lv_victim* __restrict__ v, const int32_t* __restrict__ slots,
            long long n, lv_remap_entry* __restrict__ commit) {
+  pdl_wait();
   const long long units = n * p.J;
   const int nvec = (int)(p.P >> 4);
   for (long long u = blockIdx.x; u < units; u += gridDim.x) {
@@ -695,12 +573,14 @@ k_swap_out(DevPool p, const lv_victim* __restrict__ v, const int32_t* __restrict
     int4* dst = reinterpret_cast<int4*>(p.host + ((size_t)slot * p.J + j) * p.P);
     copy_subpage(src, dst, nvec);
   }
+  pdl_trigger();
 }
 
 // Unit u = (block i, sub-page j): host[slot(blk_i)][j] -> hbm_kv[j][page_i].
 __global__ void __launch_bounds__(kCopyThreads)
 k_swap_in(DevPool p, int32_t sid, const int32_t* __restrict__ blks,
           const int32_t* __restrict__ pages, long long n, lv_remap_entry* __restrict__ commit) {
+  pdl_wait();
   const long long units = n * p.J;
   const int nvec = (int)(p.P >> 4);
   const bool sid_ok = sid >= 0 && sid < p.S;
@@ -728,6 +608,7 @@ k_swap_in(DevPool p, int32_t sid, const int32_t* __restrict__ blks,
     int4* dst = reinterpret_cast<int4*>(p.kv[j] + (size_t)page * p.P);
     copy_subpage(src, dst, nvec);
   }
+  pdl_trigger();
 }
 
 // ------------------------------------------------------- one-CTA decisions
@@ -849,8 +730,10 @@ __device__ __forceinline__ int nth_bit(uint32_t f, int k) {
 // The n lowest free bits, ascending, into out[0..n); sets them.  Each thread owns a
 // contiguous run of words and counts its free bits; then thread i finds the i-th one by
 // binary search among the threads' counts (in `base`), so that a tier with whole free words
-// takes as long as one with a free bit here and there.  The caller has checked that n are
-// free; other threads may read out when it returns.
+// takes as long as one with a free bit here and there.  Without a copy of the bitmap each
+// thread writes its own words' bits, and no more than it counted: a free on another stream
+// may add bits meanwhile.  The caller has checked that n are free; other threads may read
+// out when it returns.
 __device__ void take_lowest(const TierBits& t, int n, int32_t* out, BlockScan& scan, int* base) {
   const int W = (int)((t.nbits + 31) >> 5);
   const int per = (W + kStepThreads - 1) / kStepThreads;
@@ -862,6 +745,23 @@ __device__ void take_lowest(const TierBits& t, int n, int32_t* out, BlockScan& s
   for (int i = 0; i < per; ++i) cnt += __popc(free_of(w0 + i));
   int total;
   int r = scan.sum(cnt, &total);
+  if (LV_RARE(t.cur == t.gl)) {
+    const int r_end = min(n, r + cnt);
+#pragma unroll 1
+    for (int i = 0; i < per && r < r_end; ++i) {
+      uint32_t f = free_of(w0 + i), take = 0;
+#pragma unroll 1
+      while (f && r < r_end) {
+        const int b = __ffs(f) - 1;
+        f &= f - 1;
+        out[r++] = (w0 + i) * 32 + b;
+        take |= 1u << b;
+      }
+      if (take) t.set(w0 + i, take);
+    }
+    __syncthreads();
+    return;
+  }
   base[threadIdx.x] = r;
   __syncthreads();
 #pragma unroll 1
@@ -888,6 +788,67 @@ __device__ void take_lowest(const TierBits& t, int n, int32_t* out, BlockScan& s
     if (take) t.set(w0 + i, take);
     r += c;
   }
+}
+
+// Spreads the nd slots out[0..nd) so that the r-th victim without a clean copy has the r-th of
+// them and every other victim its copy.  In place, from the last chunk to the first: a
+// victim's rank among those without a copy is at most its index, so each read position
+// still holds its compact value when it is read.
+__device__ void spread_slots(const DevPool& p, const lv_victim* v, long long n, int nd, int32_t* out,
+                             BlockScan& scan) {
+  long long after = 0;   // victims without a copy in the chunks already spread
+#pragma unroll 1
+  for (long long c = (n + kStepThreads - 1) / kStepThreads - 1; c >= 0; --c) {
+    const long long i = c * kStepThreads + threadIdx.x;
+    const int32_t cp = i < n ? clean_copy_of(p, v[i]) : 0;
+    int chunk;
+    const int excl = scan.rank(cp < 0, &chunk);
+    const int32_t val = cp < 0 ? out[nd - after - chunk + excl] : cp;
+    __syncthreads();
+    if (i < n) out[i] = val;
+    __syncthreads();
+    after += chunk;
+  }
+}
+
+// ------------------------------------------------------------ allocation
+// Reserves n pages or slots, the lowest free ones (one CTA).  v: a swap-out's victims under
+// inclusive tiers -- those with a clean copy take it, only the others count against the
+// host tier.
+__global__ void __launch_bounds__(kStepThreads, 1)
+k_alloc(DevPool p, bool in_hbm, const lv_victim* v, long long n, int32_t* out, bool injected_fail,
+        int copy_bits) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ int ws[2 * kStepWarps];
+  __shared__ int base[kStepThreads];
+  pdl_entry();
+  BlockScan scan{ws, 0};
+  uint32_t* copy = copy_bits ? reinterpret_cast<uint32_t*>(dyn) : nullptr;
+  const TierBits t = in_hbm ? bits_copy(p.bits_hbm, p.hbm_pages, copy) : bits_copy(p.bits_host, p.host_pages, copy);
+  const long long before = p.ctl[in_hbm ? C_HBM_ALLOC : C_HOST_ALLOC];
+  int nd = (int)n;
+  if (LV_RARE(v != nullptr)) {
+    int cnt = 0;
+#pragma unroll 1
+    for (long long i = threadIdx.x; i < n; i += kStepThreads) cnt += clean_copy_of(p, v[i]) < 0 ? 1 : 0;
+    scan.sum(cnt, &nd);
+  }
+  if (LV_RARE(before + nd > (in_hbm ? p.budget : p.host_pages) || injected_fail)) {
+    if (threadIdx.x == 0) set_error(p.ctl, in_hbm ? LV_ERR_NO_HBM : LV_ERR_NO_HOST, nd);
+#pragma unroll 1
+    for (long long i = threadIdx.x; i < n; i += kStepThreads) out[i] = -1;
+    return;
+  }
+  __syncthreads();             // the bitmap's copy is complete
+  if (nd > 0) take_lowest(t, nd, out, scan, base);
+  uint32_t* own = in_hbm ? p.own_hbm : p.own_host;
+#pragma unroll 1
+  for (int i = threadIdx.x; i < nd; i += kStepThreads) own[out[i]] = kOwnerReserved;
+  __syncthreads();
+  if (LV_RARE(nd < n)) spread_slots(p, v, n, nd, out, scan);
+  bits_back(t);
+  if (threadIdx.x == 0)
+    atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[in_hbm ? C_HBM_ALLOC : C_HOST_ALLOC]), (unsigned long long)nd);
 }
 
 // -------------------------------------------------------------- exchange
@@ -1018,25 +979,11 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
     if (threadIdx.x == 0) *m.n_tasks = 0;
     return false;
   }
-  // host slots for the victims: a clean copy, or the lowest free slots in victim order.
-  // The compact list of new slots is spread in place from the last chunk to the first: a
-  // victim's rank among those without a copy is at most its index, so each read position
-  // still holds its compact value when it is read.
+  // host slots for the victims: a clean copy, or the lowest free slots in victim order
   if (n_dirty > 0) take_lowest(host, n_dirty, m.slots, scan, sh.base);
   if (LV_RARE(n_dirty < n_out)) {
-    long long after = 0;   // victims without a copy in the chunks already spread
-#pragma unroll 1
-    for (long long c = (n_out + kStepThreads - 1) / kStepThreads - 1; c >= 0; --c) {
-      const long long i = c * kStepThreads + threadIdx.x;
-      const int32_t cp = i < n_out ? clean_copy_of(p, m.v[i]) : 0;
-      int chunk;
-      const int excl = scan.rank(cp < 0, &chunk);
-      const int32_t val = cp < 0 ? m.slots[n_dirty - after - chunk + excl] : cp;
-      __syncthreads();
-      if (i < n_out) m.slots[i] = val;
-      __syncthreads();
-      after += chunk;
-    }
+    __syncthreads();
+    spread_slots(p, m.v, n_out, n_dirty, m.slots, scan);
   }
   // out-commit: victims now live in their slots, their pages are free.  A page that an
   // incoming block takes pairs that block's task with its victim's: found by looking the
@@ -1157,10 +1104,7 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
     *m.n_tasks = n_in + run;
     const long long n_clean = n_out - n_dirty;
     const long long host_delta = p.incl ? n_dirty : n_dirty - n_in;
-    if (n_in) {
-      atomicAdd(&p.cnt[m.sid].x, (int)n_in);
-      atomicAdd(&p.cnt[m.sid].y, -(int)n_in);
-    }
+    if (n_in) add_counts(p, m.sid, (int)n_in, -(int)n_in);
     atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HOST_ALLOC]), (unsigned long long)host_delta);
     if (LV_RARE(p.incl)) {
       atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_CLEAN]), (unsigned long long)(n_in - n_clean));
@@ -1238,7 +1182,7 @@ __device__ long long append_tokens_to(const DevPool& p, int32_t sid, int32_t ctx
   if (threadIdx.x == 0) {
     if (m > 0) {
       atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]), (unsigned long long)m);
-      atomicAdd(&p.cnt[sid].x, (int)m);
+      add_counts(p, sid, (int)m, 0);
     }
     // inclusive tiers: the partially filled last block gains rows, its clean copy is stale
     if (LV_RARE(p.incl) && n_tokens > 0 && nb > 0 && ctx % p.T != 0) {
@@ -1260,18 +1204,23 @@ __device__ long long append_tokens_to(const DevPool& p, int32_t sid, int32_t ctx
 }
 
 __global__ void __launch_bounds__(kStepThreads)
-k_append(DevPool p, int32_t sid, int32_t n_tokens, int32_t* pages, int32_t* count) {
+k_append(DevPool p, int32_t sid, int32_t n_tokens, int32_t* pages, int32_t* count, int copy_bits) {
+  extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ int ws[2 * kStepWarps];
   __shared__ int32_t near[kStepItems];
   __shared__ int base[kStepThreads];
   pdl_entry();
   BlockScan scan{ws, 0};
-  const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, nullptr);
-  const TierBits host = bits_copy(p.bits_host, p.host_pages, nullptr);
+  const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, copy_bits ? reinterpret_cast<uint32_t*>(dyn) : nullptr);
+  const TierBits host = bits_copy(p.bits_host, p.host_pages, nullptr);      // one bit of it at most
   const int32_t ctx = p.sess[sid].ctx_tokens;
   const long long hbm_alloc = p.ctl[C_HBM_ALLOC];
   __syncthreads();      // every thread has read both
   const long long m = append_tokens_to(p, sid, ctx, n_tokens, pages, hbm_alloc, hbm, host, near, scan, base);
+  if (m > 0) {
+    __syncthreads();
+    bits_back(hbm);
+  }
   if (threadIdx.x == 0 && count) *count = m > 0 ? (int32_t)m : 0;
 }
 
@@ -1777,6 +1726,7 @@ __device__ __forceinline__ int remap_judge(const RemapRead& r, int32_t epoch, in
 // no other entry of the call can see them, since only an entry for the same
 // block reads its table word (and the mark turned it away), and every claim of
 // an owned location fails, kOwnerFreeing or not.
+template <bool kDirect>
 __device__ __forceinline__ int remap_claim(const DevPool& p, const RemapRead& r, int err,
                                            uint32_t& got, uint32_t& was) {
   if (err) return err;
@@ -1796,10 +1746,10 @@ __device__ __forceinline__ int remap_claim(const DevPool& p, const RemapRead& r,
   const int32_t old = r.old;
   const long long old_slot = -(long long)old - 2;
   if (old >= 0 && old < p.hbm_pages) {
-    was = atomicExch(&p.own_hbm[old], kOwnerFreeing);
+    was = atomicExch(&p.own_hbm[old], kDirect ? kOwnerNone : kOwnerFreeing);
   } else if (old <= -2 && old_slot < p.host_pages) {
     if (p.incl && x.loc >= 0) was = p.own_host[old_slot];   // back in HBM: the slot stays as its clean copy
-    else was = atomicExch(&p.own_host[old_slot], kOwnerFreeing);
+    else was = atomicExch(&p.own_host[old_slot], kDirect ? kOwnerNone : kOwnerFreeing);
   }
   p.table[r.ti] = x.loc;
   return 0;
@@ -1809,6 +1759,7 @@ __device__ __forceinline__ int remap_claim(const DevPool& p, const RemapRead& r,
 // its entry's writes are put back; an accepted entry settles its clean copy
 // (inclusive tiers) and is counted, and a freed location that this block did not
 // own means the tables were inconsistent.
+template <bool kDirect>
 __device__ __forceinline__ void remap_settle(const DevPool& p, const RemapRead& r, int err,
                                              uint32_t got, uint32_t was, long long i,
                                              RemapCounts& c) {
@@ -1840,17 +1791,20 @@ __device__ __forceinline__ void remap_settle(const DevPool& p, const RemapRead& 
     p.shadow[r.ti] = -1;
     c.clean -= 1;
     if ((long long)g != h) {
-      atomicExch(&p.own_host[g], kOwnerFreeing);
+      atomicExch(&p.own_host[g], kDirect ? kOwnerNone : kOwnerFreeing);
+      if (kDirect) atomicAnd(&p.bits_host[g >> 5], ~(1u << (g & 31)));
       c.host += 1;
     }
   }
   if (old_hbm) {
+    if (kDirect) atomicAnd(&p.bits_hbm[old >> 5], ~(1u << (old & 31)));
     c.hbm += 1;
   } else if (old_host) {
     if (p.incl && x.loc >= 0) {
       p.shadow[r.ti] = (int32_t)old_slot;
       c.clean += 1;
     } else {
+      if (kDirect) atomicAnd(&p.bits_host[old_slot >> 5], ~(1u << (old_slot & 31)));
       c.host += 1;
     }
   }
@@ -1878,9 +1832,18 @@ __device__ __forceinline__ void remap_settle(const DevPool& p, const RemapRead& 
 // reservations), and another entry can take an owned location only through a
 // CAS, which then fails.  A thread's own entries are issued in order, so a
 // duplicate among them meets the epoch mark too.
-template <int E>
+//
+// kDirect: the freed locations' owner words and bitmap bits are cleared by the entries
+// themselves and there is no release pass.  That pass reads both tiers' owner words, whatever
+// the number of entries, and is a launch of its own: up to 2^18 entries the direct form is the
+// shorter (a pool of 2^20 pages and slots: 6.8 us against 10.9 for 1024 entries, 12.9 against
+// 15.0 for 2^18; scattered over the pool 37.5 against 39.6), at 2^20 the release pass (29.3
+// against 33.4), since it clears a run of freed pages by the word.
+template <int E, bool kDirect>
 __global__ void __launch_bounds__(kRemapThreads, 4)
 k_remap(DevPool p, const lv_remap_entry* __restrict__ e, long long n, int32_t epoch) {
+  if (kDirect) pdl_entry();
+  else pdl_wait();          // a large grid: the release pass is scheduled behind it
   const long long stride = (long long)gridDim.x * kRemapThreads;
   const long long i0 = blockIdx.x * (long long)kRemapThreads + threadIdx.x;
   RemapRead r[E];
@@ -1899,13 +1862,13 @@ k_remap(DevPool p, const lv_remap_entry* __restrict__ e, long long n, int32_t ep
     got[j] = kOwnerReserved;
     was[j] = kOwnerNone;
     err[j] = i0 + j * stride < n ? remap_judge(r[j], epoch, seen[j]) : -1;
-    if (err[j] >= 0) err[j] = remap_claim(p, r[j], err[j], got[j], was[j]);
+    if (err[j] >= 0) err[j] = remap_claim<kDirect>(p, r[j], err[j], got[j], was[j]);
   }
   RemapCounts c{0, 0, 0, 0, 0, 0};
 #pragma unroll
   for (int j = 0; j < E; ++j) {
     c.dh = c.dd = 0;
-    if (err[j] >= 0) remap_settle(p, r[j], err[j], got[j], was[j], i0 + j * stride, c);
+    if (err[j] >= 0) remap_settle<kDirect>(p, r[j], err[j], got[j], was[j], i0 + j * stride, c);
     warp_count(p, r[j].x.sid, c.dh, c.dd);
   }
   // block totals: warp sums, one shared atomic per warp, one global atomic per block
@@ -2734,8 +2697,7 @@ k_step(DevPool p, StepArgs a) {
       const int32_t s = sel.sorted ? session_of_key(keys[r]) : sh.sel_sid[r];
       const long long at = sel.sorted ? off[r] : sh.sel_off[r];
       const int take = (int)(n_out - at < cnt[s] ? n_out - at : cnt[s]);
-      atomicAdd(&p.cnt[s].x, -take);
-      atomicAdd(&p.cnt[s].y, take);
+      add_counts(p, s, -take, take);
     }
   }
   long long appended = 0;
@@ -2989,18 +2951,22 @@ k_counts(DevPool p, int32_t* __restrict__ hbm, int32_t* __restrict__ host) {
   }
 }
 
-__global__ void __launch_bounds__(kCensusThreads)
-k_blocks(DevPool p, int32_t sid, int32_t where, int32_t* __restrict__ out, long long* count) {
+__global__ void __launch_bounds__(kStepThreads)
+k_blocks(DevPool p, int32_t sid, int32_t where, int32_t* out, long long* count) {
+  __shared__ int ws[2 * kStepWarps];
+  pdl_entry();
+  BlockScan scan{ws, 0};
   const int32_t nb = nblocks_of(p, sid);
   const int32_t* row = p.table + (size_t)sid * p.maxB;
-  long long run = 0;
-  for (int32_t q0 = 0; q0 < nb; q0 += kCensusThreads) {
+  int run = 0;
+#pragma unroll 1
+  for (int32_t q0 = 0; q0 < nb; q0 += kStepThreads) {
     const int32_t b = q0 + threadIdx.x;
-    long long flag = 0;
-    if (b < nb) flag = where == 0 ? row[b] >= 0 : row[b] <= -2;
-    long long chunk;
-    const long long pos = run + block_excl_scan<kCensusThreads>(flag, &chunk);
-    if (flag) out[pos] = b;
+    const int32_t e = b < nb ? row[b] : -1;
+    const bool in = where == 0 ? e >= 0 : e <= -2;
+    int chunk;
+    const int pos = run + scan.rank(in, &chunk);
+    if (in) out[pos] = b;
     run += chunk;
   }
   if (threadIdx.x == 0 && count) *count = run;
@@ -3101,27 +3067,26 @@ cudaError_t launch_select(const DevPool& p, int64_t now_us, int64_t k, bool fall
   return launch_pdl(k_rank_emit, (unsigned)p.S, kEmitThreads, 0, s, p, (long long)k, fallback, count_dev, out);
 }
 
-cudaError_t launch_alloc(const DevPool& p, bool hbm, int64_t n, int32_t* out, cudaStream_t s,
-                         bool injected_fail) {
-  k_alloc<<<1, kAllocThreads, 0, s>>>(p, hbm, n, out, injected_fail);
-  return cudaGetLastError();
-}
+// The largest dynamic shared memory of the one-CTA kernels beside their static lists.
+constexpr size_t kStepDynamic = 180 * 1024;
 
-cudaError_t launch_alloc_out(const DevPool& p, const lv_victim* v, int64_t n, int32_t* out,
-                             cudaStream_t s, bool injected_fail) {
+cudaError_t launch_alloc(const DevPool& p, bool in_hbm, const lv_victim* v, int64_t n, int32_t* out,
+                         cudaStream_t s, bool injected_fail) {
   if (n <= 0) return cudaSuccess;
-  k_alloc_out<<<1, kAllocThreads, 0, s>>>(p, v, n, out, injected_fail);
-  return cudaGetLastError();
+  const size_t smem = 8 * (size_t)(((in_hbm ? p.hbm_pages : p.host_pages) + 31) >> 5);
+  const bool fit = smem <= kStepDynamic;
+  return launch_pdl(k_alloc, 1, kStepThreads, fit ? smem : 0, s, p, in_hbm, p.incl ? v : nullptr, (long long)n, out,
+                    injected_fail, fit ? 1 : 0);
 }
 
 cudaError_t launch_swap_out(const DevPool& p, const lv_victim* v, const int32_t* slots, int64_t n,
                             lv_remap_entry* commit, cudaStream_t s, int num_sms, const EventPair* ev) {
   const long long units = (long long)n * p.J;
   if (ev) cudaEventRecord(ev->start, s);
-  k_swap_out<<<blocks_for(units, 1, (long long)num_sms * 8), kCopyThreads, 0, s>>>(
-      p, v, slots, n, commit);
+  const cudaError_t e = launch_pdl(k_swap_out, blocks_for(units, 1, (long long)num_sms * 8), kCopyThreads, 0, s, p, v,
+                                   slots, (long long)n, commit);
   if (ev) cudaEventRecord(ev->end, s);
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_swap_in(const DevPool& p, int32_t sid, const int32_t* blks, const int32_t* pages,
@@ -3129,14 +3094,11 @@ cudaError_t launch_swap_in(const DevPool& p, int32_t sid, const int32_t* blks, c
                            const EventPair* ev) {
   const long long units = (long long)n * p.J;
   if (ev) cudaEventRecord(ev->start, s);
-  k_swap_in<<<blocks_for(units, 1, (long long)num_sms * 8), kCopyThreads, 0, s>>>(
-      p, sid, blks, pages, n, commit);
+  const cudaError_t e = launch_pdl(k_swap_in, blocks_for(units, 1, (long long)num_sms * 8), kCopyThreads, 0, s, p, sid,
+                                   blks, pages, (long long)n, commit);
   if (ev) cudaEventRecord(ev->end, s);
-  return cudaGetLastError();
+  return e;
 }
-
-// The largest dynamic shared memory of the one-CTA kernels beside their static lists.
-constexpr size_t kStepDynamic = 180 * 1024;
 
 bool bits_fit(const DevPool& p, size_t others) {
   return others + bits_words(p) * 4 <= kStepDynamic;
@@ -3144,6 +3106,10 @@ bool bits_fit(const DevPool& p, size_t others) {
 
 cudaError_t configure_step_kernels() {
   cudaError_t e = cudaFuncSetAttribute(k_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStepDynamic);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_alloc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStepDynamic);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_append, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStepDynamic);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_select<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)select_layout(4096).total);
   if (e != cudaSuccess) return e;
@@ -3347,6 +3313,8 @@ cudaError_t launch_tasks_pages(const DevPool& p, const int32_t* pages, int64_t n
   return cudaGetLastError();
 }
 
+constexpr long long kRemapDirect = 1 << 18;
+
 cudaError_t launch_remap(const DevPool& p, const lv_remap_entry* e, int64_t n, int32_t epoch,
                          cudaStream_t s, int num_sms, int per_thread) {
   if (n <= 0) return cudaSuccess;
@@ -3356,10 +3324,13 @@ cudaError_t launch_remap(const DevPool& p, const lv_remap_entry* e, int64_t n, i
   int E = per_thread;
   if (E != 1 && E != 2 && E != 4) E = n <= resident ? 1 : (n <= 2 * resident ? 2 : 4);
   const unsigned grid = blocks_for((n + E - 1) / E, kRemapThreads, 1ll << 30);
-  if (E == 1) k_remap<1><<<grid, kRemapThreads, 0, s>>>(p, e, n, epoch);
-  else if (E == 2) k_remap<2><<<grid, kRemapThreads, 0, s>>>(p, e, n, epoch);
-  else k_remap<4><<<grid, kRemapThreads, 0, s>>>(p, e, n, epoch);
-  cudaError_t err = cudaGetLastError();
+  cudaError_t err;
+  const unsigned T = kRemapThreads;
+  if (n <= kRemapDirect && per_thread == 0)
+    return launch_pdl(k_remap<1, true>, (unsigned)((n + T - 1) / T), T, 0, s, p, e, (long long)n, epoch);
+  if (E == 1) err = launch_pdl(k_remap<1, false>, grid, T, 0, s, p, e, (long long)n, epoch);
+  else if (E == 2) err = launch_pdl(k_remap<2, false>, grid, T, 0, s, p, e, (long long)n, epoch);
+  else err = launch_pdl(k_remap<4, false>, grid, T, 0, s, p, e, (long long)n, epoch);
   if (err != cudaSuccess) return err;
   // the release pass over both tiers' owner words (8 quads of 4 per bitmap word)
   const long long qh = (long long)((p.hbm_pages + 31) / 32) * 8;
@@ -3380,7 +3351,9 @@ cudaError_t launch_cancel(const DevPool& p, const int32_t* locs, int64_t n, cuda
 
 cudaError_t launch_append(const DevPool& p, int32_t sid, int32_t n_tokens, int32_t* pages,
                           int32_t* count, cudaStream_t s) {
-  return launch_pdl(k_append, 1, kStepThreads, 0, s, p, sid, n_tokens, pages, count);
+  const size_t smem = 8 * (size_t)((p.hbm_pages + 31) >> 5);
+  const bool fit = smem <= kStepDynamic;
+  return launch_pdl(k_append, 1, kStepThreads, fit ? smem : 0, s, p, sid, n_tokens, pages, count, fit ? 1 : 0);
 }
 
 cudaError_t launch_counts(const DevPool& p, int32_t* hbm, int32_t* host, cudaStream_t s) {
@@ -3390,8 +3363,7 @@ cudaError_t launch_counts(const DevPool& p, int32_t* hbm, int32_t* host, cudaStr
 
 cudaError_t launch_blocks(const DevPool& p, int32_t sid, int32_t where, int32_t* out,
                           long long* count, cudaStream_t s) {
-  k_blocks<<<1, kCensusThreads, 0, s>>>(p, sid, where, out, count);
-  return cudaGetLastError();
+  return launch_pdl(k_blocks, 1, kStepThreads, 0, s, p, sid, where, out, count);
 }
 
 }  // namespace lv

@@ -162,7 +162,7 @@ class KVPool:
 
     def remap(self, entries, n: int):
         lv.lv_remap(self.handle, entries, n, self.stream)
-        self.launches += 2 if n > 0 else 0
+        self.launches += (n > 0) + (n > lv.REMAP_DIRECT)   # the release pass of larger commits
 
     def cancel(self, locs, n: int):
         lv.lv_cancel(self.handle, locs, n, self.stream)
