@@ -162,13 +162,16 @@ class Staging {
     for (void* t : temps_) cudaFreeAsync(t, s_);
   }
 
-  lv_status in(const void* user, size_t bytes, const void** dev) {
+  // near: page-locked host memory is copied in too (for an argument that is read often)
+  lv_status in(const void* user, size_t bytes, const void** dev, bool near = false) {
     *dev = nullptr;
     if (bytes == 0) return LV_OK;
     if (user == nullptr) return LV_ERR_INVALID;
     if (const void* v = gpu_view(user)) {
-      *dev = v;
-      return LV_OK;
+      if (!near || is_device_ptr(user)) {
+        *dev = v;
+        return LV_OK;
+      }
     }
     void* t = nullptr;
     lv_status st = temp(bytes, &t);
@@ -389,7 +392,7 @@ lv_status staged_move_inner(lv_pool* pool, const int4* tasks_dev, int64_t n, cud
   // pack every chunk on s; the D2H runs of chunk c follow its pack
   for (int64_t c = 0; c * chunk < n_out; ++c) {
     const int64_t a = c * chunk, b = std::min(n_out, a + chunk);
-    LV_TRY(lv::launch_stage(d, true, tout_dev, a, b, stg_out, s, pool->stage_ctas,
+    LV_TRY(lv::launch_stage(d, true, false, tout_dev, a, b, stg_out, s, pool->stage_ctas,
                             timing_pair(pool, LV_TIMING_PACK), pool->stage_tma));
     LV_TRY(cudaEventRecord(ev_pack[c], s));
     LV_TRY(cudaStreamWaitEvent(pool->s_d2h, ev_pack[c], 0));
@@ -413,7 +416,7 @@ lv_status staged_move_inner(lv_pool* pool, const int4* tasks_dev, int64_t n, cud
   for (int64_t c = 0; c * chunk < n_in; ++c) {
     const int64_t a = c * chunk, b = std::min(n_in, a + chunk);
     LV_TRY(cudaStreamWaitEvent(us, ev_h2d[c], 0));
-    LV_TRY(lv::launch_stage(d, false, tin_dev, a, b, stg_in, us, pool->stage_ctas,
+    LV_TRY(lv::launch_stage(d, false, false, tin_dev, a, b, stg_in, us, pool->stage_ctas,
                             timing_pair(pool, LV_TIMING_UNPACK), pool->stage_tma));
   }
   return LV_OK;
@@ -1248,15 +1251,11 @@ lv_status pack_impl(lv_pool* pool, const int32_t* pages, int64_t n, void* run, b
   LV_TRY(join_copies(pool, s));
   Staging st(pool, s);
   const void* pin = nullptr;
-  void* tdev = nullptr;
-  lv_status r;
-  if ((r = st.in(pages, (size_t)n * 4, &pin)) != LV_OK) return r;
-  if ((r = st.out(nullptr, (size_t)n * sizeof(int4), &tdev, true)) != LV_OK) return r;
-  LV_TRY(lv::launch_tasks_pages(pool->d, static_cast<const int32_t*>(pin), n, pack,
-                                static_cast<int4*>(tdev), s));
-  LV_TRY(lv::launch_stage(pool->d, pack, static_cast<int4*>(tdev), 0, n, static_cast<uint8_t*>(rdev), s,
-                          pool->stage_ctas, timing_pair(pool, pack ? LV_TIMING_PACK : LV_TIMING_UNPACK),
-                          pool->stage_tma));
+  // every unit reads its page's id: a list in host memory is copied in
+  lv_status r = st.in(pages, (size_t)n * 4, &pin, true);
+  if (r != LV_OK) return r;
+  LV_TRY(lv::launch_stage(pool->d, pack, true, pin, 0, n, static_cast<uint8_t*>(rdev), s, pool->stage_ctas,
+                          timing_pair(pool, pack ? LV_TIMING_PACK : LV_TIMING_UNPACK), pool->stage_tma));
   return st.finish();
 }
 }  // namespace
@@ -1301,13 +1300,14 @@ lv_status lv_page_checksums(lv_pool* pool, const int32_t* pages, int64_t n, uint
     lv_status r;
     if ((r = st.in(pages, (size_t)n * 4, &pin)) != LV_OK) return r;
     if ((r = st.out(sums_out, (size_t)n * 8, &sdev, true)) != LV_OK) return r;
+    const int ctas = pool->num_sms * 8;
     void* cdev = nullptr;   // the kernel's unit cursor
-    if ((r = st.out(nullptr, sizeof(unsigned long long), &cdev, true)) != LV_OK) return r;
-    LV_TRY(cudaMemsetAsync(cdev, 0, sizeof(unsigned long long), s));
-    LV_TRY(lv::launch_zero(sdev, n * 8, s));
+    if (lv::checksums_need_cursor(pool->d, n, ctas) &&
+        (r = st.out(nullptr, sizeof(unsigned long long), &cdev, true)) != LV_OK)
+      return r;
     LV_TRY(lv::launch_checksums(pool->d, static_cast<const int32_t*>(pin), n,
                                 static_cast<unsigned long long*>(sdev),
-                                static_cast<unsigned long long*>(cdev), s, pool->num_sms * 8));
+                                static_cast<unsigned long long*>(cdev), s, ctas));
     return st.finish();
   } catch (const std::bad_alloc&) {
     return LV_ERR_OOM;

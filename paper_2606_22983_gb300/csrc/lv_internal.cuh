@@ -162,7 +162,9 @@ cudaError_t configure_step_kernels();
 cudaError_t launch_step(const DevPool& p, const ResidentScratch& rs, const StepCall& c, int32_t epoch,
                         cudaStream_t s, int copy_ctas, const EventPair* ev, const CopyOffload* off);
 cudaError_t launch_counts(const DevPool& p, int32_t* hbm, int32_t* host, cudaStream_t s);
-// sums[i] = position-weighted 64-bit sum of page pages[i] (sums zeroed by the caller)
+// sums[i] = position-weighted 64-bit sum of page pages[i]; cursor: a word of the call's own
+// where checksums_need_cursor says so, else null
+bool checksums_need_cursor(const DevPool& p, int64_t n, int ctas);
 cudaError_t launch_checksums(const DevPool& p, const int32_t* pages, int64_t n,
                              unsigned long long* sums, unsigned long long* cursor, cudaStream_t s,
                              int ctas);
@@ -178,12 +180,11 @@ cudaError_t launch_exchange_plan(const DevPool& p, const lv_victim* v, int64_t n
                                  const int32_t* blks, int64_t n_in, int32_t* slots, int32_t* pages,
                                  int4* tasks, long long* n_tasks, int32_t epoch,
                                  unsigned long long* page_tag, cudaStream_t s, long long* cursor = nullptr);
-// pack (staging[t] <- out pages) or unpack (in pages <- staging[t]) for tasks [t_begin, t_end)
-cudaError_t launch_stage(const DevPool& p, bool pack, const int4* tasks, int64_t t_begin,
-                         int64_t t_end, uint8_t* staging, cudaStream_t s, int ctas,
-                         const EventPair* ev, bool tma);
-cudaError_t launch_tasks_pages(const DevPool& p, const int32_t* pages, int64_t n, bool pack,
-                               int4* tasks, cudaStream_t s);
+// pack (staging[t] <- out pages) or unpack (in pages <- staging[t]) for entries [t_begin, t_end)
+// of a task list, or of a list of page ids (page_list)
+cudaError_t launch_stage(const DevPool& p, bool pack, bool page_list, const void* list, int64_t t_begin,
+                         int64_t t_end, uint8_t* staging, cudaStream_t s, int ctas, const EventPair* ev,
+                         bool tma);
 cudaError_t configure_stage_kernels(const DevPool& p);
 // The largest number of exchange-copy TMA stages (2P bytes each) for sub-pages of P
 // bytes (0 when two do not fit in a CTA's shared memory), and the kernel's set-up.

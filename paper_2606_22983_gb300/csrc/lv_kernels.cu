@@ -1442,16 +1442,33 @@ constexpr int kStageThreads = 32;     // one warp per CTA; lane 0 issues the bul
 constexpr int kMaxStages = 16;
 constexpr long long kWaitLimitNs = 1000000000ll;   // one second per stage wait
 
+// The HBM page of unit (t, j) of a stage kernel, -1 when the unit is skipped.
+template <bool kPack, bool kPages>
+__device__ __forceinline__ int32_t stage_page(const DevPool& p, const void* __restrict__ list, long long t, int j) {
+  if (kPages) {
+    const int32_t pg = static_cast<const int32_t*>(list)[t];
+    if (pg >= 0 && pg < p.hbm_pages) return pg;
+    if (j == 0) set_error(p.ctl, LV_ERR_BOUNDS, t);
+    return -1;
+  }
+  const int4 tk = static_cast<const int4*>(list)[t];
+  if (kPack) return tk.x;
+  return tk.z < 0 ? -1 : tk.w;
+}
+
 // Moves units u = (task t, sub-page j) of P bytes through `stages` shared-memory
 // buffers: unit i's load is issued `stages` units ahead of its store.
 // pack:   staging[t][j] <- hbm_kv[j][task.x]   for tasks with task.x >= 0
 // unpack: hbm_kv[j][task.w] <- staging[t][j]   for tasks with task.z >= 0
-template <bool kPack>
+// kPages: `list` holds page ids instead of tasks (lv_pack_pages, lv_unpack_pages); a page
+// outside the pool is reported and skipped.
+template <bool kPack, bool kPages>
 __global__ void __launch_bounds__(kStageThreads)
-k_stage_tasks(DevPool p, const int4* __restrict__ tasks, long long t_begin, long long t_end,
+k_stage_tasks(DevPool p, const void* __restrict__ list, long long t_begin, long long t_end,
               uint8_t* __restrict__ staging, int stages) {
   extern __shared__ __align__(128) unsigned char stage_mem[];
   __shared__ __align__(8) uint64_t bars[kMaxStages];
+  pdl_wait();
   if (threadIdx.x != 0) return;
   const uint32_t P = (uint32_t)p.P;
   for (int s = 0; s < stages; ++s) mbar_init(&bars[s], 1);
@@ -1462,17 +1479,12 @@ k_stage_tasks(DevPool p, const int4* __restrict__ tasks, long long t_begin, long
     const long long u = blockIdx.x + k * (long long)gridDim.x;
     const long long t = t_begin + u / p.J;
     const int j = (int)(u % p.J);
-    const int4 tk = tasks[t];
     uint8_t* st = staging + ((size_t)t * p.J + j) * P;
-    if (kPack) {
-      if (tk.x < 0) return false;
-      *src = p.kv[j] + (size_t)tk.x * P;
-      *dst = st;
-    } else {
-      if (tk.z < 0) return false;
-      *src = st;
-      *dst = p.kv[j] + (size_t)tk.w * P;
-    }
+    const int32_t pg = stage_page<kPack, kPages>(p, list, t, j);
+    if (pg < 0) return false;
+    uint8_t* page = p.kv[j] + (size_t)pg * P;
+    *src = kPack ? page : st;
+    *dst = kPack ? st : page;
     return true;
   };
   const long long mine = units > blockIdx.x ? (units - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
@@ -1618,40 +1630,23 @@ k_exchange_copy_tma(DevPool p, const int4* __restrict__ tasks, const long long* 
 }
 
 // The same moves with plain 16-byte loads and stores (256 threads per CTA).
-template <bool kPack>
+template <bool kPack, bool kPages>
 __global__ void __launch_bounds__(kCopyThreads)
-k_stage_tasks_lsu(DevPool p, const int4* __restrict__ tasks, long long t_begin, long long t_end,
+k_stage_tasks_lsu(DevPool p, const void* __restrict__ list, long long t_begin, long long t_end,
                   uint8_t* __restrict__ staging) {
+  pdl_wait();
   const long long units = (t_end - t_begin) * p.J;
   const int nvec = (int)(p.P >> 4);
   for (long long u = blockIdx.x; u < units; u += gridDim.x) {
     const long long t = t_begin + u / p.J;
     const int j = (int)(u % p.J);
-    const int4 tk = tasks[t];
-    uint8_t* st = staging + ((size_t)t * p.J + j) * p.P;
-    if (kPack) {
-      if (tk.x < 0) continue;
-      copy_subpage(reinterpret_cast<const int4*>(p.kv[j] + (size_t)tk.x * p.P), reinterpret_cast<int4*>(st), nvec);
-    } else {
-      if (tk.z < 0) continue;
-      copy_subpage(reinterpret_cast<const int4*>(st), reinterpret_cast<int4*>(p.kv[j] + (size_t)tk.w * p.P), nvec);
-    }
+    int4* st = reinterpret_cast<int4*>(staging + ((size_t)t * p.J + j) * p.P);
+    const int32_t pg = stage_page<kPack, kPages>(p, list, t, threadIdx.x == 0 ? j : 1);
+    if (pg < 0) continue;
+    int4* page = reinterpret_cast<int4*>(p.kv[j] + (size_t)pg * p.P);
+    if (kPack) copy_subpage(page, st, nvec);
+    else copy_subpage(st, page, nvec);
   }
-}
-
-// Tasks for a plain list of pages: pack reads them ({page, -1, -1, -1}), unpack
-// writes them ({-1, -1, 0, page}); an out-of-range page gives an empty task.
-__global__ void k_tasks_pages(DevPool p, const int32_t* __restrict__ pages, long long n, bool pack,
-                              int4* __restrict__ tasks) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int32_t pg = pages[i];
-  if (pg < 0 || pg >= p.hbm_pages) {
-    set_error(p.ctl, LV_ERR_BOUNDS, i);
-    tasks[i] = make_int4(-1, -1, -1, -1);
-    return;
-  }
-  tasks[i] = pack ? make_int4(pg, -1, -1, -1) : make_int4(-1, -1, 0, pg);
 }
 
 // Self-test of the bounded wait: one thread arms a stage barrier for bytes that no
@@ -2872,6 +2867,7 @@ k_checksum(DevPool p, const int32_t* __restrict__ pages, long long n, unsigned l
            unsigned long long* __restrict__ cursor) {
   __shared__ unsigned long long warp_part[kSumThreads / 32];
   __shared__ long long s_next;
+  pdl_wait();
   const long long units = n * p.J;
   const int nvec = (int)(p.P >> 4);                   // 16-byte vectors per sub-page
   // units come from a shared cursor, kSumBatch at a time, the next batch fetched while
@@ -2879,11 +2875,13 @@ k_checksum(DevPool p, const int32_t* __restrict__ pages, long long n, unsigned l
   // fewer units instead of holding up the end of the call
   // (thread 0 keeps the fetched index in a register and publishes it only at the end
   // of the batch, so that its warp does not wait for the atomic's result meanwhile)
-  if (threadIdx.x == 0) s_next = (long long)atomicAdd(cursor, (unsigned long long)kSumBatch);
+  // (null: the grid has a CTA for every batch)
+  if (threadIdx.x == 0)
+    s_next = cursor ? (long long)atomicAdd(cursor, (unsigned long long)kSumBatch) : (long long)blockIdx.x * kSumBatch;
   __syncthreads();
   for (long long b = s_next; b < units; b = s_next) {
-    unsigned long long fetched = 0;
-    if (threadIdx.x == 0) fetched = atomicAdd(cursor, (unsigned long long)kSumBatch);
+    unsigned long long fetched = (unsigned long long)units;
+    if (threadIdx.x == 0 && cursor) fetched = atomicAdd(cursor, (unsigned long long)kSumBatch);
     const long long b_end = b + kSumBatch < units ? b + kSumBatch : units;
     for (long long u = b; u < b_end; ++u) {
       const long long i = u / p.J;
@@ -3212,9 +3210,11 @@ cudaError_t launch_step(const DevPool& p, const ResidentScratch& rs, const StepC
   return launch_copy(p, rs.tasks, rs.words + R_N_TASKS, rs.words + R_CURSOR, most, s, copy_ctas, ev, off);
 }
 
-// Zeroes `words` 32-bit words at p, which may be device memory or the device alias of
-// mapped page-locked host memory (a kernel, so that either works).
-__global__ void k_zero(uint32_t* __restrict__ q, long long words) {
+// Zeroes `words` 32-bit words at q, which may be device memory or the device alias of
+// mapped page-locked host memory (a kernel, so that either works), and *cursor.
+__global__ void k_zero(uint32_t* __restrict__ q, long long words, unsigned long long* cursor) {
+  pdl_entry();
+  if (cursor && blockIdx.x == 0 && threadIdx.x == 0) *cursor = 0ull;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < words;
        i += (long long)gridDim.x * blockDim.x)
     q[i] = 0u;
@@ -3223,16 +3223,22 @@ __global__ void k_zero(uint32_t* __restrict__ q, long long words) {
 cudaError_t launch_zero(void* q, int64_t bytes, cudaStream_t s) {
   const long long words = (long long)(bytes / 4);
   if (words <= 0) return cudaSuccess;
-  k_zero<<<blocks_for(words, 256, 1024), 256, 0, s>>>(static_cast<uint32_t*>(q), words);
-  return cudaGetLastError();
+  return launch_pdl(k_zero, blocks_for(words, 256, 1024), 256, 0, s, static_cast<uint32_t*>(q), words,
+                    (unsigned long long*)nullptr);
 }
+
+bool checksums_need_cursor(const DevPool& p, int64_t n, int ctas) { return n * (long long)p.J > (long long)ctas * kSumBatch; }
 
 cudaError_t launch_checksums(const DevPool& p, const int32_t* pages, int64_t n,
                              unsigned long long* sums, unsigned long long* cursor, cudaStream_t s,
                              int ctas) {
   if (n <= 0) return cudaSuccess;
-  k_checksum<<<blocks_for(n * p.J, kSumBatch, ctas), kSumThreads, 0, s>>>(p, pages, n, sums, cursor);
-  return cudaGetLastError();
+  const long long words = 2 * (long long)n;
+  const cudaError_t e = launch_pdl(k_zero, blocks_for(words, 256, 1024), 256, 0, s, reinterpret_cast<uint32_t*>(sums),
+                                   words, cursor);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_checksum, blocks_for((n * (long long)p.J + kSumBatch - 1) / kSumBatch, 1, ctas), kSumThreads, 0, s, p,
+                    pages, (long long)n, sums, cursor);
 }
 
 cudaError_t launch_selftest_wait(const DevPool& p, long long limit_ns, cudaStream_t s) {
@@ -3263,11 +3269,17 @@ int stage_count(const DevPool& p) {
   return st < 2 ? 2 : st;
 }
 
+// Pools of different sub-page sizes share these kernels: the limit is set to what the largest
+// stages may take, never down to what one pool needs.
 cudaError_t configure_stage_kernels(const DevPool& p) {
-  const int smem = stage_count(p) * (int)p.P;
-  cudaError_t e = cudaFuncSetAttribute(k_stage_tasks<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_stage_tasks<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const int need = stage_count(p) * (int)p.P;
+  const int most = 227 * 1024 - 256 > need ? 227 * 1024 - 256 : need;
+  for (const void* f : {(const void*)k_stage_tasks<true, false>, (const void*)k_stage_tasks<false, false>,
+                        (const void*)k_stage_tasks<true, true>, (const void*)k_stage_tasks<false, true>}) {
+    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 int exchange_stage_limit(long long P) {
@@ -3283,34 +3295,29 @@ cudaError_t configure_exchange_tma(const DevPool& p) {
                               (int)((size_t)p.xstages * 2 * p.P));
 }
 
-cudaError_t launch_stage(const DevPool& p, bool pack, const int4* tasks, int64_t t_begin, int64_t t_end,
-                         uint8_t* staging, cudaStream_t s, int ctas, const EventPair* ev, bool tma) {
-  if (t_end <= t_begin) return cudaSuccess;
+template <bool kPack, bool kPages>
+static cudaError_t launch_stage_as(const DevPool& p, const void* list, int64_t t_begin, int64_t t_end,
+                                   uint8_t* staging, cudaStream_t s, int ctas, bool tma) {
   const long long units = (t_end - t_begin) * (long long)p.J;
-  if (ev) cudaEventRecord(ev->start, s);
   if (tma) {
     const int stages = stage_count(p);
-    const size_t smem = (size_t)stages * p.P;
-    const unsigned grid = blocks_for(units, 1, ctas);
-    if (pack)
-      k_stage_tasks<true><<<grid, kStageThreads, smem, s>>>(p, tasks, t_begin, t_end, staging, stages);
-    else
-      k_stage_tasks<false><<<grid, kStageThreads, smem, s>>>(p, tasks, t_begin, t_end, staging, stages);
-  } else {
-    const unsigned grid = blocks_for(units, 1, 4ll * ctas);
-    if (pack)
-      k_stage_tasks_lsu<true><<<grid, kCopyThreads, 0, s>>>(p, tasks, t_begin, t_end, staging);
-    else
-      k_stage_tasks_lsu<false><<<grid, kCopyThreads, 0, s>>>(p, tasks, t_begin, t_end, staging);
+    return launch_pdl(k_stage_tasks<kPack, kPages>, blocks_for(units, 1, ctas), kStageThreads, (size_t)stages * p.P, s,
+                      p, list, (long long)t_begin, (long long)t_end, staging, stages);
   }
-  if (ev) cudaEventRecord(ev->end, s);
-  return cudaGetLastError();
+  return launch_pdl(k_stage_tasks_lsu<kPack, kPages>, blocks_for(units, 1, 4ll * ctas), kCopyThreads, 0, s, p, list,
+                    (long long)t_begin, (long long)t_end, staging);
 }
 
-cudaError_t launch_tasks_pages(const DevPool& p, const int32_t* pages, int64_t n, bool pack, int4* tasks,
-                               cudaStream_t s) {
-  k_tasks_pages<<<blocks_for(n, 256, 1ll << 30), 256, 0, s>>>(p, pages, n, pack, tasks);
-  return cudaGetLastError();
+cudaError_t launch_stage(const DevPool& p, bool pack, bool page_list, const void* list, int64_t t_begin,
+                         int64_t t_end, uint8_t* staging, cudaStream_t s, int ctas, const EventPair* ev,
+                         bool tma) {
+  if (t_end <= t_begin) return cudaSuccess;
+  if (ev) cudaEventRecord(ev->start, s);
+  auto* launch = pack ? (page_list ? launch_stage_as<true, true> : launch_stage_as<true, false>)
+                      : (page_list ? launch_stage_as<false, true> : launch_stage_as<false, false>);
+  const cudaError_t e = launch(p, list, t_begin, t_end, staging, s, ctas, tma);
+  if (ev) cudaEventRecord(ev->end, s);
+  return e;
 }
 
 constexpr long long kRemapDirect = 1 << 18;
