@@ -898,7 +898,7 @@ struct StepLists {
 struct StepShared {
   int ws[2 * kStepWarps];
   unsigned long long best[2][kStepWarps];
-  int sums[2][kStepWarps];
+  int2 sums[kStepWarps];
   int2 pick[kStepWarps + 1];
   int sel_sid[12], sel_off[12];     // [kSelectRounds]
   uint32_t done[kStepItems / 32];   // victims that need no out task of their own
@@ -2091,20 +2091,12 @@ __device__ __forceinline__ unsigned long long warp_max(unsigned long long x) {
   return (unsigned long long)hi << 32 | lo;
 }
 
-// The largest of every thread's v and the sum of every thread's n, to all of them (one
-// barrier; two buffers as BlockScan).
-__device__ __forceinline__ unsigned long long block_max(unsigned long long v, int n, int* sum, StepShared& sh,
-                                                        int ph) {
-  const int lane = threadIdx.x & 31;
+// The largest of every thread's v, to all of them (one barrier; two buffers as BlockScan).
+__device__ __forceinline__ unsigned long long block_max(unsigned long long v, StepShared& sh, int ph) {
   v = warp_max(v);
-  n = __reduce_add_sync(0xffffffffu, n);
-  if (lane == 0) {
-    sh.best[ph][threadIdx.x >> 5] = v;
-    sh.sums[ph][threadIdx.x >> 5] = n;
-  }
+  if ((threadIdx.x & 31) == 0) sh.best[ph][threadIdx.x >> 5] = v;
   __syncthreads();
-  *sum = __reduce_add_sync(0xffffffffu, lane < kStepWarps ? sh.sums[ph][lane] : 0);
-  return warp_max(lane < kStepWarps ? sh.best[ph][lane] : 0ull);
+  return warp_max((threadIdx.x & 31) < kStepWarps ? sh.best[ph][threadIdx.x & 31] : 0ull);
 }
 
 __device__ __forceinline__ int32_t session_of_key(unsigned long long key) {
@@ -2241,9 +2233,8 @@ __device__ unsigned long long threshold_key(const DevPool& p, const unsigned lon
       if (in && x > high) high = x;
       if (in && ~x > low) low = ~x;
     }
-    int unused;
-    high = block_max(high, 0, &unused, sh, 0);
-    low = ~block_max(low, 0, &unused, sh, 1);
+    high = block_max(high, sh, 0);
+    low = ~block_max(low, sh, 1);
     if (low == high) return low;
     const int bits = 64 - __clzll((long long)(high - low));
     const int shift = bits > 9 ? bits - 9 : 0;
@@ -2277,33 +2268,36 @@ __device__ unsigned long long threshold_key(const DevPool& p, const unsigned lon
 // the first k victims.  Where few sessions should hold k blocks they are found by repeated
 // maximum, one barrier each; else, or when kSelectRounds were not enough, by the threshold
 // key, and the sessions' places by comparing them with one another, or by a sort of more
-// than kCompared.  (4096 sessions, 1500 victims of 7 or 8 sessions: 9.1 us by maximum, 12.6
-// by the threshold; 256 victims of 128 sessions: 48 us by maximum and a sort of all keys,
-// 13.1 by the threshold.)  Keys are distinct (each holds its session).  A thread may call it with
+// than kCompared.  (4096 sessions, 1500 victims of 7 or 8 sessions: 7.5 us by maximum -- 9.3
+// when every round read all keys again instead of a thread's two largest -- and 12.6 by the
+// threshold; 256 victims of 128 sessions: 48 us by maximum and a sort of all keys, 13.1 by
+// the threshold.)  Keys are distinct (each holds its session).  A thread may call it with
 // only its own sessions' keys and counts (s = thread, thread + kStepThreads, ...) written.
 constexpr int kCompared = 256;
 __device__ Selected select_sessions(const DevPool& p, unsigned long long* keys, int* off, const int* cnt,
                                     long long k, int32_t running, StepShared& sh, BlockScan& scan) {
   Selected r{};
   int mine = 0, cand = 0;
-  unsigned long long v = 0;
+  // a thread's two largest keys: when one of them is taken the other is at hand
+  unsigned long long v = 0, v2 = 0;
 #pragma unroll 1
   for (int s = threadIdx.x; s < p.S; s += kStepThreads) {
     if (s == running) keys[s] = 0ull;
     const unsigned long long x = keys[s];
-    if (x) {
-      mine += cnt[s];
-      ++cand;
-    }
-    if (x > v) v = x;
+    mine += x ? cnt[s] : 0;
+    cand += x ? 1 : 0;
+    v2 = x > v ? v : x > v2 ? x : v2;
+    v = x > v ? x : v;
   }
-  int total;
-  unsigned long long last = block_max(v, mine, &total, sh, 0);
+  mine = __reduce_add_sync(0xffffffffu, mine);
+  cand = __reduce_add_sync(0xffffffffu, cand);
+  if ((threadIdx.x & 31) == 0) sh.sums[threadIdx.x >> 5] = make_int2(mine, cand);
+  unsigned long long last = block_max(v, sh, 0);
+  const int2 part = (threadIdx.x & 31) < kStepWarps ? sh.sums[threadIdx.x & 31] : make_int2(0, 0);
+  const int total = __reduce_add_sync(0xffffffffu, part.x), cands = __reduce_add_sync(0xffffffffu, part.y);
   r.total = total;
   r.n_out = k < total ? k : total;
   long long at = 0;
-  int cands;
-  scan.sum(cand, &cands);
   const bool few = r.n_out * cands <= 8ll * total;      // eight sessions of average size
   if (LV_MOSTLY(few)) {
 #pragma unroll 1
@@ -2316,14 +2310,19 @@ __device__ Selected select_sessions(const DevPool& p, unsigned long long* keys, 
       at += cnt[s];
       ++r.m;
       if (at >= r.n_out || r.m == kSelectRounds) break;
-      v = 0;
+      if (v == last) {
+        v = v2;
+        v2 = ~0ull;                               // not known
+        if (LV_RARE(v == ~0ull)) {
+          v = 0;
 #pragma unroll 1
-      for (int s2 = threadIdx.x; s2 < p.S; s2 += kStepThreads) {
-        const unsigned long long x = keys[s2];
-        if (x < last && x > v) v = x;
+          for (int s2 = threadIdx.x; s2 < p.S; s2 += kStepThreads) {
+            const unsigned long long x = keys[s2];
+            if (x < last && x > v) v = x;
+          }
+        }
       }
-      int unused;
-      last = block_max(v, 0, &unused, sh, r.m & 1);
+      last = block_max(v, sh, r.m & 1);
     }
   }
   if (LV_RARE(at < r.n_out)) {
@@ -2752,7 +2751,7 @@ k_step(DevPool p, StepArgs a) {
 // the sessions chosen, where the census reads every row.  kCensus: no counts are kept for
 // these tables (lv_select_victims_noalloc); one CTA takes keys and counts from the census.
 // 256 victims of 1024 sessions with 1024 blocks each: 7.1 us as census and emission, 3.9 as
-// one kernel; 1500 of 4096 sessions with 256 blocks: 20.7 and 9.1 us.
+// one kernel; 1500 of 4096 sessions with 256 blocks: 20.7 and 7.5 us.
 // More victims, or victims of some hundred sessions, are written by many CTAs: 4096 victims
 // of 1024 sessions take 11.8 us here and 9.2 there, 2048 of at least 1024 sessions with two
 // blocks each 32 and 9.2, 256 of 128 such sessions 10.1 and 9.2 (13.1 and 14.9 with 4096
