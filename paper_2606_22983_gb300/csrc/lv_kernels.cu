@@ -2749,7 +2749,7 @@ k_step(DevPool p, StepArgs a) {
 // sessions are made by each CTA of a cluster and written into the first CTA's shared memory,
 // which then selects and lists the victims; it reads one count per session and the rows of
 // the sessions chosen, where the census reads every row.  kCensus: no counts are kept for
-// these tables (lv_select_victims_noalloc); one CTA takes keys and counts from the census.
+// these tables (lv_select_victims_noalloc, many sessions); one CTA takes both from the census.
 // 256 victims of 1024 sessions with 1024 blocks each: 7.1 us as census and emission, 3.9 as
 // one kernel; 1500 of 4096 sessions with 256 blocks: 20.7 and 7.5 us.
 // More victims, or victims of some hundred sessions, are written by many CTAs: 4096 victims
@@ -3018,12 +3018,15 @@ cudaError_t launch_events(const DevPool& p, const lv_event* ev, int64_t n, cudaS
   return launch_pdl(k_events, blocks_for(p.S, kEventThreads, 1 << 20), kEventThreads, 0, s, p, ev, (long long)n);
 }
 
-// One kernel up to kSelectMost victims (after a census where no counts are kept); more are
-// written by a CTA per session.
+// One kernel up to kSelectMost victims; more are written by a CTA per session.  Where no
+// counts are kept the census comes first, and up to kEmitScanMax sessions the CTAs that then
+// write place their own session: 1890 victims of 25 sessions 8.4 us so, 10.0 by one CTA after
+// the census, 256 of 1024 sessions 11.6 and 12.6; above, a third kernel would place them: 256
+// of 2048 sessions 13.8 us so and 12.6 by one CTA, of 4096 18.2 and 12.9.
 cudaError_t launch_select(const DevPool& p, int64_t now_us, int64_t k, bool fallback,
                           lv_victim* out, long long* count_dev, cudaStream_t s) {
   const size_t smem = select_layout(p.S).total;
-  const bool one = k <= kSelectMost && k <= (long long)kSelectSessions * p.maxB;
+  const bool one = k <= kSelectMost && k <= (long long)kSelectSessions * p.maxB && (p.cnt || p.S > kEmitScanMax);
   if (one && p.cnt) {
     unsigned ctas = 1;
     while ((int)ctas * kStepThreads < p.S) ctas *= 2;
