@@ -76,7 +76,8 @@ struct lv_pool {
   uint32_t st_seq = 0;
   // staged path: side streams for the copy engines, a host copy of the tasks, sync events
   cudaStream_t s_d2h = nullptr, s_h2d = nullptr;
-  int4* tasks_host = nullptr;
+  int4* tasks_host = nullptr;      // written by the kernels in place (tasks_dev: their address of it)
+  void* tasks_dev = nullptr;
   size_t tasks_host_cap = 0;
   std::vector<cudaEvent_t> sync_events;
   int stage_ctas = 0;
@@ -282,21 +283,43 @@ cudaError_t prune_marks(cudaEvent_t ev, MarkSet& m) {
   return cudaSuccess;
 }
 
+// Where the kernels leave the number of tasks, behind the task buffer's three parts.
+long long* task_count(lv_pool* pool) {
+  return reinterpret_cast<long long*>(pool->tasks_host + 3 * pool->tasks_host_cap);
+}
+
+// The GPU's address of a place in the task buffer.
+template <typename T>
+T* task_view(lv_pool* pool, T* place) {
+  return reinterpret_cast<T*>(reinterpret_cast<char*>(place) - reinterpret_cast<char*>(pool->tasks_host) +
+                              static_cast<char*>(pool->tasks_dev));
+}
+
 // The staged data movement of n validated tasks {out page, out slot, in slot, in page}
-// on `s`.  The task list is read back once; its out halves are sorted by host slot and
+// on `s`, which the kernels queued there have written into the pool's page-locked task buffer
+// (counted: n at most, and their number behind them).  Its out halves are sorted by host slot and
 // so are its in halves, so that consecutive slots become one copy-engine transfer
 // whatever order the blocks were listed in (a session evicted suffix first sits in
 // descending slots).  Then: pack the out pages into staging in slot order; copy-engine
 // runs in each direction on the side streams; unpack into the in pages; joined back
 // into `s`.  Every pack precedes every unpack on `s`, so a page that an incoming block
 // takes is read before it is overwritten.
-lv_status staged_move_inner(lv_pool* pool, const int4* tasks_dev, int64_t n, cudaStream_t s,
-                            void** staging_out, bool async) {
+//
+// What bounds it: the copy engines, about 1.9 us per transfer beside the bytes, and for small
+// moves the one wait for the task list.  The two directions' transfers are issued in turn, and
+// the packs, in chunks of 24 MiB, before them, so that both run from the start (66 runs of 1 to
+// 6 pages of 1.5 MiB each way by themselves: 1616 us issued in turn, 1813 with one direction
+// first; more streams per direction 1676 to 1841).  An exchange with its ranking: 5 pages of
+// 16 KiB 68.5 us with the task list copied back in two waits and 47 now, 37 of 192 KiB 151 and
+// 128, 25 of 1.5 MiB 358 and 332, 150 of 1.5 MiB 1890 and 1850.
+lv_status staged_move_inner(lv_pool* pool, int64_t n, bool counted, cudaStream_t s, void** staging_out,
+                            bool async) {
   const lv::DevPool& d = pool->d;
   if (n <= 0) return LV_OK;
   if ((size_t)n > pool->tasks_host_cap) return LV_ERR_INVALID;
-  LV_TRY(cudaMemcpyAsync(pool->tasks_host, tasks_dev, (size_t)n * sizeof(int4), cudaMemcpyDeviceToHost, s));
   LV_TRY(cudaStreamSynchronize(s));
+  if (counted) n = *task_count(pool) < n ? *task_count(pool) : n;
+  if (n <= 0) return LV_OK;
   // split and sort, in the second and third thirds of the page-locked task buffer
   const int4* t = pool->tasks_host;
   int4* tout = pool->tasks_host + n;
@@ -310,7 +333,7 @@ lv_status staged_move_inner(lv_pool* pool, const int4* tasks_dev, int64_t n, cud
   std::stable_sort(tin, tin + n_in, [](const int4& u, const int4& v) { return u.z < v.z; });
   if (n_out + n_in == 0) return LV_OK;      // every task was refused (errors already set)
   const size_t pb = (size_t)d.J * d.P;
-  const int64_t chunk = std::max<int64_t>(1, (int64_t)((96u << 20) / pb));
+  const int64_t chunk = std::max<int64_t>(1, (int64_t)((24u << 20) / pb));
   const int64_t nchunks = (std::max(n_out, n_in) + chunk - 1) / chunk;
   lv_status st = sync_events(pool, (size_t)(2 * nchunks + 3));
   if (st != LV_OK) return st;
@@ -376,33 +399,38 @@ lv_status staged_move_inner(lv_pool* pool, const int4* tasks_dev, int64_t n, cud
     }
     for (int64_t i = 0; i < n_out; ++i) pool->st_written.add(tout[i].y);
   }
-  // H2D first so that the inbound copies start at once: runs of consecutive slots
-  for (int64_t c = 0; c * chunk < n_in; ++c) {
-    const int64_t a = c * chunk, b = std::min(n_in, a + chunk);
-    for (int64_t i = a; i < b;) {
+  // pack every chunk on s
+  for (int64_t c = 0; c * chunk < n_out; ++c) {
+    LV_TRY(lv::launch_stage(d, true, false, tout_dev, c * chunk, std::min(n_out, (c + 1) * chunk), stg_out, s,
+                            pool->stage_ctas, timing_pair(pool, LV_TIMING_PACK), pool->stage_tma));
+    LV_TRY(cudaEventRecord(ev_pack[c], s));
+  }
+  // the transfers, one run of consecutive slots of each direction in turn: a D2H run follows
+  // the pack of its last page, and the H2D run that completes a chunk is followed by its event
+  int64_t arrived = 0, packed = 0;            // chunks whose event is recorded / waited for
+  for (int64_t i = 0, o = 0; i < n_in || o < n_out;) {
+    if (i < n_in) {
       int64_t j = i + 1;
-      while (j < b && tin[j].z == tin[j - 1].z + 1) ++j;
+      while (j < n_in && tin[j].z == tin[j - 1].z + 1) ++j;
       if (fault_fires(pool, LV_FAULT_COPY)) return LV_ERR_CUDA;
       LV_TRY(cudaMemcpyAsync(stg_in + (size_t)i * pb, host + (size_t)tin[i].z * pb, (size_t)(j - i) * pb,
                              cudaMemcpyHostToDevice, pool->s_h2d));
+      for (; arrived * chunk < n_in && std::min(n_in, (arrived + 1) * chunk) <= j; ++arrived)
+        LV_TRY(cudaEventRecord(ev_h2d[arrived], pool->s_h2d));
       i = j;
     }
-    LV_TRY(cudaEventRecord(ev_h2d[c], pool->s_h2d));
-  }
-  // pack every chunk on s; the D2H runs of chunk c follow its pack
-  for (int64_t c = 0; c * chunk < n_out; ++c) {
-    const int64_t a = c * chunk, b = std::min(n_out, a + chunk);
-    LV_TRY(lv::launch_stage(d, true, false, tout_dev, a, b, stg_out, s, pool->stage_ctas,
-                            timing_pair(pool, LV_TIMING_PACK), pool->stage_tma));
-    LV_TRY(cudaEventRecord(ev_pack[c], s));
-    LV_TRY(cudaStreamWaitEvent(pool->s_d2h, ev_pack[c], 0));
-    for (int64_t i = a; i < b;) {
-      int64_t j = i + 1;
-      while (j < b && tout[j].y == tout[j - 1].y + 1) ++j;
+    if (o < n_out) {
+      int64_t j = o + 1;
+      while (j < n_out && tout[j].y == tout[j - 1].y + 1) ++j;
       if (fault_fires(pool, LV_FAULT_COPY)) return LV_ERR_CUDA;
-      LV_TRY(cudaMemcpyAsync(host + (size_t)tout[i].y * pb, stg_out + (size_t)i * pb, (size_t)(j - i) * pb,
+      const int64_t c = (j - 1) / chunk;
+      if (c >= packed) {
+        LV_TRY(cudaStreamWaitEvent(pool->s_d2h, ev_pack[c], 0));
+        packed = c + 1;
+      }
+      LV_TRY(cudaMemcpyAsync(host + (size_t)tout[o].y * pb, stg_out + (size_t)o * pb, (size_t)(j - o) * pb,
                              cudaMemcpyDeviceToHost, pool->s_d2h));
-      i = j;
+      o = j;
     }
   }
   // unpack each chunk once it has arrived, after every pack (on s, or on s_unpack
@@ -424,10 +452,9 @@ lv_status staged_move_inner(lv_pool* pool, const int4* tasks_dev, int64_t n, cud
 
 // staged_move_inner, then (also after an early error) join the side streams back
 // into `s` and mark the staging run free in stream order.
-lv_status staged_move(lv_pool* pool, const int4* tasks_dev, int64_t n, cudaStream_t s,
-                      bool async = false) {
+lv_status staged_move(lv_pool* pool, int64_t n, cudaStream_t s, bool async = false, bool counted = false) {
   void* slot = nullptr;   // &pool->st_buf[b] once the call has taken run b
-  const lv_status st = staged_move_inner(pool, tasks_dev, n, s, &slot, async);
+  const lv_status st = staged_move_inner(pool, n, counted, s, &slot, async);
   if (!slot) return st;
   const int b = static_cast<void**>(slot) == &pool->st_buf[0] ? 0 : 1;
   if (async && st == LV_OK) {
@@ -722,12 +749,14 @@ lv_status create_impl(const lv_pool_desc* desc, cudaStream_t s, lv_pool** out) {
   pool->st_loaded.resize(d.hbm_pages);
   pool->st_written.resize(d.host_pages);
   pool->st_read.resize(d.host_pages);
-  // the task list read back, then its sorted out and in halves
-  if (cudaHostAlloc((void**)&pool->tasks_host, 3 * pool->tasks_host_cap * sizeof(int4), cudaHostAllocDefault) !=
+  // the task list read back, then its sorted out and in halves, then the number of tasks
+  if (cudaHostAlloc((void**)&pool->tasks_host, (3 * pool->tasks_host_cap + 1) * sizeof(int4),
+                    cudaHostAllocMapped) !=
       cudaSuccess) {
     pool->tasks_host = nullptr;
     return fail(LV_ERR_OOM);
   }
+  if (cudaHostGetDevicePointer(&pool->tasks_dev, pool->tasks_host, 0) != cudaSuccess) return fail(LV_ERR_CUDA);
   pool->stage_ctas = 2 * pool->num_sms;   // two TMA pack/unpack CTAs per SM (see stage_count)
   if (const char* env = std::getenv("LV_STAGE_CTAS_PER_SM")) {
     const int per = std::atoi(env);
@@ -987,11 +1016,9 @@ lv_status lv_swap_out(lv_pool* pool, const lv_victim* victims, int64_t n, int32_
     const bool fail_alloc = fault_fires(pool, LV_FAULT_HOST_ALLOC);
     LV_TRY(lv::launch_alloc(pool->d, false, static_cast<const lv_victim*>(vin), n, slots, s, fail_alloc));
     if (mode == LV_MODE_STAGED) {
-      void* tdev = nullptr;
-      if ((r = st.out(nullptr, (size_t)n * sizeof(int4), &tdev, true)) != LV_OK) return r;
       LV_TRY(lv::launch_tasks_out(pool->d, static_cast<const lv_victim*>(vin), slots, n,
-                                  static_cast<int4*>(tdev), static_cast<lv_remap_entry*>(cdev), s));
-      if ((r = staged_move(pool, static_cast<int4*>(tdev), n, s)) != LV_OK) return r;
+                                  task_view(pool, pool->tasks_host), static_cast<lv_remap_entry*>(cdev), s));
+      if ((r = staged_move(pool, n, s)) != LV_OK) return r;
       return st.finish();
     }
     LV_TRY(lv::launch_swap_out(pool->d, static_cast<const lv_victim*>(vin), slots, n,
@@ -1025,11 +1052,9 @@ lv_status lv_swap_in(lv_pool* pool, int32_t sid, const int32_t* blks, int64_t n,
     int32_t* pages = static_cast<int32_t*>(pdev);
     LV_TRY(lv::launch_alloc(pool->d, true, nullptr, n, pages, s, fault_fires(pool, LV_FAULT_HBM_ALLOC)));
     if (mode == LV_MODE_STAGED) {
-      void* tdev = nullptr;
-      if ((r = st.out(nullptr, (size_t)n * sizeof(int4), &tdev, true)) != LV_OK) return r;
       LV_TRY(lv::launch_tasks_in(pool->d, sid, static_cast<const int32_t*>(bin), pages, n,
-                                 static_cast<int4*>(tdev), static_cast<lv_remap_entry*>(cdev), s));
-      if ((r = staged_move(pool, static_cast<int4*>(tdev), n, s)) != LV_OK) return r;
+                                 task_view(pool, pool->tasks_host), static_cast<lv_remap_entry*>(cdev), s));
+      if ((r = staged_move(pool, n, s)) != LV_OK) return r;
       return st.finish();
     }
     LV_TRY(lv::launch_swap_in(pool->d, sid, static_cast<const int32_t*>(bin), pages, n,
@@ -1070,21 +1095,18 @@ lv_status lv_swap_exchange(lv_pool* pool, const lv_victim* victims, int64_t n_ou
     if ((r = st.in(blks, (size_t)n_in * 4, &bin)) != LV_OK) return r;
     if ((r = st.out(slots_out, (size_t)n_out * 4, &sdev, true)) != LV_OK) return r;
     if ((r = st.out(pages_out, (size_t)n_in * 4, &pdev, true)) != LV_OK) return r;
-    if ((r = st.out(nullptr, (size_t)(n_out + n_in) * sizeof(int4), &tdev, true)) != LV_OK) return r;
-    // the task count, and the copy kernel's cursor
-    if ((r = st.out(nullptr, 2 * sizeof(long long), &ndev, true)) != LV_OK) return r;
     if (++pool->epoch <= 0) pool->epoch = 1;
     if (mode == LV_MODE_STAGED) {
       LV_TRY(lv::launch_exchange_plan(pool->d, static_cast<const lv_victim*>(vin), n_out, sid,
                                       static_cast<const int32_t*>(bin), n_in, static_cast<int32_t*>(sdev),
-                                      static_cast<int32_t*>(pdev), static_cast<int4*>(tdev),
-                                      static_cast<long long*>(ndev), pool->epoch, pool->d.page_tag, s));
-      long long nt = 0;
-      LV_TRY(cudaMemcpyAsync(&nt, ndev, sizeof(nt), cudaMemcpyDeviceToHost, s));
-      LV_TRY(cudaStreamSynchronize(s));
-      if ((r = staged_move(pool, static_cast<int4*>(tdev), nt, s, async)) != LV_OK) return r;
+                                      static_cast<int32_t*>(pdev), task_view(pool, pool->tasks_host),
+                                      task_view(pool, task_count(pool)), pool->epoch, pool->d.page_tag, s));
+      if ((r = staged_move(pool, n_out + n_in, s, async, true)) != LV_OK) return r;
       return st.finish();
     }
+    // the tasks, their number, and the copy kernel's cursor
+    if ((r = st.out(nullptr, (size_t)(n_out + n_in) * sizeof(int4), &tdev, true)) != LV_OK) return r;
+    if ((r = st.out(nullptr, 2 * sizeof(long long), &ndev, true)) != LV_OK) return r;
     LV_TRY(lv::launch_exchange(pool->d, static_cast<const lv_victim*>(vin), n_out, sid,
                                static_cast<const int32_t*>(bin), n_in, static_cast<int32_t*>(sdev),
                                static_cast<int32_t*>(pdev), static_cast<int4*>(tdev),
