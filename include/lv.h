@@ -224,8 +224,10 @@ typedef struct lv_stats {
    the SMs) or LV_EXCHANGE_CTAS_PER_SM; LV_STAGE_STAGES and LV_STAGE_CTAS_PER_SM
    (the TMA pack/unpack kernel, default about 48 KiB of stages per CTA and two
    CTAs per SM); LV_STAGE_KERNEL=lsu (16-byte copies instead of TMA);
-   LV_REMAP_ENTRIES_PER_THREAD = 1, 2 or 4 (lv_remap's entries per thread,
-   default 1 while the GPU holds one thread per entry at once, else 2 or 4);
+   LV_REMAP_ENTRIES_PER_THREAD = 1, 2 or 4 (lv_remap's entries per thread, with
+   a release pass; by default up to 2^18 entries take a thread each and need no
+   such pass, more take 1 while the GPU holds one thread per entry at once, else
+   2 or 4);
    LV_EXCHANGE_KERNEL=tma (the exchange copy by TMA bulk copies, one issuing
    thread per CTA, with LV_EXCHANGE_STAGES stages of 2P bytes, default 4). */
 lv_status lv_pool_create(const lv_pool_desc* desc, lv_stream stream, lv_pool** out);

@@ -749,7 +749,7 @@ lv_status create_impl(const lv_pool_desc* desc, cudaStream_t s, lv_pool** out) {
   pool->st_loaded.resize(d.hbm_pages);
   pool->st_written.resize(d.host_pages);
   pool->st_read.resize(d.host_pages);
-  // the task list read back, then its sorted out and in halves, then the number of tasks
+  // the task list the kernels write, then its sorted out and in halves, then the number of tasks
   if (cudaHostAlloc((void**)&pool->tasks_host, (3 * pool->tasks_host_cap + 1) * sizeof(int4),
                     cudaHostAllocMapped) !=
       cudaSuccess) {

@@ -1,11 +1,11 @@
 // CUDA kernels of the KV swap path (sm_103a).
 //
 //   ranking   k_select; k_rank_census -> k_rank_emit          (Section 5.1, Eq. 4)
-//   allocate  k_alloc, k_alloc_out                           (lowest free, Section 5.1)
+//   allocate  k_alloc                                        (lowest free, Section 5.1)
 //   move      k_swap_out / k_swap_in                         (Section 5, Fig. 6; Section 5.2)
 //             k_exchange_plan -> k_exchange_copy             (both directions in one step)
 //             k_stage_tasks (TMA) / k_stage_tasks_lsu         (staged copy-engine path)
-//   commit    k_remap, k_cancel, k_append                    (Section 6 side tables)
+//   commit    k_remap (-> k_release), k_cancel, k_append     (Section 6 side tables)
 //   monitor   k_events                                       (Section 3, Sections 5.1-5.2)
 //   step      k_step -> k_exchange_copy                      (a whole turn, preload or eviction
 //                                                             decided on the device)
