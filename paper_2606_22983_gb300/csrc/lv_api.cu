@@ -399,15 +399,21 @@ lv_status staged_move_inner(lv_pool* pool, int64_t n, bool counted, cudaStream_t
     }
     for (int64_t i = 0; i < n_out; ++i) pool->st_written.add(tout[i].y);
   }
-  // pack every chunk on s
-  for (int64_t c = 0; c * chunk < n_out; ++c) {
-    LV_TRY(lv::launch_stage(d, true, false, tout_dev, c * chunk, std::min(n_out, (c + 1) * chunk), stg_out, s,
-                            pool->stage_ctas, timing_pair(pool, LV_TIMING_PACK), pool->stage_tma));
-    LV_TRY(cudaEventRecord(ev_pack[c], s));
-  }
-  // the transfers, one run of consecutive slots of each direction in turn: a D2H run follows
-  // the pack of its last page, and the H2D run that completes a chunk is followed by its event
-  int64_t arrived = 0, packed = 0;            // chunks whose event is recorded / waited for
+  // the transfers, one run of consecutive slots of each direction in turn: an H2D run that
+  // completes a chunk is followed by its event; a D2H run follows the pack of its last page.
+  // The first chunk's pack is issued ahead of the transfers, the others' (on s too) with the
+  // first run that needs them.
+  int64_t arrived = 0, packed = 0, ordered = 0;   // chunks recorded / packed / waited for by s_d2h
+  auto pack = [&](int64_t end) -> cudaError_t {   // the pages before `end`
+    for (; packed * chunk < end; ++packed) {
+      cudaError_t e = lv::launch_stage(d, true, false, tout_dev, packed * chunk, std::min(n_out, (packed + 1) * chunk),
+                                       stg_out, s, pool->stage_ctas, timing_pair(pool, LV_TIMING_PACK), pool->stage_tma);
+      if (e == cudaSuccess) e = cudaEventRecord(ev_pack[packed], s);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  };
+  LV_TRY(pack(std::min(n_out, chunk)));
   for (int64_t i = 0, o = 0; i < n_in || o < n_out;) {
     if (i < n_in) {
       int64_t j = i + 1;
@@ -422,12 +428,12 @@ lv_status staged_move_inner(lv_pool* pool, int64_t n, bool counted, cudaStream_t
     if (o < n_out) {
       int64_t j = o + 1;
       while (j < n_out && tout[j].y == tout[j - 1].y + 1) ++j;
-      if (fault_fires(pool, LV_FAULT_COPY)) return LV_ERR_CUDA;
-      const int64_t c = (j - 1) / chunk;
-      if (c >= packed) {
-        LV_TRY(cudaStreamWaitEvent(pool->s_d2h, ev_pack[c], 0));
-        packed = c + 1;
+      LV_TRY(pack(j));
+      if (ordered < packed) {
+        LV_TRY(cudaStreamWaitEvent(pool->s_d2h, ev_pack[packed - 1], 0));
+        ordered = packed;
       }
+      if (fault_fires(pool, LV_FAULT_COPY)) return LV_ERR_CUDA;
       LV_TRY(cudaMemcpyAsync(host + (size_t)tout[o].y * pb, stg_out + (size_t)o * pb, (size_t)(j - o) * pb,
                              cudaMemcpyDeviceToHost, pool->s_d2h));
       o = j;
