@@ -341,8 +341,8 @@ lv_status lv_swap_in(lv_pool* pool, int32_t sid, const int32_t* blks, int64_t n,
    thread right after it read the old bytes), so the host link carries data
    both ways at once.  LV_MODE_STAGED instead packs the evicted pages into HBM
    staging and unpacks the loaded ones, with the copy engines carrying one
-   transfer per contiguous slot run in each direction on two side streams (it
-   waits on the host for the plan).  Either list may be empty.  The whole call is validated
+   transfer per contiguous slot run (long runs in pieces) in each direction on
+   two side streams (it waits on the host for the plan).  Either list may be empty.  The whole call is validated
    before anything changes: on LV_ERR_STATE / LV_ERR_BOUNDS (a victim not
    resident where it says, a block not in the host tier, a block listed twice),
    LV_ERR_NO_HOST or LV_ERR_NO_HBM (device-detected) nothing is reserved,

@@ -80,6 +80,8 @@ struct lv_pool {
   void* tasks_dev = nullptr;
   size_t tasks_host_cap = 0;
   std::vector<cudaEvent_t> sync_events;
+  std::vector<std::pair<int64_t, int64_t>> st_runs;   // kept from call to call for its storage,
+  std::vector<int4> st_order;                         // as is this
   int stage_ctas = 0;
   bool stage_tma = true;           // pack/unpack with TMA bulk copies (else 16-byte LSU copies)
   int32_t fault_kind = LV_FAULT_NONE;   // lv_inject_fault: one-shot, after `fault_after` more events
@@ -295,23 +297,45 @@ T* task_view(lv_pool* pool, T* place) {
                               static_cast<char*>(pool->tasks_dev));
 }
 
+// m tasks in the order of their slots, by runs of consecutive slots, the longest run first.
+void longest_runs_first(lv_pool* pool, int4* t, int64_t m, int int4::*slot) {
+  std::vector<std::pair<int64_t, int64_t>>& runs = pool->st_runs;     // minus its length, first task
+  runs.clear();
+  for (int64_t i = 0, j; i < m; i = j) {
+    for (j = i + 1; j < m && t[j].*slot == t[j - 1].*slot + 1;) ++j;
+    runs.emplace_back(i - j, i);
+  }
+  if (runs.size() < 2) return;
+  std::sort(runs.begin(), runs.end());
+  pool->st_order.assign(t, t + m);
+  for (const auto& r : runs) {
+    const int4* from = pool->st_order.data() + r.second;
+    t = std::copy(from, from - r.first, t);
+  }
+}
+
 // The staged data movement of n validated tasks {out page, out slot, in slot, in page}
 // on `s`, which the kernels queued there have written into the pool's page-locked task buffer
 // (counted: n at most, and their number behind them).  Its out halves are sorted by host slot and
 // so are its in halves, so that consecutive slots become one copy-engine transfer
 // whatever order the blocks were listed in (a session evicted suffix first sits in
-// descending slots).  Then: pack the out pages into staging in slot order; copy-engine
+// descending slots), and the longest runs come first.  Then: pack the out pages into staging in slot order; copy-engine
 // runs in each direction on the side streams; unpack into the in pages; joined back
 // into `s`.  Every pack precedes every unpack on `s`, so a page that an incoming block
 // takes is read before it is overwritten.
 //
 // What bounds it: the copy engines, about 1.9 us per transfer beside the bytes, and for small
 // moves the one wait for the task list.  The two directions' transfers are issued in turn, and
-// the packs, in chunks of 24 MiB, before them, so that both run from the start (66 runs of 1 to
+// the packs, in chunks of 24 MiB, with the runs that need them, so that both run from the start (66 runs of 1 to
 // 6 pages of 1.5 MiB each way by themselves: 1616 us issued in turn, 1813 with one direction
-// first; more streams per direction 1676 to 1841).  An exchange with its ranking: 5 pages of
-// 16 KiB 68.5 us with the task list copied back in two waits and 47 now, 37 of 192 KiB 151 and
-// 128, 25 of 1.5 MiB 358 and 332, 150 of 1.5 MiB 1890 and 1850.
+// first; more streams per direction 1676 to 1841).  A transfer that ends while the other
+// direction's is under way is followed by a gap of up to 9 us, and a long run at the end keeps
+// its direction busy alone with its unpacks behind it; so long runs go first, in pieces of a
+// chunk (150 pages of 1.5 MiB: 1826 us in slot order, 1776 so; 50 by swap-out and swap-in: 965
+// and 947), but runs are not cut to let both directions end together (1880).  An exchange with
+// its ranking, with the task list copied back in two waits and one direction issued first, and
+// now: 5 pages of 16 KiB 68.5 us and 47, 37 of 192 KiB 151 and 126, 25 of 1.5 MiB 358 and 324,
+// 150 of 1.5 MiB 1890 and 1776.
 lv_status staged_move_inner(lv_pool* pool, int64_t n, bool counted, cudaStream_t s, void** staging_out,
                             bool async) {
   const lv::DevPool& d = pool->d;
@@ -332,6 +356,8 @@ lv_status staged_move_inner(lv_pool* pool, int64_t n, bool counted, cudaStream_t
   std::stable_sort(tout, tout + n_out, [](const int4& u, const int4& v) { return u.y < v.y; });
   std::stable_sort(tin, tin + n_in, [](const int4& u, const int4& v) { return u.z < v.z; });
   if (n_out + n_in == 0) return LV_OK;      // every task was refused (errors already set)
+  longest_runs_first(pool, tout, n_out, &int4::y);
+  longest_runs_first(pool, tin, n_in, &int4::z);
   const size_t pb = (size_t)d.J * d.P;
   const int64_t chunk = std::max<int64_t>(1, (int64_t)((24u << 20) / pb));
   const int64_t nchunks = (std::max(n_out, n_in) + chunk - 1) / chunk;
@@ -399,8 +425,9 @@ lv_status staged_move_inner(lv_pool* pool, int64_t n, bool counted, cudaStream_t
     }
     for (int64_t i = 0; i < n_out; ++i) pool->st_written.add(tout[i].y);
   }
-  // the transfers, one run of consecutive slots of each direction in turn: an H2D run that
-  // completes a chunk is followed by its event; a D2H run follows the pack of its last page.
+  // the transfers, one run of consecutive slots (or a chunk's length of it) of each direction in
+  // turn: an H2D run that completes a chunk is followed by its event; a D2H run follows the pack
+  // of its last page.
   // The first chunk's pack is issued ahead of the transfers, the others' (on s too) with the
   // first run that needs them.
   int64_t arrived = 0, packed = 0, ordered = 0;   // chunks recorded / packed / waited for by s_d2h
@@ -415,28 +442,27 @@ lv_status staged_move_inner(lv_pool* pool, int64_t n, bool counted, cudaStream_t
   };
   LV_TRY(pack(std::min(n_out, chunk)));
   for (int64_t i = 0, o = 0; i < n_in || o < n_out;) {
-    if (i < n_in) {
-      int64_t j = i + 1;
-      while (j < n_in && tin[j].z == tin[j - 1].z + 1) ++j;
+    int64_t ni = i < n_in, no = o < n_out;      // pages of the next run each way
+    while (ni && ni < chunk && i + ni < n_in && tin[i + ni].z == tin[i + ni - 1].z + 1) ++ni;
+    while (no && no < chunk && o + no < n_out && tout[o + no].y == tout[o + no - 1].y + 1) ++no;
+    if (ni) {
       if (fault_fires(pool, LV_FAULT_COPY)) return LV_ERR_CUDA;
-      LV_TRY(cudaMemcpyAsync(stg_in + (size_t)i * pb, host + (size_t)tin[i].z * pb, (size_t)(j - i) * pb,
+      LV_TRY(cudaMemcpyAsync(stg_in + (size_t)i * pb, host + (size_t)tin[i].z * pb, (size_t)ni * pb,
                              cudaMemcpyHostToDevice, pool->s_h2d));
-      for (; arrived * chunk < n_in && std::min(n_in, (arrived + 1) * chunk) <= j; ++arrived)
+      i += ni;
+      for (; arrived * chunk < n_in && std::min(n_in, (arrived + 1) * chunk) <= i; ++arrived)
         LV_TRY(cudaEventRecord(ev_h2d[arrived], pool->s_h2d));
-      i = j;
     }
-    if (o < n_out) {
-      int64_t j = o + 1;
-      while (j < n_out && tout[j].y == tout[j - 1].y + 1) ++j;
-      LV_TRY(pack(j));
+    if (no) {
+      LV_TRY(pack(o + no));
       if (ordered < packed) {
         LV_TRY(cudaStreamWaitEvent(pool->s_d2h, ev_pack[packed - 1], 0));
         ordered = packed;
       }
       if (fault_fires(pool, LV_FAULT_COPY)) return LV_ERR_CUDA;
-      LV_TRY(cudaMemcpyAsync(host + (size_t)tout[o].y * pb, stg_out + (size_t)o * pb, (size_t)(j - o) * pb,
+      LV_TRY(cudaMemcpyAsync(host + (size_t)tout[o].y * pb, stg_out + (size_t)o * pb, (size_t)no * pb,
                              cudaMemcpyDeviceToHost, pool->s_d2h));
-      o = j;
+      o += no;
     }
   }
   // unpack each chunk once it has arrived, after every pack (on s, or on s_unpack
