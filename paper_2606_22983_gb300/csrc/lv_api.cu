@@ -326,13 +326,16 @@ void longest_runs_first(lv_pool* pool, int4* t, int64_t m, int int4::*slot) {
 //
 // What bounds it: the copy engines, about 1.9 us per transfer beside the bytes, and for small
 // moves the one wait for the task list.  The two directions' transfers are issued in turn, and
-// the packs, in chunks of 24 MiB, with the runs that need them, so that both run from the start (66 runs of 1 to
+// the packs, in chunks, with the runs that need them, so that both run from the start (66 runs of 1 to
 // 6 pages of 1.5 MiB each way by themselves: 1616 us issued in turn, 1813 with one direction
 // first; more streams per direction 1676 to 1841).  A transfer that ends while the other
 // direction's is under way is followed by a gap of up to 9 us, and a long run at the end keeps
 // its direction busy alone with its unpacks behind it; so long runs go first, in pieces of a
 // chunk (150 pages of 1.5 MiB: 1826 us in slot order, 1776 so; 50 by swap-out and swap-in: 965
-// and 947), but runs are not cut to let both directions end together (1880).  An exchange with
+// and 947), but runs are not cut to let both directions end together (1880).  A small chunk
+// leaves little packing before the first transfer and little unpacking after the last (50 pages:
+// 947 us with 24 MiB, 963 with 48, 985 with 96), a large one fewer events and pieces (turns of 0.6
+// GB each way in a row: 281, 288 and 292 GB/s).  An exchange with
 // its ranking, with the task list copied back in two waits and one direction issued first, and
 // now: 5 pages of 16 KiB 68.5 us and 47, 37 of 192 KiB 151 and 126, 25 of 1.5 MiB 358 and 324,
 // 150 of 1.5 MiB 1890 and 1776.
@@ -359,7 +362,9 @@ lv_status staged_move_inner(lv_pool* pool, int64_t n, bool counted, cudaStream_t
   longest_runs_first(pool, tout, n_out, &int4::y);
   longest_runs_first(pool, tin, n_in, &int4::z);
   const size_t pb = (size_t)d.J * d.P;
-  const int64_t chunk = std::max<int64_t>(1, (int64_t)((24u << 20) / pb));
+  // a chunk is an eighth of the larger direction, 24 to 96 MiB of it
+  const int64_t chunk_bytes = std::min<int64_t>(std::max<int64_t>(std::max(n_out, n_in) * (int64_t)pb / 8, 24 << 20), 96 << 20);
+  const int64_t chunk = std::max<int64_t>(1, chunk_bytes / (int64_t)pb);
   const int64_t nchunks = (std::max(n_out, n_in) + chunk - 1) / chunk;
   lv_status st = sync_events(pool, (size_t)(2 * nchunks + 3));
   if (st != LV_OK) return st;
