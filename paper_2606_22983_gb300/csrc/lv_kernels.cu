@@ -2797,16 +2797,25 @@ k_select(DevPool p, long long now_us, long long k, bool fallback, long long* cou
     __syncthreads();
   } else {
     cg::cluster_group cluster = cg::this_cluster();
+    // every CTA says that it runs; nobody writes into the first one before all have said so
+    // (the reads of the states lie between, so the wait costs nothing)
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
     const int x = blockIdx.x * kStepThreads + tid, s0 = x & ~31;
+    unsigned long long key = 0ull;
+    int c = 0, nb = 0;
     if (s0 < p.S) {
-      const int c = x < p.S ? p.cnt[x].x : 0;
+      if (x < p.S) c = p.cnt[x].x;
       const lv_session_state st = load_states(p.sess + s0, p.S - s0, sh.states[tid >> 5]);
       if (x < p.S) {
-        const unsigned long long key = c > 0 ? session_key(p, st, x, now_us, fallback) : 0ull;
-        cluster.map_shared_rank(keys, 0)[x] = key;
-        cluster.map_shared_rank(cnt, 0)[x] = c;
-        cluster.map_shared_rank(nblk, 0)[x] = blocks_of_context(p, st.ctx_tokens);
+        if (c > 0) key = session_key(p, st, x, now_us, fallback);
+        nb = blocks_of_context(p, st.ctx_tokens);
       }
+    }
+    asm volatile("barrier.cluster.wait;" ::: "memory");
+    if (x < p.S) {
+      cluster.map_shared_rank(keys, 0)[x] = key;
+      cluster.map_shared_rank(cnt, 0)[x] = c;
+      cluster.map_shared_rank(nblk, 0)[x] = nb;
     }
     cluster.sync();
     if (blockIdx.x > 0) return;
