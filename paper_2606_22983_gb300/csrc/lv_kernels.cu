@@ -676,11 +676,16 @@ struct BlockScan {
 // One tier's allocation bitmap: the pool's words, and what this kernel works on: a copy in
 // shared memory (with the words as they were beside it, for bits_back), or where that does
 // not fit the pool's words themselves.
+// Which pages are free is read off these words alone, not off the tier's allocation count in
+// p.ctl: a free on another stream may run meanwhile, and it clears a bit and lowers that count
+// one after the other, so the two read apart may disagree, and two threads may read different
+// counts.
 struct TierBits {
   uint32_t* gl;
   uint32_t* cur;
   uint32_t* old;
   long long nbits;
+  int taken;       // set bits among the words that this thread read
   __device__ uint32_t word(int w) const { return cur != gl ? cur[w] : __ldcg(&gl[w]); }
   __device__ bool has(int32_t i) const { return word(i >> 5) >> (i & 31) & 1u; }
   __device__ void set(int w, uint32_t m) const {           // a word only this thread changes now
@@ -693,10 +698,21 @@ struct TierBits {
 // Reads a bitmap of W words into shared memory at `copy` (2 W words; null: used in place).
 __device__ __forceinline__ TierBits bits_copy(uint32_t* gl, long long nbits, uint32_t* copy) {
   const int W = (int)((nbits + 31) >> 5);
-  if (!copy) return TierBits{gl, gl, gl, nbits};
+  TierBits t{gl, gl, gl, nbits, 0};
+  if (LV_RARE(!copy)) {
+#pragma unroll 8
+    for (int w = threadIdx.x; w < W; w += kStepThreads) t.taken += __popc(gl[w]);
+    return t;
+  }
+  t.cur = copy;
+  t.old = copy + W;
 #pragma unroll 1
-  for (int w = threadIdx.x; w < W; w += kStepThreads) copy[w] = copy[W + w] = gl[w];
-  return TierBits{gl, copy, copy + W, nbits};
+  for (int w = threadIdx.x; w < W; w += kStepThreads) {
+    const uint32_t x = gl[w];
+    copy[w] = copy[W + w] = x;
+    t.taken += __popc(x);
+  }
+  return t;
 }
 
 // Writes the words that changed, as reductions of the bits that changed: a free of other
@@ -732,9 +748,10 @@ __device__ __forceinline__ int nth_bit(uint32_t f, int k) {
 // binary search among the threads' counts (in `base`), so that a tier with whole free words
 // takes as long as one with a free bit here and there.  Without a copy of the bitmap each
 // thread writes its own words' bits, and no more than it counted: a free on another stream
-// may add bits meanwhile.  The caller has checked that n are free; other threads may read
-// out when it returns.
-__device__ void take_lowest(const TierBits& t, int n, int32_t* out, BlockScan& scan, int* base) {
+// may add bits meanwhile.  Returns false, with nothing changed, when n and `spare` more are
+// not free (the searches below end only because n are); other threads may read out when it
+// returns.
+__device__ bool take_lowest(const TierBits& t, int n, long long spare, int32_t* out, BlockScan& scan, int* base) {
   const int W = (int)((t.nbits + 31) >> 5);
   const int per = (W + kStepThreads - 1) / kStepThreads;
   const int w0 = threadIdx.x * per;
@@ -745,6 +762,8 @@ __device__ void take_lowest(const TierBits& t, int n, int32_t* out, BlockScan& s
   for (int i = 0; i < per; ++i) cnt += __popc(free_of(w0 + i));
   int total;
   int r = scan.sum(cnt, &total);
+  const bool enough = total - spare >= n;
+  if (!enough) n = 0;
   if (LV_RARE(t.cur == t.gl)) {
     const int r_end = min(n, r + cnt);
 #pragma unroll 1
@@ -760,7 +779,7 @@ __device__ void take_lowest(const TierBits& t, int n, int32_t* out, BlockScan& s
       if (take) t.set(w0 + i, take);
     }
     __syncthreads();
-    return;
+    return enough;
   }
   base[threadIdx.x] = r;
   __syncthreads();
@@ -788,6 +807,7 @@ __device__ void take_lowest(const TierBits& t, int n, int32_t* out, BlockScan& s
     if (take) t.set(w0 + i, take);
     r += c;
   }
+  return enough;
 }
 
 // Spreads the nd slots out[0..nd) so that the r-th victim without a clean copy has the r-th of
@@ -825,7 +845,6 @@ k_alloc(DevPool p, bool in_hbm, const lv_victim* v, long long n, int32_t* out, b
   BlockScan scan{ws, 0};
   uint32_t* copy = copy_bits ? reinterpret_cast<uint32_t*>(dyn) : nullptr;
   const TierBits t = in_hbm ? bits_copy(p.bits_hbm, p.hbm_pages, copy) : bits_copy(p.bits_host, p.host_pages, copy);
-  const long long before = p.ctl[in_hbm ? C_HBM_ALLOC : C_HOST_ALLOC];
   int nd = (int)n;
   if (LV_RARE(v != nullptr)) {
     int cnt = 0;
@@ -833,14 +852,14 @@ k_alloc(DevPool p, bool in_hbm, const lv_victim* v, long long n, int32_t* out, b
     for (long long i = threadIdx.x; i < n; i += kStepThreads) cnt += clean_copy_of(p, v[i]) < 0 ? 1 : 0;
     scan.sum(cnt, &nd);
   }
-  if (LV_RARE(before + nd > (in_hbm ? p.budget : p.host_pages) || injected_fail)) {
+  __syncthreads();             // the bitmap's copy is complete
+  const long long spare = in_hbm ? p.hbm_pages - p.budget : 0;
+  if (LV_RARE(injected_fail || (nd > 0 && !take_lowest(t, nd, spare, out, scan, base)))) {
     if (threadIdx.x == 0) set_error(p.ctl, in_hbm ? LV_ERR_NO_HBM : LV_ERR_NO_HOST, nd);
 #pragma unroll 1
     for (long long i = threadIdx.x; i < n; i += kStepThreads) out[i] = -1;
     return;
   }
-  __syncthreads();             // the bitmap's copy is complete
-  if (nd > 0) take_lowest(t, nd, out, scan, base);
   uint32_t* own = in_hbm ? p.own_hbm : p.own_host;
 #pragma unroll 1
   for (int i = threadIdx.x; i < nd; i += kStepThreads) own[out[i]] = kOwnerReserved;
@@ -899,6 +918,7 @@ struct StepShared {
   int ws[2 * kStepWarps];
   unsigned long long best[2][kStepWarps];
   int2 sums[kStepWarps];
+  int taken[kStepWarps];            // HBM pages allocated, by the warps that read their bits
   int2 pick[kStepWarps + 1];
   int sel_sid[12], sel_off[12];     // [kSelectRounds]
   uint32_t done[kStepItems / 32];   // victims that need no out task of their own
@@ -915,12 +935,13 @@ struct StepShared {
 // else they were just read from the tables, and checked there: bad_out and bad_in are a
 // thread's first wrong victim and load, or -1.  Returns false, with nothing changed, the
 // outputs -1 and no tasks, when an item is refused or a tier is too full.
-// hbm_alloc and host_alloc: the tiers' allocation counts as the kernel found them.
+// hbm_alloc: the HBM pages allocated as the kernel found them.
 template <bool kListed>
 __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& hbm, const TierBits& host,
-                           long long hbm_alloc, long long host_alloc, long long bad_out, long long bad_in,
+                           long long hbm_alloc, long long bad_out, long long bad_in,
                            StepShared& sh, BlockScan& scan) {
-  const long long n_out = m.n_out, n_in = m.n_in;
+  const long long n_out = m.n_out;
+  long long n_in = m.n_in;
   const bool sid_ok = m.sid >= 0 && m.sid < p.S;
   const size_t row = sid_ok ? (size_t)m.sid * p.maxB : 0;
   const int32_t nb_in = kListed && sid_ok ? nblocks_of(p, m.sid) : 0;
@@ -967,8 +988,18 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
   if (LV_RARE(p.incl)) scan.sum(dirty, &n_dirty);
   // capacity, as the sequential calls see it: host slots before any is freed,
   // HBM pages after the victims' pages are freed
-  const bool no_host = host_alloc + n_dirty > p.host_pages;
   const bool no_hbm = hbm_alloc - n_out + n_in > p.budget;
+  bool no_host = false;
+  if (LV_RARE(no_hbm)) {
+    int mine = 0, used;
+#pragma unroll 1
+    for (int w = threadIdx.x; w < (int)((p.host_pages + 31) >> 5); w += kStepThreads) mine += __popc(host.word(w));
+    scan.sum(mine, &used);
+    no_host = used + (long long)n_dirty > p.host_pages;
+  } else if (LV_MOSTLY(n_dirty > 0 && !bad)) {
+    // host slots for the victims: a clean copy, or the lowest free slots in victim order
+    no_host = !take_lowest(host, n_dirty, 0, m.slots, scan, sh.base);
+  }
   if (LV_RARE(bad || no_host || no_hbm)) {
     if (!bad && threadIdx.x == 0)
       set_error(p.ctl, no_host ? LV_ERR_NO_HOST : LV_ERR_NO_HBM, no_host ? (long long)n_dirty : n_in);
@@ -979,8 +1010,6 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
     if (threadIdx.x == 0) *m.n_tasks = 0;
     return false;
   }
-  // host slots for the victims: a clean copy, or the lowest free slots in victim order
-  if (n_dirty > 0) take_lowest(host, n_dirty, m.slots, scan, sh.base);
   if (LV_RARE(n_dirty < n_out)) {
     __syncthreads();
     spread_slots(p, m.v, n_out, n_dirty, m.slots, scan);
@@ -1019,7 +1048,8 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
   __syncthreads();
   // HBM pages for the incoming blocks
   if (n_in > 0) {
-    take_lowest(hbm, (int)n_in, m.pages, scan, sh.base);
+    // (too few only if a victim's page had no bit: then nothing is loaded)
+    n_in = take_lowest(hbm, (int)n_in, 0, m.pages, scan, sh.base) ? n_in : 0;
     __syncthreads();
   }
   // a victim's page is now taken again, or free
@@ -1101,6 +1131,7 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
     run += chunk;
   }
   if (threadIdx.x == 0) {
+    if (LV_RARE(n_in < m.n_in)) set_error(p.ctl, LV_ERR_STATE, n_out);
     *m.n_tasks = n_in + run;
     const long long n_clean = n_out - n_dirty;
     const long long host_delta = p.incl ? n_dirty : n_dirty - n_in;
@@ -1136,23 +1167,22 @@ k_exchange_plan(DevPool p, const lv_victim* __restrict__ v, long long n_out, int
   uint32_t* copy = copy_bits ? reinterpret_cast<uint32_t*>(dyn) : nullptr;
   const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, copy);
   const TierBits host = bits_copy(p.bits_host, p.host_pages, copy ? copy + 2 * ((p.hbm_pages + 31) >> 5) : nullptr);
-  const long long hbm_alloc = p.ctl[C_HBM_ALLOC], host_alloc = p.ctl[C_HOST_ALLOC];
   if (threadIdx.x == 0 && cursor) *cursor = 0;
+  int hbm_alloc;
+  scan.sum(hbm.taken, &hbm_alloc);
   MovePlan m{v, n_out, sid, blks, nullptr, n_in, n_out <= kStepItems ? sh.l.slots : slots,
              n_in <= kStepItems ? sh.l.pages : pages, slots, pages, tasks, n_tasks, epoch, page_tag};
-  plan_moves<true>(p, m, hbm, host, hbm_alloc, host_alloc, -1, -1, sh, scan);
+  plan_moves<true>(p, m, hbm, host, hbm_alloc, -1, -1, sh, scan);
   __syncthreads();
   bits_back(hbm);
   bits_back(host);
 }
 
 // Grows session sid, of ctx tokens, by n_tokens (every thread of the CTA calls it): the new
-// blocks take the lowest free HBM pages, in block order.  hbm_alloc: pages allocated now.
-// near: room for kStepItems page ids in shared memory.  Returns the pages appended, -1 on an
-// error.
+// blocks take the lowest free HBM pages, in block order.  near: room for kStepItems page ids
+// in shared memory.  Returns the pages appended, -1 on an error.
 __device__ long long append_tokens_to(const DevPool& p, int32_t sid, int32_t ctx, int32_t n_tokens,
-                                      int32_t* pages, long long hbm_alloc, const TierBits& hbm,
-                                      const TierBits& host,
+                                      int32_t* pages, const TierBits& hbm, const TierBits& host,
                                       int32_t* near, BlockScan& scan, int* base) {
   const int32_t nb = (int32_t)(((uint32_t)ctx + (uint32_t)p.T - 1u) / (uint32_t)p.T);
   const uint32_t nctx = (uint32_t)ctx + (uint32_t)n_tokens;
@@ -1163,13 +1193,12 @@ __device__ long long append_tokens_to(const DevPool& p, int32_t sid, int32_t ctx
     if (threadIdx.x == 0) set_error(p.ctl, LV_ERR_BOUNDS, sid);
     return -1;
   }
-  if (LV_RARE(m > 0 && hbm_alloc + m > p.budget)) {
-    if (threadIdx.x == 0) set_error(p.ctl, LV_ERR_NO_HBM, sid);
-    return -1;
-  }
   if (m > 0) {
     int32_t* list = m <= kStepItems ? near : pages;
-    take_lowest(hbm, (int)m, list, scan, base);
+    if (LV_RARE(!take_lowest(hbm, (int)m, p.hbm_pages - p.budget, list, scan, base))) {
+      if (threadIdx.x == 0) set_error(p.ctl, LV_ERR_NO_HBM, sid);
+      return -1;
+    }
 #pragma unroll 1
     for (long long i = threadIdx.x; i < m; i += kStepThreads) {
       const int32_t pg = list[i];
@@ -1214,9 +1243,8 @@ k_append(DevPool p, int32_t sid, int32_t n_tokens, int32_t* pages, int32_t* coun
   const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, copy_bits ? reinterpret_cast<uint32_t*>(dyn) : nullptr);
   const TierBits host = bits_copy(p.bits_host, p.host_pages, nullptr);      // one bit of it at most
   const int32_t ctx = p.sess[sid].ctx_tokens;
-  const long long hbm_alloc = p.ctl[C_HBM_ALLOC];
-  __syncthreads();      // every thread has read both
-  const long long m = append_tokens_to(p, sid, ctx, n_tokens, pages, hbm_alloc, hbm, host, near, scan, base);
+  __syncthreads();      // every thread has read it and the bitmap
+  const long long m = append_tokens_to(p, sid, ctx, n_tokens, pages, hbm, host, near, scan, base);
   if (m > 0) {
     __syncthreads();
     bits_back(hbm);
@@ -2436,12 +2464,11 @@ k_step(DevPool p, StepArgs a) {
   long long* R = a.rs.words;
   const bool evict = a.evict >= 0;
 
-  // reads that depend on nothing: the candidates, allocation counts, bitmaps, every session's
-  // state (whole, before anything is decided from it) and counts
+  // reads that depend on nothing: the candidates, bitmaps, every session's state (whole,
+  // before anything is decided from it) and counts
   const bool picks = a.turn && a.sid < 0 && a.part != kStepMove;
   int32_t first_cand = -1;
   if (picks && tid < a.n_cand) first_cand = a.cand[tid];
-  const long long hbm_alloc = p.ctl[C_HBM_ALLOC], host_alloc = p.ctl[C_HOST_ALLOC];
   uint32_t* copy = a.copy_bits && a.part != kStepList ? reinterpret_cast<uint32_t*>(dyn + lay.bits) : nullptr;
   const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, copy);
   const TierBits host = bits_copy(p.bits_host, p.host_pages, copy ? copy + 2 * ((p.hbm_pages + 31) >> 5) : nullptr);
@@ -2458,8 +2485,11 @@ k_step(DevPool p, StepArgs a) {
       keys[x] = c.x > 0 ? session_key(p, st, x, a.now_us, fallback) : 0ull;
     }
   }
+  const int part = __reduce_add_sync(0xffffffffu, hbm.taken);
+  if (lane == 0) sh.taken[tid >> 5] = part;
   if (tid == 0) R[R_CURSOR] = 0;
   __syncthreads();
+  const int hbm_alloc = __reduce_add_sync(0xffffffffu, lane < kStepWarps ? sh.taken[lane] : 0);
 
   // the session: given, picked (the first candidate with a host-tier block, else the first), or none
   int32_t sid = a.sid;
@@ -2683,7 +2713,7 @@ k_step(DevPool p, StepArgs a) {
   out_check.settle();
   in_check.settle();
   const bool planned =
-      plan_moves<false>(p, m, hbm, host, hbm_alloc, host_alloc, out_check.bad, in_check.bad, sh, scan);
+      plan_moves<false>(p, m, hbm, host, hbm_alloc, out_check.bad, in_check.bad, sh, scan);
   if (LV_MOSTLY(planned && n_out > 0)) {
     // the victims' sessions: fewer blocks in HBM, more in the host tier
 #pragma unroll 1
@@ -2697,9 +2727,7 @@ k_step(DevPool p, StepArgs a) {
   long long appended = 0;
   if (LV_RARE(grow && a.append_tokens > 0)) {
     __syncthreads();                            // the commits of the plan
-    appended = append_tokens_to(p, sid, ctx, a.append_tokens, a.rs.append,
-                                planned ? hbm_alloc - n_out + n_in : hbm_alloc, hbm, host, sh.l.pages, scan,
-                                sh.base);
+    appended = append_tokens_to(p, sid, ctx, a.append_tokens, a.rs.append, hbm, host, sh.l.pages, scan, sh.base);
     if (appended < 0) appended = 0;
   }
   __syncthreads();
