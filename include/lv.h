@@ -40,6 +40,12 @@
  * output after the stream has completed.
  * Calls that allocate from the same tier (swap-out: host slots; swap-in and
  * append: HBM pages) must be ordered with respect to each other.
+ * A free (lv_cancel, the old locations of lv_remap) may overlap an allocation.
+ * A device-driven step (lv_turn, lv_make_resident, lv_evict) and
+ * lv_swap_exchange must also be ordered with calls that change the table of a
+ * session they may take blocks from or load (lv_remap, lv_session_append,
+ * another step): where such a call falls between their reads, they report
+ * LV_ERR_STATE and move nothing.
  *
  * Threads.  A pool keeps host-side state (scratch alternation, pending
  * asynchronous copies, staging runs, timing records): calls on one pool must

@@ -2164,34 +2164,38 @@ struct VictimList {
   }
 };
 
-// The blocks of session s (nb of them) in victim order: positions pos0.. of the list, by the
-// whole CTA.  A block's page has to be its own.
-__device__ void emit_whole(const DevPool& p, int32_t s, int32_t nb, long long pos0, const VictimList& l,
-                           OwnerCheck& check, BlockScan& scan) {
+// The blocks of session s (nb of them) in victim order, by the whole CTA: positions pos0 to
+// end of the list, which the session's count gave it.  A block's page has to be its own, and
+// every position has to be filled: a row that holds fewer blocks than were counted (a commit
+// on another stream between the two) is a wrong victim, of one that holds more the first are
+// taken.
+__device__ void emit_whole(const DevPool& p, int32_t s, int32_t nb, long long pos0, long long end,
+                           const VictimList& l, OwnerCheck& check, BlockScan& scan) {
   const int32_t* row = p.table + (size_t)s * p.maxB;
   const bool suffix = p.within == LV_SUFFIX_FIRST;
 #pragma unroll 1
-  for (int32_t q0 = 0; q0 < nb && pos0 < l.n_out; q0 += kStepThreads) {
+  for (int32_t q0 = 0; q0 < nb && pos0 < end; q0 += kStepThreads) {
     const int32_t q = q0 + threadIdx.x;
     const int32_t b = suffix ? nb - 1 - q : q;
     const int32_t e = q < nb ? row[b] : -1;
     check.read(l.own, e, l.n_own);
     int chunk;
     const long long pos = pos0 + scan.rank(e >= 0, &chunk);
-    if (e >= 0 && pos < l.n_out) {
+    if (e >= 0 && pos < end) {
       l.put(pos, s, b, e);
       if (l.own) check.expect(owner_key(s, b), pos);
     }
     pos0 += chunk;
   }
+  if (LV_RARE(pos0 < end)) check.bad = pos0;
 }
 
 // The same for sessions `of(r)`, r = first, first + kStepWarps, ... below m, by one warp, four
 // sessions at a time: the first 32 blocks of each are read together (a session of a few
 // blocks costs a read's latency, whoever reads it).
 template <typename Of>
-__device__ void emit_warp(const DevPool& p, const int* nblk, int m, const VictimList& l, OwnerCheck& check,
-                          Of of) {
+__device__ void emit_warp(const DevPool& p, const int* nblk, const int* cnt, int m, const VictimList& l,
+                          OwnerCheck& check, Of of) {
   const int lane = threadIdx.x & 31;
   const bool suffix = p.within == LV_SUFFIX_FIRST;
 #pragma unroll 1
@@ -2214,6 +2218,7 @@ __device__ void emit_warp(const DevPool& p, const int* nblk, int m, const Victim
       const int32_t s = so.x, nb = nblk[s];
       const int32_t* row = p.table + (size_t)s * p.maxB;
       long long pos0 = so.y;
+      const long long end = pos0 + cnt[s] < l.n_out ? pos0 + cnt[s] : l.n_out;
       int32_t x = e[u];
 #pragma unroll 1
       for (int32_t q0 = 0;; ) {
@@ -2221,16 +2226,17 @@ __device__ void emit_warp(const DevPool& p, const int* nblk, int m, const Victim
         check.read(l.own, x, l.n_own);
         const unsigned has = __ballot_sync(0xffffffffu, x >= 0);
         const long long pos = pos0 + __popc(has & ((1u << lane) - 1u));
-        if (x >= 0 && pos < l.n_out) {
+        if (x >= 0 && pos < end) {
           const int32_t b = suffix ? nb - 1 - q : q;
           l.put(pos, s, b, x);
           if (l.own) check.expect(owner_key(s, b), pos);
         }
         pos0 += __popc(has);
         q0 += 32;
-        if (q0 >= nb || pos0 >= l.n_out) break;
+        if (q0 >= nb || pos0 >= end) break;
         x = q0 + lane < nb ? row[suffix ? nb - 1 - q0 - lane : q0 + lane] : -1;
       }
+      if (LV_RARE(pos0 < end)) check.bad = pos0;
     }
   }
 }
@@ -2409,16 +2415,19 @@ __device__ Selected select_sessions(const DevPool& p, unsigned long long* keys, 
 
 // Writes the victims of the selected sessions.
 __device__ void emit_selected(const DevPool& p, const Selected& sel, const unsigned long long* keys,
-                              const int* off, const int* nblk, const VictimList& l, OwnerCheck& check,
-                              StepShared& sh, BlockScan& scan) {
+                              const int* off, const int* nblk, const int* cnt, const VictimList& l,
+                              OwnerCheck& check, StepShared& sh, BlockScan& scan) {
   if (LV_MOSTLY(sel.m <= 2 && !sel.sorted)) {
 #pragma unroll 1
-    for (int r = 0; r < sel.m; ++r)
-      emit_whole(p, sh.sel_sid[r], nblk[sh.sel_sid[r]], sh.sel_off[r], l, check, scan);
+    for (int r = 0; r < sel.m; ++r) {
+      const int32_t s = sh.sel_sid[r];
+      const long long at = sh.sel_off[r];
+      emit_whole(p, s, nblk[s], at, at + cnt[s] < l.n_out ? at + cnt[s] : l.n_out, l, check, scan);
+    }
   } else if (sel.sorted) {
-    emit_warp(p, nblk, sel.m, l, check, [&](int r) { return make_int2(session_of_key(keys[r]), off[r]); });
+    emit_warp(p, nblk, cnt, sel.m, l, check, [&](int r) { return make_int2(session_of_key(keys[r]), off[r]); });
   } else {
-    emit_warp(p, nblk, sel.m, l, check, [&](int r) { return make_int2(sh.sel_sid[r], sh.sel_off[r]); });
+    emit_warp(p, nblk, cnt, sel.m, l, check, [&](int r) { return make_int2(sh.sel_sid[r], sh.sel_off[r]); });
   }
 }
 
@@ -2564,8 +2573,11 @@ k_step(DevPool p, StepArgs a) {
       nh = R[R_N_IN];
 #pragma unroll 1
       for (long long i = tid; i < nh; i += kStepThreads) {
+        // (the order was made by another kernel, from keys read more than once: each block once)
         const int32_t b = a.rs.loads[i];
-        const long long h = -(long long)p.table[(size_t)sid * p.maxB + b] - 2;
+        const size_t ti = (size_t)sid * p.maxB + b;
+        long long h = -1;
+        if (b >= 0 && b < nb && atomicExch(&p.mark[ti], a.epoch) != a.epoch) h = -(long long)p.table[ti] - 2;
         in_check.read(p.own_host, h, p.host_pages);
         in_check.expect(owner_key(sid, b), i);
       }
@@ -2687,7 +2699,7 @@ k_step(DevPool p, StepArgs a) {
   // the victims of the order's first n_out positions
   lv_victim* near = sel.n_out <= kStepItems ? sh.l.v : nullptr;
   const VictimList list{near, a.rs.victims, p.own_hbm, p.hbm_pages, sel.n_out};
-  emit_selected(p, sel, keys, off, nblk, list, out_check, sh, scan);
+  emit_selected(p, sel, keys, off, nblk, cnt, list, out_check, sh, scan);
   // the gate: a shortfall stops the step (a preload is skipped, a foreground turn fails);
   // lv_evict takes what there is
   long long n_out = sel.n_out, n_in = go ? nh : 0;
@@ -2851,7 +2863,7 @@ k_select(DevPool p, long long now_us, long long k, bool fallback, long long* cou
   const Selected sel = select_sessions(p, keys, off, cnt, k, -1, sh, scan);
   OwnerCheck check{0, 0, -1, -1};
   const VictimList list{nullptr, out, nullptr, 0, sel.n_out};
-  emit_selected(p, sel, keys, off, nblk, list, check, sh, scan);
+  emit_selected(p, sel, keys, off, nblk, cnt, list, check, sh, scan);
   if (tid == 0) {
     p.ctl[C_SEL_COUNT] = sel.n_out;
     p.ctl[C_SEL_TOTAL] = sel.total;
