@@ -231,7 +231,7 @@ typedef struct lv_stats {
    (the TMA pack/unpack kernel, default about 48 KiB of stages per CTA and two
    CTAs per SM); LV_STAGE_KERNEL=lsu (16-byte copies instead of TMA);
    LV_REMAP_ENTRIES_PER_THREAD = 1, 2 or 4 (lv_remap's entries per thread, with
-   a release pass; by default up to 2^18 entries take a thread each and need no
+   a release pass; by default up to 2^14 entries take a thread each and need no
    such pass, more take 1 while the GPU holds one thread per entry at once, else
    2 or 4);
    LV_EXCHANGE_KERNEL=tma (the exchange copy by TMA bulk copies, one issuing

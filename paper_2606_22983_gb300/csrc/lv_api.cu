@@ -627,6 +627,8 @@ lv_status create_impl(const lv_pool_desc* desc, cudaStream_t s, lv_pool** out) {
     return fail(LV_ERR_CUDA);
   d.S = desc->max_sessions;
   d.maxB = desc->max_blocks;
+  // 2^14 words: one session's changes go to many, many sessions' to four each
+  for (d.spread_copies = 1; 2 * d.spread_copies * d.S <= 1 << 14;) d.spread_copies *= 2;
   d.T = desc->page_tokens;
   d.J = 2 * desc->num_layers;
   d.P = (int64_t)desc->page_tokens * desc->num_kv_heads * desc->head_dim * desc->elem_bytes;
@@ -684,6 +686,7 @@ lv_status create_impl(const lv_pool_desc* desc, cudaStream_t s, lv_pool** out) {
       (st = dev_alloc(pool, &d.mark, tb)) != LV_OK ||
       (st = dev_alloc(pool, &d.shadow, tb)) != LV_OK ||
       (st = dev_alloc(pool, &d.cnt, d.S)) != LV_OK ||
+      (st = dev_alloc(pool, &d.spread, (size_t)d.spread_copies * d.S)) != LV_OK ||
       (st = dev_alloc(pool, &d.own_hbm, (size_t)d.hbm_pages)) != LV_OK ||
       (st = dev_alloc(pool, &d.own_host, (size_t)d.host_pages)) != LV_OK ||
       (st = dev_alloc(pool, &d.bits_hbm, wh)) != LV_OK ||
@@ -725,6 +728,7 @@ lv_status create_impl(const lv_pool_desc* desc, cudaStream_t s, lv_pool** out) {
       cudaMemsetAsync(d.mark, 0, tb * sizeof(int32_t), s) != cudaSuccess ||
       cudaMemsetAsync(d.shadow, 0xff, tb * sizeof(int32_t), s) != cudaSuccess ||
       cudaMemsetAsync(d.cnt, 0, d.S * sizeof(int2), s) != cudaSuccess ||
+      cudaMemsetAsync(d.spread, 0, (size_t)d.spread_copies * d.S * sizeof(unsigned long long), s) != cudaSuccess ||
       cudaMemsetAsync(d.own_hbm, 0xff, (size_t)d.hbm_pages * 4, s) != cudaSuccess ||
       cudaMemsetAsync(d.own_host, 0xff, (size_t)(d.host_pages ? d.host_pages : 1) * 4, s) != cudaSuccess ||
       cudaMemsetAsync(d.bits_hbm, 0, wh * 4, s) != cudaSuccess ||

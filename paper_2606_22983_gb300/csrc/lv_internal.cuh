@@ -65,6 +65,8 @@ struct DevPool {
   int32_t* mark;          // [S][maxB] epoch of the last remap that touched the block
   int32_t* shadow;        // [S][maxB] host slot holding the block's clean copy, or -1
   int2* cnt;              // [S] blocks in HBM (x) and in the host tier (y), kept with the table
+  unsigned long long* spread;  // [spread_copies][S] changes of cnt that a large commit has not added yet
+  int32_t spread_copies;  // a power of two
   uint32_t* own_hbm;      // [hbm_pages] owner word (kOwnerNone / kOwnerReserved / sid << 16 | blk)
   uint32_t* own_host;     // [host_pages]
   uint32_t* bits_hbm;     // allocation bitmap, 1 = reserved or owned

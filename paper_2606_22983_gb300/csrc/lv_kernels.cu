@@ -114,15 +114,18 @@ __device__ __forceinline__ int2 tier_of(int32_t e) { return make_int2(e >= 0 ? 1
 
 // Both counts change by one 64-bit addition of dd * 2^32 + dh (a negative dh borrows from the
 // upper half what the sum gives back).
-__device__ __forceinline__ void add_counts(const DevPool& p, int32_t s, int dh, int dd) {
-  atomicAdd(reinterpret_cast<unsigned long long*>(&p.cnt[s]),
-            ((unsigned long long)(unsigned)dd << 32) + (unsigned long long)(long long)dh);
+__device__ __forceinline__ void add_counts(unsigned long long* cnt, int dh, int dd) {
+  atomicAdd(cnt, ((unsigned long long)(unsigned)dd << 32) + (unsigned long long)(long long)dh);
+}
+__device__ __forceinline__ unsigned long long* counts_of(const DevPool& p, int32_t s) {
+  return reinterpret_cast<unsigned long long*>(&p.cnt[s]);
 }
 
 // Adds (dh, dd) to the counts of session s, for the whole warp at once: lanes that share the
 // first adding lane's session add through one reduction, the others by themselves.
-// All 32 lanes must call it; a lane with nothing to add passes zeros.
-__device__ __forceinline__ void warp_count(const DevPool& p, int32_t s, int dh, int dd) {
+// All 32 lanes must call it; a lane with nothing to add passes zeros.  cnt: where this lane
+// adds, [S] words.
+__device__ __forceinline__ void warp_count(unsigned long long* cnt, int32_t s, int dh, int dd) {
   const unsigned act = __ballot_sync(0xffffffffu, dh != 0 || dd != 0);
   if (!act) return;
   const int lead = __ffs(act) - 1;
@@ -131,10 +134,31 @@ __device__ __forceinline__ void warp_count(const DevPool& p, int32_t s, int dh, 
   const int h = __reduce_add_sync(0xffffffffu, mine ? dh : 0);
   const int d = __reduce_add_sync(0xffffffffu, mine ? dd : 0);
   if ((int)(threadIdx.x & 31) == lead) {
-    add_counts(p, s0, h, d);
+    add_counts(cnt + s0, h, d);
   } else if (adds && !mine) {
-    add_counts(p, s, dh, dd);
+    add_counts(cnt + s, dh, dd);
   }
+}
+
+// The same for the E changes of each lane, v[j] = dd * 2^16 + dh for session s[j]: where the
+// warp's sessions are all one, through one reduction.
+template <int E>
+__device__ __forceinline__ void warp_counts(unsigned long long* cnt, const int32_t* s, const int* v) {
+  const int32_t s0 = __shfl_sync(0xffffffffu, s[0], 0);
+  bool one = true;
+  int sum = 0;
+#pragma unroll
+  for (int j = 0; j < E; ++j) {
+    one = one && (v[j] == 0 || s[j] == s0);
+    sum += v[j];
+  }
+  if (__all_sync(0xffffffffu, one)) {
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if ((threadIdx.x & 31) == 0 && sum) add_counts(cnt + s0, (int)(int16_t)sum, (sum - (int)(int16_t)sum) >> 16);
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < E; ++j) warp_count(cnt, s[j], (int)(int16_t)v[j], (v[j] - (int)(int16_t)v[j]) >> 16);
 }
 
 // ---------------------------------------------------------------- import
@@ -156,7 +180,7 @@ __global__ void k_import(DevPool p, const int32_t* __restrict__ placement,
       e = import_block(p, placement, ctx, idx, s, (int32_t)(idx % p.maxB));
     }
     const int2 t = tier_of(e);
-    warp_count(p, s, t.x, t.y);
+    warp_count(counts_of(p, 0), s, t.x, t.y);
     in_hbm += t.x;
     in_host += t.y;
   }
@@ -1039,7 +1063,7 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
     }
     if (kListed) {
       const bool mine = i < n_out;
-      warp_count(p, mine ? m.v[i].sid : 0, mine ? -1 : 0, mine ? 1 : 0);
+      warp_count(counts_of(p, 0), mine ? m.v[i].sid : 0, mine ? -1 : 0, mine ? 1 : 0);
     }
   }
   if (LV_MOSTLY(look_up))
@@ -1135,7 +1159,7 @@ __device__ bool plan_moves(const DevPool& p, const MovePlan& m, const TierBits& 
     *m.n_tasks = n_in + run;
     const long long n_clean = n_out - n_dirty;
     const long long host_delta = p.incl ? n_dirty : n_dirty - n_in;
-    if (n_in) add_counts(p, m.sid, (int)n_in, -(int)n_in);
+    if (n_in) add_counts(counts_of(p, m.sid), (int)n_in, -(int)n_in);
     atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HOST_ALLOC]), (unsigned long long)host_delta);
     if (LV_RARE(p.incl)) {
       atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_CLEAN]), (unsigned long long)(n_in - n_clean));
@@ -1211,7 +1235,7 @@ __device__ long long append_tokens_to(const DevPool& p, int32_t sid, int32_t ctx
   if (threadIdx.x == 0) {
     if (m > 0) {
       atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctl[C_HBM_ALLOC]), (unsigned long long)m);
-      add_counts(p, sid, (int)m, 0);
+      add_counts(counts_of(p, sid), (int)m, 0);
     }
     // inclusive tiers: the partially filled last block gains rows, its clean copy is stale
     if (LV_RARE(p.incl) && n_tokens > 0 && nb > 0 && ctx % p.T != 0) {
@@ -1835,8 +1859,8 @@ __device__ __forceinline__ void remap_settle(const DevPool& p, const RemapRead& 
   c.ok += 1;
 }
 
-// Each thread commits E entries, i0, i0 + stride, ... (stride = the grid's
-// threads, so a warp's entries stay contiguous).  The allocation counts and the
+// Each thread commits E entries, a CTA's threads apart, so that a warp's entries are
+// contiguous and a CTA's mostly of one session.  The allocation counts and the
 // commit counter change by block totals (one atomic per block and counter).
 // Inclusive tiers: a host location may be the block's own clean copy; a block
 // committed to HBM from the host tier keeps its slot as its clean copy; a
@@ -1858,21 +1882,27 @@ __device__ __forceinline__ void remap_settle(const DevPool& p, const RemapRead& 
 //
 // kDirect: the freed locations' owner words and bitmap bits are cleared by the entries
 // themselves and there is no release pass.  That pass reads both tiers' owner words, whatever
-// the number of entries, and is a launch of its own: up to 2^18 entries the direct form is the
-// shorter (a pool of 2^20 pages and slots: 6.8 us against 10.9 for 1024 entries, 12.9 against
-// 15.0 for 2^18; scattered over the pool 37.5 against 39.6), at 2^20 the release pass (29.3
-// against 33.4), since it clears a run of freed pages by the word.
+// the number of entries, and is a launch of its own: a commit of 1024 of 2^20 pages takes 7 to
+// 9 us without it and 11 with it.
+//
+// The sessions' counts are what many entries wait for one another at: a warp whose entries
+// are of one session adds once, but a warp of mixed ones adds 32 times to a few lines, and 16
+// sessions of 65536 blocks each in order 8192 times to each of 16 words.  So the form with a
+// release pass adds to one of spread_copies arrays, which that pass adds up: 2^20 entries of
+// 16 sessions 57 us without the copies and 25.7 with them, in mixed order 310 and 50; of 512
+// sessions 27.5 and 25.7, in mixed order 106 and 45 (26 and 37.5 when no counts were kept).
+// The direct form has no such pass, so it ends where mixed orders make it the longer one:
+// 2^14 entries of 16 sessions 11.5 us, of 2 13, and 2^16 25, against 13 to 15.
 template <int E, bool kDirect>
 __global__ void __launch_bounds__(kRemapThreads, 4)
 k_remap(DevPool p, const lv_remap_entry* __restrict__ e, long long n, int32_t epoch) {
   if (kDirect) pdl_entry();
   else pdl_wait();          // a large grid: the release pass is scheduled behind it
-  const long long stride = (long long)gridDim.x * kRemapThreads;
-  const long long i0 = blockIdx.x * (long long)kRemapThreads + threadIdx.x;
+  const long long i0 = blockIdx.x * (long long)(E * kRemapThreads) + threadIdx.x;
   RemapRead r[E];
   int32_t seen[E];
 #pragma unroll
-  for (int j = 0; j < E; ++j) remap_read_entry(p, e, i0 + j * stride, n, r[j]);
+  for (int j = 0; j < E; ++j) remap_read_entry(p, e, i0 + j * kRemapThreads, n, r[j]);
 #pragma unroll
   for (int j = 0; j < E; ++j) {
     remap_read_table(p, r[j]);
@@ -1884,16 +1914,22 @@ k_remap(DevPool p, const lv_remap_entry* __restrict__ e, long long n, int32_t ep
   for (int j = 0; j < E; ++j) {
     got[j] = kOwnerReserved;
     was[j] = kOwnerNone;
-    err[j] = i0 + j * stride < n ? remap_judge(r[j], epoch, seen[j]) : -1;
+    err[j] = i0 + j * kRemapThreads < n ? remap_judge(r[j], epoch, seen[j]) : -1;
     if (err[j] >= 0) err[j] = remap_claim<kDirect>(p, r[j], err[j], got[j], was[j]);
   }
   RemapCounts c{0, 0, 0, 0, 0, 0};
+  unsigned long long* cnt = counts_of(p, 0);
+  if (!kDirect) cnt = p.spread + (size_t)(i0 & (p.spread_copies - 1)) * p.S;
+  int32_t sid[E];
+  int change[E];
 #pragma unroll
   for (int j = 0; j < E; ++j) {
     c.dh = c.dd = 0;
-    if (err[j] >= 0) remap_settle<kDirect>(p, r[j], err[j], got[j], was[j], i0 + j * stride, c);
-    warp_count(p, r[j].x.sid, c.dh, c.dd);
+    if (err[j] >= 0) remap_settle<kDirect>(p, r[j], err[j], got[j], was[j], i0 + j * kRemapThreads, c);
+    sid[j] = r[j].x.sid;
+    change[j] = c.dd * 65536 + c.dh;
   }
+  warp_counts<E>(cnt, sid, change);
   // block totals: warp sums, one shared atomic per warp, one global atomic per block
   __shared__ int tot[4];
   if (threadIdx.x < 4) tot[threadIdx.x] = 0;
@@ -1971,6 +2007,13 @@ k_release(DevPool p, long long qh, long long qo) {
   const long long total = qh + qo;
   const long long step = (long long)gridDim.x * kReleaseThreads;
   const int lane8 = threadIdx.x & 7;
+  // the sessions' counts (whichever commit's changes they are, each is taken once)
+  const int changes = p.spread_copies * p.S;
+  for (long long i = (long long)blockIdx.x * kReleaseThreads + threadIdx.x; i < changes; i += step) {
+    if (p.spread[i] == 0ull) continue;
+    const unsigned long long x = atomicExch(&p.spread[i], 0ull);
+    if (x) atomicAdd(counts_of(p, (int32_t)(i % p.S)), x);
+  }
   for (long long q0 = (long long)blockIdx.x * kReleaseThreads + threadIdx.x;
        q0 - threadIdx.x < total; q0 += kReleaseUnroll * step) {
     uint4 v[kReleaseUnroll];
@@ -2733,7 +2776,7 @@ k_step(DevPool p, StepArgs a) {
       const int32_t s = sel.sorted ? session_of_key(keys[r]) : sh.sel_sid[r];
       const long long at = sel.sorted ? off[r] : sh.sel_off[r];
       const int take = (int)(n_out - at < cnt[s] ? n_out - at : cnt[s]);
-      add_counts(p, s, -take, take);
+      add_counts(counts_of(p, s), -take, take);
     }
   }
   long long appended = 0;
@@ -3371,7 +3414,7 @@ cudaError_t launch_stage(const DevPool& p, bool pack, bool page_list, const void
   return e;
 }
 
-constexpr long long kRemapDirect = 1 << 18;
+constexpr long long kRemapDirect = 1 << 14;
 
 cudaError_t launch_remap(const DevPool& p, const lv_remap_entry* e, int64_t n, int32_t epoch,
                          cudaStream_t s, int num_sms, int per_thread) {

@@ -35,7 +35,7 @@ LV_VERSION = 3                     # include/lv.h
 STEP_ITEMS = 1024                  # loads of one turn that a device-driven step orders by itself
 SELECT_MOST = 2048                 # a ranking of at most this many victims, and of at most
 SELECT_SESSIONS = 128              # this many per block of a table row, is one kernel
-REMAP_DIRECT = 1 << 18             # a commit of at most this many entries is one kernel
+REMAP_DIRECT = 1 << 14             # a commit of at most this many entries is one kernel
 EMIT_SCAN_MAX = 1024               # above this many sessions a larger ranking runs one more kernel
 LV_MODE_ASYNC = 16
 LV_RUNNING, LV_IMMEDIATE, LV_RESP_OPEN, LV_DONE_VALID = 1, 2, 4, 8

@@ -1,6 +1,7 @@
 """lv_remap's forms -- the entries free their old locations themselves, or a release pass does,
 with 1, 2 or 4 entries per thread -- leave the same tables, owners, counts and free pages,
-with wrong entries among the right ones and under both tier modes."""
+with wrong entries among the right ones and under both tier modes; and the default form on both
+sides of the line between them, in session order and in any other."""
 import numpy as np
 import pytest
 
@@ -72,3 +73,49 @@ def test_forms_agree(tiers, n_sessions, blocks, monkeypatch):
         for w, g in zip(want, got):
             for x, y in zip(w, g):
                 assert np.array_equal(x, y) if isinstance(x, np.ndarray) else x == y
+
+
+@pytest.mark.parametrize("order", ["sessions", "mixed"])
+@pytest.mark.parametrize("n", [2**14 - 1, 2**14, 2**14 + 1, 2**18 + 1, 700_001])
+@pytest.mark.parametrize("S", [1, 16, 700, 4096])
+def test_default_form(S, n, order, tmp_path):
+    """The kernel's per-session counts after a commit of n entries, and the pages it freed."""
+    import torch
+    from paper_2606_22983_gb300 import lv
+    from paper_2606_22983_gb300.pool import KVPool
+    from ._pool_words import pool_words
+    blocks = -(-(n + 3) // S)
+    if blocks > 65536:
+        return
+    N = S * blocks
+    pool = KVPool(layers=1, kv_heads=1, head_dim=8, page_tokens=1, max_sessions=S, max_blocks=blocks, hbm_pages=N,
+                  hbm_budget_pages=N, host_pages=N)
+    try:
+        rng = np.random.default_rng(n + S)
+        table = rng.permutation(N).astype(np.int32).reshape(S, blocks)
+        pool.import_placement(table, np.full(S, blocks, np.int32))
+        pick = rng.permutation(N)[:n] if order == "mixed" else np.arange(n)
+        s, b = pick // blocks, pick % blocks
+        v = torch.from_numpy(np.stack([s, b, table[s, b]], 1).astype(np.int32)).cuda()
+        _, commit = pool.swap_out(v, n)
+        pool.remap(commit, n)
+        assert pool.sync() == 0
+        free = np.sort(table[s, b])
+        table[s, b] = -(np.arange(n) + 2)
+        t, own_hbm, own_host = pool.tables()
+        assert np.array_equal(t, table)
+        assert np.array_equal(np.nonzero(own_hbm == -1)[0], free) and (own_host[:n] == (s << 16 | b)).all()
+        _, _, cnt = pool_words(pool, tmp_path)
+        assert np.array_equal(cnt.cpu().numpy(), np.stack([(t >= 0).sum(1), (t <= -2).sum(1)], 1))
+        # the freed pages, and no others, are there to be taken
+        sid = int(s[0])
+        back = np.nonzero(t[sid] <= -2)[0].astype(np.int32)
+        pages, commit = pool.swap_in(sid, torch.from_numpy(back).cuda(), len(back))
+        assert pool.sync() == 0 and np.array_equal(pages.cpu().numpy(), free[:len(back)])
+        pool.remap(commit, len(back))
+        assert pool.sync() == 0
+        a, d = pool.counts()
+        assert np.array_equal(cnt.cpu().numpy(), np.stack([a, d], 1))
+        assert pool.stats()["hbm_allocated"] == N - n + len(back)
+    finally:
+        pool.close()
