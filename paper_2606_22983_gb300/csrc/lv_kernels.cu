@@ -3043,9 +3043,13 @@ k_counts(DevPool p, int32_t* __restrict__ hbm, int32_t* __restrict__ host) {
 __global__ void __launch_bounds__(kStepThreads)
 k_blocks(DevPool p, int32_t sid, int32_t where, int32_t* out, long long* count) {
   __shared__ int ws[2 * kStepWarps];
+  __shared__ int32_t blocks;
   pdl_entry();
   BlockScan scan{ws, 0};
-  const int32_t nb = nblocks_of(p, sid);
+  // (by one thread: growth on another stream may change it, and it says how many barriers follow)
+  if (threadIdx.x == 0) blocks = nblocks_of(p, sid);
+  __syncthreads();
+  const int32_t nb = blocks;
   const int32_t* row = p.table + (size_t)sid * p.maxB;
   int run = 0;
 #pragma unroll 1

@@ -161,3 +161,27 @@ def test_cancel_on_another_stream(call, large):
                 assert set((-(slots[:R] + 2)).tolist()) == held
     finally:
         pool.close()
+
+
+def test_blocks_while_the_session_grows():
+    """The blocks of a session read on one stream while it grows on another, past several times
+    the reader's threads: those that it had, and any of the new ones."""
+    import torch
+    from paper_2606_22983_gb300 import lv
+    pool = _pool(1, 4096, 4096, 4096, 1)
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    try:
+        pool.import_placement(np.where(np.arange(4096) < 10, np.arange(4096), -1).astype(np.int32)[None], np.array([10], np.int32))
+        pool.sync()
+        torch.cuda.synchronize()
+        blks, count = torch.empty(4096, dtype=torch.int32).cuda(), torch.zeros(1, dtype=torch.int64).cuda()
+        for rnd in range(200):
+            lv.lv_session_append(pool.handle, 0, 20, None, None, a)
+            lv.lv_session_blocks(pool.handle, 0, 0, blks, count, b)
+            torch.cuda.synchronize()
+            had, got = 10 + 20 * rnd, blks[:int(count)].cpu().numpy()
+            assert np.array_equal(got[:had], np.arange(had))       # and any of the twenty new ones
+            assert (np.diff(got) > 0).all() and len(got) <= had + 20 and got[-1] < had + 20
+        assert pool.sync() == 0
+    finally:
+        pool.close()
