@@ -736,11 +736,6 @@ lv_status create_impl(const lv_pool_desc* desc, cudaStream_t s, lv_pool** out) {
       cudaMemsetAsync(d.ctl, 0, lv::C_N * sizeof(long long), s) != cudaSuccess ||
       cudaMemsetAsync(d.page_tag, 0, (size_t)d.hbm_pages * 8, s) != cudaSuccess)
     return fail(LV_ERR_CUDA);
-  // A fifth of the SMs (30 CTAs on GB300) keeps both link directions saturated (338 GB/s,
-  // the same as 50 CTAs or one per SM; 25 CTAs fall to 326) and leaves the rest of the
-  // GPU to the serving work that runs meanwhile: next to a consumer reading resident KV
-  // at HBM speed, 30 CTAs moved 211 GB/s and left it 0.88 of its rate, against 197 GB/s
-  // and 0.835 for 50 CTAs and 167 GB/s and 0.67 for 152.
   // 3/10 of the SMs (45 on GB300): the fewest CTAs that keep both link directions busy
   // alone, and most of the link next to a kernel that reads HBM on every SM
   pool->exchange_ctas = pool->num_sms * 3 / 10 > 0 ? pool->num_sms * 3 / 10 : 1;

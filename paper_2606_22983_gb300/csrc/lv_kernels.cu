@@ -36,13 +36,13 @@ __device__ __forceinline__ void set_error(long long* ctl, int code, long long de
   }
 }
 
-// Programmatic dependent launch.  The kernels of a device-driven step are
-// launched so that each may be scheduled while the previous kernel on the
-// stream still runs (its launch latency overlaps that kernel).  Each of them
-// begins with pdl_entry(): it waits until the previous kernel has completed
-// and its writes are visible -- nothing of the kernel runs earlier -- and then
-// lets the next kernel of the stream be scheduled.  In a kernel launched the
-// ordinary way both instructions have no effect.
+// Programmatic dependent launch.  Most kernels are launched so that each may be
+// scheduled while the previous kernel on the stream still runs (its launch
+// latency overlaps that kernel).  pdl_entry() waits until the previous kernel
+// has completed and its writes are visible, and then lets the next kernel of
+// the stream be scheduled.  Before it a kernel may read only what never changes
+// after the pool's creation (k_exchange_copy: the sub-page arrays' addresses).
+// In a kernel launched the ordinary way both instructions have no effect.
 __device__ __forceinline__ void pdl_entry() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1362,8 +1362,8 @@ k_exchange_copy(DevPool p, const int4* __restrict__ tasks, const long long* __re
 // The staged path moves pages through a contiguous HBM staging run so that the
 // copy engines can carry them over the host link: tasks (the exchange's
 // {out page, out slot, in slot, in page}) are built and validated first, then
-// k_pack_tasks gathers every out page's 2L sub-pages into staging[t] and
-// k_unpack_tasks scatters staging[t] into every in page.  Both kernels move
+// k_stage_tasks<true> gathers every out page's 2L sub-pages into staging[t] and
+// k_stage_tasks<false> scatters staging[t] into every in page.  Both move
 // whole sub-pages with TMA bulk copies (global -> shared -> global), issued by
 // one thread per CTA through a ring of shared-memory stages.
 
@@ -2116,44 +2116,38 @@ __host__ __device__ inline StepLayout step_layout(const DevPool& p, bool ordered
 }
 
 // Bitonic sort of n (a power of two) entries in shared memory: keys descending, or, with an
-// index per key, (key, index) ascending.  Up to 64 entries take one warp.
+// index per key, (key, index) ascending.
 template <bool kIndexed>
 __device__ void sort_entries(unsigned long long* key, int* idx, int n) {
-  const bool one_warp = n <= 64;
-  const int step = one_warp ? 32 : kStepThreads;
-  if (!one_warp || threadIdx.x < 32) {
 #pragma unroll 1
-    for (int k = 2; k <= n; k <<= 1) {
+  for (int k = 2; k <= n; k <<= 1) {
 #pragma unroll 1
-      for (int j = k >> 1; j > 0; j >>= 1) {
+    for (int j = k >> 1; j > 0; j >>= 1) {
 #pragma unroll 1
-        for (int i = threadIdx.x; i < n / 2; i += step) {
-          const int lo = ((i & ~(j - 1)) << 1) | (i & (j - 1)), hi = lo | j;
-          const unsigned long long x = key[lo], y = key[hi];
-          const bool first = (lo & k) == 0;
-          bool less = x < y;                     // lo's entry belongs after hi's in descending order
-          bool more = x > y;
-          if (kIndexed && x == y) {
-            less = idx[lo] < idx[hi];
-            more = idx[lo] > idx[hi];
-          }
-          const bool swap = kIndexed ? (first ? more : less) : (first ? less : more);
-          if (swap) {
-            key[lo] = y;
-            key[hi] = x;
-            if (kIndexed) {
-              const int t = idx[lo];
-              idx[lo] = idx[hi];
-              idx[hi] = t;
-            }
+      for (int i = threadIdx.x; i < n / 2; i += kStepThreads) {
+        const int lo = ((i & ~(j - 1)) << 1) | (i & (j - 1)), hi = lo | j;
+        const unsigned long long x = key[lo], y = key[hi];
+        const bool first = (lo & k) == 0;
+        bool less = x < y;                     // lo's entry belongs after hi's in descending order
+        bool more = x > y;
+        if (kIndexed && x == y) {
+          less = idx[lo] < idx[hi];
+          more = idx[lo] > idx[hi];
+        }
+        const bool swap = kIndexed ? (first ? more : less) : (first ? less : more);
+        if (swap) {
+          key[lo] = y;
+          key[hi] = x;
+          if (kIndexed) {
+            const int t = idx[lo];
+            idx[lo] = idx[hi];
+            idx[hi] = t;
           }
         }
-        if (one_warp) __syncwarp();
-        else __syncthreads();
       }
+      __syncthreads();
     }
   }
-  __syncthreads();
 }
 
 __device__ __forceinline__ unsigned long long warp_max(unsigned long long x) {
@@ -3093,7 +3087,8 @@ cudaError_t launch_session_set(const DevPool& p, const lv_session_state* in, int
 }
 
 // A launch that lets the kernel be scheduled while the previous kernel on `s`
-// still runs; the kernel must begin with pdl_entry() or pdl_wait().
+// still runs; the kernel must call pdl_entry() or pdl_wait() before it reads anything that
+// changes after the pool's creation.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem,
                        cudaStream_t s, Args&&... args) {
