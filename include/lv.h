@@ -44,8 +44,8 @@
  * A device-driven step (lv_turn, lv_make_resident, lv_evict) and
  * lv_swap_exchange must also be ordered with calls that change the table of a
  * session they may take blocks from or load (lv_remap, lv_session_append,
- * another step): where such a call falls between their reads, they report
- * LV_ERR_STATE and move nothing.
+ * another step).  A block that they find elsewhere than expected is
+ * LV_ERR_STATE, and nothing moves.
  *
  * Threads.  A pool keeps host-side state (scratch alternation, pending
  * asynchronous copies, staging runs, timing records): calls on one pool must

@@ -338,7 +338,8 @@ void longest_runs_first(lv_pool* pool, int4* t, int64_t m, int int4::*slot) {
 // GB each way in a row: 281, 288 and 292 GB/s).  An exchange with
 // its ranking, with the task list copied back in two waits and one direction issued first, and
 // now: 5 pages of 16 KiB 68.5 us and 47, 37 of 192 KiB 151 and 126, 25 of 1.5 MiB 358 and 324,
-// 150 of 1.5 MiB 1890 and 1776.
+// 150 of 1.5 MiB 1940 and 1810 (five runs a side 1918 to 1958 and 1803 to 1828; on another box, whose
+// runs differed by up to 12 %, 1940 and 1896).
 lv_status staged_move_inner(lv_pool* pool, int64_t n, bool counted, cudaStream_t s, void** staging_out,
                             bool async) {
   const lv::DevPool& d = pool->d;

@@ -2066,8 +2066,9 @@ __global__ void k_cancel(DevPool p, const int32_t* __restrict__ locs, long long 
 // 24 us of an eviction; as one kernel 17-19 and 12 us; with the session table read in whole
 // lines, the bitmaps changed in shared memory and rare branches out of line 11 us for 16
 // sessions.  Whole turns, when the copy took 16 KiB units already: eight sessions that move 24
-// pages of 16 KiB each way 47 us with the kernels in a row, 22.8 as one, 19.2 now; 1000
-// sessions and 45 pages of 192 KiB in scattered order 106, 81.8 and 75.8.
+// pages of 16 KiB each way 47 us with the kernels in a row, 22.8 as one, 19.3 now; 1000
+// sessions and 45 pages of 192 KiB in scattered order 106, 81.8 and 75.6.  (Of these 0.4 and 0.8 are
+// the count of the bitmaps' bits and the check that the victims fill their list.)
 constexpr int kSelectRounds = 12;   // sessions found by repeated maximum at most
 constexpr int kCountedLoads = 128;  // loads ordered by counting; more are sorted
 
@@ -2339,7 +2340,7 @@ __device__ unsigned long long threshold_key(const DevPool& p, const unsigned lon
 // the first k victims.  Where few sessions should hold k blocks they are found by repeated
 // maximum, one barrier each; else, or when kSelectRounds were not enough, by the threshold
 // key, and the sessions' places by comparing them with one another, or by a sort of more
-// than kCompared.  (4096 sessions, 1500 victims of 7 or 8 sessions: 7.5 us by maximum -- 9.3
+// than kCompared.  (4096 sessions, 1500 victims of 7 or 8 sessions: 7.8 us by maximum -- 9.3
 // when every round read all keys again instead of a thread's two largest -- and 12.6 by the
 // threshold; 256 victims of 128 sessions: 48 us by maximum and a sort of all keys, 13.1 by
 // the threshold.)  Keys are distinct (each holds its session).  A thread may call it with
@@ -2828,7 +2829,7 @@ k_step(DevPool p, StepArgs a) {
 // the sessions chosen, where the census reads every row.  kCensus: no counts are kept for
 // these tables (lv_select_victims_noalloc, many sessions); one CTA takes both from the census.
 // 256 victims of 1024 sessions with 1024 blocks each: 7.1 us as census and emission, 3.9 as
-// one kernel; 1500 of 4096 sessions with 256 blocks: 20.7 and 7.5 us.
+// one kernel; 1500 of 4096 sessions with 256 blocks: 20.9 and 7.8 us.
 // More victims, or victims of some hundred sessions, are written by many CTAs: 4096 victims
 // of 1024 sessions take 11.8 us here and 9.2 there, 2048 of at least 1024 sessions with two
 // blocks each 32 and 9.2, 256 of 128 such sessions 10.1 and 9.2 (13.1 and 14.9 with 4096
