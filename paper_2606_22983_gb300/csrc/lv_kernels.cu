@@ -720,7 +720,9 @@ struct TierBits {
 };
 
 // Reads a bitmap of W words into shared memory at `copy` (2 W words; null: used in place).
-__device__ __forceinline__ TierBits bits_copy(uint32_t* gl, long long nbits, uint32_t* copy) {
+// me: the thread's place in a permutation of the CTA's threads, of which the first copy the
+// first words.
+__device__ __forceinline__ TierBits bits_copy(uint32_t* gl, long long nbits, uint32_t* copy, int me) {
   const int W = (int)((nbits + 31) >> 5);
   TierBits t{gl, gl, gl, nbits, 0};
   if (LV_RARE(!copy)) {
@@ -731,7 +733,7 @@ __device__ __forceinline__ TierBits bits_copy(uint32_t* gl, long long nbits, uin
   t.cur = copy;
   t.old = copy + W;
 #pragma unroll 1
-  for (int w = threadIdx.x; w < W; w += kStepThreads) {
+  for (int w = me; w < W; w += kStepThreads) {
     const uint32_t x = gl[w];
     copy[w] = copy[W + w] = x;
     t.taken += __popc(x);
@@ -868,7 +870,8 @@ k_alloc(DevPool p, bool in_hbm, const lv_victim* v, long long n, int32_t* out, b
   pdl_entry();
   BlockScan scan{ws, 0};
   uint32_t* copy = copy_bits ? reinterpret_cast<uint32_t*>(dyn) : nullptr;
-  const TierBits t = in_hbm ? bits_copy(p.bits_hbm, p.hbm_pages, copy) : bits_copy(p.bits_host, p.host_pages, copy);
+  const TierBits t = in_hbm ? bits_copy(p.bits_hbm, p.hbm_pages, copy, threadIdx.x)
+                            : bits_copy(p.bits_host, p.host_pages, copy, threadIdx.x);
   int nd = (int)n;
   if (LV_RARE(v != nullptr)) {
     int cnt = 0;
@@ -1189,8 +1192,9 @@ k_exchange_plan(DevPool p, const lv_victim* __restrict__ v, long long n_out, int
   pdl_entry();
   BlockScan scan{sh.ws, 0};
   uint32_t* copy = copy_bits ? reinterpret_cast<uint32_t*>(dyn) : nullptr;
-  const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, copy);
-  const TierBits host = bits_copy(p.bits_host, p.host_pages, copy ? copy + 2 * ((p.hbm_pages + 31) >> 5) : nullptr);
+  const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, copy, threadIdx.x);
+  const TierBits host = bits_copy(p.bits_host, p.host_pages, copy ? copy + 2 * ((p.hbm_pages + 31) >> 5) : nullptr,
+                                  threadIdx.x);
   if (threadIdx.x == 0 && cursor) *cursor = 0;
   int hbm_alloc;
   scan.sum(hbm.taken, &hbm_alloc);
@@ -1264,8 +1268,9 @@ k_append(DevPool p, int32_t sid, int32_t n_tokens, int32_t* pages, int32_t* coun
   __shared__ int base[kStepThreads];
   pdl_entry();
   BlockScan scan{ws, 0};
-  const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, copy_bits ? reinterpret_cast<uint32_t*>(dyn) : nullptr);
-  const TierBits host = bits_copy(p.bits_host, p.host_pages, nullptr);      // one bit of it at most
+  const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, copy_bits ? reinterpret_cast<uint32_t*>(dyn) : nullptr,
+                                 threadIdx.x);
+  const TierBits host = bits_copy(p.bits_host, p.host_pages, nullptr, 0);   // one bit of it at most
   const int32_t ctx = p.sess[sid].ctx_tokens;
   __syncthreads();      // every thread has read it and the bitmap
   const long long m = append_tokens_to(p, sid, ctx, n_tokens, pages, hbm, host, near, scan, base);
@@ -2066,9 +2071,8 @@ __global__ void k_cancel(DevPool p, const int32_t* __restrict__ locs, long long 
 // 24 us of an eviction; as one kernel 17-19 and 12 us; with the session table read in whole
 // lines, the bitmaps changed in shared memory and rare branches out of line 11 us for 16
 // sessions.  Whole turns, when the copy took 16 KiB units already: eight sessions that move 24
-// pages of 16 KiB each way 47 us with the kernels in a row, 22.8 as one, 19.3 now; 1000
-// sessions and 45 pages of 192 KiB in scattered order 106, 81.8 and 75.6.  (Of these 0.4 and 0.8 are
-// the count of the bitmaps' bits and the check that the victims fill their list.)
+// pages of 16 KiB each way 47 us with the kernels in a row, 22.8 as one, 19.1 now; 1000
+// sessions and 45 pages of 192 KiB in scattered order 106, 81.8 and 75.9.
 constexpr int kSelectRounds = 12;   // sessions found by repeated maximum at most
 constexpr int kCountedLoads = 128;  // loads ordered by counting; more are sorted
 
@@ -2517,8 +2521,11 @@ k_step(DevPool p, StepArgs a) {
   int32_t first_cand = -1;
   if (picks && tid < a.n_cand) first_cand = a.cand[tid];
   uint32_t* copy = a.copy_bits && a.part != kStepList ? reinterpret_cast<uint32_t*>(dyn + lay.bits) : nullptr;
-  const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, copy);
-  const TierBits host = bits_copy(p.bits_host, p.host_pages, copy ? copy + 2 * ((p.hbm_pages + 31) >> 5) : nullptr);
+  // (the few words of a small pool by warps that have no states to read, each tier's by others:
+  // eight sessions 19.1 us a turn so, 19.4 when the first warp reads all three one after the other)
+  const TierBits hbm = bits_copy(p.bits_hbm, p.hbm_pages, copy, kStepThreads - 1 - tid);
+  const TierBits host = bits_copy(p.bits_host, p.host_pages, copy ? copy + 2 * ((p.hbm_pages + 31) >> 5) : nullptr,
+                                  tid ^ (kStepThreads / 2));
   const bool fallback = !evict && !a.preload;
 #pragma unroll 1
   for (int s0 = tid & ~31; s0 < p.S; s0 += kStepThreads) {      // 32 sessions of a warp
