@@ -2199,8 +2199,8 @@ struct VictimList {
   lv_victim* far;
   const uint32_t* own;      // null: not checked
   long long n_own;
-  long long n_out;          // positions below this are written
-  __device__ void put(long long pos, int32_t s, int32_t b, int32_t e) const {
+  int n_out;          // positions below this are written
+  __device__ void put(int pos, int32_t s, int32_t b, int32_t e) const {
     if (near) near[pos] = lv_victim{s, b, e};
     far[pos] = lv_victim{s, b, e};
   }
@@ -2211,7 +2211,7 @@ struct VictimList {
 // every position has to be filled: a row that holds fewer blocks than were counted (a commit
 // on another stream between the two) is a wrong victim, of one that holds more the first are
 // taken.
-__device__ void emit_whole(const DevPool& p, int32_t s, int32_t nb, long long pos0, long long end,
+__device__ void emit_whole(const DevPool& p, int32_t s, int32_t nb, int pos0, int end,
                            const VictimList& l, OwnerCheck& check, BlockScan& scan) {
   const int32_t* row = p.table + (size_t)s * p.maxB;
   const bool suffix = p.within == LV_SUFFIX_FIRST;
@@ -2222,7 +2222,7 @@ __device__ void emit_whole(const DevPool& p, int32_t s, int32_t nb, long long po
     const int32_t e = q < nb ? row[b] : -1;
     check.read(l.own, e, l.n_own);
     int chunk;
-    const long long pos = pos0 + scan.rank(e >= 0, &chunk);
+    const int pos = pos0 + scan.rank(e >= 0, &chunk);
     if (e >= 0 && pos < end) {
       l.put(pos, s, b, e);
       if (l.own) check.expect(owner_key(s, b), pos);
@@ -2259,15 +2259,15 @@ __device__ void emit_warp(const DevPool& p, const int* nblk, const int* cnt, int
       const int2 so = of(r);
       const int32_t s = so.x, nb = nblk[s];
       const int32_t* row = p.table + (size_t)s * p.maxB;
-      long long pos0 = so.y;
-      const long long end = pos0 + cnt[s] < l.n_out ? pos0 + cnt[s] : l.n_out;
+      int pos0 = so.y;
+      const int end = min(pos0 + cnt[s], l.n_out);
       int32_t x = e[u];
 #pragma unroll 1
       for (int32_t q0 = 0;; ) {
         const int32_t q = q0 + lane;
         check.read(l.own, x, l.n_own);
         const unsigned has = __ballot_sync(0xffffffffu, x >= 0);
-        const long long pos = pos0 + __popc(has & ((1u << lane) - 1u));
+        const int pos = pos0 + __popc(has & ((1u << lane) - 1u));
         if (x >= 0 && pos < end) {
           const int32_t b = suffix ? nb - 1 - q : q;
           l.put(pos, s, b, x);
@@ -2463,8 +2463,8 @@ __device__ void emit_selected(const DevPool& p, const Selected& sel, const unsig
 #pragma unroll 1
     for (int r = 0; r < sel.m; ++r) {
       const int32_t s = sh.sel_sid[r];
-      const long long at = sh.sel_off[r];
-      emit_whole(p, s, nblk[s], at, at + cnt[s] < l.n_out ? at + cnt[s] : l.n_out, l, check, scan);
+      const int at = sh.sel_off[r];
+      emit_whole(p, s, nblk[s], at, min(at + cnt[s], l.n_out), l, check, scan);
     }
   } else if (sel.sorted) {
     emit_warp(p, nblk, cnt, sel.m, l, check, [&](int r) { return make_int2(session_of_key(keys[r]), off[r]); });
@@ -2743,7 +2743,7 @@ k_step(DevPool p, StepArgs a) {
   }
   // the victims of the order's first n_out positions
   lv_victim* near = sel.n_out <= kStepItems ? sh.l.v : nullptr;
-  const VictimList list{near, a.rs.victims, p.own_hbm, p.hbm_pages, sel.n_out};
+  const VictimList list{near, a.rs.victims, p.own_hbm, p.hbm_pages, (int)sel.n_out};
   emit_selected(p, sel, keys, off, nblk, cnt, list, out_check, sh, scan);
   // the gate: a shortfall stops the step (a preload is skipped, a foreground turn fails);
   // lv_evict takes what there is
@@ -2907,7 +2907,7 @@ k_select(DevPool p, long long now_us, long long k, bool fallback, long long* cou
   }
   const Selected sel = select_sessions(p, keys, off, cnt, k, -1, sh, scan);
   OwnerCheck check{0, 0, -1, -1};
-  const VictimList list{nullptr, out, nullptr, 0, sel.n_out};
+  const VictimList list{nullptr, out, nullptr, 0, (int)sel.n_out};
   emit_selected(p, sel, keys, off, nblk, cnt, list, check, sh, scan);
   if (tid == 0) {
     p.ctl[C_SEL_COUNT] = sel.n_out;
