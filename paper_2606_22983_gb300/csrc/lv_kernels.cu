@@ -2072,7 +2072,7 @@ __global__ void k_cancel(DevPool p, const int32_t* __restrict__ locs, long long 
 // lines, the bitmaps changed in shared memory and rare branches out of line 11 us for 16
 // sessions.  Whole turns, when the copy took 16 KiB units already: eight sessions that move 24
 // pages of 16 KiB each way 47 us with the kernels in a row, 22.8 as one, 19.1 now; 1000
-// sessions and 45 pages of 192 KiB in scattered order 106, 81.8 and 75.9.
+// sessions and 45 pages of 192 KiB in scattered order 106, 81.8 and 75.2.
 constexpr int kSelectRounds = 12;   // sessions found by repeated maximum at most
 constexpr int kCountedLoads = 128;  // loads ordered by counting; more are sorted
 
@@ -2836,7 +2836,7 @@ k_step(DevPool p, StepArgs a) {
 // the sessions chosen, where the census reads every row.  kCensus: no counts are kept for
 // these tables (lv_select_victims_noalloc, many sessions); one CTA takes both from the census.
 // 256 victims of 1024 sessions with 1024 blocks each: 7.1 us as census and emission, 3.9 as
-// one kernel; 1500 of 4096 sessions with 256 blocks: 20.9 and 7.8 us.
+// one kernel; 1500 of 4096 sessions with 256 blocks: 20.7 and 7.8 us.
 // More victims, or victims of some hundred sessions, are written by many CTAs: 4096 victims
 // of 1024 sessions take 11.8 us here and 9.2 there, 2048 of at least 1024 sessions with two
 // blocks each 32 and 9.2, 256 of 128 such sessions 10.1 and 9.2 (13.1 and 14.9 with 4096
